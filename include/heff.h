@@ -61,7 +61,7 @@ extern "C" {
 #define HEFF_ERR_WORKSPACE -7       /* workspace too small or misaligned (256 B)     */
 
 /* ---- precisions and element types ----------------------------------------- */
-#define HEFF_PREC_FP64 0   /* FP64 CUDA-core block GEMMs (reference GPU path)        */
+#define HEFF_PREC_FP64 0   /* FP64 accuracy: 62-bit fixed-point digits, exact sums      */
 #define HEFF_PREC_BF16X3 1 /* tcgen05 BF16 hi/lo split, 3 products, FP32 accumulate   */
 #define HEFF_PREC_TF32X3 2 /* tcgen05 TF32 hi/lo split, 3 products, FP32 accumulate   */
 
@@ -312,7 +312,7 @@ int heff_davidson(heff_plan* plan, const void* L, const void* W1, const void* W2
 
 /*
  * Environment extension (Section II-C: the left environment A and right environment B
- * are grown one site at a time as the sweep moves).  FP64 block products on the GPU.
+ * are grown one site at a time as the sweep moves).
  *   side 0 (left):  Lnew[c,v,d] = sum A[a,t,c] L[a,w,b] W[w,t,s,v] A[b,s,d]
  *   side 1 (right): Rnew[c,w,d] = sum B[c,t,a] R[a,v,b] W[w,t,s,v] B[d,s,b]
  * Layouts: site (a, s, b) flows (+1, +1, -1); W (w, t, s, v) flows (+1, +1, -1, -1);
@@ -334,7 +334,7 @@ void heff_env_plan_destroy(heff_env_plan* plan);
 
 /*
  * Arithmetic of the environment update's block products.  HEFF_PREC_FP64 (the default):
- * FP64 on the CUDA cores.  HEFF_PREC_BF16X3: on the tensor cores, each operand element split
+ * FP64 accuracy, from fixed-point digits.  HEFF_PREC_BF16X3: on the tensor cores, each operand element split
  * into bf16 hi + lo and three products per K block, FP32 accumulation (about 1e-5 relative
  * per product); the tensors stay FP64 buffers (the update converts env_old and the site
  * tensor to FP32 copies in the workspace, whose size covers both precisions) and the call
@@ -346,7 +346,7 @@ int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precision);
 /*
  * Read and clear the sticky error flag of an environment-update workspace: HEFF_ERR_TIMEOUT
  * when a bounded wait of a tensor-core product expired in the last update (its output is
- * then incomplete; the context stays usable), else HEFF_OK (always for FP64 plans).
+ * then incomplete; the context stays usable), else HEFF_OK.
  * Synchronises `stream`.  Errors: INVALID_ARG, WORKSPACE, CUDA.
  */
 int heff_env_status(const heff_env_plan* plan, void* workspace, size_t workspace_bytes, void* stream);
@@ -400,8 +400,8 @@ int heff_backward(heff_grad_plan* g, heff_plan* plan, const double* L, const dou
 void heff_grad_plan_destroy(heff_grad_plan* g);
 
 /*
- * Arithmetic of the gradients' block products (U, T1, dL, dR): HEFF_PREC_FP64 (the default,
- * CUDA cores) or HEFF_PREC_BF16X3 (tensor cores, bf16 hi/lo split, FP32-accumulated; about
+ * Arithmetic of the gradients' block products (U, T1, dL, dR): HEFF_PREC_FP64 (the default)
+ * or HEFF_PREC_BF16X3 (tensor cores, bf16 hi/lo split, FP32-accumulated; about
  * 1e-5 relative).  The scalars, dx and the W gradients' reductions stay FP64; buffers stay
  * FP64.  With HEFF_PREC_BF16X3 the workspace also holds FP32 copies of x, L and R (the
  * products' operands, converted once per call) and the intermediates in FP32, so
@@ -539,7 +539,7 @@ int heff_plan_timings(heff_plan* plan, float* ms);
  * tensor memory and returns, so its outputs are incomplete but the context stays usable.
  * A GEMM launch clears the flag when the workspace is not one of the last two the plan
  * used.  Synchronises `stream`.  Returns HEFF_ERR_TIMEOUT if the flag was set (and clears
- * it), else HEFF_OK; always HEFF_OK for FP64 plans, whose kernels do not wait.
+ * it), else HEFF_OK (also, for an FP64 plan, when no apply has run in this workspace).
  * workspace: device, at least heff_plan_workspace_size bytes.  Errors: INVALID_ARG,
  * WORKSPACE (too small), CUDA.
  */

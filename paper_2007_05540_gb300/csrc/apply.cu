@@ -1,11 +1,11 @@
-// Packing, operator preparation, the FP64 CUDA-core block GEMMs, and the C-ABI compute
-// entry points of the two-site H_eff matvec (Section II-C / Fig. 1d).
+// Packing, operator preparation, and the C-ABI compute entry points of the two-site H_eff
+// matvec (Section II-C / Fig. 1d).
 //
 // One apply is four launches on the caller's stream:
 //   mix_kernel   LW = L.W1 and RW = W2.R into the workspace (operator preparation)
 //   pack_kernel  x -> XT (per charge sector, transposed so the contraction index is
 //                contiguous; hi/lo split for the tensor-core precisions)
-//   GEMM 1       T = LW . XT^T              (tensor cores: tc_gemm.cu; FP64: below)
+//   GEMM 1       T = LW . XT^T              (split precisions: tc_gemm.cu; FP64: fx_gemm.cu)
 //   GEMM 2       y = T . RW^T               (written straight into y's block layout)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "convert.cuh"
+#include "fixed.cuh"
 #include "internal.h"
 
 using heff::fail;
@@ -89,7 +90,8 @@ constexpr int PACK_WARPS = 4;
 template <typename In, int PREC>
 __global__ void __launch_bounds__(32 * PACK_WARPS) pack_kernel(const PackTile* __restrict__ tiles, int ntiles,
                                                                PtrBatch xs, char* __restrict__ xt, int64_t ld,
-                                                               int64_t batch_elems) {
+                                                               int64_t batch_elems, uint16_t* __restrict__ codes,
+                                                               int64_t code_rows, int64_t batch_rows) {
     using E = typename Plane<PREC>::T;
     constexpr bool SPLIT = PREC != HEFF_PREC_FP64;
     constexpr int KB = 64 / (int)sizeof(E);          // elements per K block of one half
@@ -114,6 +116,16 @@ __global__ void __launch_bounds__(32 * PACK_WARPS) pack_kernel(const PackTile* _
             sw[r][lane] = (bv && r < na) ? to_acc<Acc>(x[(int64_t)(t.a0 + r) * t.m_b + b]) : (Acc)0;
     }
     __syncwarp();
+    if constexpr (!SPLIT) {
+        // exponent codes of the tile's XT rows (lane = row) over these 32 columns
+        if (codes && t.b0 + lane < t.m_b) {
+            int e = 0;
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+                e = max(e, fx::exp_code((uint32_t)__double2hiint(sw[r][lane]), (uint32_t)__double2loint(sw[r][lane])));
+            codes[(t.xt_col0 + t.a0) / KPAD * code_rows + bz * batch_rows + t.xt_row0 + t.b0 + lane] = (uint16_t)e;
+        }
+    }
     E* base = reinterpret_cast<E*>(xt) + (int64_t)bz * batch_elems;
     const int c = 2 * (lane & 15), h = lane >> 4;
     const int nb = t.m_b - t.b0;                    // XT rows of this tile
@@ -145,6 +157,8 @@ struct MixArgs {
     const void *L, *W1, *W2, *R;
     char* lw; int64_t ld_lw;
     char* rw; int64_t ld_rw;
+    uint16_t *elw, *erw;        // FP64: exponent codes [column / KPAD][row], or null
+    int64_t rows_lw, rows_rw;
 };
 
 template <typename In, int PREC>
@@ -192,6 +206,9 @@ __device__ __forceinline__ void mix_tile(const MixTile& t, const MixArgs& a) {
             rv[i] = rr + i < t.nrows;
             rc[i] = (int64_t)(t.r0 + rr + i) * t.cols;
         }
+        // both half warps run the column loop to the same end: their lanes cover one 32-column
+        // block each (cols_pad is a multiple of 32, not of 64)
+        const unsigned half_mask = 0xffffu << (lane & 16);
         for (int cb = 2 * lane; cb < t.cols_pad; cb += 64 * U) {
             Acc a0[RW][U], a1[RW][U];
 #pragma unroll
@@ -233,6 +250,19 @@ __device__ __forceinline__ void mix_tile(const MixTile& t, const MixArgs& a) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int c = cb + 64 * u;
+                    if (!SPLIT && (t.which ? a.erw : a.elw)) {
+                        // the largest code of a 32-column block: 16 lanes (a block is all inside
+                        // or all outside the padded columns)
+                        int e = 0;
+                        if constexpr (!SPLIT) {
+                            e = max(fx::exp_code((uint32_t)__double2hiint(a0[i][u]), (uint32_t)__double2loint(a0[i][u])),
+                                    fx::exp_code((uint32_t)__double2hiint(a1[i][u]), (uint32_t)__double2loint(a1[i][u])));
+                        }
+                        for (int o = 1; o < 16; o <<= 1) e = max(e, __shfl_xor_sync(half_mask, e, o));
+                        if ((lane & 15) == 0 && c < t.cols_pad)
+                            (t.which ? a.erw : a.elw)[(t.dst_col0 + c) / KPAD * (t.which ? a.rows_rw : a.rows_lw) +
+                                                      t.dst_row0 + t.r0 + rr + i] = (uint16_t)e;
+                    }
                     if (c >= t.cols_pad) break;
                     E h0, l0, h1, l1;
                     Plane<PREC>::split(a0[i][u], h0, l0);
@@ -254,64 +284,6 @@ template <typename In, int PREC>
 __global__ void __launch_bounds__(256, HEFF_MIX_MINB) mix_kernel(MixArgs a) {
     pdl_trigger();                                  // the pack kernel may be scheduled behind it
     mix_tile<In, PREC>(a.tiles[blockIdx.x], a);
-}
-
-// ------------------------------------------------------------------ FP64 CUDA-core GEMM
-// C[m x n] = sum_seg A[a_row + r, k] B[b_row + c, k] over 64 x 64 tiles, 4 x 4 per thread.
-struct GemmArgs {
-    const GemmTask* tasks;
-    const KSeg* segs;
-    int ntasks;
-    const char* A; int64_t a_batch_rows;    // operand arrays and their per-batch row offsets
-    const char* B; int64_t b_batch_rows;
-    int64_t ld;                             // shared row pitch of A and B
-    char* C; int64_t c_batch_elems;         // GEMM 1 output (T) and per-batch offset
-    PtrBatch y;                             // GEMM 2 outputs (one per batch entry)
-    int mode;                               // 0: write T (operand type), 1: write y (io type)
-};
-
-__global__ void __launch_bounds__(256) gemm_fp64_kernel(GemmArgs g) {
-    __shared__ double As[16][64 + 1];
-    __shared__ double Bs[16][64 + 1];
-    const GemmTask t = g.tasks[blockIdx.x];
-    const int bz = blockIdx.y;
-    const double* A = reinterpret_cast<const double*>(g.A) + (int64_t)bz * g.a_batch_rows * g.ld;
-    const double* B = reinterpret_cast<const double*>(g.B) + (int64_t)bz * g.b_batch_rows * g.ld;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    double acc[4][4] = {};
-    for (int s = 0; s < t.seg_count; ++s) {
-        const KSeg sg = g.segs[t.seg_begin + s];
-        for (int k0 = sg.k0; k0 < sg.k0 + sg.klen; k0 += 16) {
-            for (int l = 0; l < 4; ++l) {
-                int idx = tid + 256 * l, row = idx >> 4, kk = idx & 15;
-                As[kk][row] = row < t.m ? A[(t.a_row + row) * g.ld + k0 + kk] : 0.0;
-                Bs[kk][row] = row < t.n ? B[(t.b_row + row) * g.ld + k0 + kk] : 0.0;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < 16; ++kk) {
-                double a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty * 4 + i]; b[i] = Bs[kk][tx * 4 + i]; }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-    }
-    double* C = g.mode == 0 ? reinterpret_cast<double*>(g.C) + (int64_t)bz * g.c_batch_elems
-                            : static_cast<double*>(const_cast<void*>(g.y.p[bz]));
-    for (int i = 0; i < 4; ++i) {
-        int r = ty * 4 + i;
-        if (r >= t.m) continue;
-        for (int j = 0; j < 4; ++j) {
-            int c = tx * 4 + j;
-            if (c < t.n) C[t.c_off + (int64_t)r * t.ldc + c] = acc[i][j];
-            else if (c < t.n + t.n_zero) C[t.c_off + (int64_t)r * t.ldc + c] = 0.0;
-        }
-    }
 }
 
 // ------------------------------------------------------------------ host side
@@ -343,7 +315,8 @@ int plan_upload(heff_plan* p) {
     if ((rc = upload(p->pack, &p->d_pack)) != HEFF_OK) return rc;
     if ((rc = upload(p->mix, &p->d_mix)) != HEFF_OK) return rc;
     if ((rc = upload(p->terms, &p->d_terms)) != HEFF_OK) return rc;
-    for (GemmList* g : {&p->g1, &p->g2, &p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair}) {
+    for (GemmList* g : {&p->g1, &p->g2, &p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->fx1, &p->fx2}) {
+        if (p->opts.precision == HEFF_PREC_FP64 && (g == &p->g1 || g == &p->g2)) continue;   // fx1, fx2 run
         if ((rc = upload(g->tasks, &g->d_tasks)) != HEFF_OK) return rc;
         if ((rc = upload(g->segs, &g->d_segs)) != HEFF_OK) return rc;
     }
@@ -366,7 +339,7 @@ void plan_free_device(heff_plan* p) {
     p->d_w1_zero = p->d_w2_zero = nullptr;
     p->d_wcount = nullptr;
     cudaFree(p->g1.d_tasks); cudaFree(p->g1.d_segs); cudaFree(p->g2.d_tasks); cudaFree(p->g2.d_segs);
-    for (GemmList* g : {&p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair}) {
+    for (GemmList* g : {&p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->fx1, &p->fx2}) {
         cudaFree(g->d_tasks); cudaFree(g->d_segs);
         g->d_tasks = nullptr; g->d_segs = nullptr;
     }
@@ -376,7 +349,7 @@ void plan_free_device(heff_plan* p) {
 
 
 template <typename In, int PREC>
-static void launch_pack_t(heff_plan* p, const PtrBatch& xs, int nb, char* ws, cudaStream_t st) {
+static void launch_pack_t(heff_plan* p, const PtrBatch& xs, int nb, char* ws, uint16_t* codes, cudaStream_t st) {
     const int nt = (int)p->pack.size();
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
@@ -388,10 +361,11 @@ static void launch_pack_t(heff_plan* p, const PtrBatch& xs, int nb, char* ws, cu
     cfg.attrs = at;
     cfg.numAttrs = HEFF_PDL ? 1 : 0;
     cudaLaunchKernelEx(&cfg, pack_kernel<In, PREC>, static_cast<const PackTile*>(p->d_pack), nt, xs,
-                       ws + p->off_xt, p->ld_x, (int64_t)p->planes * p->rows_x * p->ld_x);
+                       ws + p->off_xt, p->ld_x, (int64_t)p->planes * p->rows_x * p->ld_x, codes,
+                       p->opts.max_batch * p->rows_x, p->rows_x);
 }
 
-int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, void* stream) {
+int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, bool codes, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (p->pack.empty()) return HEFF_OK;
     for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
@@ -400,15 +374,17 @@ int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, 
         for (int b = 0; b < nb; ++b) xs.p[b] = x[b0 + b];
         char* w = static_cast<char*>(ws) + (size_t)b0 * p->rows_x * p->ld_x * p->esize * p->planes;
         const bool f32 = p->opts.io_dtype == HEFF_DTYPE_F32;
+        uint16_t* e = codes ? reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + p->off_ex) + (int64_t)b0 * p->rows_x
+                            : nullptr;
         switch (p->opts.precision) {
-            case HEFF_PREC_FP64: launch_pack_t<double, HEFF_PREC_FP64>(p, xs, nb, w, st); break;
+            case HEFF_PREC_FP64: launch_pack_t<double, HEFF_PREC_FP64>(p, xs, nb, w, e, st); break;
             case HEFF_PREC_BF16X3:
-                if (f32) launch_pack_t<float, HEFF_PREC_BF16X3>(p, xs, nb, w, st);
-                else launch_pack_t<double, HEFF_PREC_BF16X3>(p, xs, nb, w, st);
+                if (f32) launch_pack_t<float, HEFF_PREC_BF16X3>(p, xs, nb, w, nullptr, st);
+                else launch_pack_t<double, HEFF_PREC_BF16X3>(p, xs, nb, w, nullptr, st);
                 break;
             default:
-                if (f32) launch_pack_t<float, HEFF_PREC_TF32X3>(p, xs, nb, w, st);
-                else launch_pack_t<double, HEFF_PREC_TF32X3>(p, xs, nb, w, st);
+                if (f32) launch_pack_t<float, HEFF_PREC_TF32X3>(p, xs, nb, w, nullptr, st);
+                else launch_pack_t<double, HEFF_PREC_TF32X3>(p, xs, nb, w, nullptr, st);
         }
         count_launches(1);
     }
@@ -416,24 +392,27 @@ int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, 
     return HEFF_OK;
 }
 
-static MixArgs mix_args(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, char* ws) {
-    return MixArgs{p->d_mix, p->d_terms, L, W1, W2, R, ws + p->off_lw, p->ld_x, ws + p->off_rw, p->ld_t};
+static MixArgs mix_args(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, char* ws,
+                        bool codes) {
+    return MixArgs{p->d_mix, p->d_terms, L, W1, W2, R, ws + p->off_lw, p->ld_x, ws + p->off_rw, p->ld_t,
+                   codes ? reinterpret_cast<uint16_t*>(ws + p->off_elw) : nullptr,
+                   codes ? reinterpret_cast<uint16_t*>(ws + p->off_erw) : nullptr, p->rows_lw, p->rows_rw};
 }
 
 template <typename In, int PREC>
 static void launch_mix_t(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R,
-                         char* ws, cudaStream_t st) {
-    mix_kernel<In, PREC><<<(unsigned)p->mix.size(), 256, 0, st>>>(mix_args(p, L, W1, W2, R, ws));
+                         char* ws, cudaStream_t st, bool codes = false) {
+    mix_kernel<In, PREC><<<(unsigned)p->mix.size(), 256, 0, st>>>(mix_args(p, L, W1, W2, R, ws, codes));
 }
 
 int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, void* ws,
-               void* stream) {
+               bool codes, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (p->mix.empty()) return HEFF_OK;
     char* w = static_cast<char*>(ws);
     const bool f32 = p->opts.io_dtype == HEFF_DTYPE_F32;
     switch (p->opts.precision) {
-        case HEFF_PREC_FP64: launch_mix_t<double, HEFF_PREC_FP64>(p, L, W1, W2, R, w, st); break;
+        case HEFF_PREC_FP64: launch_mix_t<double, HEFF_PREC_FP64>(p, L, W1, W2, R, w, st, codes); break;
         case HEFF_PREC_BF16X3:
             if (f32) launch_mix_t<float, HEFF_PREC_BF16X3>(p, L, W1, W2, R, w, st);
             else launch_mix_t<double, HEFF_PREC_BF16X3>(p, L, W1, W2, R, w, st);
@@ -449,37 +428,9 @@ int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, cons
 
 int launch_tc_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
 
-int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream) {
-    if (p->opts.precision != HEFF_PREC_FP64) return launch_tc_gemm(p, which, ws, y, nbatch, stream);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const GemmList& gl = which == 1 ? p->g1 : p->g2;
-    if (gl.tasks.empty()) return HEFF_OK;
-    char* w = static_cast<char*>(ws);
-    for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
-        int nb = nbatch - b0 < MAXB ? nbatch - b0 : MAXB;
-        GemmArgs g{};
-        g.tasks = gl.d_tasks;
-        g.segs = gl.d_segs;
-        g.ntasks = (int)gl.tasks.size();
-        if (which == 1) {
-            g.A = w + p->off_lw; g.a_batch_rows = 0;
-            g.B = w + p->off_xt + (size_t)b0 * p->rows_x * p->ld_x * 8; g.b_batch_rows = p->rows_x;
-            g.ld = p->ld_x;
-            g.C = w + p->off_t + (size_t)b0 * p->rows_t * p->ld_t * 8; g.c_batch_elems = p->rows_t * p->ld_t;
-            g.mode = 0;
-        } else {
-            g.A = w + p->off_t + (size_t)b0 * p->rows_t * p->ld_t * 8; g.a_batch_rows = p->rows_t;
-            g.B = w + p->off_rw; g.b_batch_rows = 0;
-            g.ld = p->ld_t;
-            for (int b = 0; b < nb; ++b) g.y.p[b] = y[b0 + b];
-            g.mode = 1;
-        }
-        dim3 grid((unsigned)gl.tasks.size(), nb);
-        gemm_fp64_kernel<<<grid, 256, 0, st>>>(g);
-        count_launches(1);
-    }
-    CK(cudaGetLastError());
-    return HEFF_OK;
+int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream) {
+    return p->opts.precision == HEFF_PREC_FP64 ? launch_fx_matvec(p, which, ws, y, nbatch, codes, stream)
+                                               : launch_tc_gemm(p, which, ws, y, nbatch, stream);
 }
 
 }  // namespace heff
@@ -506,36 +457,54 @@ static int check_ws(const heff_plan* p, void* ws, size_t bytes) {
     return HEFF_OK;
 }
 
+// FP64 plans: the sticky error flag of a workspace new to the plan starts at zero (caller memory,
+// contents unknown); the split precisions do this when they encode the workspace's tensor maps
+static int fresh_workspace(heff_plan* p, void* ws, void* stream) {
+    if (p->opts.precision != HEFF_PREC_FP64 || p->tmap_ws[0] == ws || p->tmap_ws[1] == ws) return HEFF_OK;
+    CK(cudaMemsetAsync(static_cast<char*>(ws) + p->off_flags, 0, sizeof(int), static_cast<cudaStream_t>(stream)));
+    p->tmap_ws[p->tmap_next] = ws;
+    p->tmap_next ^= 1;
+    return HEFF_OK;
+}
+
 static int do_prepare(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
-                      void* workspace, void* stream) {
+                      void* workspace, bool codes, void* stream) {
     heff::record_phase(plan, 0, stream);
-    int rc = heff::launch_mix(plan, L, W1, W2, R, workspace, stream);
+    int rc = heff::launch_mix(plan, L, W1, W2, R, workspace, codes, stream);
     heff::record_phase(plan, 1, stream);
     return rc;
 }
 
-static int do_gemms(heff_plan* plan, void* const* y, int nbatch, void* workspace, void* stream) {
+static int do_gemms(heff_plan* plan, void* const* y, int nbatch, void* workspace, bool codes, void* stream) {
     int rc;
-    if ((rc = heff::launch_gemm(plan, 1, workspace, y, nbatch, stream))) return rc;
+    if ((rc = heff::launch_gemm(plan, 1, workspace, y, nbatch, codes, stream))) return rc;
     heff::record_phase(plan, 3, stream);
-    if ((rc = heff::launch_gemm(plan, 2, workspace, y, nbatch, stream))) return rc;
+    if ((rc = heff::launch_gemm(plan, 2, workspace, y, nbatch, codes, stream))) return rc;
     heff::record_phase(plan, 4, stream);
     return HEFF_OK;
 }
 
 static int do_matvec(heff_plan* plan, const void* const* x, void* const* y, int nbatch, void* workspace,
-                     void* stream) {
+                     bool codes, void* stream) {
     int rc;
-    if ((rc = heff::launch_pack_batch(plan, x, nbatch, workspace, stream))) return rc;
+    if ((rc = fresh_workspace(plan, workspace, stream))) return rc;
+    if ((rc = heff::launch_pack_batch(plan, x, nbatch, workspace, codes, stream))) return rc;
     heff::record_phase(plan, 2, stream);
-    return do_gemms(plan, y, nbatch, workspace, stream);
+    return do_gemms(plan, y, nbatch, workspace, codes, stream);
 }
 
 static int do_apply(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
-                    const void* const* x, void* const* y, int nbatch, void* workspace, void* stream) {
+                    const void* const* x, void* const* y, int nbatch, void* workspace, bool codes, void* stream) {
     plan->ev_prepare = true;
-    int rc = do_prepare(plan, L, W1, W2, R, workspace, stream);
-    return rc ? rc : do_matvec(plan, x, y, nbatch, workspace, stream);
+    int rc = do_prepare(plan, L, W1, W2, R, workspace, codes, stream);
+    return rc ? rc : do_matvec(plan, x, y, nbatch, workspace, codes, stream);
+}
+
+int heff::apply_in(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, const void* x,
+                   void* y, void* ws, size_t bytes, void* stream) {
+    const void* xs[1] = {x};
+    void* ys[1] = {y};
+    return do_apply(p, L, W1, W2, R, xs, ys, 1, ws, bytes >= p->ws_bytes, stream);
 }
 
 extern "C" int heff_prepare(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
@@ -545,7 +514,7 @@ extern "C" int heff_prepare(heff_plan* plan, const void* L, const void* W1, cons
     int rc = check_ws(plan, workspace, workspace_bytes);
     if (rc) return rc;
     plan->ev_prepare = true;
-    return do_prepare(plan, L, W1, W2, R, workspace, stream);
+    return do_prepare(plan, L, W1, W2, R, workspace, true, stream);
 }
 
 extern "C" int heff_apply_prepared(heff_plan* plan, const void* x, void* y, void* workspace,
@@ -560,7 +529,7 @@ extern "C" int heff_apply_prepared(heff_plan* plan, const void* x, void* y, void
     void* ys[1] = {y};
     plan->ev_prepare = false;
     heff::record_phase(plan, 1, stream);
-    return do_matvec(plan, xs, ys, 1, workspace, stream);
+    return do_matvec(plan, xs, ys, 1, workspace, true, stream);
 }
 
 extern "C" int heff_apply(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
@@ -571,9 +540,7 @@ extern "C" int heff_apply(heff_plan* plan, const void* L, const void* W1, const 
     if (x == y) return fail(HEFF_ERR_INVALID_ARG, "y must not alias x");
     int rc = check_ws(plan, workspace, workspace_bytes);
     if (rc) return rc;
-    const void* xs[1] = {x};
-    void* ys[1] = {y};
-    return do_apply(plan, L, W1, W2, R, xs, ys, 1, workspace, stream);
+    return heff::apply_in(plan, L, W1, W2, R, x, y, workspace, workspace_bytes, stream);
 }
 
 namespace {
@@ -643,7 +610,7 @@ extern "C" int heff_apply_batched(heff_plan* plan, const void* L, const void* W1
     int rc = check_ws(plan, workspace, workspace_bytes);
     if (rc) return rc;
     plan->ev_prepare = true;
-    return do_apply(plan, L, W1, W2, R, x, y, nbatch, workspace, stream);
+    return do_apply(plan, L, W1, W2, R, x, y, nbatch, workspace, true, stream);
 }
 
 // Tile-shape autotuner: time each GEMM with every task list the plan built (N = 256, N = 128,
@@ -680,8 +647,8 @@ extern "C" int heff_plan_autotune(heff_plan* plan, const void* L, const void* W1
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         const void* xs[1] = {x};
         void* ys[1] = {y};
-        if ((rc = heff::launch_mix(plan, L, W1, W2, R, workspace, stream))) return rc;
-        if ((rc = heff::launch_pack_batch(plan, xs, 1, workspace, stream))) return rc;
+        if ((rc = heff::launch_mix(plan, L, W1, W2, R, workspace, false, stream))) return rc;
+        if ((rc = heff::launch_pack_batch(plan, xs, 1, workspace, false, stream))) return rc;
         // each candidate: one warm-up launch, then the median of 5 separately timed launches
         cudaEvent_t e[6];
         for (auto& ev : e) CK(cudaEventCreate(&ev));
@@ -694,10 +661,10 @@ extern "C" int heff_plan_autotune(heff_plan* plan, const void* L, const void* W1
                 ms[c] = 0.f;
                 if (v[c]->tasks.empty() && !v[0]->tasks.empty()) continue;
                 std::swap(*v[0], *v[c]);
-                rc = heff::launch_gemm(plan, which, workspace, ys, 1, stream);
+                rc = heff::launch_gemm(plan, which, workspace, ys, 1, false, stream);
                 CK(cudaEventRecord(e[0], st));
                 for (int r = 0; r < 5 && !rc; ++r) {
-                    rc = heff::launch_gemm(plan, which, workspace, ys, 1, stream);
+                    rc = heff::launch_gemm(plan, which, workspace, ys, 1, false, stream);
                     CK(cudaEventRecord(e[r + 1], st));
                 }
                 if (!rc) {

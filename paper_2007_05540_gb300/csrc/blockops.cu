@@ -1,9 +1,10 @@
-// FP64 block-product engine: lists of strided dense block products summed into output
-// tiles, and block dot products.  Used by the environment update and the Rayleigh-quotient
+// Block-product engine: lists of strided dense block products summed into output tiles (run by
+// fx_gemm.cu in FP64 accuracy, or by blockops_tc.cu in BF16x3), and block dot products.  Used by the environment update and the Rayleigh-quotient
 // gradients (the block-pair contractions of Algorithm 2 with charge-matched blocks, each
 // product a small dense GEMM, Section IV "list" algorithm).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "convert.cuh"
@@ -14,6 +15,14 @@ namespace heff {
 void BList::add_block(int64_t c_off, int32_t ldc, int32_t m, int32_t n, const std::vector<BProd>& ps) {
     blocks.push_back(Block{c_off, ldc, m, n, (int32_t)block_prods.size(), (int32_t)ps.size()});
     block_prods.insert(block_prods.end(), ps.begin(), ps.end());
+    const bool fx = tile_n == FX_TILE_N;
+    std::vector<std::pair<int32_t, int32_t>> codes(ps.size());
+    int32_t steps = 0;
+    for (size_t i = 0; fx && i < ps.size(); ++i) {
+        const BProd& p = ps[i];
+        codes[i] = {view_codes(0, p.a_off, p.a_rs, p.a_cs, m, p.K), view_codes(1, p.b_off, p.b_cs, p.b_rs, n, p.K)};
+        steps += (p.K + 15) / 16;
+    }
     for (int r0 = 0; r0 < m; r0 += tile_m)
         for (int c0 = 0; c0 < n; c0 += tile_n) {
             BTile t{};
@@ -23,8 +32,12 @@ void BList::add_block(int64_t c_off, int32_t ldc, int32_t m, int32_t n, const st
             t.n = n - c0 < tile_n ? n - c0 : tile_n;
             t.prod_begin = (int32_t)prods.size();
             t.prod_count = (int32_t)ps.size();
-            for (const BProd& p : ps) {
+            t.steps = steps;
+            for (size_t i = 0; i < ps.size(); ++i) {
+                const BProd& p = ps[i];
                 BProd q = p;
+                q.ea = codes[i].first + r0;
+                q.eb = codes[i].second + c0;
                 q.a_off += (int64_t)r0 * p.a_rs;
                 q.b_off += (int64_t)c0 * p.b_cs;
                 prods.push_back(q);
@@ -34,6 +47,16 @@ void BList::add_block(int64_t c_off, int32_t ldc, int32_t m, int32_t n, const st
         }
 }
 
+int32_t BList::view_codes(int which, int64_t off, int32_t rs, int32_t ks, int32_t n, int32_t K) {
+    auto ins = views.insert({{which, off, rs, ks, n, K}, ncodes});
+    if (ins.second) {
+        for (int32_t r = 0; r < n; r += 32)
+            rows.push_back({off + (int64_t)r * rs, rs, ks, n - r < 32 ? n - r : 32, K, ncodes + r, which});
+        ncodes += n;
+    }
+    return ins.first->second;
+}
+
 void BList::retile(int tm, int tn) {
     std::vector<Block> bl;
     std::vector<BProd> bp;
@@ -41,6 +64,9 @@ void BList::retile(int tm, int tn) {
     bp.swap(block_prods);
     tiles.clear();
     prods.clear();
+    rows.clear();
+    views.clear();
+    ncodes = 0;
     flops = 0;
     tile_m = tm;
     tile_n = tn;
@@ -52,82 +78,40 @@ void BList::retile(int tm, int tn) {
 int blist_upload(BList& b) {
     b.d_tiles = nullptr;
     b.d_prods = nullptr;
-    if (!b.tiles.empty()) {
-        if (cudaMalloc((void**)&b.d_tiles, b.tiles.size() * sizeof(BTile)) != cudaSuccess ||
-            cudaMemcpy(b.d_tiles, b.tiles.data(), b.tiles.size() * sizeof(BTile), cudaMemcpyHostToDevice) != cudaSuccess)
-            return fail(HEFF_ERR_CUDA, "block tile upload failed");
-    }
-    if (!b.prods.empty()) {
-        if (cudaMalloc((void**)&b.d_prods, b.prods.size() * sizeof(BProd)) != cudaSuccess ||
-            cudaMemcpy(b.d_prods, b.prods.data(), b.prods.size() * sizeof(BProd), cudaMemcpyHostToDevice) != cudaSuccess)
-            return fail(HEFF_ERR_CUDA, "block product upload failed");
-    }
+    b.d_rows = nullptr;
+    b.d_codes = nullptr;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&b.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return fail(HEFF_ERR_CUDA, "device query failed");
+    // the longest tiles first
+    if (b.tile_n == FX_TILE_N)
+        std::stable_sort(b.tiles.begin(), b.tiles.end(), [](const BTile& x, const BTile& y) {
+            return (int64_t)x.steps * (x.n + 32) > (int64_t)y.steps * (y.n + 32);
+        });
+    auto up = [](const auto& v, auto** d) {
+        return v.empty() || (cudaMalloc((void**)d, v.size() * sizeof(v[0])) == cudaSuccess &&
+                             cudaMemcpy(*d, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice) == cudaSuccess);
+    };
+    if (!up(b.tiles, &b.d_tiles) || !up(b.prods, &b.d_prods) || !up(b.rows, &b.d_rows))
+        return fail(HEFF_ERR_CUDA, "block list upload failed");
+    if (b.ncodes && cudaMalloc((void**)&b.d_codes, b.ncodes * sizeof(uint16_t)) != cudaSuccess)
+        return fail(HEFF_ERR_CUDA, "block list upload failed");
     return HEFF_OK;
 }
 
 void blist_free(BList& b) {
     cudaFree(b.d_tiles);
     cudaFree(b.d_prods);
+    cudaFree(b.d_rows);
+    cudaFree(b.d_codes);
     b.d_tiles = nullptr;
     b.d_prods = nullptr;
+    b.d_rows = nullptr;
+    b.d_codes = nullptr;
 }
 
 namespace {
-
-// 64 x 64 output tile, 256 threads with 4 x 4 outputs each, K in steps of 16 through
-// shared memory.  Loads follow whichever operand stride is unit so they coalesce.
-__global__ void __launch_bounds__(256) bgemm_kernel(const BTile* __restrict__ tiles, const BProd* __restrict__ prods,
-                                                    const double* __restrict__ A, const double* __restrict__ B,
-                                                    double* __restrict__ C, const double* __restrict__ coef1,
-                                                    const double* __restrict__ coef2, double scale,
-                                                    const double* __restrict__ inv_scale, int accumulate) {
-    __shared__ double As[16][64 + 1];
-    if (inv_scale) scale /= inv_scale[0];
-    __shared__ double Bs[16][64 + 1];
-    const BTile t = tiles[blockIdx.x];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    double acc[4][4] = {};
-    for (int pi = 0; pi < t.prod_count; ++pi) {
-        const BProd p = prods[t.prod_begin + pi];
-        const double coef = (p.c1 < 0 ? 1.0 : coef1[p.c1]) * (p.c2 < 0 ? 1.0 : coef2[p.c2]);
-        for (int k0 = 0; k0 < p.K; k0 += 16) {
-            for (int l = 0; l < 4; ++l) {
-                const int idx = tid + 256 * l;
-                // A: (row, kk); unit stride along k -> kk fastest, else rows fastest
-                int row, kk;
-                if (p.a_cs == 1) { row = idx >> 4; kk = idx & 15; } else { row = idx & 63; kk = idx >> 6; }
-                As[kk][row] = (row < t.m && k0 + kk < p.K)
-                                  ? coef * A[p.a_off + (int64_t)row * p.a_rs + (int64_t)(k0 + kk) * p.a_cs] : 0.0;
-                int col, kb;
-                if (p.b_cs == 1) { col = idx & 63; kb = idx >> 6; } else { col = idx >> 4; kb = idx & 15; }
-                Bs[kb][col] = (col < t.n && k0 + kb < p.K)
-                                  ? B[p.b_off + (int64_t)(k0 + kb) * p.b_rs + (int64_t)col * p.b_cs] : 0.0;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                double a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { a[i] = As[k][ty * 4 + i]; b[i] = Bs[k][tx * 4 + i]; }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-    }
-    for (int i = 0; i < 4; ++i) {
-        const int r = ty * 4 + i;
-        if (r >= t.m) continue;
-        for (int j = 0; j < 4; ++j) {
-            const int c = tx * 4 + j;
-            if (c >= t.n) continue;
-            double* cp = C + t.c_off + (int64_t)r * t.ldc + c;
-            *cp = accumulate ? *cp + scale * acc[i][j] : scale * acc[i][j];
-        }
-    }
-}
 
 // one CTA per dot: partial[d] = <X[x_off..], Y[y_off..]>, accumulated in the element type
 // (FP32 vectors come from the tensor-core products, whose values carry ~1e-5 anyway)
@@ -161,17 +145,6 @@ __global__ void gather_dots_kernel(const int32_t* __restrict__ off, const double
 }
 
 }  // namespace
-
-int launch_bgemm(const BList& b, const double* A, const double* B, double* C, const double* coef1,
-                 const double* coef2, double scale, void* stream, const double* inv_scale) {
-    if (b.tiles.empty()) return HEFF_OK;
-    bgemm_kernel<<<(unsigned)b.tiles.size(), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        b.d_tiles, b.d_prods, A, B, C, coef1, coef2, scale, inv_scale, b.accumulate ? 1 : 0);
-    count_launches(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "bgemm launch: %s", cudaGetErrorString(e));
-    return HEFF_OK;
-}
 
 template <typename T>
 static int block_dots_t(const BDot* d_dots, int ndots, const int32_t* d_off, const T* X, const T* Y, double* out,

@@ -1,5 +1,5 @@
 // Environment extension on the GPU (Section II-C: the left environment A and right
-// environment B grow by one site as the sweep moves), in FP64 on the block-product engine.
+// environment B grow by one site as the sweep moves), on the block-product engine.
 //
 // Left (site tensor A[a, s, b], flows (+1, +1, -1); environment L[a', w, a]):
 //   X[(a', w), (s, b)]  = L[a', w, a] . A[a, s, b]                      (step 1)
@@ -34,6 +34,7 @@ struct heff_env_plan {
     size_t off_x = 256, off_env32 = 0, off_site32 = 0;
     size_t ws_bytes = 0;
     bool uploaded = false;
+    const void* last_ws = nullptr;    // workspace of the last update (its error flag is initialised)
 };
 
 namespace {
@@ -247,13 +248,14 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
     char* ws = static_cast<char*>(workspace);
     int* err = reinterpret_cast<int*>(ws);
     int rc;
-    if (plan->precision == HEFF_PREC_FP64) {
-        double* X = reinterpret_cast<double*>(ws + plan->off_x);
-        if ((rc = heff::launch_bgemm(plan->step1, env_old, site, X, nullptr, nullptr, 1.0, stream))) return rc;
-        return heff::launch_bgemm(plan->step2, site, X, env_new, W, nullptr, 1.0, stream);
-    }
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+    plan->last_ws = workspace;
+    if (plan->precision == HEFF_PREC_FP64) {
+        double* X = reinterpret_cast<double*>(ws + plan->off_x);
+        if ((rc = heff::launch_bgemm(plan->step1, env_old, site, X, nullptr, nullptr, 1.0, stream, err))) return rc;
+        return heff::launch_bgemm(plan->step2, site, X, env_new, W, nullptr, 1.0, stream, err);
+    }
     float* X = reinterpret_cast<float*>(ws + plan->off_x);
     float* E32 = reinterpret_cast<float*>(ws + plan->off_env32);
     float* S32 = reinterpret_cast<float*>(ws + plan->off_site32);
@@ -270,11 +272,11 @@ extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precisio
     if (precision != HEFF_PREC_FP64 && precision != HEFF_PREC_BF16X3)
         return fail(HEFF_ERR_UNSUPPORTED, "environment updates run in HEFF_PREC_FP64 or HEFF_PREC_BF16X3");
     if (precision == plan->precision) return HEFF_OK;
-    const int tile = precision == HEFF_PREC_FP64 ? 64 : 128;
+    const bool fx = precision == HEFF_PREC_FP64;
     heff::blist_free(plan->step1);
     heff::blist_free(plan->step2);
-    plan->step1.retile(tile, tile);
-    plan->step2.retile(tile, tile);
+    plan->step1.retile(fx ? heff::FX_TILE_M : 128, fx ? heff::FX_TILE_N : 128);
+    plan->step2.retile(fx ? heff::FX_TILE_M : 128, fx ? heff::FX_TILE_N : 128);
     plan->precision = precision;
     if (plan->uploaded) {
         int rc;
@@ -289,7 +291,8 @@ extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precisio
 extern "C" int heff_env_status(const heff_env_plan* plan, void* workspace, size_t workspace_bytes, void* stream) {
     heff::clear_error();
     if (!plan || !workspace) return fail(HEFF_ERR_INVALID_ARG, "heff_env_status: null argument");
-    if (plan->precision == HEFF_PREC_FP64) return HEFF_OK;
+    // an FP64 plan's flag exists once an update has run in this workspace
+    if (plan->precision == HEFF_PREC_FP64 && workspace != plan->last_ws) return HEFF_OK;
     if (workspace_bytes < plan->ws_bytes) return fail(HEFF_ERR_WORKSPACE, "heff_env_status: workspace too small");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int* d = static_cast<int*>(workspace);
@@ -318,6 +321,7 @@ extern "C" void heff_env_plan_destroy(heff_env_plan* plan) {
 struct heff_two_site {
     BList prods;
     bool uploaded = false;
+    int* err = nullptr;        // host memory mapped to the device: a bounded wait expired
 };
 
 extern "C" int heff_two_site_create(const heff_layout* A, const heff_layout* B, const heff_layout* x,
@@ -365,11 +369,14 @@ extern "C" int heff_two_site_create(const heff_layout* A, const heff_layout* B, 
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) {
         int rc = heff::blist_upload(P->prods);
+        if (!rc && cudaHostAlloc((void**)&P->err, sizeof(int), cudaHostAllocMapped) != cudaSuccess)
+            rc = fail(HEFF_ERR_OOM, "heff_two_site_create: host allocation failed");
         if (rc) {
             heff::blist_free(P->prods);
             delete P;
             return rc;
         }
+        *P->err = 0;
         P->uploaded = true;
     } else {
         cudaGetLastError();
@@ -382,11 +389,16 @@ extern "C" int heff_two_site_apply(heff_two_site* P, const double* A, const doub
     heff::clear_error();
     if (!P || !A || !B || !x) return fail(HEFF_ERR_INVALID_ARG, "heff_two_site_apply: null argument");
     if (!P->uploaded) return fail(HEFF_ERR_UNSUPPORTED, "two-site plan was created without a CUDA device");
-    return heff::launch_bgemm(P->prods, A, B, x, nullptr, nullptr, 1.0, stream);
+    if (*static_cast<volatile int*>(P->err)) {
+        *P->err = 0;
+        return fail(HEFF_ERR_TIMEOUT, "heff_two_site_apply: a bounded device-side wait of an earlier call expired");
+    }
+    return heff::launch_bgemm(P->prods, A, B, x, nullptr, nullptr, 1.0, stream, P->err);
 }
 
 extern "C" void heff_two_site_destroy(heff_two_site* P) {
     if (!P) return;
     heff::blist_free(P->prods);
+    cudaFreeHost(P->err);
     delete P;
 }

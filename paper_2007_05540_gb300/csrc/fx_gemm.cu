@@ -1,0 +1,816 @@
+// FP64 block products on the sm_103a tensor cores: fixed-point digits on the FP16 pipe.
+//
+// GB300 does about two FP64 multiply-adds per SM and clock (1.2 TFLOP/s in all), while its FP16
+// tensor pipe does about 4000.  So a product of FP64 operands is computed here from integer
+// digits, the error-free splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012):
+// every row of A and every column of B gets one scale (a power of two from its largest
+// element), each element becomes a 62-bit fixed-point number of eight signed 8-bit digits
+// (fixed.cuh), and
+//   C = sum_g 2^(-8 g) sum_{i + j = g} A_i B_j^T,      g = 0 .. 7,
+// where the digit planes A_i, B_j are FP16 operands of tcgen05 MMAs.  The 36 digit products of a
+// K step land in 8 accumulators (one per g) in tensor memory.  All sums that matter at FP64
+// precision are exact: a digit product is at most 2^14, and a chunk of 256 contraction steps
+// keeps the accumulators g <= 4 below 2^24, where FP32 adds integers exactly; the later ones
+// weigh 2^-40 and less.  After each chunk the accumulators are added into 96-bit integers, and
+// the sum is rounded to FP64 once at the end.  What is dropped is the part of an element below
+// 2^-62 of the largest in its row, and the digit products g >= 8: together about
+// 2^-61 K max|a row| max|b column|, against 2^-53 per addition of a running FP64 sum.
+//
+// Rows that the scale cannot hold (infinities, NaNs, magnitudes beyond 2^+-400) make their tile
+// run in FP64 arithmetic on the CUDA cores inside the same kernel.
+//
+// Two sources of work share the kernel: the matvec's task lists over the workspace operands
+// (MODE 0; K contiguous, one pitch) and the block-product lists with arbitrary strides and
+// scalar coefficients (MODE 1).
+//
+// One persistent CTA per SM, 128 x 64 output tiles, 20 warps:
+//   warps 0-7    producers: load 128 + 64 rows x 16 K of FP64, convert to digits, write the FP16
+//                planes into the 64-byte-swizzled K-major layout (a ring of 4 steps, 48 KB each)
+//   warps 8-15   drain: 8 accumulators -> 96-bit integers in registers -> FP64 -> global
+//   warp 16      allocates the 512 tensor-memory columns; one thread issues the MMAs: digit
+//                plane A_i times the planes B_0 .. B_{7-i}, which lie one after another in shared
+//                memory and so are one wide B operand, whose products go to the accumulators
+//                i .. 7, which lie one after another in tensor memory
+// Registers are moved from the other warps to the drain warps (96 integers a thread).
+//
+// Bound by the 36 digit products: 1.9 PFLOP/s of FP16 / 36 = 53 TFLOP/s, less the ragged tiles and
+// the drain of the accumulators every 256 steps.  Against the FP64 units (64 x 64 tiles on the
+// CUDA cores), whole calls: prepared matvec m = 1024, k = 14, 6.24 -> 0.65 ms; environment update
+// m = 1024, 4.9 -> 0.59 ms; gradients m = 320, 9.2 -> 1.46 ms.
+// Every mbarrier wait is bounded; on expiry the CTA raises the error flag, stops issuing work,
+// waits (bounded) for its MMAs in flight, frees its tensor memory and returns.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include "fixed.cuh"
+#include "internal.h"
+#include "tc_ptx.cuh"
+
+namespace heff {
+namespace {
+
+using namespace ptx;
+
+constexpr int FM = FX_TILE_M, FN = FX_TILE_N;     // output tile
+constexpr int FKS = 16;                           // contraction elements per step
+constexpr int FD = 8;                             // digits
+constexpr int FST = 4;                            // steps in the ring (two per 64-byte K block)
+constexpr int FCH = 16;                           // steps per exact accumulation chunk (256 elements)
+constexpr int PW = 8, EW = 8;                     // producer and drain warps
+constexpr int FTHREADS = 32 * (PW + EW + 4);      // + the MMA warp's warpgroup
+constexpr int A_PLANE = FM * 64;                  // one digit plane of A, 32 K elements
+constexpr int A_BLK = FD * A_PLANE;               // 64 KB
+constexpr int B_BLK = FD * FN * 64;               // 32 KB
+constexpr int BLK = A_BLK + B_BLK;
+constexpr int OFF_TR = (FST / 2) * BLK;           // drain transposes: 32 rows x 8 columns per warp
+constexpr int TR_WARP = 32 * 9 * 8;
+constexpr int OFF_DF = OFF_TR + EW * TR_WARP;     // FP64 tiles: 8 K x (64 + 1) for A and for B
+constexpr int OFF_E = OFF_DF + 2 * 8 * 65 * 8;    // row and column scales, two tiles
+constexpr int OFF_BAR = OFF_E + 2 * (FM + FN + PW) * 4;
+constexpr int FSMEM = OFF_BAR + 256 + 1024;
+static_assert(FSMEM <= 227 * 1024, "shared memory of one CTA");
+// register split (per thread): producers, drain, MMA warpgroup; the kernel is compiled for
+// R_ALL, and each SM partition holds two producer, two drain and one other warp
+constexpr int R_ALL = 96, R_PROD = 80, R_DRAIN = 136, R_MMA = 48;
+static_assert(2 * R_PROD + 2 * R_DRAIN + R_MMA <= 5 * R_ALL, "registers of a partition");
+
+struct FxArgs {
+    // MODE 0
+    const GemmTask* tasks;
+    const KSeg* segs;
+    int64_t ld, a_batch_rows, b_batch_rows;
+    const uint16_t *ea, *eb;             // exponent codes [column / 32][row]; null: all tiles in FP64
+    int64_t ea_rows, eb_rows;
+    uint16_t* et;                        // codes of the output T (null for y)
+    int64_t et_rows, c_batch_rows, c_batch_elems;
+    PtrBatch y;                          // outputs (mode y), or y.p[0] unused
+    int nbatch, b0, to_y;
+    // MODE 1
+    const BTile* tiles;
+    const BProd* prods;
+    const uint16_t* e;                   // exponent codes per operand row (BProd.ea, eb)
+    const double *coef1, *coef2, *inv_scale;
+    double scale;
+    int accumulate;
+    // both
+    int ntiles;
+    const double *A, *B;
+    double* C;
+    int* err;
+};
+
+struct Tile {
+    int m, n, n_zero, ldc, steps, pbeg, pcnt, bat;
+    int64_t c_off, a_row, b_row;
+};
+
+template <int MODE>
+__device__ __forceinline__ Tile get_tile(const FxArgs& g, long item) {
+    Tile t;
+    if constexpr (MODE == 0) {
+        const int b = (int)(item % g.nbatch);
+        const GemmTask k = g.tasks[item / g.nbatch];
+        t.m = k.m; t.n = k.n; t.n_zero = k.n_zero; t.ldc = k.ldc; t.steps = k.ktotal / FKS;
+        t.pbeg = k.seg_begin; t.pcnt = k.seg_count; t.bat = b;
+        t.c_off = k.c_off;
+        t.a_row = k.a_row + (g.b0 + b) * g.a_batch_rows;
+        t.b_row = k.b_row + (g.b0 + b) * g.b_batch_rows;
+    } else {
+        const BTile k = g.tiles[item];
+        t.m = k.m; t.n = k.n; t.n_zero = 0; t.ldc = k.ldc; t.steps = k.steps;
+        t.pbeg = k.prod_begin; t.pcnt = k.prod_count; t.bat = 0;
+        t.c_off = k.c_off; t.a_row = 0; t.b_row = 0;
+    }
+    return t;
+}
+
+// round i of this CTA: block lists run in a snake over the sorted tiles; task lists are laid
+// out for a plain round robin by the planner
+template <int MODE>
+__device__ __forceinline__ long item_of(long i) {
+    const long G = gridDim.x, c = blockIdx.x;
+    return MODE == 0 ? i * G + c : i * G + ((i & 1) ? G - 1 - c : c);
+}
+
+__device__ __forceinline__ double prod_coef(const FxArgs& g, const BProd& p) {
+    return (p.c1 < 0 ? 1.0 : g.coef1[p.c1]) * (p.c2 < 0 ? 1.0 : g.coef2[p.c2]);
+}
+
+// One product (a contraction segment) of a tile: element (r, k) of A at a[r ars + k acs], column
+// c's element k of B at b[c bcs + k brs].
+struct Prod {
+    const double *a, *b;
+    int64_t ars, bcs;
+    int acs, brs, K;
+    double coef;
+};
+
+template <int MODE>
+__device__ __forceinline__ Prod get_prod(const FxArgs& g, const Tile& t, int i) {
+    Prod p;
+    if constexpr (MODE == 0) {
+        const KSeg s = g.segs[t.pbeg + i];
+        p.a = g.A + t.a_row * g.ld + s.k0;
+        p.b = g.B + t.b_row * g.ld + s.k0;
+        p.ars = p.bcs = g.ld;
+        p.acs = p.brs = 1;
+        p.K = s.klen;
+        p.coef = 1.0;
+    } else {
+        const BProd q = g.prods[t.pbeg + i];
+        p.a = g.A + q.a_off;
+        p.b = g.B + q.b_off;
+        p.ars = q.a_rs; p.acs = q.a_cs;
+        p.bcs = q.b_cs; p.brs = q.b_rs;
+        p.K = q.K;
+        p.coef = prod_coef(g, q);
+    }
+    return p;
+}
+
+// Scale of row r of A (side 0) or column r of B (side 1) over the tile's products; ok: cleared
+// when the row needs FP64.
+template <int MODE>
+__device__ __forceinline__ int row_scale(const FxArgs& g, const Tile& t, int side, int r, bool& ok) {
+    int E = 0;
+    if constexpr (MODE == 0) {
+        const uint16_t* e = side ? g.eb : g.ea;
+        const int64_t rows = side ? g.eb_rows : g.ea_rows;
+        if (!e) { ok = false; return fx::E_ZERO; }
+        e += (side ? t.b_row : t.a_row) + r;
+        for (int s = 0; s < t.pcnt; ++s) {
+            const KSeg sg = g.segs[t.pbeg + s];
+            const int kb0 = sg.k0 / KPAD, nkb = sg.klen / KPAD;
+#pragma unroll 4
+            for (int j = 0; j < nkb; ++j) E = max(E, (int)e[(kb0 + j) * rows]);
+        }
+    } else {
+        for (int s = 0; s < t.pcnt; ++s) {
+            const BProd& p = g.prods[t.pbeg + s];
+            int v = g.e[(side ? p.eb : p.ea) + r];
+            if (side == 0 && (p.c1 >= 0 || p.c2 >= 0)) {
+                const double c = prod_coef(g, p);
+                const int ec = fx::exp_code((uint32_t)__double2hiint(c), (uint32_t)__double2loint(c));
+                if (ec == 0x7ff) ok = false;
+                // |c v| < 2^(ec - 1022) 2^(v - 1022)
+                v = (v == 0 || ec == 0) && v != 0x7ff ? 0 : (v == 0x7ff ? v : max(v + ec - 1022, 1));
+            }
+            E = max(E, v);
+        }
+    }
+    if (!fx::exp_plain(E)) ok = false;
+    return E ? E : fx::E_ZERO;
+}
+
+// Eight K values k0 .. k0 + 7 of one row (zeros beyond K or for an absent row).
+__device__ __forceinline__ void load8(double (&v)[8], const double* row, int ks, int k0, int K, bool have, bool vec) {
+    if (have && k0 + 8 <= K) {
+        if (vec) {
+            const double2* p = reinterpret_cast<const double2*>(row + k0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const double2 d = __ldg(p + i);
+                v[2 * i] = d.x;
+                v[2 * i + 1] = d.y;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = row[(int64_t)(k0 + i) * ks];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = have && k0 + i < K ? row[(int64_t)(k0 + i) * ks] : 0.0;
+    }
+}
+
+// Digits of eight K values into the eight planes (plane bytes apart), 16 bytes each at addr.
+__device__ __forceinline__ void digits8(const double (&v)[8], int E, uint32_t addr, uint32_t plane) {
+    uint32_t d[FD][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        uint64_t q[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const double x = v[2 * p + u];
+            q[u] = fx::to_fixed((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x), E);
+        }
+        // bytes of the two elements side by side, each in the low byte of an FP16 1024 + b;
+        // 1024 + b - 1152 is the digit
+        const __half2 off = __half2half2(__ushort_as_half((unsigned short)0x6480));
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            const uint32_t x = (uint32_t)(q[0] >> (32 * w)), y = (uint32_t)(q[1] >> (32 * w));
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const uint32_t t = __byte_perm(x, y, b ? 0x7362 : 0x5140);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const uint32_t f = __byte_perm(t, 0x64646464u, c ? 0x4342 : 0x4140);
+                    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&f), off);
+                    d[7 - (4 * w + 2 * b + c)][p] = *reinterpret_cast<const uint32_t*>(&h);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < FD; ++s) st_shared_v4(addr + s * plane, d[s][0], d[s][1], d[s][2], d[s][3]);
+}
+
+// byte offset of the 8-element chunk (half step h of the ring step st) of row r in a plane
+__device__ __forceinline__ uint32_t chunk_off(int r, uint32_t st, int h) {
+    return (uint32_t)r * 64 + (((2 * (st & 1) + h) ^ ((r >> 1) & 3)) << 4);
+}
+
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t& a, uint32_t& b) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(taddr));
+}
+// the loads have landed (the registers pass through, so that nothing reads them earlier)
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&d)[FD][2]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(d[0][0]), "+r"(d[0][1]), "+r"(d[1][0]), "+r"(d[1][1]), "+r"(d[2][0]), "+r"(d[2][1]),
+                   "+r"(d[3][0]), "+r"(d[3][1]), "+r"(d[4][0]), "+r"(d[4][1]), "+r"(d[5][0]), "+r"(d[5][1]),
+                   "+r"(d[6][0]), "+r"(d[6][1]), "+r"(d[7][0]), "+r"(d[7][1])
+                 :
+                 : "memory");
+}
+
+// FP16 operands, FP32 accumulate, K-major, M x N
+__device__ __forceinline__ uint32_t idesc_f16(uint32_t M, uint32_t N) {
+    return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
+}
+
+template <int MODE>
+__device__ __forceinline__ double* out_ptr(const FxArgs& g, const Tile& t) {
+    if constexpr (MODE == 0)
+        return (g.to_y ? static_cast<double*>(const_cast<void*>(g.y.p[t.bat]))
+                       : g.C + (int64_t)(g.b0 + t.bat) * g.c_batch_elems) + t.c_off;
+    return g.C + t.c_off;
+}
+
+// exponent codes of T: the 32-column block of column c (of the tile) in row r (of the tile)
+__device__ __forceinline__ uint16_t* code_ptr(const FxArgs& g, const Tile& t, int r, int c) {
+    const int64_t row = t.c_off / t.ldc + r + (int64_t)(g.b0 + t.bat) * g.c_batch_rows;
+    return g.et + ((t.c_off % t.ldc + c) / KPAD) * g.et_rows + row;
+}
+
+// Producer warps meet (bounded, so that a CTA that gives up does not hang here).
+struct PSync {
+    uint64_t* bar;
+    uint32_t n;
+    volatile int* abort_flag;
+    int* err;
+    __device__ __forceinline__ bool operator()() {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+        return mbar_wait(bar, n++ & 1, abort_flag, err);
+    }
+};
+
+// A tile in FP64 arithmetic on the producer warps (256 threads, 4 x 4 outputs each, two halves
+// of 64 rows).
+template <int MODE>
+__device__ __forceinline__ bool fp64_tile(const FxArgs& g, const Tile& t, double* sh, PSync& psync, double scale) {
+    double (*As)[65] = reinterpret_cast<double (*)[65]>(sh);
+    double (*Bs)[65] = As + 8;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    double* C = out_ptr<MODE>(g, t);
+    for (int half = 0; half < t.m; half += 64) {
+        const int m = t.m - half < 64 ? t.m - half : 64;
+        double acc[4][4] = {};
+        for (int s = 0; s < t.pcnt; ++s) {
+            const Prod p = get_prod<MODE>(g, t, s);
+            for (int k0 = 0; k0 < p.K; k0 += 8) {
+                for (int l = 0; l < 2; ++l) {
+                    const int idx = tid + 256 * l;
+                    int r, k;
+                    if (p.acs == 1) { r = idx >> 3; k = idx & 7; } else { r = idx & 63; k = idx >> 6; }
+                    As[k][r] = r < m && k0 + k < p.K
+                                   ? p.coef * p.a[(int64_t)(half + r) * p.ars + (int64_t)(k0 + k) * p.acs] : 0.0;
+                    if (p.brs == 1) { r = idx >> 3; k = idx & 7; } else { r = idx & 63; k = idx >> 6; }
+                    Bs[k][r] = r < t.n && k0 + k < p.K
+                                   ? p.b[(int64_t)r * p.bcs + (int64_t)(k0 + k) * p.brs] : 0.0;
+                }
+                if (!psync()) return false;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    double a[4], b[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { a[i] = As[k][ty * 4 + i]; b[i] = Bs[k][tx * 4 + i]; }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                }
+                if (!psync()) return false;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = ty * 4 + i;
+            int code = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = tx * 4 + j;
+                const double v = c < t.n ? acc[i][j] : 0.0;
+                if (r < m && c < t.n + t.n_zero) {
+                    double* cp = C + (int64_t)(half + r) * t.ldc + c;
+                    if (MODE == 0) *cp = v;
+                    else *cp = g.accumulate ? *cp + scale * v : scale * v;
+                }
+                code = max(code, fx::exp_code((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v)));
+            }
+            if (MODE == 0 && !g.to_y && g.et) {
+                // eight lanes hold one row's 32 columns
+                for (int o = 1; o < 8; o <<= 1) code = max(code, __shfl_xor_sync(0xffffffffu, code, o));
+                if ((tx & 7) == 0 && r < m && tx * 4 < t.n + t.n_zero)
+                    *code_ptr(g, t, half + r, tx * 4) = (uint16_t)code;
+            }
+        }
+    }
+    return true;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_constant__ FxArgs g) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
+    uint64_t* empty = full + FST;
+    uint64_t* tready = empty + FST;      // [2] scales of a tile are in shared memory
+    uint64_t* edone = tready + 2;        // [2] the drain and the MMA issuer are done with them
+    uint64_t* tfull = edone + 2;         // a chunk's sums are in tensor memory
+    uint64_t* tempty = tfull + 1;        // they have been read
+    uint64_t* pbar = tempty + 1;
+    uint64_t* drain = pbar + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    int* escale = reinterpret_cast<int*>(smem + OFF_E);          // [2][FM + FN]
+    int* ebad = escale + 2 * (FM + FN);                          // [2][PW]
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < FST; ++s) { mbar_init(&full[s], PW); mbar_init(&empty[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&tready[b], 1); mbar_init(&edone[b], EW + 1); }
+        mbar_init(tfull, 1);
+        mbar_init(tempty, EW);
+        mbar_init(pbar, PW);
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == PW + EW) tmem_alloc(tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t base = su32(smem);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const long total = (long)g.ntiles * (MODE == 0 ? g.nbatch : 1);
+    const long rounds = (total + gridDim.x - 1) / gridDim.x;
+
+    if (warp < PW) {
+        // ------------------------------------------------ producers
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_PROD));
+        PSync psync{pbar, 0, abort_flag, g.err};
+        const double scale = MODE == 1 ? (g.inv_scale ? g.scale / g.inv_scale[0] : g.scale) : 1.0;
+        uint32_t step = 0, tcount = 0;
+        bool ok = true;
+        // rows of a warp's 16-row group in an order that spreads its stores over the banks
+        const int rl = ((lane >> 1) & 1) | ((lane >> 2) & 1) << 2 | ((lane >> 3) & 1) << 1 | ((lane >> 4) & 1) << 3;
+        for (long i = 0; i < rounds && ok; ++i) {
+            const long item = item_of<MODE>(i);
+            if (item >= total) continue;
+            const Tile t = get_tile<MODE>(g, item);
+            if (t.m == 0) continue;
+            const int b = tcount & 1;
+            if (!(ok = mbar_wait(&edone[b], ((tcount >> 1) & 1) ^ 1, abort_flag, g.err))) break;
+            ++tcount;
+            // scales: one thread per row of A, then per column of B
+            int* es = escale + b * (FM + FN);
+            {
+                const int side = threadIdx.x >= FM, r = side ? threadIdx.x - FM : threadIdx.x;
+                bool plain = true;
+                if (threadIdx.x < FM + FN)
+                    es[threadIdx.x] = r < (side ? t.n : t.m) ? row_scale<MODE>(g, t, side, r, plain) : fx::E_ZERO;
+                const bool bad = __any_sync(0xffffffffu, !plain);
+                if (lane == 0) ebad[b * PW + warp] = bad;
+            }
+            if (!(ok = psync())) break;
+            if (threadIdx.x == 0) mbar_arrive(&tready[b]);
+            bool bad = false;
+#pragma unroll
+            for (int w = 0; w < PW; ++w) bad |= ebad[b * PW + w] != 0;
+            if (bad) {
+                ok = fp64_tile<MODE>(g, t, reinterpret_cast<double*>(smem + OFF_DF), psync, scale);
+                continue;
+            }
+            if (t.steps == 0) continue;
+            const int n16 = (t.n + 15) & ~15;
+            const uint32_t bplane = (uint32_t)n16 * 64;
+            // warp w converts A rows (two 8-element halves of 16 rows, or one half of 32 rows);
+            // B (64 rows) takes four warps: warps 0-3 on even steps, 4-7 on odd steps
+            Prod p = get_prod<MODE>(g, t, 0);
+            int pi = 0, k = 0;
+            double va[8], vb[8];
+            auto load_a = [&](const Prod& q, int kk) {
+                if (q.acs == 1) {
+                    const int r = warp * 16 + rl;
+                    const double* row = q.a + (int64_t)r * q.ars;
+                    load8(va, row, 1, kk + 8 * (lane & 1), q.K, r < t.m,
+                          MODE == 0 || (reinterpret_cast<uintptr_t>(row) & 15) == 0);
+                } else {
+                    const int r = (warp & 3) * 32 + lane;
+                    load8(va, q.a + (int64_t)r * q.ars, q.acs, kk + 8 * (warp >> 2), q.K, r < t.m, false);
+                }
+            };
+            auto load_b = [&](const Prod& q, int kk) {
+                const int w = warp & 3;
+                if (q.brs == 1) {
+                    const int r = w * 16 + rl;
+                    const double* row = q.b + (int64_t)r * q.bcs;
+                    load8(vb, row, 1, kk + 8 * (lane & 1), q.K, r < t.n,
+                          MODE == 0 || (reinterpret_cast<uintptr_t>(row) & 15) == 0);
+                } else {
+                    const int r = (w & 1) * 32 + lane;
+                    load8(vb, q.b + (int64_t)r * q.bcs, q.brs, kk + 8 * (w >> 1), q.K, r < t.n, false);
+                }
+            };
+            load_a(p, 0);
+            for (int s = 0; s < t.steps; ++s, ++step) {
+                const uint32_t st = step % FST;
+                const bool mine_b = ((step & 1) != 0) == (warp >= 4);
+                const bool ka = p.acs == 1, kb = p.brs == 1;
+                const double coef = p.coef;
+                if (mine_b) load_b(p, k);
+                const uint32_t blk = base + (st >> 1) * BLK;
+                if (!(ok = mbar_wait(&empty[st], ((step / FST) & 1) ^ 1, abort_flag, g.err))) break;
+                {
+                    const int r = ka ? warp * 16 + rl : (warp & 3) * 32 + lane;
+                    const int h = ka ? lane & 1 : warp >> 2;
+                    if (MODE == 1 && coef != 1.0) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) va[e] *= coef;
+                    }
+                    if (r < t.m) digits8(va, es[r], blk + chunk_off(r, st, h), A_PLANE);
+                }
+                // the next step's A rows are on their way while this step's B is converted
+                k += FKS;
+                if (k >= p.K && s + 1 < t.steps) {
+                    k = 0;
+                    p = get_prod<MODE>(g, t, ++pi);
+                }
+                if (s + 1 < t.steps) load_a(p, k);
+                if (mine_b) {
+                    const int w = warp & 3;
+                    const int r = kb ? w * 16 + rl : (w & 1) * 32 + lane;
+                    const int h = kb ? lane & 1 : w >> 1;
+                    if (r < t.n) digits8(vb, es[FM + r], blk + A_BLK + chunk_off(r, st, h), bplane);
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full[st]);
+            }
+        }
+    } else if (warp < PW + EW) {
+        // ------------------------------------------------ drain
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_DRAIN));
+        const double scale = MODE == 1 ? (g.inv_scale ? g.scale / g.inv_scale[0] : g.scale) : 1.0;
+        const int q = warp & 3, h = (warp - PW) >> 2;       // tensor-memory lanes, column half
+        double* tr = reinterpret_cast<double*>(smem + OFF_TR + (warp - PW) * TR_WARP);
+        uint32_t ccount = 0, tcount = 0;
+        bool ok = true;
+        for (long i = 0; i < rounds && ok; ++i) {
+            const long item = item_of<MODE>(i);
+            if (item >= total) continue;
+            const Tile t = get_tile<MODE>(g, item);
+            if (t.m == 0) continue;
+            const int b = tcount & 1;
+            if (!(ok = mbar_wait(&tready[b], (tcount >> 1) & 1, abort_flag, g.err))) break;
+            ++tcount;
+            bool bad = false;
+#pragma unroll
+            for (int w = 0; w < PW; ++w) bad |= ebad[b * PW + w] != 0;
+            if (!bad) {
+                const int n16 = (t.n + 15) & ~15;
+                uint32_t w0[32], w1[32], w2[32];
+#pragma unroll
+                for (int c = 0; c < 32; ++c) { w0[c] = 0; w1[c] = 0; w2[c] = 0; }
+                for (int s = 0; s < t.steps; s += FCH) {
+                    if (!(ok = mbar_wait(tfull, ccount & 1, abort_flag, g.err))) break;
+                    ++ccount;
+                    tc_fence_after();
+                    const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + 32 * h;
+#pragma unroll
+                    for (int c = 0; c < 32; c += 2) {
+                        if (32 * h + c < n16) {
+                            uint32_t d[FD][2];
+#pragma unroll
+                            for (int e = 0; e < FD; ++e) tmem_ld2(ta + e * n16 + c, d[e][0], d[e][1]);
+                            tmem_ld_wait(d);
+#pragma unroll
+                            for (int u = 0; u < 2; ++u) {
+                                int64_t hi = 0, lo = 0;
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    hi += (int64_t)__float2int_rn(__uint_as_float(d[e][u])) * (1 << (8 * (3 - e)));
+                                    lo += (int64_t)__float2int_rn(__uint_as_float(d[4 + e][u])) * (1 << (8 * (3 - e)));
+                                }
+                                hi += lo >> 32;
+                                // (w2, w1, w0) += hi 2^32 + low word of lo
+                                asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+                                    : "+r"(w0[c + u]), "+r"(w1[c + u]), "+r"(w2[c + u])
+                                    : "r"((uint32_t)lo), "r"((uint32_t)hi), "r"((uint32_t)(hi >> 32)));
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty);
+                }
+                if (!ok) break;
+                // round to FP64 and store, 8 columns at a time
+                const int* es = escale + b * (FM + FN);
+                const int er = es[q * 32 + lane] - 2112;
+                const int rows = t.m - q * 32 < 32 ? t.m - q * 32 : 32;
+                double* C = out_ptr<MODE>(g, t) + (int64_t)(q * 32) * t.ldc;
+                const int ncols = t.n + t.n_zero;
+                int code = 0;
+#pragma unroll
+                for (int c0 = 0; c0 < 32; c0 += 8) {
+                    const int col0 = 32 * h + c0;
+                    if (col0 < ncols && rows > 0) {
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            double v = 0.0;
+                            if (col0 + c < t.n) {
+                                v = fx::from_fixed(w2[c0 + c], w1[c0 + c], w0[c0 + c], er + es[FM + col0 + c]);
+                                if (MODE == 1 && scale != 1.0) v *= scale;
+                            }
+                            if (MODE == 0)
+                                code = max(code, fx::exp_code((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v)));
+                            tr[lane * 9 + c] = v;
+                        }
+                        __syncwarp();
+                        const int c = lane & 7;
+                        for (int r = lane >> 3; r < rows; r += 4)
+                            if (col0 + c < ncols) {
+                                double* cp = C + (int64_t)r * t.ldc + col0 + c;
+                                const double v = tr[r * 9 + c];
+                                *cp = MODE == 1 && g.accumulate ? *cp + v : v;
+                            }
+                        __syncwarp();
+                    }
+                }
+                if (MODE == 0 && !g.to_y && lane < rows && 32 * h < ncols)
+                    *code_ptr(g, t, q * 32 + lane, 32 * h) = (uint16_t)code;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&edone[b]);
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_MMA));
+        if (warp == PW + EW && lane == 0) {
+            // -------------------------------------------- MMA issuer
+            uint32_t step = 0, ccount = 0, tcount = 0;
+            bool ok = true;
+            for (long i = 0; i < rounds && ok; ++i) {
+                const long item = item_of<MODE>(i);
+                if (item >= total) continue;
+                const Tile t = get_tile<MODE>(g, item);
+                if (t.m == 0) continue;
+                const int b = tcount & 1;
+                if (!(ok = mbar_wait(&tready[b], (tcount >> 1) & 1, abort_flag, g.err))) break;
+                ++tcount;
+                bool bad = false;
+                for (int w = 0; w < PW; ++w) bad |= ebad[b * PW + w] != 0;
+                mbar_arrive(&edone[b]);
+                if (bad) continue;
+                const uint32_t n16 = (uint32_t)((t.n + 15) & ~15);
+                for (int s = 0; s < t.steps; ++s, ++step) {
+                    const uint32_t st = step % FST;
+                    const bool first = s % FCH == 0;
+                    if (first) {
+                        if (!(ok = mbar_wait(tempty, (ccount & 1) ^ 1, abort_flag, g.err))) break;
+                        tc_fence_after();
+                    }
+                    if (!(ok = mbar_wait(&full[st], (step / FST) & 1, abort_flag, g.err))) break;
+                    tc_fence_after();
+                    const uint32_t blk = base + (st >> 1) * BLK + 32 * (st & 1);
+                    const uint64_t da = sdesc64(blk), db = sdesc64(blk + A_BLK);
+                    for (uint32_t d = 0; d < (uint32_t)FD; ++d) {
+                        const uint64_t a = da + d * (A_PLANE >> 4);
+                        const uint32_t cols = (FD - d) * n16;
+                        for (uint32_t c = 0; c < cols; c += 256) {
+                            const uint32_t n = cols - c < 256 ? cols - c : 256;
+                            umma_bf16(tmem + d * n16 + c, a, db + (c * 64 >> 4), idesc_f16(FM, n),
+                                      first && d == 0 ? 0u : 1u);
+                        }
+                    }
+                    umma_commit(&empty[st]);
+                    if (s % FCH == FCH - 1 || s + 1 == t.steps) {
+                        umma_commit(tfull);
+                        ++ccount;
+                    }
+                }
+            }
+            if (!ok) {
+                umma_commit(drain);
+                mbar_wait_drain(drain, 0);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == PW + EW) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
+// Exponent codes of operand rows: unit u covers up to 32 rows of one operand view, element
+// (r, k) at off + r rs + k ks; out[r] = the largest code of row r.
+__global__ void __launch_bounds__(256) row_code_kernel(const FxRows* __restrict__ units, const double* __restrict__ A,
+                                                       const double* __restrict__ B, uint16_t* __restrict__ out) {
+    __shared__ int part[8][32];
+    const FxRows u = units[blockIdx.x];
+    const double* src = (u.which ? B : A) + u.off;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto code = [](double v) { return fx::exp_code((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v)); };
+    if (u.ks == 1) {
+        // lanes along K; each warp four rows, loads of the four in flight together
+        int e[4] = {0, 0, 0, 0};
+        for (int k = lane; k < u.K; k += 32)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int r = warp + 8 * j;
+                if (r < u.rows) e[j] = max(e[j], code(src[(int64_t)r * u.rs + k]));
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            for (int o = 16; o > 0; o >>= 1) e[j] = max(e[j], __shfl_xor_sync(0xffffffffu, e[j], o));
+            if (lane == 0 && warp + 8 * j < u.rows) out[u.out + warp + 8 * j] = (uint16_t)e[j];
+        }
+    } else {
+        // lanes along the rows, warps along K
+        int e = 0;
+        if (lane < u.rows) {
+#pragma unroll 4
+            for (int k = warp; k < u.K; k += 8) e = max(e, code(src[(int64_t)lane * u.rs + (int64_t)k * u.ks]));
+        }
+        part[warp][lane] = e;
+        __syncthreads();
+        if (warp == 0 && lane < u.rows) {
+#pragma unroll
+            for (int w = 1; w < 8; ++w) e = max(e, part[w][lane]);
+            out[u.out + lane] = (uint16_t)e;
+        }
+    }
+}
+
+template <int MODE>
+int launch_fx(const FxArgs& g, int num_sms, cudaStream_t st) {
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(fx_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
+        if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+        attr = true;
+    }
+    const long total = (long)g.ntiles * (MODE == 0 ? g.nbatch : 1);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(total < num_sms ? total : num_sms));
+    cfg.blockDim = dim3(FTHREADS);
+    cfg.dynamicSmemBytes = FSMEM;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = HEFF_PDL ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fx_gemm_kernel<MODE>, g);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "fx_gemm launch: %s", cudaGetErrorString(e));
+    count_launches(1);
+    return HEFF_OK;
+}
+
+}  // namespace
+
+int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream) {
+    const GemmList& gl = which == 1 ? p->fx1 : p->fx2;
+    if (gl.tasks.empty()) return HEFF_OK;
+    char* w = static_cast<char*>(ws);
+    for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
+        FxArgs g{};
+        g.tasks = gl.d_tasks;
+        g.segs = gl.d_segs;
+        g.ntiles = (int)gl.tasks.size();
+        g.nbatch = nbatch - b0 < MAXB ? nbatch - b0 : MAXB;
+        g.b0 = b0;
+        g.err = reinterpret_cast<int*>(w + p->off_flags);
+        uint16_t* e_t = reinterpret_cast<uint16_t*>(w + p->off_et);
+        const int64_t t_rows = p->opts.max_batch * p->rows_t;
+        if (which == 1) {
+            g.A = reinterpret_cast<const double*>(w + p->off_lw);
+            g.B = reinterpret_cast<const double*>(w + p->off_xt);
+            g.ld = p->ld_x;
+            g.b_batch_rows = p->rows_x;
+            g.C = reinterpret_cast<double*>(w + p->off_t);
+            g.c_batch_elems = p->rows_t * p->ld_t;
+            g.c_batch_rows = p->rows_t;
+            if (codes) {
+                g.ea = reinterpret_cast<const uint16_t*>(w + p->off_elw);
+                g.ea_rows = p->rows_lw;
+                g.eb = reinterpret_cast<const uint16_t*>(w + p->off_ex);
+                g.eb_rows = p->opts.max_batch * p->rows_x;
+                g.et = e_t;
+                g.et_rows = t_rows;
+            }
+        } else {
+            g.A = reinterpret_cast<const double*>(w + p->off_t);
+            g.B = reinterpret_cast<const double*>(w + p->off_rw);
+            g.ld = p->ld_t;
+            g.a_batch_rows = p->rows_t;
+            for (int b = 0; b < g.nbatch; ++b) g.y.p[b] = y[b0 + b];
+            g.to_y = 1;
+            if (codes) {
+                g.ea = e_t;
+                g.ea_rows = t_rows;
+                g.eb = reinterpret_cast<const uint16_t*>(w + p->off_erw);
+                g.eb_rows = p->rows_rw;
+            }
+        }
+        int rc = launch_fx<0>(g, p->num_sms > 0 ? p->num_sms : 148, static_cast<cudaStream_t>(stream));
+        if (rc) return rc;
+    }
+    return HEFF_OK;
+}
+
+int launch_bgemm(const BList& b, const double* A, const double* B, double* C, const double* coef1,
+                 const double* coef2, double scale, void* stream, int* err, const double* inv_scale) {
+    if (b.tiles.empty()) return HEFF_OK;
+    if (b.tile_m != FM || b.tile_n != FN)
+        return fail(HEFF_ERR_INVALID_ARG, "FP64 block products need %d x %d tiles", FM, FN);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (!b.rows.empty()) {
+        row_code_kernel<<<(unsigned)b.rows.size(), 256, 0, st>>>(b.d_rows, A, B, b.d_codes);
+        count_launches(1);
+    }
+    FxArgs g{};
+    g.tiles = b.d_tiles;
+    g.prods = b.d_prods;
+    g.e = b.d_codes;
+    g.coef1 = coef1;
+    g.coef2 = coef2;
+    g.inv_scale = inv_scale;
+    g.scale = scale;
+    g.accumulate = b.accumulate ? 1 : 0;
+    g.ntiles = (int)b.tiles.size();
+    g.A = A;
+    g.B = B;
+    g.C = C;
+    g.err = err;
+    return launch_fx<1>(g, b.num_sms > 0 ? b.num_sms : 148, st);
+}
+
+}  // namespace heff

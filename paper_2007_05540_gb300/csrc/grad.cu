@@ -1,5 +1,5 @@
 // Gradients of the Rayleigh quotient rho = <x|K|x> / <x|x> of the two-site effective
-// Hamiltonian K (Section II-C), in FP64 on the block-product engine.  With n = <x|x>,
+// Hamiltonian K (Section II-C), on the block-product engine.  With n = <x|x>,
 // y = K x (computed by heff_apply on the caller's plan, any precision):
 //   d rho / d x = 2 (y - rho x) / n
 //   U[a', (t1 t2 wr), b]  = sum_b' x[a',t1,t2,b'] R[b',wr,b]
@@ -57,6 +57,7 @@ struct heff_grad_plan {
     int32_t *d_w12_off = nullptr, *d_w12_terms = nullptr;
     int32_t *d_dw1_off = nullptr, *d_dw1_terms = nullptr, *d_dw2_off = nullptr, *d_dw2_terms = nullptr;
     bool uploaded = false;
+    const void* last_ws = nullptr;    // workspace of the last call (its error flag is initialised)
 };
 
 namespace {
@@ -441,8 +442,9 @@ extern "C" int heff_backward(heff_grad_plan* g, heff_plan* plan, const double* L
     float* x32 = reinterpret_cast<float*>(ws + g->off_x32);
     float* L32 = reinterpret_cast<float*>(ws + g->off_L32);
     float* R32 = reinterpret_cast<float*>(ws + g->off_R32);
-    if (tc && cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess)
+    if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess)
         return fail(HEFF_ERR_CUDA, "heff_backward: memset failed");
+    g->last_ws = grad_ws;
     // y = K x into dx (dx is overwritten by the gradient below)
     int rc = heff_apply(plan, L, W1, W2, R, x, dx, apply_ws, apply_ws_bytes, stream);
     if (rc) return rc;
@@ -487,10 +489,10 @@ extern "C" int heff_backward(heff_grad_plan* g, heff_plan* plan, const double* L
             continue;
         }
         double *U = Ureg, *T1 = Ureg;
-        if ((rc = heff::launch_bgemm(c.U, x, R, U, nullptr, nullptr, 1.0, stream))) return rc;
-        if ((rc = heff::launch_bgemm(c.T1, L, x, T1, nullptr, nullptr, 1.0, stream))) return rc;
-        if ((rc = heff::launch_bgemm(c.dL, U, x, dL, W12, nullptr, 1.0, stream, sc))) return rc;
-        if ((rc = heff::launch_bgemm(c.dR, x, T1, dR, W12, nullptr, 1.0, stream, sc))) return rc;
+        if ((rc = heff::launch_bgemm(c.U, x, R, U, nullptr, nullptr, 1.0, stream, err))) return rc;
+        if ((rc = heff::launch_bgemm(c.T1, L, x, T1, nullptr, nullptr, 1.0, stream, err))) return rc;
+        if ((rc = heff::launch_bgemm(c.dL, U, x, dL, W12, nullptr, 1.0, stream, err, sc))) return rc;
+        if ((rc = heff::launch_bgemm(c.dR, x, T1, dR, W12, nullptr, 1.0, stream, err, sc))) return rc;
         if ((rc = heff::launch_block_dots(c.d_gdots, (int)c.gdots.size(), c.d_goff, T1, U, G, (int)g->ng, part, 1.0,
                                           stream, streamed)))
             return rc;
@@ -513,12 +515,12 @@ extern "C" int heff_grad_plan_set_precision(heff_grad_plan* g, int32_t precision
     if (precision != HEFF_PREC_FP64 && precision != HEFF_PREC_BF16X3)
         return fail(HEFF_ERR_UNSUPPORTED, "gradient block products run in HEFF_PREC_FP64 or HEFF_PREC_BF16X3");
     if (precision == g->precision) return HEFF_OK;
-    const int tile = precision == HEFF_PREC_FP64 ? 64 : 128;
+    const bool fx = precision == HEFF_PREC_FP64;
     int rc = HEFF_OK;
     for (GradChunk& c : g->chunks)
         for (BList* b : {&c.U, &c.T1, &c.dL, &c.dR}) {
             heff::blist_free(*b);
-            b->retile(tile, tile);
+            b->retile(fx ? heff::FX_TILE_M : 128, fx ? heff::FX_TILE_N : 128);
             if (g->uploaded && !rc) rc = heff::blist_upload(*b);
         }
     g->precision = precision;
@@ -530,7 +532,8 @@ extern "C" int heff_grad_plan_set_precision(heff_grad_plan* g, int32_t precision
 extern "C" int heff_grad_status(const heff_grad_plan* g, void* grad_ws, size_t grad_ws_bytes, void* stream) {
     heff::clear_error();
     if (!g || !grad_ws) return fail(HEFF_ERR_INVALID_ARG, "heff_grad_status: null argument");
-    if (g->precision == HEFF_PREC_FP64) return HEFF_OK;
+    // an FP64 plan's flag exists once a call has run in this workspace
+    if (g->precision == HEFF_PREC_FP64 && grad_ws != g->last_ws) return HEFF_OK;
     if (grad_ws_bytes < g->ws_bytes) return fail(HEFF_ERR_WORKSPACE, "heff_grad_status: workspace too small");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int* d = reinterpret_cast<int*>(static_cast<double*>(grad_ws) + g->off_flag);

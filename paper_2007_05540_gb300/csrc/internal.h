@@ -2,6 +2,7 @@
 // CUDA translation units.  Nothing here is part of the C ABI.
 #pragma once
 
+#include <array>
 #include <cstddef>
 #include <cstdint>
 #include <map>
@@ -87,22 +88,31 @@ struct KSeg {
 };
 
 // ---------------------------------------------------------------- block-product engine
-// One output tile C[m x n] (m, n <= 64) = scale * sum over its products of
+// One output tile C[m x n] = scale * sum over its products of
 //   coef * A[a_off + r * a_rs + k * a_cs] * B[b_off + k * b_rs + c * b_cs],  k < K,
-// coef = (c1 < 0 ? 1 : coef1[c1]) * (c2 < 0 ? 1 : coef2[c2]).  FP64 throughout.
+// coef = (c1 < 0 ? 1 : coef1[c1]) * (c2 < 0 ? 1 : coef2[c2]).
 struct BProd {
     int64_t a_off, b_off;
     int32_t a_rs, a_cs, b_rs, b_cs;
     int32_t K;
     int32_t c1, c2;
-    int32_t pad_;
+    int32_t ea, eb;         // FP64 lists: exponent codes of the A rows and of the B columns
 };
 struct BTile {
     int64_t c_off;
     int32_t ldc, m, n;
     int32_t prod_begin, prod_count;
-    int32_t pad_;
+    int32_t steps;          // FP64 lists: steps of 16 contraction elements, each product rounded up
 };
+// up to 32 rows of one operand view whose exponent codes an FP64 list needs
+struct FxRows {
+    int64_t off;
+    int32_t rs, ks, rows, K;
+    int32_t out;            // first code
+    int32_t which;          // 0: A, 1: B
+};
+// output tile of the FP64 products (fx_gemm.cu)
+constexpr int FX_TILE_M = 128, FX_TILE_N = 64;
 struct BList {
     std::vector<BTile> tiles;
     std::vector<BProd> prods;
@@ -110,7 +120,17 @@ struct BList {
     BProd* d_prods = nullptr;
     double flops = 0;
     bool accumulate = false;   // C += result instead of C = result
-    int tile_m = 64, tile_n = 64;   // output tile shape the block list is cut into
+    // output tile shape the block list is cut into: FP64 products, or 128 x 128 (tensor cores, BF16x3)
+    int tile_m = FX_TILE_M, tile_n = FX_TILE_N;
+    // FP64 products: the operand rows and columns whose exponent codes they need, one slot per
+    // row of each distinct view of an operand block; the codes are recomputed on every call
+    std::vector<FxRows> rows;
+    FxRows* d_rows = nullptr;
+    uint16_t* d_codes = nullptr;
+    int32_t ncodes = 0;
+    std::map<std::array<int64_t, 6>, int32_t> views;
+    int num_sms = 0;
+    int32_t view_codes(int which, int64_t off, int32_t rs, int32_t ks, int32_t n, int32_t K);
     // the output blocks as added (products given for the block origin), kept for re-tiling
     struct Block { int64_t c_off; int32_t ldc, m, n, prod_begin, prod_count; };
     std::vector<Block> blocks;
@@ -122,8 +142,10 @@ struct BList {
 };
 int blist_upload(BList& b);
 void blist_free(BList& b);
+// the list's products in FP64 accuracy (fixed-point digits on the tensor cores, fx_gemm.cu); err:
+// device int raised when a bounded wait expires
 int launch_bgemm(const BList& b, const double* A, const double* B, double* C, const double* coef1,
-                 const double* coef2, double scale, void* stream, const double* inv_scale = nullptr);
+                 const double* coef2, double scale, void* stream, int* err, const double* inv_scale = nullptr);
 // the same products on the tensor cores (BF16x3 split, FP32 accumulation; blockops_tc.cu)
 // on FP32 copies of the operands (launch_convert_f64_f32), with an FP32 (c_f64 false) or
 // FP64 output; needs 128 x 128 tiles (retile); err: device int raised when a bounded wait
@@ -204,6 +226,10 @@ struct heff_plan {
     heff::GemmList g1, g2;            // active task lists
     heff::GemmList g1_alt, g2_alt;    // the other tile width (tensor-core paths), see heff_plan_autotune
     heff::GemmList g1_pair, g2_pair;  // N = 256 tiles in CTA pairs sharing B (tensor-core paths)
+    heff::GemmList fx1, fx2;          // FP64 plans: the task lists that run (FX_TILE_M x FX_TILE_N tiles)
+    // FP64 plans: exponent codes of the operand arrays, [column / KPAD][row]; they come last in the
+    // workspace (ws_min: its size without them, when every tile runs in FP64 arithmetic)
+    size_t off_ex = 0, off_elw = 0, off_et = 0, off_erw = 0, ws_min = 0;
     int64_t stats[24] = {0};
     // tensor-map cache for the tensor-core path: two entries keyed by workspace pointer
     // (two streams alternating workspaces reuse their maps), replaced round-robin
@@ -221,10 +247,15 @@ struct heff_plan {
 
 namespace heff {
 // launchers (apply.cu)
-int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, void* stream);
+// (codes: FP64 plans keep the operands' exponent codes in the workspace)
+int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, bool codes, void* stream);
 int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R,
-               void* ws, void* stream);
-int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
+               void* ws, bool codes, void* stream);
+int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream);
+int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream);
+// one apply in the first `bytes` of ws, which may hold less than ws_bytes but at least ws_min
+int apply_in(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, const void* x, void* y,
+             void* ws, size_t bytes, void* stream);
 // clusters of two tensor-core CTAs resident at once (tc_gemm.cu; num_sms / 2 without a device)
 int tc_pair_clusters(int num_sms, int precision);
 // one block waiting at the SVD sweeps' grid barrier set up for two (svd.cu; wait self-test)

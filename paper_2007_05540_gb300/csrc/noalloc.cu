@@ -45,8 +45,9 @@ extern "C" int heff_apply_noalloc(heff_plan* plan, const void* L, const void* W1
                                   const void* R, const void* x, void* y, void* stream) {
     heff::clear_error();
     if (!plan) return fail(HEFF_ERR_INVALID_ARG, "heff_apply_noalloc: null plan");
-    size_t need = 0;
-    heff_plan_workspace_size(plan, &need);
+    // an FP64 plan also fits without the room for its operands' exponent codes (it then runs every
+    // tile in FP64 arithmetic)
+    const size_t need = plan->ws_min;
     if (need > (size_t)HEFF_NOALLOC_WORKSPACE_BYTES)
         return fail(HEFF_ERR_WORKSPACE,
                     "heff_apply_noalloc: the plan needs %zu bytes of workspace, the built-in array holds %zu "
@@ -66,6 +67,12 @@ extern "C" int heff_apply_noalloc(heff_plan* plan, const void* L, const void* W1
     e = cudaMemsetAsync(static_cast<char*>(ws) + plan->off_flags, 0, 256,
                         static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+    if (plan->ws_bytes > (size_t)HEFF_NOALLOC_WORKSPACE_BYTES && plan->nelem_x > 0) {
+        if (!L || !W1 || !W2 || !R || !x || !y) return fail(HEFF_ERR_INVALID_ARG, "heff_apply: null argument");
+        if (x == y) return fail(HEFF_ERR_INVALID_ARG, "y must not alias x");
+        if (!plan->uploaded) return fail(HEFF_ERR_UNSUPPORTED, "plan was created without a CUDA device");
+        return heff::apply_in(plan, L, W1, W2, R, x, y, ws, (size_t)HEFF_NOALLOC_WORKSPACE_BYTES, stream);
+    }
     return heff_apply(plan, L, W1, W2, R, x, y, ws, (size_t)HEFF_NOALLOC_WORKSPACE_BYTES, stream);
 }
 

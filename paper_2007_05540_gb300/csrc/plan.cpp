@@ -597,7 +597,8 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
         };
         const bool tc = opts->precision != HEFF_PREC_FP64;
         if (!build_lists(tc ? 128 : 64, tc ? 256 : 64, P->g1, P->g2) ||
-            (tc && !build_lists(128, 128, P->g1_alt, P->g2_alt))) {
+            (tc ? !build_lists(128, 128, P->g1_alt, P->g2_alt)
+                : !build_lists(heff::FX_TILE_M, heff::FX_TILE_N, P->fx1, P->fx2))) {
             delete P;
             return fail(HEFF_ERR_CHARGE_MISMATCH, "internal: y block missing");
         }
@@ -631,7 +632,7 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
             P->stats[16] = (int64_t)c1;
             P->stats[17] = (int64_t)c2;
         }
-        for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt}) keep_owned(*G, owned);
+        for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->fx1, &P->fx2}) keep_owned(*G, owned);
         // ---- CTA pairs (tensor-core paths): N = 256 tiles with the same B rows, width and K
         // segments go two to an entry, so that one read of each B box serves both CTAs of a
         // cluster.  A tile left without a partner gets a ghost (no rows: it loads its half of
@@ -697,8 +698,9 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
         // time ~ (K blocks + a fixed overhead) x MMA width) and interleave the per-CTA lists
         // in that pattern, padding short lists with empty tasks (no rows, no segments).
         // CTA pairs are scheduled the same way, an entry (two tasks) per cluster.
-        if (tc && HEFF_LPT_SCHEDULE) {
-            for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->g1_pair, &P->g2_pair}) {
+        if (HEFF_LPT_SCHEDULE) {
+            for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->g1_pair, &P->g2_pair, &P->fx1, &P->fx2}) {
+                if (!tc && (G == &P->g1 || G == &P->g2)) continue;    // 64 x 64 tiles: only described, not run
                 const int model = (G == &P->g1 || G == &P->g1_alt || G == &P->g1_pair) ? HEFF_TILE_COST_G1
                                                                                         : HEFF_TILE_COST_G2;
                 const size_t CLn = (size_t)G->cl;
@@ -709,7 +711,8 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
                 for (size_t t = 0; t < nt; ++t)
                     for (size_t r = 0; r < CLn; ++r) {
                         const heff::GemmTask& k = G->tasks[t * CLn + r];
-                        work[t] = std::max(work[t], (double)(k.ktotal / KPAD + 4) * tile_width_cost(k.m, k.n, model));
+                        work[t] = std::max(work[t], tc ? (double)(k.ktotal / KPAD + 4) * tile_width_cost(k.m, k.n, model)
+                                                       : (double)(k.ktotal / KPAD + 4) * (k.n + 32));
                     }
                 std::vector<size_t> ord(nt);
                 for (size_t t = 0; t < nt; ++t) ord[t] = t;
@@ -764,6 +767,14 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
         P->off_t = off;  off = al(off + e * (size_t)opts->max_batch * P->rows_t * P->ld_t);
         P->off_rw = off; off = al(off + e * (size_t)P->rows_rw * P->ld_t);
         P->off_flags = off; off = al(off + 256);
+        P->ws_min = off;
+        if (!tc) {
+            const size_t kx = (size_t)(P->ld_x / KPAD) * sizeof(uint16_t), kt = (size_t)(P->ld_t / KPAD) * sizeof(uint16_t);
+            P->off_ex = off;  off = al(off + kx * opts->max_batch * P->rows_x);
+            P->off_elw = off; off = al(off + kx * P->rows_lw);
+            P->off_et = off;  off = al(off + kt * opts->max_batch * P->rows_t);
+            P->off_erw = off; off = al(off + kt * P->rows_rw);
+        }
         P->ws_bytes = off;
         int64_t* st = P->stats;
         st[0] = (int64_t)Q.size(); st[1] = (int64_t)rgs.size(); st[2] = (int64_t)rws.size();

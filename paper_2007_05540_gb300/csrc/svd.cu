@@ -904,12 +904,12 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
     svd_v_to_f64_kernel<<<dim3(128, nsec), 256, 0, st>>>(S->d_sec, f32, ws);
     heff::count_launches(1);
     for (int it = 0; it < 2; ++it) {
-        if ((rc = heff::launch_bgemm(S->gram, ws, ws, ws, nullptr, nullptr, 1.0, stream))) return rc;
-        if ((rc = heff::launch_bgemm(S->vg, ws, ws, ws, nullptr, nullptr, -0.5, stream))) return rc;
+        if ((rc = heff::launch_bgemm(S->gram, ws, ws, ws, nullptr, nullptr, 1.0, stream, d_err))) return rc;
+        if ((rc = heff::launch_bgemm(S->vg, ws, ws, ws, nullptr, nullptr, -0.5, stream, d_err))) return rc;
         svd_ns_kernel<<<dim3(128, nsec), 256, 0, st>>>(S->d_sec, ws);
         heff::count_launches(1);
     }
-    if ((rc = heff::launch_bgemm(S->jv, ws, ws, ws, nullptr, nullptr, 1.0, stream))) return rc;
+    if ((rc = heff::launch_bgemm(S->jv, ws, ws, ws, nullptr, nullptr, 1.0, stream, d_err))) return rc;
     svd_copy_w_kernel<<<dim3(128, nsec), 256, 0, st>>>(S->d_sec, ws);
     heff::count_launches(1);
     // FP64 sweeps to convergence: off-diagonal measure 1e-14, i.e. stop after the sweep that

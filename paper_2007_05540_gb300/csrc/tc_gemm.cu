@@ -948,7 +948,9 @@ extern "C" int heff_workspace_status(const heff_plan* plan, void* workspace, siz
                                      void* stream) {
     using namespace heff;
     if (!plan || !workspace) return fail(HEFF_ERR_INVALID_ARG, "heff_workspace_status: null plan/workspace");
-    if (plan->opts.precision == HEFF_PREC_FP64) return HEFF_OK;
+    // an FP64 plan's flag exists once an apply has run in this workspace
+    if (plan->opts.precision == HEFF_PREC_FP64 && plan->tmap_ws[0] != workspace && plan->tmap_ws[1] != workspace)
+        return HEFF_OK;
     if (workspace_bytes < plan->off_flags + 256)
         return fail(HEFF_ERR_WORKSPACE, "heff_workspace_status: workspace smaller than the plan's");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
