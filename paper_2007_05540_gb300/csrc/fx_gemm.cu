@@ -202,63 +202,123 @@ __device__ __forceinline__ int row_scale(const FxArgs& g, const Tile& t, int sid
     return E ? E : fx::E_ZERO;
 }
 
-// Eight K values k0 .. k0 + 7 of one row (zeros beyond K or for an absent row).
-__device__ __forceinline__ void load8(double (&v)[8], const double* row, int ks, int k0, int K, bool have, bool vec) {
-    if (have && k0 + 8 <= K) {
-        if (vec) {
-            const double2* p = reinterpret_cast<const double2*>(row + k0);
+// byte offset of the 8-element chunk h of row r in a plane, on the even steps of the ring (the
+// odd ones lie 32 bytes further in the swizzled row: the offset ^ 32)
+__device__ __forceinline__ uint32_t chunk_off(int r, int h) {
+    return (uint32_t)r * 64 + ((uint32_t)(h ^ ((r >> 1) & 3)) << 4);
+}
+
+// A producer thread's walk over one operand of a tile: its row, and the eight K values of each
+// step that it loads and converts.  SIDE 0: A, SIDE 1: B.
+template <int MODE, int SIDE>
+struct Walk {
+    const double* p;        // this thread's first element of the step
+    int ks;                 // stride along K (MODE 0: 1)
+    int left;               // elements of the product from there on (beyond them: zeros)
+    int i, end;             // product, and the elements of it that the step's first half starts at
+    int h;                  // which 8 of the step's 16 elements
+    int E;                  // scale of the row
+    uint32_t off;           // where the digits go; ~0 for an absent row
+    double coef;
+
+    __device__ __forceinline__ void place(int r, int rows, const int* es) {
+        off = r < rows ? chunk_off(r, h) : ~0u;
+        E = es[SIDE * FM + r];
+    }
+    // the first step of product n
+    __device__ __forceinline__ void set(const FxArgs& g, const Tile& t, const int* es, int n) {
+        i = n;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        // K contiguous: 16 rows x 2 halves a warp, in an order that spreads its stores over the
+        // banks; rows contiguous: 32 rows, one half
+        const int rl = ((lane >> 1) & 1) | ((lane >> 2) & 1) << 2 | ((lane >> 3) & 1) << 1 | ((lane >> 4) & 1) << 3;
+        if constexpr (MODE == 0) {
+            const KSeg s = g.segs[t.pbeg + n];
+            end = s.klen;
+            h = lane & 1;
+            const int r = (SIDE ? warp & 3 : warp) * 16 + rl;
+            p = (SIDE ? g.B : g.A) + ((SIDE ? t.b_row : t.a_row) + r) * g.ld + s.k0 + 8 * h;
+            ks = 1;
+            place(r, SIDE ? t.n : t.m, es);
+        } else {
+            const BProd& q = g.prods[t.pbeg + n];
+            end = q.K;
+            ks = SIDE ? q.b_rs : q.a_cs;
+            const int w = SIDE ? warp & 3 : warp;
+            int r;
+            if (ks == 1) {
+                r = w * 16 + rl;
+                h = lane & 1;
+            } else {
+                r = (SIDE ? w & 1 : w & 3) * 32 + lane;
+                h = SIDE ? w >> 1 : w >> 2;
+            }
+            p = (SIDE ? g.B + q.b_off : g.A + q.a_off) + (int64_t)r * (SIDE ? q.b_cs : q.a_rs) + (int64_t)8 * h * ks;
+            if (SIDE == 0) coef = prod_coef(g, q);
+            place(r, SIDE ? t.n : t.m, es);
+        }
+        left = off != ~0u ? end - 8 * h : 0;
+    }
+    // the next step (pcnt products in all)
+    __device__ __forceinline__ void next(const FxArgs& g, const Tile& t, const int* es) {
+        end -= FKS;
+        if (end > 0) {
+            p += MODE == 0 ? (int64_t)FKS : (int64_t)FKS * ks;
+            left -= FKS;
+        } else if (i + 1 < t.pcnt) {
+            set(g, t, es, i + 1);
+        } else {
+            left = 0;
+        }
+    }
+    __device__ __forceinline__ void load(double (&v)[8]) const {
+        if (left >= 8) {
+            if (MODE == 0 || (ks == 1 && (reinterpret_cast<uintptr_t>(p) & 15) == 0)) {
+                const double2* q = reinterpret_cast<const double2*>(p);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const double2 d = __ldg(p + i);
-                v[2 * i] = d.x;
-                v[2 * i + 1] = d.y;
+                for (int e = 0; e < 4; ++e) {
+                    const double2 d = __ldg(q + e);
+                    v[2 * e] = d.x;
+                    v[2 * e + 1] = d.y;
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = __ldg(p + (int64_t)e * ks);
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = row[(int64_t)(k0 + i) * ks];
+            for (int e = 0; e < 8; ++e) v[e] = e < left ? __ldg(p + (int64_t)e * ks) : 0.0;
         }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = have && k0 + i < K ? row[(int64_t)(k0 + i) * ks] : 0.0;
     }
-}
+};
 
 // Digits of eight K values into the eight planes (plane bytes apart), 16 bytes each at addr.
 __device__ __forceinline__ void digits8(const double (&v)[8], int E, uint32_t addr, uint32_t plane) {
-    uint32_t d[FD][4];
+    uint64_t q[8];
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        uint64_t q[2];
+    for (int e = 0; e < 8; ++e)
+        q[e] = fx::to_fixed((uint32_t)__double2hiint(v[e]), (uint32_t)__double2loint(v[e]), E);
+    // bytes of two elements side by side, each in the low byte of an FP16 1024 + b, of which
+    // 1152 is taken off: the digit.  Planes in pairs, to keep few registers alive.
+    const __half2 bias = __half2half2(__ushort_as_half((unsigned short)0x6480));
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const double x = v[2 * p + u];
-            q[u] = fx::to_fixed((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x), E);
-        }
-        // bytes of the two elements side by side, each in the low byte of an FP16 1024 + b;
-        // 1024 + b - 1152 is the digit
-        const __half2 off = __half2half2(__ushort_as_half((unsigned short)0x6480));
+    for (int pair = 3; pair >= 0; --pair) {
+        uint32_t d[2][4];
 #pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            const uint32_t x = (uint32_t)(q[0] >> (32 * w)), y = (uint32_t)(q[1] >> (32 * w));
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t x = (uint32_t)(q[2 * e] >> (32 * (pair >> 1)));
+            const uint32_t y = (uint32_t)(q[2 * e + 1] >> (32 * (pair >> 1)));
+            const uint32_t t = __byte_perm(x, y, (pair & 1) ? 0x7362 : 0x5140);
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const uint32_t t = __byte_perm(x, y, b ? 0x7362 : 0x5140);
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const uint32_t f = __byte_perm(t, 0x64646464u, c ? 0x4342 : 0x4140);
-                    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&f), off);
-                    d[7 - (4 * w + 2 * b + c)][p] = *reinterpret_cast<const uint32_t*>(&h);
-                }
+            for (int c = 0; c < 2; ++c) {
+                const uint32_t f = __byte_perm(t, 0x64646464u, c ? 0x4342 : 0x4140);
+                const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&f), bias);
+                d[c][e] = *reinterpret_cast<const uint32_t*>(&hv);
             }
         }
+        st_shared_v4(addr + (6 - 2 * pair) * plane, d[1][0], d[1][1], d[1][2], d[1][3]);
+        st_shared_v4(addr + (7 - 2 * pair) * plane, d[0][0], d[0][1], d[0][2], d[0][3]);
     }
-#pragma unroll
-    for (int s = 0; s < FD; ++s) st_shared_v4(addr + s * plane, d[s][0], d[s][1], d[s][2], d[s][3]);
-}
-
-// byte offset of the 8-element chunk (half step h of the ring step st) of row r in a plane
-__device__ __forceinline__ uint32_t chunk_off(int r, uint32_t st, int h) {
-    return (uint32_t)r * 64 + (((2 * (st & 1) + h) ^ ((r >> 1) & 3)) << 4);
 }
 
 __device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t& a, uint32_t& b) {
@@ -277,6 +337,31 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t (&d)[FD][2]) {
 // FP16 operands, FP32 accumulate, K-major, M x N
 __device__ __forceinline__ uint32_t idesc_f16(uint32_t M, uint32_t N) {
     return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
+}
+
+// The digit products of one step (16 contraction elements) or, with NK = 2, of the two steps of a
+// 64-byte block, for B planes of N16 rows: A plane d times the B planes 0 .. 7 - d.  The two steps
+// follow each other on the same operand shape, and everything but the base addresses is a
+// constant: issued from a plain loop over the planes a step takes 1600 cycles at N16 = 64 (the
+// tensor pipe needs 1152), in this order 1250.
+template <int N16, int NK>
+__device__ __forceinline__ void issue_planes(uint32_t tmem, uint64_t a, uint64_t b, uint32_t fresh) {
+#pragma unroll
+    for (int d = 0; d < FD; ++d)
+#pragma unroll
+        for (int c = 0; c < (FD - d) * N16; c += 256)
+#pragma unroll
+            for (int k = 0; k < NK; ++k)
+                umma_bf16(tmem + d * N16 + c, a + d * (A_PLANE >> 4) + 2 * k, b + (c * 64 >> 4) + 2 * k,
+                          idesc_f16(FM, (FD - d) * N16 - c < 256 ? (FD - d) * N16 - c : 256),
+                          d == 0 && k == 0 ? (fresh ? 0u : 1u) : 1u);
+}
+template <int NK>
+__device__ __forceinline__ void issue_step(int n16, uint32_t tmem, uint64_t a, uint64_t b, uint32_t fresh) {
+    if (n16 == 64) issue_planes<64, NK>(tmem, a, b, fresh);
+    else if (n16 == 48) issue_planes<48, NK>(tmem, a, b, fresh);
+    else if (n16 == 32) issue_planes<32, NK>(tmem, a, b, fresh);
+    else issue_planes<16, NK>(tmem, a, b, fresh);
 }
 
 template <int MODE>
@@ -416,8 +501,6 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
         const double scale = MODE == 1 ? (g.inv_scale ? g.scale / g.inv_scale[0] : g.scale) : 1.0;
         uint32_t step = 0, tcount = 0;
         bool ok = true;
-        // rows of a warp's 16-row group in an order that spreads its stores over the banks
-        const int rl = ((lane >> 1) & 1) | ((lane >> 2) & 1) << 2 | ((lane >> 3) & 1) << 1 | ((lane >> 4) & 1) << 3;
         for (long i = 0; i < rounds && ok; ++i) {
             const long item = item_of<MODE>(i);
             if (item >= total) continue;
@@ -446,66 +529,42 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                 continue;
             }
             if (t.steps == 0) continue;
-            const int n16 = (t.n + 15) & ~15;
-            const uint32_t bplane = (uint32_t)n16 * 64;
-            // warp w converts A rows (two 8-element halves of 16 rows, or one half of 32 rows);
-            // B (64 rows) takes four warps: warps 0-3 on even steps, 4-7 on odd steps
-            Prod p = get_prod<MODE>(g, t, 0);
-            int pi = 0, k = 0;
+            const uint32_t bplane = (uint32_t)((t.n + 15) & ~15) * 64;
+            // warp w converts 16 (or half of 32) rows of A on every step; B has half as many rows:
+            // warps 0-3 convert it on even steps, warps 4-7 on odd steps.  The loads of the next
+            // item are issued before an item is converted.
+            Walk<MODE, 0> wa;
+            Walk<MODE, 1> wb;
             double va[8], vb[8];
-            auto load_a = [&](const Prod& q, int kk) {
-                if (q.acs == 1) {
-                    const int r = warp * 16 + rl;
-                    const double* row = q.a + (int64_t)r * q.ars;
-                    load8(va, row, 1, kk + 8 * (lane & 1), q.K, r < t.m,
-                          MODE == 0 || (reinterpret_cast<uintptr_t>(row) & 15) == 0);
-                } else {
-                    const int r = (warp & 3) * 32 + lane;
-                    load8(va, q.a + (int64_t)r * q.ars, q.acs, kk + 8 * (warp >> 2), q.K, r < t.m, false);
-                }
-            };
-            auto load_b = [&](const Prod& q, int kk) {
-                const int w = warp & 3;
-                if (q.brs == 1) {
-                    const int r = w * 16 + rl;
-                    const double* row = q.b + (int64_t)r * q.bcs;
-                    load8(vb, row, 1, kk + 8 * (lane & 1), q.K, r < t.n,
-                          MODE == 0 || (reinterpret_cast<uintptr_t>(row) & 15) == 0);
-                } else {
-                    const int r = (w & 1) * 32 + lane;
-                    load8(vb, q.b + (int64_t)r * q.bcs, q.brs, kk + 8 * (w >> 1), q.K, r < t.n, false);
-                }
-            };
-            load_a(p, 0);
+            wa.set(g, t, es, 0);
+            wa.load(va);
+            wb.set(g, t, es, 0);
+            if (((step & 1) != 0) != (warp >= 4)) wb.next(g, t, es);
+            wb.load(vb);
             for (int s = 0; s < t.steps; ++s, ++step) {
                 const uint32_t st = step % FST;
-                const bool mine_b = ((step & 1) != 0) == (warp >= 4);
-                const bool ka = p.acs == 1, kb = p.brs == 1;
-                const double coef = p.coef;
-                if (mine_b) load_b(p, k);
+                double cur[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) cur[e] = va[e];
+                const int E = wa.E;
+                const uint32_t off = wa.off, odd = 32 * (st & 1);
+                if (MODE == 1) {
+                    const double coef = wa.coef;
+                    if (coef != 1.0) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) cur[e] *= coef;
+                    }
+                }
+                wa.next(g, t, es);
+                wa.load(va);
                 const uint32_t blk = base + (st >> 1) * BLK;
                 if (!(ok = mbar_wait(&empty[st], ((step / FST) & 1) ^ 1, abort_flag, g.err))) break;
-                {
-                    const int r = ka ? warp * 16 + rl : (warp & 3) * 32 + lane;
-                    const int h = ka ? lane & 1 : warp >> 2;
-                    if (MODE == 1 && coef != 1.0) {
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) va[e] *= coef;
-                    }
-                    if (r < t.m) digits8(va, es[r], blk + chunk_off(r, st, h), A_PLANE);
-                }
-                // the next step's A rows are on their way while this step's B is converted
-                k += FKS;
-                if (k >= p.K && s + 1 < t.steps) {
-                    k = 0;
-                    p = get_prod<MODE>(g, t, ++pi);
-                }
-                if (s + 1 < t.steps) load_a(p, k);
-                if (mine_b) {
-                    const int w = warp & 3;
-                    const int r = kb ? w * 16 + rl : (w & 1) * 32 + lane;
-                    const int h = kb ? lane & 1 : w >> 1;
-                    if (r < t.n) digits8(vb, es[FM + r], blk + A_BLK + chunk_off(r, st, h), bplane);
+                if (off != ~0u) digits8(cur, E, blk + (off ^ odd), A_PLANE);
+                if (((step & 1) != 0) == (warp >= 4)) {
+                    if (wb.off != ~0u) digits8(vb, wb.E, blk + A_BLK + (wb.off ^ odd), bplane);
+                    wb.next(g, t, es);
+                    wb.next(g, t, es);
+                    wb.load(vb);
                 }
                 fence_async_smem();
                 __syncwarp();
@@ -626,29 +685,28 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                 for (int w = 0; w < PW; ++w) bad |= ebad[b * PW + w] != 0;
                 mbar_arrive(&edone[b]);
                 if (bad) continue;
-                const uint32_t n16 = (uint32_t)((t.n + 15) & ~15);
-                for (int s = 0; s < t.steps; ++s, ++step) {
+                const int n16 = (t.n + 15) & ~15;
+                for (int s = 0; s < t.steps;) {
                     const uint32_t st = step % FST;
                     const bool first = s % FCH == 0;
+                    // both steps of a 64-byte block, unless the tile or its chunk ends in between
+                    const bool two = !(st & 1) && s + 1 < t.steps && s % FCH != FCH - 1;
                     if (first) {
                         if (!(ok = mbar_wait(tempty, (ccount & 1) ^ 1, abort_flag, g.err))) break;
                         tc_fence_after();
                     }
                     if (!(ok = mbar_wait(&full[st], (step / FST) & 1, abort_flag, g.err))) break;
+                    if (two && !(ok = mbar_wait(&full[st + 1], (step / FST) & 1, abort_flag, g.err))) break;
                     tc_fence_after();
                     const uint32_t blk = base + (st >> 1) * BLK + 32 * (st & 1);
                     const uint64_t da = sdesc64(blk), db = sdesc64(blk + A_BLK);
-                    for (uint32_t d = 0; d < (uint32_t)FD; ++d) {
-                        const uint64_t a = da + d * (A_PLANE >> 4);
-                        const uint32_t cols = (FD - d) * n16;
-                        for (uint32_t c = 0; c < cols; c += 256) {
-                            const uint32_t n = cols - c < 256 ? cols - c : 256;
-                            umma_bf16(tmem + d * n16 + c, a, db + (c * 64 >> 4), idesc_f16(FM, n),
-                                      first && d == 0 ? 0u : 1u);
-                        }
-                    }
+                    if (two) issue_step<2>(n16, tmem, da, db, first);
+                    else issue_step<1>(n16, tmem, da, db, first);
                     umma_commit(&empty[st]);
-                    if (s % FCH == FCH - 1 || s + 1 == t.steps) {
+                    if (two) umma_commit(&empty[st + 1]);
+                    s += two ? 2 : 1;
+                    step += two ? 2 : 1;
+                    if (s % FCH == 0 || s == t.steps) {
                         umma_commit(tfull);
                         ++ccount;
                     }
