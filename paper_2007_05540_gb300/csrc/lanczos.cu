@@ -3,7 +3,7 @@
 // the Davidson routine of Algorithm 1).
 //
 // Every vector operation runs in FP64 on the device and the loop never synchronises with
-// the host.  Per iteration k:
+// the host.  Per iteration k, the matvec and one cooperative kernel (lz_step_kernel):
 //   w = H v_k                       (heff_apply_prepared; any precision, FP64 vectors)
 //   a = v_k . (w - beta_{k-1} v_{k-1}),  w -= beta_{k-1} v_{k-1} + a v_k
 //                                   (the three-term recurrence, with ||w||^2 after it)
@@ -22,10 +22,15 @@
 // normalised.  If beta_k falls below 1e-13 |alpha_k| the Krylov space is invariant: the
 // remaining iterations become no-ops and the eigenproblem uses the k + 1 vectors built.
 // Reductions are two-stage with a fixed order, so results are deterministic.
+//
+// One step's vector work was twelve launches whose kernels ran 3-16 us each; at m = 1024 (n =
+// 232k) they took 120 us of a 216 us step.  In one kernel the phases meet at grid barriers (about
+// 2 us each) and w stays in shared memory between them.
 #include <cuda_runtime.h>
 
 #include <cmath>
 
+#include "barrier.cuh"
 #include "internal.h"
 
 using heff::fail;
@@ -37,18 +42,15 @@ constexpr int RT = 256;          // threads per reduction block
 constexpr int RB = 456;          // reduction blocks (partial sums per vector): 3 per SM on 152 SMs
 constexpr int VT = 8;            // vectors per multi-dot pass
 
-constexpr int GMAX = 4096;       // largest grid of the element-wise kernels (grid_for)
 constexpr int NVMAX = 128;       // basis vectors of one Lanczos workspace, at most
 
 // State in the Lanczos workspace (doubles): [0] n_eff (as double), [1] active flag,
-// [2] theta, [3] residual estimate, [4] second Gram-Schmidt pass needed (this step),
-// [8..8+NMAX) alpha, [8+NMAX..) beta, then h (NMAX), s (NMAX), partials (RB * NVMAX), the
-// partial sums of ||w||^2 after the three-term update (RB) and after a Gram-Schmidt pass
-// (GMAX), and a (the three-term projection of the current step).
+// [2] theta, [3] residual estimate, [8..8+NMAX) alpha, [8+NMAX..) beta; then s (NMAX), partial
+// sums (RB blocks x (NVMAX + 2)), the grid barrier's words, and the vectors.
 struct LzLayout {
     int nmax;
     int64_t n;
-    size_t off_state, off_h, off_s, off_part, off_wn, off_sq, off_a, off_T, off_V, bytes;
+    size_t off_state, off_s, off_part, off_bar, off_V, bytes;
 };
 
 LzLayout lz_layout(int64_t n, int n_iter) {
@@ -58,31 +60,23 @@ LzLayout lz_layout(int64_t n, int n_iter) {
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     size_t o = 0;
     l.off_state = o; o = al(o + sizeof(double) * (8 + 2 * (size_t)l.nmax));
-    l.off_h = o;     o = al(o + sizeof(double) * (size_t)l.nmax);
     l.off_s = o;     o = al(o + sizeof(double) * (size_t)l.nmax);
-    l.off_part = o;  o = al(o + sizeof(double) * (size_t)RB * NVMAX);
-    l.off_wn = o;    o = al(o + sizeof(double) * (size_t)RB);
-    l.off_sq = o;    o = al(o + sizeof(double) * (size_t)GMAX);
-    l.off_a = o;     o = al(o + sizeof(double));
-    l.off_T = o;     o = al(o + sizeof(double) * 2 * (size_t)l.nmax * l.nmax);
+    l.off_part = o;  o = al(o + sizeof(double) * (size_t)RB * (NVMAX + 2));
+    l.off_bar = o;   o = al(o + 3 * sizeof(unsigned int));
     l.off_V = o;     o = al(o + sizeof(double) * (size_t)(l.nmax + 1) * (size_t)n);   // V + w
     l.bytes = o;
     return l;
 }
 
 struct Lz {
-    double* state;   // n_eff, active, theta, resid, second pass, alpha[nmax], beta[nmax]
-    double* h;
-    double* s;
-    double* part;
-    double* wn;      // partial sums of ||w||^2 after the three-term update (RB)
-    double* sq;      // partial sums of ||w||^2 after a combine (one per block of its grid)
-    double* a;       // the three-term projection a of the current step
-    double* T;       // nmax x nmax matrix + nmax x nmax eigenvectors
+    double* state;   // n_eff, active, theta, resid, -, ..., alpha[nmax], beta[nmax]
+    double* s;       // eigenvector of the tridiagonal matrix
+    double* part;    // partial sums, [quantity][block]
+    unsigned int* bar;   // grid barrier: counter, generation, error
     double* V;       // (nmax) basis vectors, then w
     int64_t n;
     int nmax;
-    double* w() const { return V + (int64_t)nmax * n; }
+    __host__ __device__ double* w() const { return V + (int64_t)nmax * n; }
 };
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
@@ -95,12 +89,6 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     __syncthreads();
     return v;
-}
-
-// Whether a gated kernel runs: gate 0 while the iteration is active, gate 1 only when the
-// active step also needs its second Gram-Schmidt pass (state[4]).
-__device__ __forceinline__ bool gated_off(const double* state, int gate) {
-    return state[1] == 0.0 || (gate == 1 && state[4] == 0.0);
 }
 
 // partial[b * VT + t] = sum over block b's chunk of V[j0 + t] . w, t < nv
@@ -141,39 +129,6 @@ __global__ void __launch_bounds__(RT) multidot_kernel(const double* __restrict__
     }
 }
 
-// The three-term recurrence of step k, in two launches: mode 0 writes partial sums of
-// v_k . (w - beta_{k-1} v_{k-1}) to part[b * VT] (a = their sum, by finish_dots into
-// *ap); mode 1 updates w -= beta_{k-1} v_{k-1} + a v_k and writes the partial sums of the
-// new ||w||^2 to wn[b].  k = 0 has no v_{k-1} term.
-__global__ void __launch_bounds__(RT) three_term_kernel(const double* __restrict__ V, double* __restrict__ w,
-                                                        int64_t n, int k, int nmax, double* __restrict__ part,
-                                                        double* __restrict__ wn, const double* __restrict__ state,
-                                                        const double* __restrict__ ap, int mode) {
-    __shared__ double sh[RT / 32];
-    if (state[1] == 0.0) return;
-    const double* vk = V + (int64_t)k * n;
-    const double* vp = k > 0 ? V + (int64_t)(k - 1) * n : vk;
-    const double b = k > 0 ? state[8 + nmax + k - 1] : 0.0;
-    const double a = mode == 1 ? *ap : 0.0;
-    double acc = 0.0;
-    const int64_t stride = (int64_t)gridDim.x * RT;
-    for (int64_t i = (int64_t)blockIdx.x * RT + threadIdx.x; i < n; i += stride) {
-        const double x = w[i] - b * vp[i];
-        if (mode == 0) {
-            acc = fma(vk[i], x, acc);
-        } else {
-            const double y = x - a * vk[i];
-            w[i] = y;
-            acc = fma(y, y, acc);
-        }
-    }
-    acc = block_sum(acc, sh);
-    if (threadIdx.x == 0) {
-        if (mode == 0) part[blockIdx.x * VT] = acc;
-        else wn[blockIdx.x] = acc;
-    }
-}
-
 // out[j0 + t] = (accumulate ? out : 0) + sum_b partial[b * VT + t]
 __global__ void finish_dots_kernel(const double* __restrict__ part, int nb, int j0, int nv, double* out,
                                    int accumulate, const double* __restrict__ state) {
@@ -187,25 +142,17 @@ __global__ void finish_dots_kernel(const double* __restrict__ part, int nb, int 
     }
 }
 
-// y[i] = (beta_y * y[i]) + sign * sum_{j < nv} c[j] V[j][i]   (c from device memory); with
-// sq, also sq[b] = block b's sum of the new y[i]^2.  With clamp, only the first state[0]
-// rows (the Krylov dimension reached) enter: rows never written after a breakdown are not
-// read.
+// y[i] = (beta_y * y[i]) + sign * sum_{j < nv} c[j] V[j][i]   (c from device memory)
 __global__ void __launch_bounds__(RT) combine_kernel(const double* __restrict__ V, int64_t n, int nv,
                                                      const double* __restrict__ c, double sign, double beta_y,
-                                                     double* __restrict__ y, const double* __restrict__ state,
-                                                     int ignore_active, int gate = 0,
-                                                     double* __restrict__ sq = nullptr, int clamp = 0) {
+                                                     double* __restrict__ y, const double* __restrict__ state) {
     __shared__ double cs[128];
-    __shared__ double sh[RT / 32];
-    if (!ignore_active && gated_off(state, gate)) return;
-    if (clamp) nv = min(nv, (int)state[0]);
+    if (state[1] == 0.0) return;
     for (int j = threadIdx.x; j < nv; j += blockDim.x) cs[j] = c[j];
     __syncthreads();
     // two elements per iteration (their loads in flight together), then the remainder
     const int64_t stride = (int64_t)gridDim.x * RT;
     int64_t i = (int64_t)blockIdx.x * RT + threadIdx.x;
-    double yy = 0.0;
     for (; i + stride < n; i += 2 * stride) {
         double a0 = 0.0, a1 = 0.0;
 #pragma unroll 8
@@ -213,23 +160,14 @@ __global__ void __launch_bounds__(RT) combine_kernel(const double* __restrict__ 
             a0 = fma(cs[j], V[(int64_t)j * n + i], a0);
             a1 = fma(cs[j], V[(int64_t)j * n + i + stride], a1);
         }
-        const double y0 = (beta_y == 0.0 ? 0.0 : beta_y * y[i]) + sign * a0;
-        const double y1 = (beta_y == 0.0 ? 0.0 : beta_y * y[i + stride]) + sign * a1;
-        y[i] = y0;
-        y[i + stride] = y1;
-        yy = fma(y1, y1, fma(y0, y0, yy));
+        y[i] = (beta_y == 0.0 ? 0.0 : beta_y * y[i]) + sign * a0;
+        y[i + stride] = (beta_y == 0.0 ? 0.0 : beta_y * y[i + stride]) + sign * a1;
     }
     for (; i < n; i += stride) {
         double a = 0.0;
 #pragma unroll 8
         for (int j = 0; j < nv; ++j) a = fma(cs[j], V[(int64_t)j * n + i], a);
-        const double y0 = (beta_y == 0.0 ? 0.0 : beta_y * y[i]) + sign * a;
-        y[i] = y0;
-        yy = fma(y0, y0, yy);
-    }
-    if (sq) {                                        // block-uniform
-        yy = block_sum(yy, sh);
-        if (threadIdx.x == 0) sq[blockIdx.x] = yy;
+        y[i] = (beta_y == 0.0 ? 0.0 : beta_y * y[i]) + sign * a;
     }
 }
 
@@ -266,223 +204,401 @@ __global__ void __launch_bounds__(RT) normalize_kernel(const double* __restrict_
     for (int64_t i = (int64_t)blockIdx.x * RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) dst[i] = src[i] * inv;
 }
 
-// All the projections of one Gram-Schmidt pass in one launch: block (b, g) computes the
-// dots of basis vectors g VT .. g VT + VT - 1 (those below nvec) with w over chunk b, into
-// part[j * gridDim.x + b]; vec_finish_kernel adds each vector's partials in a fixed order.
-__global__ void __launch_bounds__(RT) multidot_all_kernel(const double* __restrict__ V,
-                                                          const double* __restrict__ w, int64_t n, int nvec,
-                                                          double* __restrict__ part,
-                                                          const double* __restrict__ state, int gate) {
-    __shared__ double sh[RT / 32];
-    if (gated_off(state, gate)) return;
-    const int j0 = blockIdx.y * VT;
-    const int nv = nvec - j0 < VT ? nvec - j0 : VT;
-    const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t beg = (int64_t)blockIdx.x * chunk, end = beg + chunk < n ? beg + chunk : n;
-    double acc[VT];
+// ---------------------------------------------------------------- Lanczos step
+// The cooperative kernels run at most one block of LT threads per SM; block b owns the
+// elements [b chunk, (b + 1) chunk) of every vector, and its piece of w lives in shared memory
+// when it fits (LW_MAX doubles), else in place.
+constexpr int LT = 512, LWARPS = LT / 32;
+constexpr int LW_MAX = 25600;
+
+struct LzArgs {
+    Lz z;
+    const double* x0;       // start vector (lz_start)
+    double* x_out;          // Ritz vector (lz_finish)
+    double* result;
+    int64_t chunk;
+    int k, w_shared;
+    int* apply_err;         // the matvec workspace's error flag, raised with the barrier's
+};
+
+struct LzBlock {
+    double* h;              // [NVMAX + 1] sums over all blocks, shared memory
+    double* red;            // [LWARPS * 2]
+    int64_t beg;
+    int len;
+};
+
+// Sum over the block, for thread 0 (a warp's FP64 addition takes 16 cycles of the SM's FP64 unit:
+// only one warp adds the warps' sums).
+__device__ __forceinline__ double lz_block_sum(double v, double* red) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = threadIdx.x < LWARPS ? red[threadIdx.x] : 0.0;
+        for (int o = LWARPS / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    __syncthreads();
+    return v;
+}
+
+__device__ __forceinline__ bool lz_barrier(const LzArgs& a) {
+    if (gridDim.x == 1) {
+        __syncthreads();
+        return true;
+    }
+    const bool ok = grid_barrier(a.z.bar, a.z.bar + 1, gridDim.x, reinterpret_cast<int*>(a.z.bar + 2));
+    if (!ok && threadIdx.x == 0) atomicExch(a.apply_err, 1);
+    return ok;
+}
+
+// out[j] = sum over the blocks of part[j0 + j][block], j < nv: one warp per quantity, every block
+// the same sums in the same order.
+__device__ __forceinline__ void lz_gather(const LzArgs& a, int j0, int nv, double* out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int j = warp; j < nv; j += LWARPS) {
+        double v = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(a.z.part + (int64_t)(j0 + j) * RB + b);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) out[j] = v;
+    }
+    __syncthreads();
+}
+
+// part[j][this block] = V_j . w over the block's elements, j < nv, and part[nv] = w . w.  A warp
+// takes one vector over one of `seg` pieces of the chunk (all warps busy also for few vectors).
+__device__ __forceinline__ void lz_dots(const LzArgs& a, const LzBlock& b, const double* w, int nv) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q = nv + 1, seg = q >= LWARPS ? 1 : LWARPS / q;
+    const int piece = ((b.len + seg - 1) / seg + 31) & ~31;
+    for (int item = warp; item < q * seg; item += LWARPS) {
+        const int j = item / seg, s = item % seg;
+        const double* v = j < nv ? a.z.V + (int64_t)j * a.z.n + b.beg : w;
+        const int end = (s + 1) * piece < b.len ? (s + 1) * piece : b.len;
+        double acc = 0.0;
+        int i = s * piece + lane;
+        for (; i + 7 * 32 < end; i += 8 * 32) {
+            double u[8];
 #pragma unroll
-    for (int t = 0; t < VT; ++t) acc[t] = 0.0;
-    int64_t i = beg + threadIdx.x;
-    for (; i + RT < end; i += 2 * RT) {
-        const double w0 = w[i], w1 = w[i + RT];
-        double v0[VT], v1[VT];
+            for (int e = 0; e < 8; ++e) u[e] = v[i + 32 * e];
 #pragma unroll
-        for (int t = 0; t < VT; ++t) {
-            v0[t] = t < nv ? V[(int64_t)(j0 + t) * n + i] : 0.0;
-            v1[t] = t < nv ? V[(int64_t)(j0 + t) * n + i + RT] : 0.0;
+            for (int e = 0; e < 8; ++e) acc = fma(u[e], w[i + 32 * e], acc);
         }
-#pragma unroll
-        for (int t = 0; t < VT; ++t) acc[t] = fma(v1[t], w1, fma(v0[t], w0, acc[t]));
+        for (; i < end; i += 32) acc = fma(v[i], w[i], acc);
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) {
+            if (seg == 1) a.z.part[(int64_t)j * RB + blockIdx.x] = acc;
+            else b.red[item] = acc;
+        }
     }
-    for (; i < end; i += RT) {
-        const double wi = w[i];
-#pragma unroll
-        for (int t = 0; t < VT; ++t)
-            if (t < nv) acc[t] = fma(V[(int64_t)(j0 + t) * n + i], wi, acc[t]);
-    }
-#pragma unroll
-    for (int t = 0; t < VT; ++t) {
-        if (t >= nv) break;                          // block-uniform
-        const double sum = block_sum(acc[t], sh);
-        if (threadIdx.x == 0) part[(int64_t)(j0 + t) * gridDim.x + blockIdx.x] = sum;
+    if (seg > 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < q) {
+            double s = 0.0;
+            for (int e = 0; e < seg; ++e) s += b.red[threadIdx.x * seg + e];
+            a.z.part[(int64_t)threadIdx.x * RB + blockIdx.x] = s;
+        }
     }
 }
 
-// out[j] = sum over b < nb of part[j * nb + b], one block per vector j
-__global__ void vec_finish_kernel(const double* __restrict__ part, int nb, double* __restrict__ out,
-                                  const double* __restrict__ state, int gate) {
-    __shared__ double sh[RT / 32];
-    if (gated_off(state, gate)) return;
-    double v = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) v += part[(int64_t)blockIdx.x * nb + b];
-    v = block_sum(v, sh);
-    if (threadIdx.x == 0) out[blockIdx.x] = v;
+// w -= sum_{j < nv} h_j V_j over the block's elements; returns the block's new w . w
+__device__ __forceinline__ double lz_subtract(const LzArgs& a, const LzBlock& b, double* w, int nv) {
+    double sq = 0.0;
+    for (int i = threadIdx.x; i < b.len; i += LT) {
+        const double* v = a.z.V + b.beg + i;
+        double s = 0.0;
+#pragma unroll 8
+        for (int j = 0; j < nv; ++j) s = fma(b.h[j], v[(int64_t)j * a.z.n], s);
+        const double y = w[i] - s;
+        w[i] = y;
+        sq = fma(y, y, sq);
+    }
+    return lz_block_sum(sq, b.red);
 }
 
-// beta_k = ||w|| from the nb partial sums of squares; records beta_k and n_eff = k + 1 and
-// ends the iteration when beta_k <= 1e-13 |alpha_k| (an invariant Krylov space)
-__global__ void lz_beta_kernel(const double* __restrict__ sq, int nb, double* state, int k, int nmax) {
-    __shared__ double sh[RT / 32];
-    if (state[1] == 0.0) return;
-    double v = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) v += sq[b];
-    v = block_sum(v, sh);
-    if (threadIdx.x == 0) {
-        const double r = sqrt(v), a = state[8 + k];
+__device__ __forceinline__ LzBlock lz_block(const LzArgs& a, double* h, double* red) {
+    LzBlock b{h, red, (int64_t)blockIdx.x * a.chunk, 0};
+    const int64_t left = a.z.n - b.beg;
+    b.len = (int)(left < a.chunk ? (left > 0 ? left : 0) : a.chunk);
+    return b;
+}
+
+// One Lanczos step on w = H v_k (in the workspace): recurrence, one or two Gram-Schmidt passes,
+// alpha_k, beta_k and v_{k+1}.
+__global__ void __launch_bounds__(LT, 1) lz_step_kernel(LzArgs a) {
+    extern __shared__ double dyn[];
+    __shared__ double h[NVMAX + 1], red[LWARPS * 2];
+    double* state = a.z.state;
+    if (state[1] == 0.0) return;                       // the same for every block: no barrier is left open
+    const LzBlock b = lz_block(a, h, red);
+    const int k = a.k, nmax = a.z.nmax;
+    double* wg = a.z.w() + b.beg;
+    double* w = a.w_shared ? dyn : wg;
+    const double* vk = a.z.V + (int64_t)k * a.z.n + b.beg;
+    const double* vp = vk - a.z.n;
+    const double beta = k > 0 ? state[8 + nmax + k - 1] : 0.0;
+    // x = w - beta v_{k-1}, a = v_k . x
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < b.len; i += LT) {
+        const double x = k > 0 ? wg[i] - beta * vp[i] : wg[i];
+        w[i] = x;
+        acc = fma(vk[i], x, acc);
+    }
+    // slots NVMAX (||w||^2 after a pass) and NVMAX + 1 (a) are their own: no block still reads a
+    // slot that another writes, with one barrier per sum
+    acc = lz_block_sum(acc, red);
+    if (threadIdx.x == 0) a.z.part[(int64_t)(NVMAX + 1) * RB + blockIdx.x] = acc;
+    if (!lz_barrier(a)) return;
+    lz_gather(a, NVMAX + 1, 1, h);
+    double alpha = h[0];
+    for (int i = threadIdx.x; i < b.len; i += LT) w[i] -= alpha * vk[i];
+    __syncthreads();
+    // Gram-Schmidt against v_0 .. v_k; again when less than half of ||w||^2 is left
+    double sq = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+        lz_dots(a, b, w, k + 1);
+        if (!lz_barrier(a)) return;
+        lz_gather(a, 0, k + 2, h);
+        const double before = h[k + 1];
+        alpha += h[k];
+        const double mine = lz_subtract(a, b, w, k + 1);
+        if (threadIdx.x == 0) a.z.part[(int64_t)NVMAX * RB + blockIdx.x] = mine;
+        if (!lz_barrier(a)) return;
+        lz_gather(a, NVMAX, 1, h);
+        sq = h[0];
+        __syncthreads();
+        if (!(sq < 0.5 * before)) break;
+    }
+    const double r = sqrt(sq);
+    // an invariant Krylov space (beta_k <= 1e-13 |alpha_k|) ends the iteration
+    const bool go = r > 1e-13 * fabs(alpha) && r > 1e-300;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        state[8 + k] = alpha;
         state[8 + nmax + k] = r;
         state[0] = (double)(k + 1);
-        if (!(r > 1e-13 * fabs(a)) || !(r > 1e-300)) state[1] = 0.0;
+        if (!go) state[1] = 0.0;
     }
+    if (!go) return;
+    const double inv = 1.0 / r;
+    double* vn = a.z.V + (int64_t)(k + 1) * a.z.n + b.beg;
+    for (int i = threadIdx.x; i < b.len; i += LT) vn[i] = w[i] * inv;
 }
 
-// v_{k+1} = w / beta_k while the iteration is active
-__global__ void __launch_bounds__(RT) lz_scale_kernel(const double* __restrict__ w, double* __restrict__ v,
-                                                      int64_t n, const double* __restrict__ state, int k,
-                                                      int nmax) {
-    if (state[1] == 0.0) return;
-    const double inv = 1.0 / state[8 + nmax + k];
-    for (int64_t i = (int64_t)blockIdx.x * RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) v[i] = w[i] * inv;
+// v_0 = x0 / ||x0||; a zero x0 leaves the iteration inactive
+__global__ void __launch_bounds__(LT, 1) lz_start_kernel(LzArgs a) {
+    __shared__ double h[NVMAX + 1], red[LWARPS * 2];
+    const LzBlock b = lz_block(a, h, red);
+    const double* x = a.x0 + b.beg;
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < b.len; i += LT) acc = fma(x[i], x[i], acc);
+    acc = lz_block_sum(acc, red);
+    if (threadIdx.x == 0) a.z.part[blockIdx.x] = acc;
+    if (!lz_barrier(a)) return;
+    lz_gather(a, 0, 1, h);
+    const double r = sqrt(h[0]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.z.state[0] = 0.0;
+        a.z.state[1] = r > 0.0 ? 1.0 : 0.0;
+    }
+    if (!(r > 0.0)) return;
+    const double inv = 1.0 / r;
+    double* v = a.z.V + b.beg;
+    for (int i = threadIdx.x; i < b.len; i += LT) v[i] = x[i] * inv;
 }
 
-// After the first Gram-Schmidt pass of step k: whether the second runs (state[4]), i.e.
-// whether the pass left less than half of ||w||^2 (before: wn, nb1 partials; after: sq, nb2
-// partials).
-__global__ void lz_second_pass_kernel(double* state, const double* __restrict__ wn, int nb1,
-                                      const double* __restrict__ sq, int nb2) {
-    __shared__ double sh[RT / 32];
-    if (state[1] == 0.0) return;
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < nb1; i += blockDim.x) a += wn[i];
-    for (int i = threadIdx.x; i < nb2; i += blockDim.x) b += sq[i];
-    a = block_sum(a, sh);
-    b = block_sum(b, sh);
-    if (threadIdx.x == 0) state[4] = (b < 0.5 * a) ? 1.0 : 0.0;
-}
-
-// alpha_k = a + h1[k] (+ h2[k] when the second pass ran): every projection of H v_k on v_k
-__global__ void set_alpha_kernel(double* state, const double* a, const double* h1, const double* h2, int k) {
-    if (state[1] == 0.0) return;
-    state[8 + k] = *a + h1[k] + (state[4] != 0.0 ? h2[k] : 0.0);
-}
-
-// Lowest eigenpair of the n_eff x n_eff tridiagonal matrix T (diagonal alpha, off-diagonal
-// beta), in FP64 on one thread: the eigenvalue by bisection on the Sturm count (the number
-// of negative pivots of the LDL^T factorisation of T - x I equals the number of
-// eigenvalues below x), the eigenvector by inverse iteration with the tridiagonal system
-// solved by Gaussian elimination with partial pivoting.  Writes theta to state[2],
-// |beta_{n-1} s_{n-1}| (the Lanczos residual norm of the Ritz pair) to state[3], the
-// eigenvector to s; T holds 4 * nmax doubles of scratch.
-__global__ void tridiag_eig_kernel(double* state, double* T, double* s, int nmax) {
-    // one warp: the 32 lanes evaluate Sturm counts at 32 interior points of the bracket
-    // (multisection: each step shrinks it 33-fold), then lane 0 runs the inverse iteration
-    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+// Lowest eigenpair of the n x n tridiagonal matrix T (diagonal al, off-diagonal be, shared
+// memory), in FP64 by one warp: the eigenvalue by multisection on the Sturm sequence (the leading
+// principal minors p_i of T - x I change sign when an eigenvalue lies below x), the lanes at 32
+// points of the bracket; the eigenvector by inverse iteration, T - theta I factored once by Gaussian
+// elimination with partial pivoting.  Chains of FP64 operations set the time, and every warp that
+// joins slows the others (a warp's FP64 instruction holds the SM's FP64 unit for 16 cycles): the
+// minors need three multiply-adds a row and no division (rescaled when they leave 2^+-300), and
+// the factors are kept over the iterations (20 x 20: 265 us with divisions and arrays in global
+// memory, 30 us now).  Returns theta to lane 0; s gets the eigenvector; work: 5 arrays of NVMAX.
+__device__ double lz_tridiag(const double* al, const double* be, int n, double* s, double* work) {
     const int lane = threadIdx.x;
-    const int n = (int)state[0];
-    for (int i = lane; i < nmax; i += 32) s[i] = 0.0;
-    __syncwarp();                        // lane 0 writes s below: the zeros land first
-    if (n <= 0) {                        // a zero start vector: no Krylov space
-        if (lane == 0) { state[2] = 0.0; state[3] = 0.0; }
-        return;
-    }
-    const double* al = state + 8;
-    const double* be = state + 8 + nmax;
+    double *f = work, *dd = work + NVMAX, *du = work + 2 * NVMAX, *du2 = work + 3 * NVMAX, *b2 = work + 4 * NVMAX;
     double lo = al[0], hi = al[0];
-    for (int i = 0; i < n; ++i) {
+    for (int i = lane; i < n; i += 32) {
         const double r = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i + 1 < n ? fabs(be[i]) : 0.0);
         lo = fmin(lo, al[i] - r);
         hi = fmax(hi, al[i] + r);
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
     const double scale = fmax(fabs(lo), fabs(hi)) + 1e-300;
-    auto count_below = [&](double x) {
-        int c = 0;
-        double d = 1.0;
+    const double inv = 1.0 / scale;
+    // squares of the scaled off-diagonals; b2[0] = 0
+    for (int i = lane; i < n; i += 32) {
+        const double e = i > 0 ? be[i - 1] * inv : 0.0;
+        b2[i] = e * e;
+    }
+    __syncwarp();
+    // whether an eigenvalue lies below x.  The scaled entries are at most 1 (x at most 1): a row
+    // changes the minors by at most a factor of 4
+    auto below = [&](double x) {
+        double p0 = 0.0, p1 = 1.0;
+        bool neg = false;
         for (int i = 0; i < n; ++i) {
-            const double b2 = i > 0 ? be[i - 1] * be[i - 1] : 0.0;
-            d = (al[i] - x) - (i > 0 ? b2 / d : 0.0);
-            if (d == 0.0) d = -1e-300 * scale;
-            if (d < 0.0) ++c;
+            const double p2 = fma((al[i] - x) * inv, p1, -(b2[i] * p0));
+            // a vanishing minor counts with the sign opposite to its predecessor's
+            neg = neg || p2 == 0.0 || (__double2hiint(p2) ^ __double2hiint(p1)) < 0;
+            p0 = p1;
+            p1 = p2;
+            const int e = (__double2hiint(p1) >> 20) & 0x7ff;
+            if (e < 1023 - 300 || e > 1023 + 300) {
+                const int g = 1023 - e < 500 ? 1023 - e : 500;      // both times 2^g
+                const double m = __hiloint2double((g + 1023) << 20, 0);
+                p0 *= m;
+                p1 *= m;
+            }
         }
-        return c;
+        return neg;
     };
-    // the lowest eigenvalue stays in (lo, hi]: count_below(lo) = 0, count_below(hi) >= 1
+    // the lowest eigenvalue stays in (lo, hi]
     for (int it = 0; it < 60 && hi - lo > 4e-16 * scale; ++it) {
         const double step = (hi - lo) / 33.0;
         const double x = lane == 31 ? hi - 0.5 * step : lo + (lane + 1) * step;
-        const unsigned below = __ballot_sync(0xffffffffu, count_below(x) >= 1);
-        const int k = below ? __ffs(below) - 1 : 32;             // first point with an eigenvalue below
+        const unsigned m = __ballot_sync(0xffffffffu, below(x));
+        const int k = m ? __ffs(m) - 1 : 32;          // first point with an eigenvalue below it
         const double xk = __shfl_sync(0xffffffffu, x, k < 32 ? k : 31);
         const double xk1 = __shfl_sync(0xffffffffu, x, k > 0 ? (k < 32 ? k - 1 : 31) : 0);
         if (k < 32) hi = xk;
         if (k > 0) lo = xk1;
     }
-    if (lane != 0) return;
     const double theta = 0.5 * (lo + hi);
-    // inverse iteration: (T - theta I) z_new = z, banded LU with partial pivoting.  A pivot
-    // below tiny (theta is an eigenvalue to rounding, so one pivot is ~0: exactly 0 when
-    // n = 1) is replaced by +-tiny, and z is rescaled by its largest entry before it is
-    // normalised, so the large solution neither overflows nor turns into NaN.
+    // P (T - theta I) = L U: multipliers and row exchanges, U with two super-diagonals.  A pivot
+    // below tiny (theta is an eigenvalue to rounding, so one pivot is ~0) is replaced by +-tiny
+    __shared__ unsigned char swap[NVMAX];
     const double tiny = 1e-15 * scale;
-    auto guard = [&](double v) { return fabs(v) < tiny ? (v < 0.0 ? -tiny : tiny) : v; };
-    double* dl = T;              // sub-diagonal / multipliers
-    double* dd = T + nmax;       // diagonal
-    double* du = T + 2 * nmax;   // first super-diagonal
-    double* du2 = T + 3 * nmax;  // second super-diagonal (fill-in from pivoting)
-    for (int i = 0; i < n; ++i) s[i] = 1.0 / sqrt((double)n);
-    for (int iter = 0; iter < 4; ++iter) {
-        for (int i = 0; i < n; ++i) {
-            dd[i] = al[i] - theta;
-            du[i] = i + 1 < n ? be[i] : 0.0;
-            dl[i] = i + 1 < n ? be[i] : 0.0;
-            du2[i] = 0.0;
-        }
+    if (lane == 0) {
+        double d = al[0] - theta, u = n > 1 ? be[0] : 0.0;        // row i of the elimination
         for (int i = 0; i + 1 < n; ++i) {
-            if (fabs(dd[i]) >= fabs(dl[i])) {              // no row swap
-                dd[i] = guard(dd[i]);
-                const double f = dl[i] / dd[i];
-                dl[i] = f;
-                dd[i + 1] -= f * du[i];
-                s[i + 1] -= f * s[i];
-            } else {                                      // swap rows i and i+1
-                const double f = dd[i] / dl[i];
-                dd[i] = dl[i];
-                dl[i] = f;
-                const double t = du[i];
-                du[i] = dd[i + 1];
-                dd[i + 1] = t - f * dd[i + 1];
-                if (i + 2 < n) {
-                    du2[i] = du[i + 1];
-                    du[i + 1] = -f * du[i + 1];
-                }
-                const double sv = s[i];
-                s[i] = s[i + 1];
-                s[i + 1] = sv - f * s[i + 1];
+            const double l = be[i], dn = al[i + 1] - theta, un = i + 2 < n ? be[i + 1] : 0.0;
+            if (fabs(d) >= fabs(l)) {                 // no exchange
+                if (fabs(d) < tiny) d = d < 0.0 ? -tiny : tiny;
+                const double m = l / d;
+                f[i] = m; swap[i] = 0;
+                dd[i] = d; du[i] = u; du2[i] = 0.0;
+                d = dn - m * u;
+                u = un;
+            } else {                                  // rows i and i + 1 exchanged
+                const double m = d / l;
+                f[i] = m; swap[i] = 1;
+                dd[i] = l; du[i] = dn; du2[i] = un;
+                d = u - m * dn;
+                u = -m * un;
             }
         }
-        dd[n - 1] = guard(dd[n - 1]);
-        // back substitution
-        for (int i = n - 1; i >= 0; --i) {
-            double v = s[i];
-            if (i + 1 < n) v -= du[i] * s[i + 1];
-            if (i + 2 < n) v -= du2[i] * s[i + 2];
-            s[i] = v / dd[i];
+        if (fabs(d) < tiny) d = d < 0.0 ? -tiny : tiny;
+        dd[n - 1] = d;
+        du[n - 1] = du2[n - 1] = 0.0;
+    }
+    __syncwarp();
+    const double s0 = 1.0 / sqrt((double)n);
+    for (int i = lane; i < n; i += 32) {
+        dd[i] = 1.0 / dd[i];
+        s[i] = s0;
+    }
+    __syncwarp();
+    for (int iter = 0; iter < 4; ++iter) {
+        if (lane == 0) {
+            double y = s[0];
+            for (int i = 0; i + 1 < n; ++i) {
+                const double z = s[i + 1];
+                s[i] = swap[i] ? z : y;
+                y = swap[i] ? y - f[i] * z : z - f[i] * y;
+            }
+            s[n - 1] = y;
+            double x1 = 0.0, x2 = 0.0;
+            for (int i = n - 1; i >= 0; --i) {
+                const double x = (s[i] - du[i] * x1 - du2[i] * x2) * dd[i];
+                s[i] = x;
+                x2 = x1;
+                x1 = x;
+            }
         }
-        double mx = 0.0;
-        for (int i = 0; i < n; ++i) mx = fmax(mx, fabs(s[i]));
+        __syncwarp();
+        // scale by the largest entry, then by the norm: the large solution does not overflow
+        double mx = 0.0, nr = 0.0;
+        for (int i = lane; i < n; i += 32) mx = fmax(mx, fabs(s[i]));
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (!(mx > 0.0) || !isfinite(mx)) {           // cannot happen with the guards; keep e_0
-            for (int i = 0; i < n; ++i) s[i] = i == 0 ? 1.0 : 0.0;
+            for (int i = lane; i < n; i += 32) s[i] = i == 0 ? 1.0 : 0.0;
+            __syncwarp();
             break;
         }
-        double nr = 0.0;
-        for (int i = 0; i < n; ++i) { s[i] /= mx; nr += s[i] * s[i]; }
-        nr = sqrt(nr);
-        for (int i = 0; i < n; ++i) s[i] /= nr;
+        const double im = 1.0 / mx;
+        for (int i = lane; i < n; i += 32) nr = fma(s[i] * im, s[i] * im, nr);
+        for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+        nr = im / sqrt(nr);
+        for (int i = lane; i < n; i += 32) s[i] *= nr;
+        __syncwarp();
     }
-    // fix the sign (largest component positive) for reproducible Ritz vectors
-    int im = 0;
-    for (int i = 1; i < n; ++i) if (fabs(s[i]) > fabs(s[im])) im = i;
-    if (s[im] < 0) for (int i = 0; i < n; ++i) s[i] = -s[i];
-    state[2] = theta;
-    state[3] = fabs(be[n - 1] * s[n - 1]);
+    if (lane == 0) {
+        // fix the sign (largest component positive) for reproducible Ritz vectors
+        int im = 0;
+        for (int i = 1; i < n; ++i) if (fabs(s[i]) > fabs(s[im])) im = i;
+        if (s[im] < 0)
+            for (int i = 0; i < n; ++i) s[i] = -s[i];
+    }
+    __syncwarp();
+    return theta;
+}
+
+// The lowest Ritz pair: theta, the residual estimate |beta_{n-1} s_{n-1}|, x = V s normalised, and
+// the result record.
+__global__ void __launch_bounds__(LT, 1) lz_finish_kernel(LzArgs a) {
+    __shared__ double h[NVMAX + 1], red[LWARPS * 2], al[NVMAX], be[NVMAX], work[5 * NVMAX];
+    const LzBlock b = lz_block(a, h, red);
+    double* state = a.z.state;
+    const int n = (int)state[0], nmax = a.z.nmax;
+    if (blockIdx.x == 0) {
+        if (n > 0) {
+            for (int i = threadIdx.x; i < n; i += LT) {
+                al[i] = state[8 + i];
+                be[i] = state[8 + nmax + i];
+            }
+            __syncthreads();
+            if (threadIdx.x < 32) {
+                const double theta = lz_tridiag(al, be, n, h, work);
+                for (int i = threadIdx.x; i < n; i += 32) a.z.s[i] = h[i];
+                if (threadIdx.x == 0) {
+                    state[2] = theta;
+                    state[3] = fabs(be[n - 1] * h[n - 1]);
+                }
+            }
+        } else if (threadIdx.x == 0) {                // a zero start vector: no Krylov space
+            state[2] = 0.0;
+            state[3] = 0.0;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 + 2 * nmax; i += LT)
+            a.result[i] = i < 2 ? state[2 + i] : (i == 2 ? (double)n : state[8 + i - 3]);
+    }
+    if (!lz_barrier(a)) return;
+    for (int j = threadIdx.x; j < n; j += LT) h[j] = __ldcg(a.z.s + j);
+    __syncthreads();
+    double* x = a.x_out + b.beg;
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < b.len; i += LT) {
+        const double* v = a.z.V + b.beg + i;
+        double s = 0.0;
+#pragma unroll 8
+        for (int j = 0; j < n; ++j) s = fma(h[j], v[(int64_t)j * a.z.n], s);
+        x[i] = s;
+        acc = fma(s, s, acc);
+    }
+    acc = lz_block_sum(acc, red);
+    if (threadIdx.x == 0) a.z.part[blockIdx.x] = acc;
+    if (!lz_barrier(a)) return;
+    lz_gather(a, 0, 1, h);
+    const double r = sqrt(h[0]);
+    if (!(r > 0.0)) return;
+    const double inv = 1.0 / r;
+    for (int i = threadIdx.x; i < b.len; i += LT) x[i] *= inv;
 }
 
 // ---------------------------------------------------------------- Davidson (Algorithm 1)
@@ -617,66 +733,48 @@ namespace {
 
 Lz lz_view(const LzLayout& lay, void* lz_ws, int64_t n) {
     char* base = static_cast<char*>(lz_ws);
-    return Lz{reinterpret_cast<double*>(base + lay.off_state), reinterpret_cast<double*>(base + lay.off_h),
-              reinterpret_cast<double*>(base + lay.off_s), reinterpret_cast<double*>(base + lay.off_part),
-              reinterpret_cast<double*>(base + lay.off_wn), reinterpret_cast<double*>(base + lay.off_sq),
-              reinterpret_cast<double*>(base + lay.off_a),
-              reinterpret_cast<double*>(base + lay.off_T), reinterpret_cast<double*>(base + lay.off_V), n,
-              lay.nmax};
+    return Lz{reinterpret_cast<double*>(base + lay.off_state), reinterpret_cast<double*>(base + lay.off_s),
+              reinterpret_cast<double*>(base + lay.off_part), reinterpret_cast<unsigned int*>(base + lay.off_bar),
+              reinterpret_cast<double*>(base + lay.off_V), n, lay.nmax};
 }
 
 // n_iter Lanczos steps from x0 on operators already prepared in apply_ws; x0 may alias x_out
 // (it is only read into the first basis vector).
 int lanczos_core(heff_plan* plan, const double* x0, int32_t n_iter, double* x_out, double* result,
                  void* apply_ws, size_t apply_ws_bytes, const Lz& z, cudaStream_t st) {
-    void* stream = st;
     const int64_t n = z.n;
-    const int G = grid_for(n);
-    const int GN = G < 1024 ? G : 1024;      // normalize: every block re-sums the RB partials
-    int rc;
-    // v_0 = x0 / ||x0||
-    sumsq_kernel<<<RB, RT, 0, st>>>(x0, n, z.part);
-    normalize_kernel<<<GN, RT, 0, st>>>(z.part, RB, x0, z.V, n, z.state, 0);
-    count_launches(2);
-    for (int k = 0; k < n_iter; ++k) {
-        double* vk = z.V + (int64_t)k * n;
-        // w = H v_k (skipped work is harmless after breakdown: the result is not used)
-        if ((rc = heff_apply_prepared(plan, vk, z.w(), apply_ws, apply_ws_bytes, stream))) return rc;
-        // three-term recurrence: a -> z.a, w -= beta_{k-1} v_{k-1} + a v_k
-        three_term_kernel<<<RB, RT, 0, st>>>(z.V, z.w(), n, k, z.nmax, z.part, z.wn, z.state, z.a, 0);
-        finish_dots_kernel<<<1, RT, 0, st>>>(z.part, RB, 0, 1, z.a, 0, z.state);
-        three_term_kernel<<<RB, RT, 0, st>>>(z.V, z.w(), n, k, z.nmax, z.part, z.wn, z.state, z.a, 1);
-        count_launches(3);
-        // classical Gram-Schmidt: h1 -> z.h, then (when needed) h2 -> z.s; each combine also
-        // leaves the partial sums of ||w||^2 in z.sq for the test and the normalisation
-        for (int pass = 0; pass < 2; ++pass) {
-            double* hp = pass == 0 ? z.h : z.s;
-            multidot_all_kernel<<<dim3(RB, (k + VT) / VT), RT, 0, st>>>(z.V, z.w(), n, k + 1, z.part, z.state,
-                                                                         pass);
-            vec_finish_kernel<<<k + 1, RT, 0, st>>>(z.part, RB, hp, z.state, pass);
-            combine_kernel<<<G, RT, 0, st>>>(z.V, n, k + 1, hp, -1.0, 1.0, z.w(), z.state, 0, pass, z.sq);
-            count_launches(3);
-            if (pass == 0) {
-                lz_second_pass_kernel<<<1, RT, 0, st>>>(z.state, z.wn, RB, z.sq, G);
-                count_launches(1);
-            }
-        }
-        set_alpha_kernel<<<1, 1, 0, st>>>(z.state, z.a, z.h, z.s, k);
-        lz_beta_kernel<<<1, RT, 0, st>>>(z.sq, G, z.state, k, z.nmax);
-        lz_scale_kernel<<<G, RT, 0, st>>>(z.w(), z.V + (int64_t)(k + 1) * n, n, z.state, k, z.nmax);
-        count_launches(3);
+    // a block per SM, each with at least 1024 elements (two per thread)
+    int64_t blocks = (n + 1023) / 1024;
+    const int most = plan->num_sms < RB ? plan->num_sms : RB;
+    if (blocks > most) blocks = most;
+    LzArgs a{z, x0, x_out, result, (n + blocks - 1) / blocks, 0, 0,
+             reinterpret_cast<int*>(static_cast<char*>(apply_ws) + plan->off_flags)};
+    a.w_shared = a.chunk <= LW_MAX;
+    const size_t smem = a.w_shared ? (size_t)a.chunk * sizeof(double) : 0;
+    static bool attr = false;
+    cudaError_t e = cudaSuccess;
+    if (!attr) {
+        e = cudaFuncSetAttribute(lz_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 LW_MAX * (int)sizeof(double));
+        attr = e == cudaSuccess;
     }
-    tridiag_eig_kernel<<<1, 32, 0, st>>>(z.state, z.T, z.s, z.nmax);
-    // x = V s (rows beyond n_eff have s = 0), then normalise
-    combine_kernel<<<G, RT, 0, st>>>(z.V, n, z.nmax, z.s, 1.0, 0.0, x_out, z.state, 1, 0, nullptr, 1);
-    sumsq_kernel<<<RB, RT, 0, st>>>(x_out, n, z.part);
-    normalize_kernel<<<GN, RT, 0, st>>>(z.part, RB, x_out, x_out, n, z.state, 2);
-    count_launches(4);
-    // result: [theta, residual estimate, n_eff, alpha..., beta...]
-    cudaMemcpyAsync(result, z.state + 2, sizeof(double) * 2, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyAsync(result + 2, z.state, sizeof(double), cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyAsync(result + 3, z.state + 8, sizeof(double) * 2 * z.nmax, cudaMemcpyDeviceToDevice, st);
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemsetAsync(z.bar, 0, 3 * sizeof(unsigned int), st);
+    void* args[] = {&a};
+    auto launch = [&](const void* kernel, size_t bytes) {
+        if (e == cudaSuccess)
+            e = cudaLaunchCooperativeKernel(kernel, dim3((unsigned)blocks), dim3(LT), args, bytes, st);
+        count_launches(1);
+    };
+    launch((const void*)lz_start_kernel, 0);
+    for (int k = 0; k < n_iter && e == cudaSuccess; ++k) {
+        // w = H v_k (skipped work is harmless after breakdown: the result is not used)
+        int rc = heff_apply_prepared(plan, z.V + (int64_t)k * n, z.w(), apply_ws, apply_ws_bytes, st);
+        if (rc) return rc;
+        a.k = k;
+        launch((const void*)lz_step_kernel, smem);
+    }
+    launch((const void*)lz_finish_kernel, 0);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "heff_lanczos: %s", cudaGetErrorString(e));
     return HEFF_OK;
 }
@@ -916,7 +1014,7 @@ extern "C" int heff_davidson(heff_plan* plan, const void* L, const void* W1, con
             finish_dots_kernel<<<1, RT, 0, st>>>(part, RB, j0, k, h, 0, state);
             count_launches(2);
         }
-        combine_kernel<<<G, RT, 0, st>>>(V, n, nv, h, -1.0, 1.0, q, state, 0);
+        combine_kernel<<<G, RT, 0, st>>>(V, n, nv, h, -1.0, 1.0, q, state);
         count_launches(1);
     };
     for (int i = 0; i < max_vecs; ++i) {
@@ -931,8 +1029,8 @@ extern "C" int heff_davidson(heff_plan* plan, const void* L, const void* W1, con
         dav_set_m_kernel<<<1, 64, 0, st>>>(M, h, i, max_vecs, state);
         dav_eig_kernel<<<1, 32, 0, st>>>(M, E, s, state, i + 1, max_vecs);
         // x = V s, q = V^A s - lambda x, ||q||
-        combine_kernel<<<G, RT, 0, st>>>(V, n, i + 1, s, 1.0, 0.0, x_out, state, 0);
-        combine_kernel<<<G, RT, 0, st>>>(VA, n, i + 1, s, 1.0, 0.0, q, state, 0);
+        combine_kernel<<<G, RT, 0, st>>>(V, n, i + 1, s, 1.0, 0.0, x_out, state);
+        combine_kernel<<<G, RT, 0, st>>>(VA, n, i + 1, s, 1.0, 0.0, q, state);
         dav_shift_kernel<<<G, RT, 0, st>>>(q, x_out, n, state);
         sumsq_kernel<<<RB, RT, 0, st>>>(q, n, part);
         dav_check_kernel<<<1, RT, 0, st>>>(part, RB, state, i + 1 == max_vecs);

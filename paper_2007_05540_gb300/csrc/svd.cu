@@ -30,6 +30,7 @@
 #include <tuple>
 #include <type_traits>
 
+#include "barrier.cuh"
 #include "internal.h"
 
 using heff::fail;
@@ -170,36 +171,7 @@ constexpr int SVD_SWEEP_NT = 256;
 #ifndef SVD_UNROLL
 #define SVD_UNROLL 8        // column pieces per lane loaded together in a pair's loops
 #endif
-constexpr long long SVD_BARRIER_CYCLES = 2ll << 30;
-
-__device__ __forceinline__ bool grid_barrier(unsigned int* count, unsigned int* gen, unsigned int nblocks,
-                                             int* err) {
-    __syncthreads();
-    __shared__ int ok;
-    if (threadIdx.x == 0) {
-        ok = 1;
-        volatile unsigned int* vgen = gen;
-        const unsigned int g = *vgen;
-        __threadfence();
-        if (atomicAdd(count, 1u) == nblocks - 1) {
-            atomicExch(count, 0u);
-            __threadfence();
-            atomicAdd(gen, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (*vgen == g) {
-                if (*(volatile int*)err || clock64() - t0 > SVD_BARRIER_CYCLES) {
-                    atomicExch(err, 1);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
-}
+using heff::grid_barrier;
 
 template <typename T>
 __device__ __forceinline__ T warp_sum_t(T v) {
