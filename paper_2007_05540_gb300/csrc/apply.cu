@@ -325,6 +325,8 @@ int plan_upload(heff_plan* p) {
         if ((rc = upload(g->tasks, &g->d_tasks)) != HEFF_OK) return rc;
         if ((rc = upload(g->segs, &g->d_segs)) != HEFF_OK) return rc;
     }
+    for (MergeList* m : {&p->mg1, &p->mg2})
+        if ((rc = upload(m->tasks, &m->d_tasks)) != HEFF_OK) return rc;
     if ((rc = upload(p->w1_zero, &p->d_w1_zero)) != HEFF_OK) return rc;
     if ((rc = upload(p->w2_zero, &p->d_w2_zero)) != HEFF_OK) return rc;
     CK(cudaMalloc((void**)&p->d_wcount, sizeof(unsigned long long)));
@@ -347,6 +349,10 @@ void plan_free_device(heff_plan* p) {
     for (GemmList* g : {&p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->fx1, &p->fx2}) {
         cudaFree(g->d_tasks); cudaFree(g->d_segs);
         g->d_tasks = nullptr; g->d_segs = nullptr;
+    }
+    for (MergeList* m : {&p->mg1, &p->mg2}) {
+        cudaFree(m->d_tasks);
+        m->d_tasks = nullptr;
     }
     p->d_pack = nullptr; p->d_mix = nullptr; p->d_terms = nullptr;
     p->g1.d_tasks = p->g2.d_tasks = nullptr; p->g1.d_segs = p->g2.d_segs = nullptr;

@@ -183,6 +183,14 @@ struct GemmList {
     std::vector<double> task_flops, task_useful;
 };
 
+// The tasks of a GEMM list by merge class (batched launches, tc_gemm.cu): class c holds the tasks
+// [first[c], first[c + 1]), longest first
+struct MergeList {
+    std::vector<GemmTask> tasks;
+    GemmTask* d_tasks = nullptr;
+    int first[5] = {0, 0, 0, 0, 0};
+};
+
 }  // namespace heff
 
 struct heff_layout {
@@ -235,7 +243,8 @@ struct heff_plan {
     // (two streams alternating workspaces reuse their maps), replaced round-robin
     void* tmap_ws[2] = {nullptr, nullptr};
     int tmap_next = 0;
-    alignas(64) unsigned char tmaps[2][13][128];
+    alignas(64) unsigned char tmaps[2][15][128];
+    heff::MergeList mg1, mg2;  // max_batch > 1, split precisions: the N = 256 tasks by merge class
     int device = 0;
     int num_sms = 0;
     bool uploaded = false;    // false: created without a CUDA device (inspection only)

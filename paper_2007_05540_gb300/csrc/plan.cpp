@@ -633,6 +633,28 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
             P->stats[17] = (int64_t)c2;
         }
         for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->fx1, &P->fx2}) keep_owned(*G, owned);
+        // ---- merge classes (batched launches): the narrowest slot of 256, 128, 64 or 32 columns
+        // (GEMM 1; T's columns come in blocks of 32) or of 128, 64 or 32 rows (GEMM 2) that holds
+        // the tile, so that 2^class batch entries fill one tile
+        if (tc && opts->max_batch > 1) {
+            const struct { const heff::GemmList* G; heff::MergeList* M; } two[2] = {{&P->g1, &P->mg1}, {&P->g2, &P->mg2}};
+            for (const auto& w : two) {
+                auto cls = [&](const heff::GemmTask& k) {
+                    if (k.seg_count == 0) return 0;                 // a zero tile: per entry
+                    const int d = w.M == &P->mg1 ? k.n : k.m, top = w.M == &P->mg1 ? 256 : 128;
+                    int c = 0;
+                    while ((top >> (c + 1)) >= 32 && d <= (top >> (c + 1))) ++c;
+                    return c;
+                };
+                w.M->tasks = w.G->tasks;
+                std::stable_sort(w.M->tasks.begin(), w.M->tasks.end(), [&](const heff::GemmTask& a, const heff::GemmTask& b) {
+                    const int ca = cls(a), cb = cls(b);
+                    return ca != cb ? ca < cb : a.ktotal > b.ktotal;
+                });
+                for (const auto& k : w.M->tasks)
+                    for (int c = cls(k) + 1; c < 5; ++c) ++w.M->first[c];
+            }
+        }
         // ---- CTA pairs (tensor-core paths): N = 256 tiles with the same B rows, width and K
         // segments go two to an entry, so that one read of each B box serves both CTAs of a
         // cluster.  A tile left without a partner gets a ghost (no rows: it loads its half of

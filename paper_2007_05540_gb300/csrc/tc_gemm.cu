@@ -88,7 +88,18 @@ struct TcMaps {
     CUtensorMap a[2];
     CUtensorMap b[3];
     CUtensorMap c;      // T store map: 32 x 32 boxes (GEMM 1 only)
-    CUtensorMap bq;     // B operand, 32-row box (a CTA pair's half of a narrow B tile)
+    CUtensorMap bq;     // B operand, 32-row box (a CTA pair's half of a narrow B tile, merged items)
+    CUtensorMap aq;     // A operand, 32-row box (merged items)
+};
+
+// Merged items of a batched launch: the batch entries of one task that share a tile.  A task of
+// merge class c whose n (GEMM 1) or m (GEMM 2) fits a slot of 256 >> c columns or 128 >> c rows
+// is run for 2^c batch entries at once, entry e in slot e of the tile.
+constexpr int MERGE_CLASSES = 4;
+struct Merge {
+    long item0[MERGE_CLASSES + 1];       // first item of each class
+    int task0[MERGE_CLASSES];            // first task
+    int groups[MERGE_CLASSES];           // items per task: batch entries / 2^c, rounded up
 };
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
@@ -225,7 +236,11 @@ struct TcArgs {
     int y_f64;                            // y element type (mode 1)
     int b0;                               // first batch entry of this launch
     int* err;                             // sticky error flag in the workspace
+    Merge mg;                             // merged items
 };
+
+// A work item: the task, its first batch entry (of the launch) and their number, and its class.
+struct Item { long task; int first, cnt, cls; };
 
 // CL = 1: every CTA runs its own 128-row tiles.  CL = 2: the two CTAs of a cluster run the
 // two tiles of one entry (tasks 2e, 2e + 1: the same B rows and K segments) as one M = 256
@@ -235,7 +250,9 @@ struct TcArgs {
 // in its own tensor memory.  Per CTA this halves the B operand in shared memory (ring
 // stages of 32 KB instead of 48 KB) and the shared-memory bytes the tensor core reads per
 // MMA.  A pair's second task may be a ghost (m = 0: computed, not stored).
-template <int PREC, int TN, int STAGES, int SWZ, int CL>
+// MG: a batched launch whose items are merged (its own instance: the index arithmetic of the merged
+// tiles costs the single-vector launches 0.3 %).
+template <int PREC, int TN, int STAGES, int SWZ, int CL, bool MG>
 __global__ void __launch_bounds__(tc_threads<PREC>(), 1)
 tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
     static_assert(SWZ == 64, "a K block of one half is 64 bytes; hi + lo fill a 128-byte row");
@@ -282,14 +299,32 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
     const uint32_t rank = CL > 1 ? cluster_rank() : 0u;
     const long cid = (long)(blockIdx.x / CL), ncl = (long)(gridDim.x / CL);
     const long nent = g.ntasks / CL;                                 // entries per batch
-    const long total = nent * g.nbatch;
+    constexpr bool merged = MG;
+    static_assert(!MG || CL == 1, "merged items run on single-CTA tiles");
+    const long total = merged ? g.mg.item0[MERGE_CLASSES] : nent * g.nbatch;
     // work item gi -> (entry, batch entry).  Batch-inner order: the batch entries of one
     // task follow each other, so the CTAs that run them at the same time share its operand
     // tiles (the A tile of GEMM 1, the B tile of GEMM 2) through L2.  With one batch entry
     // both orders are the planner's order.
     const long nbl = g.nbatch;
-    auto ent = [&](long gi) { return HEFF_BATCH_INNER ? gi / nbl : gi % nent; };
-    auto bat = [&](long gi) { return (int)(HEFF_BATCH_INNER ? gi % nbl : gi / nent); };
+    auto item = [&](long gi) {
+        Item w{};
+        if (merged) {
+            int c = 0;
+#pragma unroll
+            for (int k = 1; k < MERGE_CLASSES; ++k) c += gi >= g.mg.item0[k];
+            const long r = gi - g.mg.item0[c];
+            w.cls = c;
+            w.task = g.mg.task0[c] + r / g.mg.groups[c];
+            w.first = (int)(r % g.mg.groups[c]) << c;
+            w.cnt = min(1 << c, g.nbatch - w.first);
+        } else {
+            w.task = HEFF_BATCH_INNER ? gi / nbl : gi % nent;
+            w.first = (int)(HEFF_BATCH_INNER ? gi % nbl : gi / nent);
+            w.cnt = 1;
+        }
+        return w;
+    };
     constexpr int KB = SWZ / (PREC == HEFF_PREC_BF16X3 ? 2 : 4);   // elements per K block
     constexpr int KSUB = SWZ / 32;                                   // MMAs (32-byte K) per block
 
@@ -305,11 +340,16 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
         bool ok = true;
         // the next task and the next segment are loaded one step ahead, so their latency
         // overlaps with the current loads instead of draining the ring
-        GemmTask tn = cid < total ? g.tasks[CL * ent(cid) + rank] : GemmTask{};
+        Item wn = cid < total ? item(cid) : Item{};
+        GemmTask tn = cid < total ? g.tasks[CL * wn.task + rank] : GemmTask{};
         for (long gi = cid; gi < total && ok; gi += ncl) {
             const GemmTask t = tn;
-            if (gi + ncl < total) tn = g.tasks[CL * ent(gi + ncl) + rank];
-            const int b = g.b0 + bat(gi);
+            const Item w = wn;
+            if (gi + ncl < total) {
+                wn = item(gi + ncl);
+                tn = g.tasks[CL * wn.task + rank];
+            }
+            const int b = g.b0 + w.first;
             const int ar = (int)(t.a_row + b * g.a_batch_rows), br = (int)(t.b_row + b * g.b_batch_rows);
             const int ia = t.m <= 64 ? 0 : 1, ib = t.n <= 64 ? 0 : (t.n <= 128 ? 1 : 2);
             const CUtensorMap* ma = &maps.a[CL == 1 ? ia : 1];   // a pair always loads 128 A rows
@@ -318,8 +358,16 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
             const int half = (t.n <= 16 ? 16 : (t.n + 15) & ~15) / 2;
             const int hb = half <= 32 ? 0 : (half <= 64 ? 1 : 2);
             const CUtensorMap* mh = hb == 0 ? &maps.bq : &maps.b[hb - 1];
-            const uint32_t bytes = CL == 1 ? 2u * (uint32_t)((64 << ia) + (64 << ib)) * SWZ
-                                           : (uint32_t)CL * 2u * (uint32_t)(128 + (32 << hb)) * SWZ;
+            uint32_t bytes = CL == 1 ? 2u * (uint32_t)((64 << ia) + (64 << ib)) * SWZ
+                                     : (uint32_t)CL * 2u * (uint32_t)(128 + (32 << hb)) * SWZ;
+            // merged: cnt slots of the B tile (GEMM 1) or of the A tile (GEMM 2), one box each
+            const int slot = (g.mode == 0 ? 256 : 128) >> w.cls;
+            const CUtensorMap* ms = nullptr;
+            if (MG && w.cls) {
+                ms = g.mode == 0 ? (slot == 128 ? &maps.b[1] : (slot == 64 ? &maps.b[0] : &maps.bq))
+                                 : (slot == 64 ? &maps.a[0] : &maps.aq);
+                bytes = 2u * (uint32_t)(w.cnt * slot + (g.mode == 0 ? 64 << ia : 64 << ib)) * SWZ;
+            }
             // a K block at column k of the rows starts at element 2 k of the interleaved rows
             KSeg sn = t.seg_count > 0 ? g.segs[t.seg_begin] : KSeg{};
             for (int s = 0; s < t.seg_count && ok; ++s) {
@@ -330,8 +378,19 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                     uint8_t* base = smem + st * S::STAGE_BYTES;
                     if constexpr (CL == 1) {
                         mbar_expect_tx(&full[st], bytes);
-                        tma_load(base, ma, &full[st], 2 * k, ar);
-                        tma_load(base + S::A_BYTES, mb, &full[st], 2 * k, br);
+                        if (!MG || w.cls == 0) {
+                            tma_load(base, ma, &full[st], 2 * k, ar);
+                            tma_load(base + S::A_BYTES, mb, &full[st], 2 * k, br);
+                        } else if (g.mode == 0) {
+                            tma_load(base, ma, &full[st], 2 * k, ar);
+                            for (int e = 0; e < w.cnt; ++e)
+                                tma_load(base + S::A_BYTES + e * slot * 2 * SWZ, ms, &full[st], 2 * k,
+                                         br + e * (int)g.b_batch_rows);
+                        } else {
+                            for (int e = 0; e < w.cnt; ++e)
+                                tma_load(base + e * slot * 2 * SWZ, ms, &full[st], 2 * k, ar + e * (int)g.a_batch_rows);
+                            tma_load(base + S::A_BYTES, mb, &full[st], 2 * k, br);
+                        }
                     } else {
                         // both CTAs' loads complete on the even CTA's barrier, which expects them all
                         const uint32_t fb = full_pair + (uint32_t)(st * sizeof(uint64_t));
@@ -374,10 +433,15 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
         // the lo half of a K block is SWZ bytes into each 128-byte row
         constexpr uint64_t O_LO = (uint64_t)SWZ >> 4, O_B = S::A_BYTES >> 4, O_STAGE = S::STAGE_BYTES >> 4;
         bool ok = true;
-        GemmTask tn = cid < total ? g.tasks[CL * ent(cid) + rank] : GemmTask{};
+        Item wn = cid < total ? item(cid) : Item{};
+        GemmTask tn = cid < total ? g.tasks[CL * wn.task + rank] : GemmTask{};
         for (long gi = cid; gi < total && ok; gi += ncl) {
             const GemmTask t = tn;
-            if (gi + ncl < total) tn = g.tasks[CL * ent(gi + ncl) + rank];
+            const Item w = wn;
+            if (gi + ncl < total) {
+                wn = item(gi + ncl);
+                tn = g.tasks[CL * wn.task + rank];
+            }
             if (t.seg_count == 0) {            // nothing to contract: the epilogue writes zeros
                 const uint32_t acc = ccount & 1, use = ccount >> 1;
                 if (!(ok = mbar_wait(&tempty[acc], (use & 1) ^ 1, abort_flag, g.err))) break;
@@ -387,7 +451,8 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                 continue;
             }
             const int nkb = t.ktotal / KB;
-            const uint32_t nmma = t.n <= 16 ? 16u : (uint32_t)((t.n + 15) & ~15);
+            const uint32_t nmma = MG && w.cls && g.mode == 0 ? (uint32_t)(w.cnt * (256 >> w.cls))
+                                                       : (t.n <= 16 ? 16u : (uint32_t)((t.n + 15) & ~15));
             const uint32_t id = idesc(FMT, TM * CL, nmma);
             uint32_t first = 1, acc = 0, d = 0;
             int left = 0;                      // K blocks left in the current chunk
@@ -464,25 +529,36 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
         uint32_t ccount = 0;
         bool live = true;
         for (long gi = cid; gi < total && live; gi += ncl) {
-            const GemmTask t = g.tasks[CL * ent(gi) + rank];
-            const int brel = bat(gi), b = g.b0 + brel;
+            const Item w = item(gi);
+            const GemmTask t = g.tasks[CL * w.task + rank];
+            // merged: GEMM 1 keeps its rows and its entries' columns lie cslot apart (a 32-column
+            // chunk is within one entry); GEMM 2 its columns, this warp's 32 rows within one entry
+            const int cslot = MG && g.mode == 0 ? 256 >> w.cls : 256, rslot = MG && g.mode != 0 ? 128 >> w.cls : 128;
+            const int re = MG ? (q * 32) / rslot : 0, r_in = MG ? (q * 32) % rslot : q * 32;
+            const int brel = w.first + re;
             const int nch = (t.seg_count > 0 && CH != 0x7fffffff) ? (t.ktotal / KB + CH - 1) / CH : 1;
           for (int ch = 0; ch < nch; ++ch) {
             const uint32_t acc = ccount & 1, use = ccount >> 1;
             if (!mbar_wait(&tfull[acc], use & 1, abort_flag, g.err)) { live = false; break; }
             tc_fence_after();
             const int ncols = t.n + t.n_zero;
-            const int rows = t.m - q * 32 < 32 ? t.m - q * 32 : 32;   // valid rows of this warp
+            // valid rows of this warp
+            const int rows = !MG || re < (g.mode == 0 ? 1 : w.cnt) ? (t.m - r_in < 32 ? t.m - r_in : 32) : 0;
             const bool boxed = g.mode == 0 && rows == 32;              // warp-uniform
-            int x0 = 0, yh = 0;
-            if (boxed) {
-                x0 = (int)(t.c_off % t.ldc);
-                yh = (int)(t.c_off / t.ldc) + q * 32 + b * g.c_batch_rows;
-            }
-            for (int c0 = 32 * h; c0 < ncols; c0 += 32 * NH) {
+            // all columns of the tile: those of the entries' slots that are written
+            const int call = MG && g.mode == 0 && w.cls ? w.cnt * cslot : ncols;
+            for (int ct = 32 * h; ct < call; ct += 32 * NH) {
+                const int ce = MG ? ct / cslot : 0, c0 = MG ? ct % cslot : ct;   // batch entry, column within it
+                if (c0 >= ncols) continue;                             // warp-uniform
+                const int b = g.b0 + brel + ce;
+                int x0 = 0, yh = 0;
+                if (boxed) {
+                    x0 = (int)(t.c_off % t.ldc);
+                    yh = (int)(t.c_off / t.ldc) + q * 32 + b * g.c_batch_rows;
+                }
                 uint32_t raw[32];
                 if (t.seg_count > 0) {
-                    tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + acc * TN + c0, raw);
+                    tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + acc * TN + ct, raw);
                 } else {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) raw[i] = 0u;
@@ -598,7 +674,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                                     lv[p] = (__float_as_uint(f - __uint_as_float(h)) + 0x1000u) & 0xffffe000u;
                                 }
                             }
-                            const int64_t o = (int64_t)(q * 32 + rr) * 2 * t.ldc;
+                            const int64_t o = (int64_t)(r_in + rr) * 2 * t.ldc;
                             *reinterpret_cast<uint4*>(hi + o) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
                             *reinterpret_cast<uint4*>(lo + o) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
                         }
@@ -614,11 +690,11 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                             double old[8];
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
-                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(q * 32 + r0 + u) * t.ldc] : 0.0;
+                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(r_in + r0 + u) * t.ldc] : 0.0;
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
                                 if (r0 + u < rows)
-                                    y[(int64_t)(q * 32 + r0 + u) * t.ldc] =
+                                    y[(int64_t)(r_in + r0 + u) * t.ldc] =
                                         old[u] + f32_to_f64(stage[(r0 + u) * 32 + (lane ^ (r0 + u))]);
                         }
                     } else {
@@ -627,11 +703,11 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                             float old[8];
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
-                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(q * 32 + r0 + u) * t.ldc] : 0.f;
+                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(r_in + r0 + u) * t.ldc] : 0.f;
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
                                 if (r0 + u < rows)
-                                    y[(int64_t)(q * 32 + r0 + u) * t.ldc] =
+                                    y[(int64_t)(r_in + r0 + u) * t.ldc] =
                                         old[u] + stage[(r0 + u) * 32 + (lane ^ (r0 + u))];
                         }
                     }
@@ -717,12 +793,12 @@ static_assert(SWZ_TC / (int)sizeof(__nv_bfloat16) <= KPAD, "a K block must not s
 constexpr int KCHUNK_BF16 = HEFF_KCHUNK_BF16;
 constexpr int KCHUNK_TF32 = HEFF_KCHUNK_TF32;
 
-template <int PREC, int TN_TC, int CL>
+template <int PREC, int TN_TC, int CL, bool MG = false>
 struct TcKernel {
     // a 192 KB ring; a CTA of a pair holds half of the B rows (TN_TC / CL)
     static constexpr int STAGES = (192 * 1024) / (2 * (128 + TN_TC / CL) * SWZ_TC);
     using S = Smem<TN_TC / CL, STAGES, SWZ_TC>;
-    static constexpr auto kern = tc_gemm_kernel<PREC, TN_TC, STAGES, SWZ_TC, CL>;
+    static constexpr auto kern = tc_gemm_kernel<PREC, TN_TC, STAGES, SWZ_TC, CL, MG>;
 
     // shared-memory opt-in (once) and, for pairs, the clusters that fit on the device at once
     static int setup(int num_sms, int* clusters) {
@@ -753,9 +829,35 @@ struct TcKernel {
     }
 };
 
-template <int PREC, int TN_TC, int CL>
-int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, cudaStream_t st) {
-    using K = TcKernel<PREC, TN_TC, CL>;
+// Items of a merged launch over nb batch entries, no class above cap.
+Merge merge_items(const MergeList& ml, int nb, int cap) {
+    Merge mg{};
+    long items = 0;
+    for (int c = 0; c < MERGE_CLASSES; ++c) {
+        mg.item0[c] = items;
+        mg.task0[c] = ml.first[c];
+        mg.groups[c] = (nb + (1 << c) - 1) >> c;
+        const int last = c < cap ? ml.first[c + 1] : ml.first[MERGE_CLASSES];
+        if (c <= cap) items += (long)(last - ml.first[c]) * mg.groups[c];
+    }
+    mg.item0[MERGE_CLASSES] = items;
+    return mg;
+}
+
+// The highest merge class of a batched launch (0: not merged).  A merged item does the work of up
+// to 2^class items in the time of about one (electron problem, m = 1000, blocks of 10-120, 16
+// vectors: GEMM 1 170k items of 1.0 us), so as many entries are merged as leave every SM two items.
+int merge_cap(const MergeList& ml, int nb, int num_sms) {
+    if (nb < 2 || !ml.d_tasks) return 0;
+    for (int cap = MERGE_CLASSES - 1; cap >= 1; --cap)
+        if (merge_items(ml, nb, cap).item0[MERGE_CLASSES] >= 2L * num_sms) return cap;
+    return 0;
+}
+
+// merge: the highest merge class of a batched launch on the N = 256 tiles, 0: one entry per item
+template <int PREC, int TN_TC, int CL, bool MG = false>
+int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, cudaStream_t st, int merge = 0) {
+    using K = TcKernel<PREC, TN_TC, CL, MG>;
     using S = typename K::S;
     const int nsm = p->num_sms > 0 ? p->num_sms : 148;
     int max_cl = 0;
@@ -799,9 +901,17 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
         if ((rc = make_map(&m[12], w + p->off_rw, PREC, (uint64_t)p->rows_rw, (uint64_t)(2 * p->ld_t), 32u,
                            2 * SWZ_TC)))
             return rc;
+        // [13] LW, [14] T with 32-row boxes
+        if ((rc = make_map(&m[13], w + p->off_lw, PREC, (uint64_t)p->rows_lw, (uint64_t)(2 * p->ld_x), 32u,
+                           2 * SWZ_TC)))
+            return rc;
+        if ((rc = make_map(&m[14], w + p->off_t, PREC, (uint64_t)(B * p->rows_t), (uint64_t)(2 * p->ld_t), 32u,
+                           2 * SWZ_TC)))
+            return rc;
         p->tmap_ws[slot] = ws;
     }
     const GemmList& gl = which == 1 ? p->g1 : p->g2;
+    const MergeList& ml = which == 1 ? p->mg1 : p->mg2;
     if (gl.tasks.empty()) return HEFF_OK;
     TcMaps maps;
     const int sa = which == 1 ? 0 : 5, sb = which == 1 ? 2 : 7;
@@ -809,6 +919,7 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
     maps.b[0] = m[sb]; maps.b[1] = m[sb + 1]; maps.b[2] = m[sb + 2];
     maps.c = m[10];
     maps.bq = m[which == 1 ? 11 : 12];
+    maps.aq = m[which == 1 ? 13 : 14];
     for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
         const int nb = nbatch - b0 < MAXB ? nbatch - b0 : MAXB;
         TcArgs g{};
@@ -831,7 +942,12 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
             g.kchunk = (PREC == HEFF_PREC_TF32X3 ? KCHUNK_TF32 : KCHUNK_BF16) * 64 / SWZ_TC;
             g.y_f64 = p->opts.io_dtype == HEFF_DTYPE_F64;
         }
-        const long total = (long)(g.ntasks / CL) * nb;        // entries (tiles, or pairs of tiles)
+        long total = (long)(g.ntasks / CL) * nb;              // entries (tiles, or pairs of tiles)
+        if (MG) {
+            g.mg = merge_items(ml, nb, merge);
+            g.tasks = ml.d_tasks;
+            total = g.mg.item0[MERGE_CLASSES];
+        }
         long units = max_cl;                                   // CTAs, or clusters of CL CTAs
         if (total < units) units = total;
         {
@@ -871,6 +987,14 @@ int launch_tc_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch
     const GemmList& gl = which == 1 ? p->g1 : p->g2;
     if (gl.tasks.empty()) return HEFF_OK;         // nothing to contract (no tensor maps needed)
     const bool wide = gl.tn == 256, pair = gl.cl == 2;
+    // batched launches whose entries share tiles run the N = 256 tiles whatever variant is active
+    // (every variant has the same contraction segments)
+    const int merge = merge_cap(which == 1 ? p->mg1 : p->mg2, nbatch < MAXB ? nbatch : MAXB,
+                                p->num_sms > 0 ? p->num_sms : 148);
+    if (merge)
+        return p->opts.precision == HEFF_PREC_BF16X3
+                   ? launch_tc_t<HEFF_PREC_BF16X3, 256, 1, true>(p, which, ws, y, nbatch, st, merge)
+                   : launch_tc_t<HEFF_PREC_TF32X3, 256, 1, true>(p, which, ws, y, nbatch, st, merge);
     if (p->opts.precision == HEFF_PREC_BF16X3)
         return pair ? launch_tc_t<HEFF_PREC_BF16X3, 256, 2>(p, which, ws, y, nbatch, st)
                     : wide ? launch_tc_t<HEFF_PREC_BF16X3, 256, 1>(p, which, ws, y, nbatch, st)
