@@ -188,7 +188,7 @@ struct GemmList {
 struct MergeList {
     std::vector<GemmTask> tasks;
     GemmTask* d_tasks = nullptr;
-    int first[5] = {0, 0, 0, 0, 0};
+    int first[7] = {0, 0, 0, 0, 0, 0, 0};
 };
 
 }  // namespace heff

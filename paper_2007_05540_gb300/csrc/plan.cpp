@@ -633,15 +633,17 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
             P->stats[17] = (int64_t)c2;
         }
         for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->fx1, &P->fx2}) keep_owned(*G, owned);
-        // ---- merge classes (batched launches): the narrowest slot of 256, 128, 64 or 32 columns
-        // (GEMM 1; T's columns come in blocks of 32) or of 128, 64 or 32 rows (GEMM 2) that holds
-        // the tile, so that 2^class batch entries fill one tile
+        // ---- merge classes (batched launches; defined in tc_gemm.cu): the narrowest slot that holds
+        // the tile, so that as many batch entries as possible fill one tile; T's columns come in
+        // blocks of 32
         if (tc && opts->max_batch > 1) {
             const struct { const heff::GemmList* G; heff::MergeList* M; } two[2] = {{&P->g1, &P->mg1}, {&P->g2, &P->mg2}};
             for (const auto& w : two) {
                 auto cls = [&](const heff::GemmTask& k) {
+                    const bool first = w.M == &P->mg1;
                     if (k.seg_count == 0) return 0;                 // a zero tile: per entry
-                    const int d = w.M == &P->mg1 ? k.n : k.m, top = w.M == &P->mg1 ? 256 : 128;
+                    if (first && k.m <= 64 && k.n <= 64) return k.n <= 32 ? 5 : 4;
+                    const int d = first ? k.n : k.m, top = first ? 256 : 128;
                     int c = 0;
                     while ((top >> (c + 1)) >= 32 && d <= (top >> (c + 1))) ++c;
                     return c;
@@ -652,7 +654,7 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
                     return ca != cb ? ca < cb : a.ktotal > b.ktotal;
                 });
                 for (const auto& k : w.M->tasks)
-                    for (int c = cls(k) + 1; c < 5; ++c) ++w.M->first[c];
+                    for (int c = cls(k) + 1; c < 7; ++c) ++w.M->first[c];
             }
         }
         // ---- CTA pairs (tensor-core paths): N = 256 tiles with the same B rows, width and K

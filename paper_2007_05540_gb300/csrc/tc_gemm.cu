@@ -36,6 +36,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <type_traits>
 
@@ -92,14 +93,20 @@ struct TcMaps {
     CUtensorMap aq;     // A operand, 32-row box (merged items)
 };
 
-// Merged items of a batched launch: the batch entries of one task that share a tile.  A task of
-// merge class c whose n (GEMM 1) or m (GEMM 2) fits a slot of 256 >> c columns or 128 >> c rows
-// is run for 2^c batch entries at once, entry e in slot e of the tile.
-constexpr int MERGE_CLASSES = 4;
+// Merged items of a batched launch: the batch entries of one task that share a tile, entry e in
+// slot e.  Merge classes of a task:
+//   0     one entry per item
+//   1-3   GEMM 1: 2, 4 or 8 entries side by side in slots of 128, 64 or 32 columns (the tile's
+//         n fits);  GEMM 2: 2 or 4 entries in slots of 64 or 32 rows (its m fits)
+//   4, 5  GEMM 1, tiles of at most 64 x 64: 2 or 4 entries in slots of 64 or 32 rows of the
+//         transposed tile (A: the vectors, B: the LW rows).  A tile of few LW rows otherwise leaves
+//         all its epilogue to the two warps of its tensor-memory lanes
+// A launch may merge fewer entries than a class allows (its shift is lowered, its slots widen).
+constexpr int MERGE_CLASSES = 6;
 struct Merge {
     long item0[MERGE_CLASSES + 1];       // first item of each class
     int task0[MERGE_CLASSES];            // first task
-    int groups[MERGE_CLASSES];           // items per task: batch entries / 2^c, rounded up
+    int shift[MERGE_CLASSES];            // log2 of the entries per item
 };
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
@@ -239,8 +246,9 @@ struct TcArgs {
     Merge mg;                             // merged items
 };
 
-// A work item: the task, its first batch entry (of the launch) and their number, and its class.
-struct Item { long task; int first, cnt, cls; };
+// A work item: the task, its first batch entry (of the launch) and their number, the slot width
+// (0: a single entry), and whether the tile is transposed.
+struct Item { long task; int first, cnt, slot; bool swap; };
 
 // CL = 1: every CTA runs its own 128-row tiles.  CL = 2: the two CTAs of a cluster run the
 // two tiles of one entry (tasks 2e, 2e + 1: the same B rows and K segments) as one M = 256
@@ -314,10 +322,12 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
 #pragma unroll
             for (int k = 1; k < MERGE_CLASSES; ++k) c += gi >= g.mg.item0[k];
             const long r = gi - g.mg.item0[c];
-            w.cls = c;
-            w.task = g.mg.task0[c] + r / g.mg.groups[c];
-            w.first = (int)(r % g.mg.groups[c]) << c;
-            w.cnt = min(1 << c, g.nbatch - w.first);
+            const int sh = g.mg.shift[c], groups = (g.nbatch + (1 << sh) - 1) >> sh;
+            w.task = g.mg.task0[c] + r / groups;
+            w.first = (int)(r % groups) << sh;
+            w.cnt = min(1 << sh, g.nbatch - w.first);
+            w.swap = c >= 4;
+            w.slot = sh ? (g.mode == 0 && !w.swap ? 256 : 128) >> sh : 0;
         } else {
             w.task = HEFF_BATCH_INNER ? gi / nbl : gi % nent;
             w.first = (int)(HEFF_BATCH_INNER ? gi % nbl : gi / nent);
@@ -361,12 +371,17 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
             uint32_t bytes = CL == 1 ? 2u * (uint32_t)((64 << ia) + (64 << ib)) * SWZ
                                      : (uint32_t)CL * 2u * (uint32_t)(128 + (32 << hb)) * SWZ;
             // merged: cnt slots of the B tile (GEMM 1) or of the A tile (GEMM 2), one box each
-            const int slot = (g.mode == 0 ? 256 : 128) >> w.cls;
-            const CUtensorMap* ms = nullptr;
-            if (MG && w.cls) {
+            const int slot = w.slot;
+            const CUtensorMap *ms = nullptr, *ml = nullptr;
+            if (MG && slot) {
                 ms = g.mode == 0 ? (slot == 128 ? &maps.b[1] : (slot == 64 ? &maps.b[0] : &maps.bq))
                                  : (slot == 64 ? &maps.a[0] : &maps.aq);
-                bytes = 2u * (uint32_t)(w.cnt * slot + (g.mode == 0 ? 64 << ia : 64 << ib)) * SWZ;
+                int other = g.mode == 0 ? 64 << ia : 64 << ib;        // rows of the shared operand
+                if (w.swap) {
+                    other = t.m <= 32 ? 32 : other;
+                    ml = other == 32 ? &maps.aq : ma;
+                }
+                bytes = 2u * (uint32_t)(w.cnt * slot + other) * SWZ;
             }
             // a K block at column k of the rows starts at element 2 k of the interleaved rows
             KSeg sn = t.seg_count > 0 ? g.segs[t.seg_begin] : KSeg{};
@@ -378,9 +393,13 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                     uint8_t* base = smem + st * S::STAGE_BYTES;
                     if constexpr (CL == 1) {
                         mbar_expect_tx(&full[st], bytes);
-                        if (!MG || w.cls == 0) {
+                        if (!MG || slot == 0) {
                             tma_load(base, ma, &full[st], 2 * k, ar);
                             tma_load(base + S::A_BYTES, mb, &full[st], 2 * k, br);
+                        } else if (w.swap) {
+                            for (int e = 0; e < w.cnt; ++e)
+                                tma_load(base + e * slot * 2 * SWZ, ms, &full[st], 2 * k, br + e * (int)g.b_batch_rows);
+                            tma_load(base + S::A_BYTES, ml, &full[st], 2 * k, ar);
                         } else if (g.mode == 0) {
                             tma_load(base, ma, &full[st], 2 * k, ar);
                             for (int e = 0; e < w.cnt; ++e)
@@ -451,8 +470,9 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                 continue;
             }
             const int nkb = t.ktotal / KB;
-            const uint32_t nmma = MG && w.cls && g.mode == 0 ? (uint32_t)(w.cnt * (256 >> w.cls))
-                                                       : (t.n <= 16 ? 16u : (uint32_t)((t.n + 15) & ~15));
+            const int nt = MG && w.swap ? t.m : t.n;
+            const uint32_t nmma = MG && w.slot && !w.swap && g.mode == 0 ? (uint32_t)(w.cnt * w.slot)
+                                                                         : (nt <= 16 ? 16u : (uint32_t)((nt + 15) & ~15));
             const uint32_t id = idesc(FMT, TM * CL, nmma);
             uint32_t first = 1, acc = 0, d = 0;
             int left = 0;                      // K blocks left in the current chunk
@@ -469,19 +489,23 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                 }
                 if (!(ok = mbar_wait(&full[st], ph, abort_flag, g.err))) break;
                 tc_fence_after();
-                const uint64_t ahi = dsc0 + st * O_STAGE, alo = ahi + O_LO;
-                const uint64_t bhi = ahi + O_B, blo = bhi + O_LO;
+                const uint64_t ahi = dsc0 + st * O_STAGE, bhi = ahi + O_B;
+                // the second and the third product, LW_hi XT_lo and LW_lo XT_hi, in this order also
+                // where a transposed tile has LW as B: the sums' bits do not depend on the merging
+                const bool sw = MG && w.swap;
+                const uint64_t a2 = sw ? ahi + O_LO : ahi, b2 = sw ? bhi : bhi + O_LO;
+                const uint64_t a3 = sw ? ahi : ahi + O_LO, b3 = sw ? bhi + O_LO : bhi;
 #pragma unroll
                 for (int kk = 0; kk < KSUB; ++kk) {
                     const uint64_t o = (uint64_t)(kk * 32) >> 4;     // 32-byte step inside the row
                     if constexpr (CL == 1) {
                         umma<PREC>(d, ahi + o, bhi + o, id, first ? 0u : 1u);
-                        umma<PREC>(d, ahi + o, blo + o, id, 1u);
-                        umma<PREC>(d, alo + o, bhi + o, id, 1u);
+                        umma<PREC>(d, a2 + o, b2 + o, id, 1u);
+                        umma<PREC>(d, a3 + o, b3 + o, id, 1u);
                     } else {
                         umma2<PREC>(d, ahi + o, bhi + o, id, first ? 0u : 1u);
-                        umma2<PREC>(d, ahi + o, blo + o, id, 1u);
-                        umma2<PREC>(d, alo + o, bhi + o, id, 1u);
+                        umma2<PREC>(d, a2 + o, b2 + o, id, 1u);
+                        umma2<PREC>(d, a3 + o, b3 + o, id, 1u);
                     }
                     first = 0;
                 }
@@ -531,9 +555,11 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
         for (long gi = cid; gi < total && live; gi += ncl) {
             const Item w = item(gi);
             const GemmTask t = g.tasks[CL * w.task + rank];
-            // merged: GEMM 1 keeps its rows and its entries' columns lie cslot apart (a 32-column
-            // chunk is within one entry); GEMM 2 its columns, this warp's 32 rows within one entry
-            const int cslot = MG && g.mode == 0 ? 256 >> w.cls : 256, rslot = MG && g.mode != 0 ? 128 >> w.cls : 128;
+            // merged: entries lie slot apart, GEMM 1's along the columns (a 32-column chunk is within
+            // one entry), GEMM 2's and the transposed tiles' along the lanes (this warp's 32 lanes
+            // are within one entry)
+            const bool bylane = MG && w.slot && (g.mode != 0 || w.swap);
+            const int cslot = MG && w.slot && !bylane ? w.slot : 256, rslot = bylane ? w.slot : 128;
             const int re = MG ? (q * 32) / rslot : 0, r_in = MG ? (q * 32) % rslot : q * 32;
             const int brel = w.first + re;
             const int nch = (t.seg_count > 0 && CH != 0x7fffffff) ? (t.ktotal / KB + CH - 1) / CH : 1;
@@ -543,12 +569,18 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
             tc_fence_after();
             const int ncols = t.n + t.n_zero;
             // valid rows of this warp
-            const int rows = !MG || re < (g.mode == 0 ? 1 : w.cnt) ? (t.m - r_in < 32 ? t.m - r_in : 32) : 0;
-            const bool boxed = g.mode == 0 && rows == 32;              // warp-uniform
-            // all columns of the tile: those of the entries' slots that are written
-            const int call = MG && g.mode == 0 && w.cls ? w.cnt * cslot : ncols;
+            const bool swap = MG && w.swap;
+            const bool mine = !bylane || re < w.cnt;
+            // all accumulator columns of the tile: those of the entries' slots, or the rows of a
+            // transposed tile
+            const int call = swap ? t.m : (MG && w.slot && !bylane ? w.cnt * cslot : ncols);
             for (int ct = 32 * h; ct < call; ct += 32 * NH) {
-                const int ce = MG ? ct / cslot : 0, c0 = MG ? ct % cslot : ct;   // batch entry, column within it
+                // batch entry and column of the output chunk, its first row and number of rows
+                const int ce = MG && !swap ? ct / cslot : 0;
+                const int c0 = swap ? r_in : (MG ? ct % cslot : ct);
+                const int row0 = swap ? ct : r_in;
+                const int rows = mine ? (t.m - row0 < 32 ? t.m - row0 : 32) : 0;
+                const bool boxed = g.mode == 0 && rows == 32 && !swap;  // warp-uniform
                 if (c0 >= ncols) continue;                             // warp-uniform
                 const int b = g.b0 + brel + ce;
                 int x0 = 0, yh = 0;
@@ -631,7 +663,8 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                 if (lane == 0) bulk_wait_read<0>();
                 __syncwarp();
 #pragma unroll
-                for (int i = 0; i < 32; ++i) stage[lane * 32 + (i ^ lane)] = __uint_as_float(raw[i]);
+                for (int i = 0; i < 32; ++i)
+                    stage[swap ? i * 32 + (lane ^ i) : lane * 32 + (i ^ lane)] = __uint_as_float(raw[i]);
                 __syncwarp();
                 const int c = c0 + lane;                       // this lane's column
                 if (g.mode == 0) {
@@ -674,7 +707,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                                     lv[p] = (__float_as_uint(f - __uint_as_float(h)) + 0x1000u) & 0xffffe000u;
                                 }
                             }
-                            const int64_t o = (int64_t)(r_in + rr) * 2 * t.ldc;
+                            const int64_t o = (int64_t)(row0 + rr) * 2 * t.ldc;
                             *reinterpret_cast<uint4*>(hi + o) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
                             *reinterpret_cast<uint4*>(lo + o) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
                         }
@@ -690,11 +723,11 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                             double old[8];
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
-                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(r_in + r0 + u) * t.ldc] : 0.0;
+                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(row0 + r0 + u) * t.ldc] : 0.0;
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
                                 if (r0 + u < rows)
-                                    y[(int64_t)(r_in + r0 + u) * t.ldc] =
+                                    y[(int64_t)(row0 + r0 + u) * t.ldc] =
                                         old[u] + f32_to_f64(stage[(r0 + u) * 32 + (lane ^ (r0 + u))]);
                         }
                     } else {
@@ -703,11 +736,11 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                             float old[8];
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
-                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(r_in + r0 + u) * t.ldc] : 0.f;
+                                old[u] = (ch && r0 + u < rows) ? y[(int64_t)(row0 + r0 + u) * t.ldc] : 0.f;
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
                                 if (r0 + u < rows)
-                                    y[(int64_t)(r_in + r0 + u) * t.ldc] =
+                                    y[(int64_t)(row0 + r0 + u) * t.ldc] =
                                         old[u] + stage[(r0 + u) * 32 + (lane ^ (r0 + u))];
                         }
                     }
@@ -829,32 +862,31 @@ struct TcKernel {
     }
 };
 
-// Items of a merged launch over nb batch entries, no class above cap.
+// Items of a merged launch over nb batch entries, at most 2^cap entries each.
 Merge merge_items(const MergeList& ml, int nb, int cap) {
     Merge mg{};
     long items = 0;
     for (int c = 0; c < MERGE_CLASSES; ++c) {
         mg.item0[c] = items;
         mg.task0[c] = ml.first[c];
-        mg.groups[c] = (nb + (1 << c) - 1) >> c;
-        const int last = c < cap ? ml.first[c + 1] : ml.first[MERGE_CLASSES];
-        if (c <= cap) items += (long)(last - ml.first[c]) * mg.groups[c];
+        mg.shift[c] = std::min(c < 4 ? c : c - 3, cap);
+        items += (long)(ml.first[c + 1] - ml.first[c]) * ((nb + (1 << mg.shift[c]) - 1) >> mg.shift[c]);
     }
     mg.item0[MERGE_CLASSES] = items;
     return mg;
 }
 
-// The highest merge class of a batched launch (0: not merged).  A merged item does the work of up
+// log2 of the most entries per item of a batched launch (0: not merged).  A merged item does the work of up
 // to 2^class items in the time of about one (electron problem, m = 1000, blocks of 10-120, 16
 // vectors: GEMM 1 170k items of 1.0 us), so as many entries are merged as leave every SM two items.
 int merge_cap(const MergeList& ml, int nb, int num_sms) {
     if (nb < 2 || !ml.d_tasks) return 0;
-    for (int cap = MERGE_CLASSES - 1; cap >= 1; --cap)
+    for (int cap = 3; cap >= 1; --cap)
         if (merge_items(ml, nb, cap).item0[MERGE_CLASSES] >= 2L * num_sms) return cap;
     return 0;
 }
 
-// merge: the highest merge class of a batched launch on the N = 256 tiles, 0: one entry per item
+// merge: log2 of the most batch entries per item (MG, on the N = 256 tiles)
 template <int PREC, int TN_TC, int CL, bool MG = false>
 int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, cudaStream_t st, int merge = 0) {
     using K = TcKernel<PREC, TN_TC, CL, MG>;
