@@ -187,7 +187,7 @@ __device__ __forceinline__ void mix_tile(const MixTile& t, const MixArgs& a) {
     const int nt = t.term_count < 64 ? t.term_count : 64;
     for (int k = threadIdx.x; k < nt; k += blockDim.x) {
         MixTerm m = terms[t.term_begin + k];
-        coef[k] = to_acc<Acc>(W[m.w_idx]);
+        coef[k] = m.w_idx < 0 ? (Acc)1 : to_acc<Acc>(W[m.w_idx]);
         srco[k] = m.src_off;
     }
     __syncthreads();
@@ -229,7 +229,7 @@ __device__ __forceinline__ void mix_tile(const MixTile& t, const MixArgs& a) {
                 } else {                                      // rare: more than 64 terms
                     const MixTerm m = terms[t.term_begin + k];
                     s = src + m.src_off;
-                    cf = to_acc<Acc>(W[m.w_idx]);
+                    cf = m.w_idx < 0 ? (Acc)1 : to_acc<Acc>(W[m.w_idx]);
                 }
                 In v0[RW][U], v1[RW][U];
 #pragma unroll
@@ -405,6 +405,10 @@ int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, 
 
 static MixArgs mix_args(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, char* ws,
                         bool codes) {
+    if (p->env)
+        return MixArgs{p->d_mix, p->d_terms, L, W1, W2, R, ws + p->off_lw, p->ld_x, ws + p->off_xt, p->ld_x,
+                       codes ? reinterpret_cast<uint16_t*>(ws + p->off_elw) : nullptr,
+                       codes ? reinterpret_cast<uint16_t*>(ws + p->off_ex) : nullptr, p->rows_lw, p->rows_x};
     return MixArgs{p->d_mix, p->d_terms, L, W1, W2, R, ws + p->off_lw, p->ld_x, ws + p->off_rw, p->ld_t,
                    codes ? reinterpret_cast<uint16_t*>(ws + p->off_elw) : nullptr,
                    codes ? reinterpret_cast<uint16_t*>(ws + p->off_erw) : nullptr, p->rows_lw, p->rows_rw};

@@ -1,19 +1,28 @@
 // Environment extension on the GPU (Section II-C: the left environment A and right
-// environment B grow by one site as the sweep moves), on the block-product engine.
+// environment B grow by one site as the sweep moves).
 //
-// Left (site tensor A[a, s, b], flows (+1, +1, -1); environment L[a', w, a]):
-//   X[(a', w), (s, b)]  = L[a', w, a] . A[a, s, b]                      (step 1)
-//   Lnew[c, v, d]       = sum W[w, t, s, v] A[a', t, c]^T . X[(a', w), (s, d)]   (step 2)
-// Right (site tensor B[a, s, b]; environment R[b', w, b]):
-//   Y[(b', v), (a, s)]  = R[b', v, b] . B[a, s, b]^T                    (step 1)
-//   Rnew[c, w, d]       = sum W[w, t, s, v] B[c, t, b'] . Y[(b', v), (d, s)]     (step 2)
-// Each charge-matched block pair is one small dense product; step 2 sums, per output
-// block, the products whose MPO coefficient is nonzero in the host copy of W.
+// Both sides have one form.  With i the sectors of env_old's bond, j those of env_new's, u and n
+// their channels, S_j[b, (s, i) a] the site tensor as a matrix (out-bond state b, columns the
+// site's state and in-bond state), and c(u, t, s, n) the entries of W:
+//   Lnew[j', n, j] = S_j' . T^T,     T[(n, j', j) b, (t, i') a'] = S_j . LW^T               (GEMMs 2, 1)
+//   LW[(n, t, i', j) a', (s, i) a] = sum_u c(u, t, s, n) env_old[i', u, i]                  (mix)
+// so the update is one operator preparation and two grouped GEMMs over workspace operands with
+// the contraction index contiguous: the kernels of the H_eff matvec (apply.cu, tc_gemm.cu,
+// fx_gemm.cu) run it from tables of the same form (heff_plan with env set).  W enters with the
+// environment, before the GEMMs: a product per entry of W, as in the list form below, contracts the
+// same site block with up to k blocks that differ by a coefficient.
+//
+// An update whose dense operands would take more than ENV_DENSE_MAX bytes of workspace runs as lists of
+// block products instead (about a quarter of the memory; blockops.cu):
+//   X[(a', w), (s, b)]  = L[a', w, a] . A[a, s, b],   Lnew[c, v, d] = sum W A[a', t, c]^T . X     (left)
+//   Y[(b', v), (a, s)]  = R[b', v, b] . B[a, s, b]^T, Rnew[c, w, d] = sum W B[c, t, b'] . Y       (right)
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <map>
+#include <memory>
 #include <new>
+#include <set>
 #include <tuple>
 
 #include "internal.h"
@@ -21,23 +30,37 @@
 using heff::fail;
 using heff::BList;
 using heff::BProd;
+using heff::GemmTask;
+using heff::KPAD;
+using heff::pad_up;
 
-// Workspace: [error flag, 256 B][intermediate X or Y][tensor-core precision only: FP32 copies
-// of env_old and of the site tensor].  The FP64 products keep the intermediate in FP64; the
-// tensor-core products read FP32 copies and keep it in FP32.
 struct heff_env_plan {
     int side = 0;
     int precision = HEFF_PREC_FP64;   // of the block products
-    BList step1, step2;
-    int64_t ws_elems = 0;      // intermediate (X or Y) elements
+    double flops = 0;                 // of the list form (the block pairs of Algorithm 2)
+    size_t ws_bytes = 0;              // covers both precisions
     int64_t n_env = 0, n_site = 0;
-    size_t off_x = 256, off_env32 = 0, off_site32 = 0;
-    size_t ws_bytes = 0;
-    bool uploaded = false;
+    bool device = false;              // created with a CUDA device
     const void* last_ws = nullptr;    // workspace of the last update (its error flag is initialised)
+    // dense form: block-level tasks, cut into the precision's tiles when the plan is first used
+    bool dense = true;
+    std::vector<GemmTask> blocks1, blocks2;
+    std::vector<heff::KSeg> segs1, segs2;
+    std::vector<heff::PackTile> pack;
+    std::vector<heff::MixTile> mix;
+    std::vector<heff::MixTerm> terms;
+    int64_t rows_sp = 0, ld = 0, rows_lw = 0, rows_t = 0;
+    std::unique_ptr<heff_plan> plan;
+    // list form.  Workspace: [error flag, 256 B][intermediate X or Y][tensor-core precision only: FP32
+    // copies of env_old and of the site tensor].  The FP64 products keep the intermediate in FP64;
+    // the tensor-core products read FP32 copies and keep it in FP32.
+    BList step1, step2;
+    size_t off_x = 256, off_env32 = 0, off_site32 = 0;
 };
 
 namespace {
+
+constexpr size_t ENV_DENSE_MAX = (size_t)64 << 30;
 
 using Charge = std::vector<int32_t>;
 
@@ -47,6 +70,235 @@ Charge add(const Charge& a, const Charge& b, int sb = 1) {
     Charge r(a);
     for (size_t c = 0; c < r.size(); ++c) r[c] += sb * b[c];
     return r;
+}
+
+// Operand layout, block-level GEMM tasks and copy / mix tiles of the dense form, and the flop count of
+// the list form.  c(u, t, s, n): index of the kept entry of W, or -1; nu: channels of env_old.
+template <typename C>
+void build_dense(heff_env_plan* P, const heff_layout* env_old, const heff_layout* site, const heff_layout* env_new,
+                 const heff::IndexDesc& sa, const heff::IndexDesc& sp, const heff::IndexDesc& sb, int d, int nu, C c) {
+    const bool left = P->side == 0;
+    const heff::IndexDesc &in = left ? sa : sb, &out = left ? sb : sa;
+    const int ni = in.nsec, nj = out.nsec, nn = env_new->idx[1].nsec;
+    // the site blocks that the products use: (i, s) -> j and (j, t) -> i by charge
+    auto off_of = [&](int i, int s, int j) { return left ? site->offset_of({i, s, j}) : site->offset_of({j, s, i}); };
+    std::vector<int> out_of((size_t)ni * d, -1), in_of((size_t)nj * d, -1);
+    for (int s = 0; s < d; ++s) {
+        for (int i = 0; i < ni; ++i) {
+            const int j = out.find(add(in.q(i), sp.q(s), left ? 1 : -1));
+            if (j >= 0 && off_of(i, s, j) >= 0) out_of[(size_t)i * d + s] = j;
+        }
+        for (int j = 0; j < nj; ++j) {
+            const int i = in.find(add(out.q(j), sp.q(s), left ? -1 : 1));
+            if (i >= 0 && off_of(i, s, j) >= 0) in_of[(size_t)j * d + s] = i;
+        }
+    }
+    // columns of S_j: one padded segment per site block
+    std::map<std::tuple<int, int, int>, int32_t> col;          // (j, s, i)
+    std::vector<int32_t> width(nj, 0);
+    std::vector<int64_t> sp_row(nj, 0);
+    int64_t rows = 0;
+    for (int j = 0; j < nj; ++j) { sp_row[j] = rows; rows += out.dims[j]; }
+    for (size_t b = 0; b < site->offsets.size(); ++b) {
+        const int i = site->keys[b * 3 + (left ? 0 : 2)], s = site->keys[b * 3 + 1], j = site->keys[b * 3 + (left ? 2 : 0)];
+        const int mi = in.dims[i], mj = out.dims[j], pad = (int)pad_up(mi, KPAD);
+        const int32_t c0 = width[j];
+        col[{j, s, i}] = c0;
+        width[j] += pad;
+        if (left) {                                             // stored a x b: transposed copy
+            for (int a0 = 0; a0 < pad; a0 += 32)
+                for (int b0 = 0; b0 < mj; b0 += 32)
+                    P->pack.push_back({site->offsets[b], sp_row[j], c0, mi, mj, pad, a0, b0});
+        } else {                                                // stored b x a: plain copy
+            const int32_t tb = (int32_t)P->terms.size();
+            P->terms.push_back({site->offsets[b], -1, 0});
+            for (int r0 = 0; r0 < mj; r0 += 32)
+                P->mix.push_back({sp_row[j], c0, mj, mi, pad, r0, std::min(32, mj - r0), tb, 1, 1});
+        }
+    }
+    P->rows_sp = std::max<int64_t>(rows, 1);
+    P->ld = KPAD;
+    for (int j = 0; j < nj; ++j) P->ld = std::max<int64_t>(P->ld, width[j]);
+    // LW row groups (n, t, i', j): segments (s, i) with their terms (u), from env_old's blocks; and the
+    // intermediate blocks (i', u, s, j) of the list form, for its flop count
+    struct Seg { int s, i; std::vector<heff::MixTerm> terms; };
+    struct Group { int64_t row = -1; std::map<std::pair<int, int>, Seg> segs; };
+    std::map<std::tuple<int, int, int, int>, Group> groups;
+    std::set<std::tuple<int, int, int, int>> inter;
+    for (size_t b = 0; b < env_old->offsets.size(); ++b) {
+        const int ip = env_old->keys[b * 3], u = env_old->keys[b * 3 + 1], i = env_old->keys[b * 3 + 2];
+        for (int s = 0; s < d; ++s) {
+            const int j = out_of[(size_t)i * d + s];
+            if (j < 0) continue;
+            bool used = false;
+            for (int t = 0; t < d; ++t)
+                for (int n = 0; n < nn; ++n) {
+                    const int32_t w = c(u, t, s, n);
+                    if (w < 0) continue;
+                    used = true;
+                    Seg& sg = groups[{n, t, ip, j}].segs[{s, i}];
+                    sg.s = s;
+                    sg.i = i;
+                    sg.terms.push_back({env_old->offsets[b], w, 0});
+                }
+            if (!used) continue;
+            inter.insert({ip, u, s, j});
+            P->flops += 2.0 * in.dims[ip] * out.dims[j] * in.dims[i];
+        }
+    }
+    // env_new's blocks: T rows, GEMM 1 (one task per site state t of the bra), GEMM 2
+    int64_t t_rows = 0, lw_rows = 0;
+    for (size_t b = 0; b < env_new->offsets.size(); ++b) {
+        const int jp = env_new->keys[b * 3], n = env_new->keys[b * 3 + 1], j = env_new->keys[b * 3 + 2];
+        const int mjp = out.dims[jp], mj = out.dims[j];
+        GemmTask g2{};
+        g2.a_row = sp_row[jp];
+        g2.b_row = t_rows;
+        g2.m = mjp;
+        g2.n = mj;
+        g2.c_off = env_new->offsets[b];
+        g2.ldc = mj;
+        g2.seg_begin = (int32_t)P->segs2.size();
+        for (int t = 0; t < d; ++t) {
+            const int ip = in_of[(size_t)jp * d + t];
+            if (ip < 0) continue;
+            for (int u = 0; u < nu; ++u)
+                for (int s = 0; s < d; ++s)
+                    if (c(u, t, s, n) >= 0 && inter.count({ip, u, s, j})) P->flops += 2.0 * mjp * mj * in.dims[ip];
+            auto it = groups.find({n, t, ip, j});
+            if (it == groups.end()) continue;
+            Group& g = it->second;
+            const int mip = in.dims[ip], pad = (int)pad_up(mip, KPAD);
+            if (g.row < 0) {
+                g.row = lw_rows;
+                lw_rows += mip;
+                for (auto& kv : g.segs) {
+                    const Seg& sg = kv.second;
+                    const int mi = in.dims[sg.i];
+                    const int32_t tb = (int32_t)P->terms.size();
+                    P->terms.insert(P->terms.end(), sg.terms.begin(), sg.terms.end());
+                    for (int r0 = 0; r0 < mip; r0 += 32)
+                        P->mix.push_back({g.row, col[{j, sg.s, sg.i}], mip, mi, (int32_t)pad_up(mi, KPAD), r0,
+                                          std::min(32, mip - r0), tb, (int32_t)sg.terms.size(), 0});
+                }
+            }
+            GemmTask g1{};
+            g1.a_row = sp_row[j];
+            g1.b_row = g.row;
+            g1.m = mj;
+            g1.n = mip;
+            const int32_t c0 = col[{jp, t, ip}];
+            g1.c_off = t_rows * P->ld + c0;
+            g1.ldc = (int32_t)P->ld;
+            g1.n_zero = pad - mip;
+            g1.seg_begin = (int32_t)P->segs1.size();
+            for (auto& kv : g.segs) {
+                const int32_t len = (int32_t)pad_up(in.dims[kv.second.i], KPAD);
+                P->segs1.push_back({col[{j, kv.second.s, kv.second.i}], len});
+                g1.ktotal += len;
+            }
+            g1.seg_count = (int32_t)P->segs1.size() - g1.seg_begin;
+            P->blocks1.push_back(g1);
+            P->segs2.push_back({c0, pad});
+            g2.ktotal += pad;
+        }
+        g2.seg_count = (int32_t)P->segs2.size() - g2.seg_begin;
+        P->blocks2.push_back(g2);
+        t_rows += mj;
+    }
+    P->rows_lw = std::max<int64_t>(lw_rows, 1);
+    P->rows_t = std::max<int64_t>(t_rows, 1);
+}
+
+// Workspace of the dense form in a precision; with p, its offsets too.
+size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
+    auto al = [](size_t v) { return (v + 255) / 256 * 256; };
+    const bool tc = precision != HEFF_PREC_FP64;
+    const size_t e = (size_t)(tc ? 4 : 8) * P->ld, kb = (size_t)(P->ld / KPAD) * sizeof(uint16_t);
+    size_t off = 0, o_sp, o_lw, o_t, o_f;
+    o_sp = off; off = al(off + e * P->rows_sp);
+    o_lw = off; off = al(off + e * P->rows_lw);
+    o_t = off;  off = al(off + e * P->rows_t);
+    o_f = off;  off = al(off + 256);
+    if (p) {
+        p->off_xt = o_sp; p->off_lw = o_lw; p->off_t = o_t; p->off_rw = o_t; p->off_flags = o_f;
+        p->ws_min = off;
+    }
+    if (!tc) {
+        size_t o_ex, o_elw, o_et;
+        o_ex = off;  off = al(off + kb * P->rows_sp);
+        o_elw = off; off = al(off + kb * P->rows_lw);
+        o_et = off;  off = al(off + kb * P->rows_t);
+        if (p) { p->off_ex = o_ex; p->off_elw = o_elw; p->off_et = o_et; p->off_erw = o_et; }
+    }
+    if (p) p->ws_bytes = off;
+    return off;
+}
+
+// The device tables of the current precision.
+int ensure_plan(heff_env_plan* P) {
+    if (P->plan) return HEFF_OK;
+    int rc;
+    try {
+        std::unique_ptr<heff_plan> p(new heff_plan());
+        const bool tc = P->precision != HEFF_PREC_FP64;
+        p->env = true;
+        p->opts.precision = P->precision;
+        p->opts.io_dtype = HEFF_DTYPE_F64;
+        p->opts.max_batch = 1;
+        p->planes = tc ? 2 : 1;
+        p->esize = tc ? 2 : 8;
+        p->nelem_x = P->n_site;
+        p->rows_x = P->rows_sp; p->ld_x = P->ld; p->rows_lw = P->rows_lw;
+        p->rows_t = P->rows_t; p->ld_t = P->ld; p->rows_rw = 0;
+        dense_bytes(P, P->precision, p.get());
+        p->pack = P->pack;
+        p->mix = P->mix;
+        p->terms = P->terms;
+        int nsm = 148, dev = 0, v = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+            nsm = v;
+        cudaGetLastError();
+        const int tm = tc ? 128 : heff::FX_TILE_M, tn = tc ? 256 : heff::FX_TILE_N;
+        auto cut = [&](const std::vector<GemmTask>& blocks, const std::vector<heff::KSeg>& segs, heff::GemmList& G,
+                       bool first) {
+            G.tm = tm;
+            G.tn = tn;
+            G.segs = segs;
+            for (const GemmTask& k : blocks)
+                for (int m0 = 0; m0 < k.m; m0 += tm)
+                    for (int n0 = 0; n0 < k.n; n0 += tn) {
+                        GemmTask t = k;
+                        t.a_row += m0;
+                        t.b_row += n0;
+                        t.m = std::min(tm, k.m - m0);
+                        t.n = std::min(tn, k.n - n0);
+                        t.c_off += (int64_t)m0 * k.ldc + n0;
+                        t.n_zero = n0 + tn >= k.n ? k.n_zero : 0;
+                        G.tasks.push_back(t);
+                    }
+            G.owner.assign(G.tasks.size(), 0);
+            G.task_flops.assign(G.tasks.size(), 0.0);
+            G.task_useful.assign(G.tasks.size(), 0.0);
+            heff::lpt_schedule(G, nsm, tc, first);
+        };
+        cut(P->blocks1, P->segs1, tc ? p->g1 : p->fx1, true);
+        cut(P->blocks2, P->segs2, tc ? p->g2 : p->fx2, false);
+        if ((rc = heff::plan_upload(p.get())) != HEFF_OK) {
+            heff::plan_free_device(p.get());
+            return rc;
+        }
+        P->plan = std::move(p);
+    } catch (const std::bad_alloc&) {
+        return fail(HEFF_ERR_OOM, "out of host memory while planning the environment update");
+    }
+    return HEFF_OK;
+}
+
+void free_plan(heff_env_plan* P) {
+    if (P->plan) heff::plan_free_device(P->plan.get());
+    P->plan.reset();
 }
 
 }  // namespace
@@ -92,6 +344,13 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
         };
         // site blocks by key
         auto site_off = [&](int a, int s, int b) { return site->offset_of({a, s, b}); };
+        P->n_env = env_old->nelem;
+        P->n_site = site->nelem;
+        build_dense(P, env_old, site, env_new, sa, sp, sb, d, side == 0 ? kw : kv,
+                    [&](int u, int t, int s, int n) { return side == 0 ? widx(u, t, s, n) : widx(n, t, s, u); });
+        P->ws_bytes = dense_bytes(P, HEFF_PREC_FP64, nullptr);
+        P->dense = P->ws_bytes <= ENV_DENSE_MAX;
+        if (!P->dense) {
         std::map<std::tuple<int, int, int, int>, int64_t> inter;   // intermediate blocks -> offset
         int64_t ioff = 0;
         if (side == 0) {
@@ -192,21 +451,21 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
                 P->step2.add_block(env_new->offsets[bk], mid, mic, mid, ps);
             }
         }
-        P->ws_elems = ioff;
-        P->n_env = env_old->nelem;
-        P->n_site = site->nelem;
         auto al = [](size_t v) { return (v + 255) / 256 * 256; };
         const size_t fp64_bytes = P->off_x + al((size_t)ioff * sizeof(double));
         P->off_env32 = P->off_x + al((size_t)ioff * sizeof(float));
         P->off_site32 = P->off_env32 + al((size_t)P->n_env * sizeof(float));
         const size_t tc_bytes = P->off_site32 + al((size_t)P->n_site * sizeof(float));
         P->ws_bytes = std::max(fp64_bytes, tc_bytes);
+        }
     } catch (const std::bad_alloc&) {
         delete P;
         return fail(HEFF_ERR_OOM, "out of host memory while planning the environment update");
     }
     int ndev = 0;
-    if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) {
+    P->device = cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0;
+    cudaGetLastError();
+    if (P->device && !P->dense) {
         int rc;
         if ((rc = heff::blist_upload(P->step1)) || (rc = heff::blist_upload(P->step2))) {
             heff::blist_free(P->step1);
@@ -214,9 +473,6 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
             delete P;
             return rc;
         }
-        P->uploaded = true;
-    } else {
-        cudaGetLastError();
     }
     *out = P;
     return HEFF_OK;
@@ -226,13 +482,15 @@ extern "C" int heff_env_workspace_size(const heff_env_plan* plan, size_t* bytes)
     heff::clear_error();
     if (!plan || !bytes) return fail(HEFF_ERR_INVALID_ARG, "heff_env_workspace_size: null argument");
     *bytes = plan->ws_bytes;
-    return HEFF_OK;
+    // the caller allocates now and updates next: build the device tables of the current precision
+    // here, so that an update neither allocates nor synchronises (stream capture)
+    return plan->dense && plan->device ? ensure_plan(const_cast<heff_env_plan*>(plan)) : HEFF_OK;
 }
 
 extern "C" int heff_env_flops(const heff_env_plan* plan, double* flops) {
     heff::clear_error();
     if (!plan || !flops) return fail(HEFF_ERR_INVALID_ARG, "heff_env_flops: null argument");
-    *flops = plan->step1.flops + plan->step2.flops;
+    *flops = plan->flops;
     return HEFF_OK;
 }
 
@@ -241,13 +499,27 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
     heff::clear_error();
     if (!plan || !env_old || !site || !W || !env_new)
         return fail(HEFF_ERR_INVALID_ARG, "heff_env_update: null argument");
-    if (!plan->uploaded) return fail(HEFF_ERR_UNSUPPORTED, "env plan was created without a CUDA device");
+    if (!plan->device) return fail(HEFF_ERR_UNSUPPORTED, "env plan was created without a CUDA device");
     if (!workspace || workspace_bytes < plan->ws_bytes || reinterpret_cast<uintptr_t>(workspace) % 256)
         return fail(HEFF_ERR_WORKSPACE, "environment workspace of %zu bytes, needs %zu (256-byte aligned)",
                     workspace_bytes, plan->ws_bytes);
     char* ws = static_cast<char*>(workspace);
-    int* err = reinterpret_cast<int*>(ws);
     int rc;
+    if (plan->dense) {
+        if ((rc = ensure_plan(plan))) return rc;
+        heff_plan* p = plan->plan.get();
+        cudaError_t ez = cudaMemsetAsync(ws + p->off_flags, 0, sizeof(int), static_cast<cudaStream_t>(stream));
+        if (ez != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(ez));
+        plan->last_ws = workspace;
+        const void* xs[1] = {site};
+        void* ys[1] = {env_new};
+        // the mix tiles read env_old as L with W as W1, and (side 1) the site tensor as R
+        if ((rc = heff::launch_mix(p, env_old, W, W, site, ws, true, stream))) return rc;
+        if ((rc = heff::launch_pack_batch(p, xs, 1, ws, true, stream))) return rc;
+        if ((rc = heff::launch_gemm(p, 1, ws, ys, 1, true, stream))) return rc;
+        return heff::launch_gemm(p, 2, ws, ys, 1, true, stream);
+    }
+    int* err = reinterpret_cast<int*>(ws);
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
     plan->last_ws = workspace;
@@ -272,16 +544,21 @@ extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precisio
     if (precision != HEFF_PREC_FP64 && precision != HEFF_PREC_BF16X3)
         return fail(HEFF_ERR_UNSUPPORTED, "environment updates run in HEFF_PREC_FP64 or HEFF_PREC_BF16X3");
     if (precision == plan->precision) return HEFF_OK;
+    if (plan->dense) {
+        free_plan(plan);
+        plan->precision = precision;
+        return HEFF_OK;
+    }
     const bool fx = precision == HEFF_PREC_FP64;
     heff::blist_free(plan->step1);
     heff::blist_free(plan->step2);
     plan->step1.retile(fx ? heff::FX_TILE_M : 128, fx ? heff::FX_TILE_N : 128);
     plan->step2.retile(fx ? heff::FX_TILE_M : 128, fx ? heff::FX_TILE_N : 128);
     plan->precision = precision;
-    if (plan->uploaded) {
+    if (plan->device) {
         int rc;
         if ((rc = heff::blist_upload(plan->step1)) || (rc = heff::blist_upload(plan->step2))) {
-            plan->uploaded = false;
+            plan->device = false;
             return rc;
         }
     }
@@ -291,11 +568,12 @@ extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precisio
 extern "C" int heff_env_status(const heff_env_plan* plan, void* workspace, size_t workspace_bytes, void* stream) {
     heff::clear_error();
     if (!plan || !workspace) return fail(HEFF_ERR_INVALID_ARG, "heff_env_status: null argument");
-    // an FP64 plan's flag exists once an update has run in this workspace
-    if (plan->precision == HEFF_PREC_FP64 && workspace != plan->last_ws) return HEFF_OK;
+    // the flag exists once an update has run in this workspace
+    if (workspace != plan->last_ws) return HEFF_OK;
     if (workspace_bytes < plan->ws_bytes) return fail(HEFF_ERR_WORKSPACE, "heff_env_status: workspace too small");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int* d = static_cast<int*>(workspace);
+    if (plan->dense && !plan->plan) return HEFF_OK;     // nothing has run since the precision was set
+    int* d = reinterpret_cast<int*>(static_cast<char*>(workspace) + (plan->dense ? plan->plan->off_flags : 0));
     int flag = 0;
     cudaError_t e = cudaMemcpyAsync(&flag, d, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -308,6 +586,7 @@ extern "C" int heff_env_status(const heff_env_plan* plan, void* workspace, size_
 
 extern "C" void heff_env_plan_destroy(heff_env_plan* plan) {
     if (!plan) return;
+    free_plan(plan);
     heff::blist_free(plan->step1);
     heff::blist_free(plan->step2);
     delete plan;

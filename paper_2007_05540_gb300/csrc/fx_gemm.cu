@@ -808,7 +808,21 @@ int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbat
         g.err = reinterpret_cast<int*>(w + p->off_flags);
         uint16_t* e_t = reinterpret_cast<uint16_t*>(w + p->off_et);
         const int64_t t_rows = p->opts.max_batch * p->rows_t;
-        if (which == 1) {
+        if (p->env) {
+            // A: XT in both; B: LW into T, then T into y
+            g.A = reinterpret_cast<const double*>(w + p->off_xt);
+            g.B = reinterpret_cast<const double*>(w + (which == 1 ? p->off_lw : p->off_t));
+            g.ld = p->ld_x;
+            g.C = reinterpret_cast<double*>(w + p->off_t);
+            g.y.p[0] = y[b0];
+            g.to_y = which == 2;
+            g.ea = reinterpret_cast<const uint16_t*>(w + p->off_ex);
+            g.ea_rows = p->rows_x;
+            g.eb = which == 1 ? reinterpret_cast<const uint16_t*>(w + p->off_elw) : e_t;
+            g.eb_rows = which == 1 ? p->rows_lw : t_rows;
+            g.et = which == 1 ? e_t : nullptr;
+            g.et_rows = t_rows;
+        } else if (which == 1) {
             g.A = reinterpret_cast<const double*>(w + p->off_lw);
             g.B = reinterpret_cast<const double*>(w + p->off_xt);
             g.ld = p->ld_x;

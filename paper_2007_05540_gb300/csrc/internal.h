@@ -68,7 +68,7 @@ struct MixTile {
 };
 struct MixTerm {
     int64_t src_off;   // element offset of the environment block
-    int32_t w_idx;     // element index into the MPO buffer
+    int32_t w_idx;     // element index into the MPO buffer; -1: coefficient 1 (a plain copy)
     int32_t pad_;
 };
 
@@ -234,6 +234,9 @@ struct heff_plan {
     heff::GemmList g1, g2;            // active task lists
     heff::GemmList g1_alt, g2_alt;    // the other tile width (tensor-core paths), see heff_plan_autotune
     heff::GemmList g1_pair, g2_pair;  // N = 256 tiles in CTA pairs sharing B (tensor-core paths)
+    // the environment update's plan (env.cu): GEMM 1 contracts XT with LW into T, GEMM 2 XT with T;
+    // there is no RW, and which = 1 mix tiles fill XT
+    bool env = false;
     heff::GemmList fx1, fx2;          // FP64 plans: the task lists that run (FX_TILE_M x FX_TILE_N tiles)
     // FP64 plans: exponent codes of the operand arrays, [column / KPAD][row]; they come last in the
     // workspace (ws_min: its size without them, when every tile runs in FP64 arithmetic)
@@ -243,7 +246,7 @@ struct heff_plan {
     // (two streams alternating workspaces reuse their maps), replaced round-robin
     void* tmap_ws[2] = {nullptr, nullptr};
     int tmap_next = 0;
-    alignas(64) unsigned char tmaps[2][15][128];
+    alignas(64) unsigned char tmaps[2][17][128];
     heff::MergeList mg1, mg2;  // max_batch > 1, split precisions: the N = 256 tasks by merge class
     int device = 0;
     int num_sms = 0;
@@ -265,6 +268,7 @@ int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbat
 // one apply in the first `bytes` of ws, which may hold less than ws_bytes but at least ws_min
 int apply_in(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, const void* x, void* y,
              void* ws, size_t bytes, void* stream);
+void lpt_schedule(GemmList& G, int units, bool tc, bool first);
 // clusters of two tensor-core CTAs resident at once (tc_gemm.cu; num_sms / 2 without a device)
 int tc_pair_clusters(int num_sms, int precision);
 // one block waiting at the SVD sweeps' grid barrier set up for two (svd.cu; wait self-test)

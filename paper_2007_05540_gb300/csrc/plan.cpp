@@ -98,6 +98,66 @@ bool check_index(const IndexDesc& a, const IndexDesc& b, int flow_a) {
 
 }  // namespace
 
+// Static schedule of the persistent kernels: CTA c of a grid of min(units, entries) runs the
+// entries c, c + grid, c + 2 grid, ...  The entries are assigned by longest-processing-time (each to
+// the least loaded CTA, longest first; a tile's time ~ (K blocks + a fixed overhead) x its width
+// cost) and the per-CTA lists interleaved in that pattern, short lists padded with empty tasks (no
+// rows, no segments).  CTA pairs are scheduled the same way, an entry (two tasks) per cluster.
+void heff::lpt_schedule(GemmList& G, int units, bool tc, bool first) {
+    const int model = first ? HEFF_TILE_COST_G1 : HEFF_TILE_COST_G2;
+    const size_t CLn = (size_t)G.cl;
+    const size_t nt = G.tasks.size() / CLn;          // entries
+    if (nt == 0) return;
+    const int grid = (int)std::min<size_t>((size_t)units, nt);
+    std::vector<double> work(nt, 0.0);
+    for (size_t t = 0; t < nt; ++t)
+        for (size_t r = 0; r < CLn; ++r) {
+            const GemmTask& k = G.tasks[t * CLn + r];
+            work[t] = std::max(work[t], tc ? (double)(k.ktotal / KPAD + 4) * tile_width_cost(k.m, k.n, model)
+                                           : (double)(k.ktotal / KPAD + 4) * (k.n + 32));
+        }
+    std::vector<size_t> ord(nt);
+    for (size_t t = 0; t < nt; ++t) ord[t] = t;
+    std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) { return work[a] > work[b]; });
+    // least loaded CTA first, the lowest index among equal loads (a min-heap on (load, CTA):
+    // O(tasks log grid))
+    std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>,
+                        std::greater<std::pair<double, int>>> heap;
+    for (int c = 0; c < grid; ++c) heap.push({0.0, c});
+    std::vector<std::vector<size_t>> per(grid);
+    for (size_t t : ord) {
+        const std::pair<double, int> top = heap.top();
+        heap.pop();
+        per[top.second].push_back(t);
+        heap.push({top.first + work[t], top.second});
+    }
+    size_t depth = 0;
+    for (auto& v : per) depth = std::max(depth, v.size());
+    GemmList s2;
+    for (size_t j = 0; j < depth; ++j)
+        for (int c = 0; c < grid; ++c)
+            for (size_t r = 0; r < CLn; ++r) {
+                if (j < per[c].size()) {
+                    const size_t t = per[c][j] * CLn + r;
+                    s2.tasks.push_back(G.tasks[t]);
+                    s2.owner.push_back(G.owner[t]);
+                    s2.task_flops.push_back(G.task_flops[t]);
+                    s2.task_useful.push_back(G.task_useful[t]);
+                } else {
+                    GemmTask e{};
+                    e.ldc = 1;
+                    s2.tasks.push_back(e);
+                    s2.owner.push_back(-1);
+                    s2.task_flops.push_back(0.0);
+                    s2.task_useful.push_back(0.0);
+                }
+            }
+    G.tasks.swap(s2.tasks);
+    G.owner.swap(s2.owner);
+    G.task_flops.swap(s2.task_flops);
+    G.task_useful.swap(s2.task_useful);
+}
+
 extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, const heff_layout* W2,
                                 const heff_layout* R, const heff_layout* x, const double* W1_host,
                                 const double* W2_host, const heff_plan_opts* opts, heff_plan** out) {
@@ -716,68 +776,11 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
             if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) ncl = heff::tc_pair_clusters(nsm, opts->precision);
             cudaGetLastError();
         }
-        // ---- static schedule of the persistent tensor-core kernels: CTA c of a grid of
-        // min(nsm, tasks) runs tasks c, c + grid, c + 2 grid, ...  Assign the tasks by
-        // longest-processing-time (each to the least loaded CTA, longest first; a tile's
-        // time ~ (K blocks + a fixed overhead) x MMA width) and interleave the per-CTA lists
-        // in that pattern, padding short lists with empty tasks (no rows, no segments).
-        // CTA pairs are scheduled the same way, an entry (two tasks) per cluster.
         if (HEFF_LPT_SCHEDULE) {
             for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->g1_pair, &P->g2_pair, &P->fx1, &P->fx2}) {
                 if (!tc && (G == &P->g1 || G == &P->g2)) continue;    // 64 x 64 tiles: only described, not run
-                const int model = (G == &P->g1 || G == &P->g1_alt || G == &P->g1_pair) ? HEFF_TILE_COST_G1
-                                                                                        : HEFF_TILE_COST_G2;
-                const size_t CLn = (size_t)G->cl;
-                const size_t nt = G->tasks.size() / CLn;          // entries
-                if (nt == 0) continue;
-                const int grid = (int)std::min<size_t>((size_t)(CLn == 2 ? ncl : nsm), nt);
-                std::vector<double> work(nt, 0.0);
-                for (size_t t = 0; t < nt; ++t)
-                    for (size_t r = 0; r < CLn; ++r) {
-                        const heff::GemmTask& k = G->tasks[t * CLn + r];
-                        work[t] = std::max(work[t], tc ? (double)(k.ktotal / KPAD + 4) * tile_width_cost(k.m, k.n, model)
-                                                       : (double)(k.ktotal / KPAD + 4) * (k.n + 32));
-                    }
-                std::vector<size_t> ord(nt);
-                for (size_t t = 0; t < nt; ++t) ord[t] = t;
-                std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) { return work[a] > work[b]; });
-                // least loaded CTA first, the lowest index among equal loads (a min-heap on
-                // (load, CTA): O(tasks log grid))
-                std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>,
-                                    std::greater<std::pair<double, int>>> heap;
-                for (int c = 0; c < grid; ++c) heap.push({0.0, c});
-                std::vector<std::vector<size_t>> per(grid);
-                for (size_t t : ord) {
-                    const std::pair<double, int> top = heap.top();
-                    heap.pop();
-                    per[top.second].push_back(t);
-                    heap.push({top.first + work[t], top.second});
-                }
-                size_t depth = 0;
-                for (auto& v : per) depth = std::max(depth, v.size());
-                heff::GemmList s2;
-                for (size_t j = 0; j < depth; ++j)
-                    for (int c = 0; c < grid; ++c)
-                        for (size_t r = 0; r < CLn; ++r) {
-                            if (j < per[c].size()) {
-                                const size_t t = per[c][j] * CLn + r;
-                                s2.tasks.push_back(G->tasks[t]);
-                                s2.owner.push_back(G->owner[t]);
-                                s2.task_flops.push_back(G->task_flops[t]);
-                                s2.task_useful.push_back(G->task_useful[t]);
-                            } else {
-                                heff::GemmTask e{};
-                                e.ldc = 1;
-                                s2.tasks.push_back(e);
-                                s2.owner.push_back(-1);
-                                s2.task_flops.push_back(0.0);
-                                s2.task_useful.push_back(0.0);
-                            }
-                        }
-                G->tasks.swap(s2.tasks);
-                G->owner.swap(s2.owner);
-                G->task_flops.swap(s2.task_flops);
-                G->task_useful.swap(s2.task_useful);
+                const bool first = G == &P->g1 || G == &P->g1_alt || G == &P->g1_pair;
+                heff::lpt_schedule(*G, G->cl == 2 ? ncl : nsm, tc, first);
             }
         }
         for (int i = 0; i < na; ++i) if (owned[i]) P->shard_sectors.push_back(i);

@@ -910,48 +910,31 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
         if (ez != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(ez));
         // Operand rows interleave the hi and lo halves by K block: 2 ld elements per row, boxes
         // of 128-byte rows (a K block of both halves).
-        // [0,1] LW (64, 128 rows)  [2,3,4] XT (64, 128, 256)  [5,6] T (64, 128)  [7,8,9] RW (64, 128, 256)
-        // [10] T store boxes: 32 rows x 128 bytes
-        struct { char* base; int64_t rows, ld; int slot, nbox; } ops[4] = {
-            {w + p->off_lw, p->rows_lw, p->ld_x, 0, 2},
-            {w + p->off_xt, B * p->rows_x, p->ld_x, 2, 3},
-            {w + p->off_t, B * p->rows_t, p->ld_t, 5, 2},
-            {w + p->off_rw, p->rows_rw, p->ld_t, 7, 3}};
-        for (auto& o : ops)
-            for (int k = 0; k < o.nbox; ++k) {
-                int rc = make_map(&m[o.slot + k], o.base, PREC, (uint64_t)o.rows, (uint64_t)(2 * o.ld), 64u << k,
-                                  2 * SWZ_TC);
+        // [4 o + k]: array o (LW, XT, T, RW) in boxes of 32 << k rows;  [16] T store boxes: 32 rows
+        struct { char* base; int64_t rows, ld; } ops[4] = {{w + p->off_lw, p->rows_lw, p->ld_x},
+                                                           {w + p->off_xt, B * p->rows_x, p->ld_x},
+                                                           {w + p->off_t, B * p->rows_t, p->ld_t},
+                                                           {w + p->off_rw, p->rows_rw, p->ld_t}};
+        for (int o = 0; o < (p->env ? 3 : 4); ++o)
+            for (int k = 0; k < 4; ++k) {
+                int rc = make_map(&m[4 * o + k], ops[o].base, PREC, (uint64_t)ops[o].rows, (uint64_t)(2 * ops[o].ld),
+                                  32u << k, 2 * SWZ_TC);
                 if (rc) return rc;
             }
-        int rc = make_map(&m[10], w + p->off_t, PREC, (uint64_t)(B * p->rows_t), (uint64_t)(2 * p->ld_t), 32u,
+        int rc = make_map(&m[16], w + p->off_t, PREC, (uint64_t)(B * p->rows_t), (uint64_t)(2 * p->ld_t), 32u,
                           2 * SWZ_TC);
         if (rc) return rc;
-        // [11] XT, [12] RW with 32-row boxes (halves of a 64-row B box for CTA pairs)
-        if ((rc = make_map(&m[11], w + p->off_xt, PREC, (uint64_t)(B * p->rows_x), (uint64_t)(2 * p->ld_x), 32u,
-                           2 * SWZ_TC)))
-            return rc;
-        if ((rc = make_map(&m[12], w + p->off_rw, PREC, (uint64_t)p->rows_rw, (uint64_t)(2 * p->ld_t), 32u,
-                           2 * SWZ_TC)))
-            return rc;
-        // [13] LW, [14] T with 32-row boxes
-        if ((rc = make_map(&m[13], w + p->off_lw, PREC, (uint64_t)p->rows_lw, (uint64_t)(2 * p->ld_x), 32u,
-                           2 * SWZ_TC)))
-            return rc;
-        if ((rc = make_map(&m[14], w + p->off_t, PREC, (uint64_t)(B * p->rows_t), (uint64_t)(2 * p->ld_t), 32u,
-                           2 * SWZ_TC)))
-            return rc;
         p->tmap_ws[slot] = ws;
     }
     const GemmList& gl = which == 1 ? p->g1 : p->g2;
     const MergeList& ml = which == 1 ? p->mg1 : p->mg2;
     if (gl.tasks.empty()) return HEFF_OK;
     TcMaps maps;
-    const int sa = which == 1 ? 0 : 5, sb = which == 1 ? 2 : 7;
-    maps.a[0] = m[sa]; maps.a[1] = m[sa + 1];
-    maps.b[0] = m[sb]; maps.b[1] = m[sb + 1]; maps.b[2] = m[sb + 2];
-    maps.c = m[10];
-    maps.bq = m[which == 1 ? 11 : 12];
-    maps.aq = m[which == 1 ? 13 : 14];
+    const int oa = p->env ? 1 : (which == 1 ? 0 : 2), ob = p->env ? (which == 1 ? 0 : 2) : (which == 1 ? 1 : 3);
+    const CUtensorMap *ma = &m[4 * oa], *mb = &m[4 * ob];
+    maps.aq = ma[0]; maps.a[0] = ma[1]; maps.a[1] = ma[2];
+    maps.bq = mb[0]; maps.b[0] = mb[1]; maps.b[1] = mb[2]; maps.b[2] = mb[3];
+    maps.c = m[16];
     for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
         const int nb = nbatch - b0 < MAXB ? nbatch - b0 : MAXB;
         TcArgs g{};
