@@ -320,10 +320,12 @@ int plan_upload(heff_plan* p) {
     if ((rc = upload(p->pack, &p->d_pack)) != HEFF_OK) return rc;
     if ((rc = upload(p->mix, &p->d_mix)) != HEFF_OK) return rc;
     if ((rc = upload(p->terms, &p->d_terms)) != HEFF_OK) return rc;
-    for (GemmList* g : {&p->g1, &p->g2, &p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->fx1, &p->fx2}) {
+    for (GemmList* g : {&p->g1, &p->g2, &p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->sp2, &p->sp2_alt, &p->fx1,
+                        &p->fx2}) {
         if (p->opts.precision == HEFF_PREC_FP64 && (g == &p->g1 || g == &p->g2)) continue;   // fx1, fx2 run
         if ((rc = upload(g->tasks, &g->d_tasks)) != HEFF_OK) return rc;
         if ((rc = upload(g->segs, &g->d_segs)) != HEFF_OK) return rc;
+        if ((rc = upload(g->split, &g->d_split)) != HEFF_OK) return rc;
     }
     for (MergeList* m : {&p->mg1, &p->mg2})
         if ((rc = upload(m->tasks, &m->d_tasks)) != HEFF_OK) return rc;
@@ -345,17 +347,16 @@ void plan_free_device(heff_plan* p) {
     cudaFree(p->d_w1_zero); cudaFree(p->d_w2_zero); cudaFree(p->d_wcount);
     p->d_w1_zero = p->d_w2_zero = nullptr;
     p->d_wcount = nullptr;
-    cudaFree(p->g1.d_tasks); cudaFree(p->g1.d_segs); cudaFree(p->g2.d_tasks); cudaFree(p->g2.d_segs);
-    for (GemmList* g : {&p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->fx1, &p->fx2}) {
-        cudaFree(g->d_tasks); cudaFree(g->d_segs);
-        g->d_tasks = nullptr; g->d_segs = nullptr;
+    for (GemmList* g : {&p->g1, &p->g2, &p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->sp2, &p->sp2_alt, &p->fx1,
+                        &p->fx2}) {
+        cudaFree(g->d_tasks); cudaFree(g->d_segs); cudaFree(g->d_split);
+        g->d_tasks = nullptr; g->d_segs = nullptr; g->d_split = nullptr;
     }
     for (MergeList* m : {&p->mg1, &p->mg2}) {
         cudaFree(m->d_tasks);
         m->d_tasks = nullptr;
     }
     p->d_pack = nullptr; p->d_mix = nullptr; p->d_terms = nullptr;
-    p->g1.d_tasks = p->g2.d_tasks = nullptr; p->g1.d_segs = p->g2.d_segs = nullptr;
 }
 
 
@@ -385,7 +386,7 @@ int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, 
         for (int b = 0; b < nb; ++b) xs.p[b] = x[b0 + b];
         char* w = static_cast<char*>(ws) + (size_t)b0 * p->rows_x * p->ld_x * p->esize * p->planes;
         const bool f32 = p->opts.io_dtype == HEFF_DTYPE_F32;
-        uint16_t* e = codes ? reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + p->off_ex) + (int64_t)b0 * p->rows_x
+        uint16_t* e = codes && p->opts.precision == HEFF_PREC_FP64 ? reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + p->off_ex) + (int64_t)b0 * p->rows_x
                             : nullptr;
         switch (p->opts.precision) {
             case HEFF_PREC_FP64: launch_pack_t<double, HEFF_PREC_FP64>(p, xs, nb, w, e, st); break;
@@ -436,6 +437,68 @@ int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, cons
             if (f32) launch_mix_t<float, HEFF_PREC_TF32X3>(p, L, W1, W2, R, w, st);
             else launch_mix_t<double, HEFF_PREC_TF32X3>(p, L, W1, W2, R, w, st);
     }
+    count_launches(1);
+    CK(cudaGetLastError());
+    return HEFF_OK;
+}
+
+// ------------------------------------------------------------------ split tiles
+// y of the split tiles: the parts of a tile added in order (block: 8 rows of a tile; lanes along the
+// columns).  Adding them in the GEMM, by whichever CTA finishes a tile last, leaves the additions to a
+// few warps and their load latency: apply m = 1024, TF32x3, 85 us of GEMM 2 unsplit, 110 us that way.
+template <typename P, typename Y>
+__global__ void __launch_bounds__(256) sum_parts_kernel(const SplitTile* __restrict__ tiles, int row_blocks,
+                                                        const P* __restrict__ scratch, int64_t scratch_elems,
+                                                        PtrBatch ys) {
+    const SplitTile t = tiles[blockIdx.x / row_blocks];
+    const int r = (int)(blockIdx.x % row_blocks) * 8 + (threadIdx.x >> 5);
+    pdl_wait();
+    pdl_trigger();
+    if (r >= t.m) return;
+    const P* sp = scratch + (int64_t)blockIdx.y * scratch_elems + t.off + (int64_t)r * t.n;
+    Y* y = static_cast<Y*>(const_cast<void*>(ys.p[blockIdx.y])) + t.c_off + (int64_t)r * t.ldc;
+    const int64_t part = (int64_t)t.m * t.n;
+    for (int c = threadIdx.x & 31; c < t.n; c += 32) {
+        P v[SPLIT_MAX];
+#pragma unroll
+        for (int k = 0; k < SPLIT_MAX; ++k) v[k] = k < t.parts ? sp[k * part + c] : (P)0;
+        auto wide = [](P f) {
+            if constexpr (std::is_same<P, float>::value && std::is_same<Y, double>::value) return f32_to_f64(f);
+            else return (Y)f;
+        };
+        Y a = wide(v[0]);
+#pragma unroll
+        for (int k = 1; k < SPLIT_MAX; ++k)
+            if (k < t.parts) a += wide(v[k]);
+        y[c] = a;
+    }
+}
+
+int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, int nbatch, void* stream) {
+    if (g.split.empty()) return HEFF_OK;
+    PtrBatch ys{};
+    for (int b = 0; b < nbatch; ++b) ys.p[b] = y[b];
+    const int row_blocks = (g.tm + 7) / 8;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(g.split.size() * row_blocks), (unsigned)nbatch);
+    cfg.blockDim = dim3(256);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cfg.attrs = at;
+    cfg.numAttrs = HEFF_PDL ? 1 : 0;
+    const char* w = static_cast<const char*>(ws) + p->off_split;
+    const SplitTile* t = g.d_split;
+    if (p->opts.precision == HEFF_PREC_FP64)
+        cudaLaunchKernelEx(&cfg, sum_parts_kernel<double, double>, t, row_blocks, reinterpret_cast<const double*>(w),
+                           g.split_elems, ys);
+    else if (p->opts.io_dtype == HEFF_DTYPE_F64)
+        cudaLaunchKernelEx(&cfg, sum_parts_kernel<float, double>, t, row_blocks, reinterpret_cast<const float*>(w),
+                           g.split_elems, ys);
+    else
+        cudaLaunchKernelEx(&cfg, sum_parts_kernel<float, float>, t, row_blocks, reinterpret_cast<const float*>(w),
+                           g.split_elems, ys);
     count_launches(1);
     CK(cudaGetLastError());
     return HEFF_OK;
@@ -662,8 +725,8 @@ extern "C" int heff_plan_autotune(heff_plan* plan, const void* L, const void* W1
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         const void* xs[1] = {x};
         void* ys[1] = {y};
-        if ((rc = heff::launch_mix(plan, L, W1, W2, R, workspace, false, stream))) return rc;
-        if ((rc = heff::launch_pack_batch(plan, xs, 1, workspace, false, stream))) return rc;
+        if ((rc = heff::launch_mix(plan, L, W1, W2, R, workspace, true, stream))) return rc;
+        if ((rc = heff::launch_pack_batch(plan, xs, 1, workspace, true, stream))) return rc;
         // each candidate: one warm-up launch, then the median of 5 separately timed launches
         cudaEvent_t e[6];
         for (auto& ev : e) CK(cudaEventCreate(&ev));
@@ -676,10 +739,10 @@ extern "C" int heff_plan_autotune(heff_plan* plan, const void* L, const void* W1
                 ms[c] = 0.f;
                 if (v[c]->tasks.empty() && !v[0]->tasks.empty()) continue;
                 std::swap(*v[0], *v[c]);
-                rc = heff::launch_gemm(plan, which, workspace, ys, 1, false, stream);
+                rc = heff::launch_gemm(plan, which, workspace, ys, 1, true, stream);
                 CK(cudaEventRecord(e[0], st));
                 for (int r = 0; r < 5 && !rc; ++r) {
-                    rc = heff::launch_gemm(plan, which, workspace, ys, 1, false, stream);
+                    rc = heff::launch_gemm(plan, which, workspace, ys, 1, true, stream);
                     CK(cudaEventRecord(e[r + 1], st));
                 }
                 if (!rc) {

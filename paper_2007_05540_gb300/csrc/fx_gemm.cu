@@ -85,6 +85,9 @@ struct FxArgs {
     int64_t et_rows, c_batch_rows, c_batch_elems;
     PtrBatch y;                          // outputs (mode y), or y.p[0] unused
     int nbatch, b0, to_y;
+    double* split;                       // scratch of the split tiles, split_elems per batch entry
+    const SplitTile* split_tiles;
+    int64_t split_elems;
     // MODE 1
     const BTile* tiles;
     const BProd* prods;
@@ -100,7 +103,7 @@ struct FxArgs {
 };
 
 struct Tile {
-    int m, n, n_zero, ldc, steps, pbeg, pcnt, bat;
+    int m, n, n_zero, ldc, steps, pbeg, pcnt, bat, split;
     int64_t c_off, a_row, b_row;
 };
 
@@ -111,14 +114,14 @@ __device__ __forceinline__ Tile get_tile(const FxArgs& g, long item) {
         const int b = (int)(item % g.nbatch);
         const GemmTask k = g.tasks[item / g.nbatch];
         t.m = k.m; t.n = k.n; t.n_zero = k.n_zero; t.ldc = k.ldc; t.steps = k.ktotal / FKS;
-        t.pbeg = k.seg_begin; t.pcnt = k.seg_count; t.bat = b;
+        t.pbeg = k.seg_begin; t.pcnt = k.seg_count; t.bat = b; t.split = k.split;
         t.c_off = k.c_off;
         t.a_row = k.a_row + (g.b0 + b) * g.a_batch_rows;
         t.b_row = k.b_row + (g.b0 + b) * g.b_batch_rows;
     } else {
         const BTile k = g.tiles[item];
         t.m = k.m; t.n = k.n; t.n_zero = 0; t.ldc = k.ldc; t.steps = k.steps;
-        t.pbeg = k.prod_begin; t.pcnt = k.prod_count; t.bat = 0;
+        t.pbeg = k.prod_begin; t.pcnt = k.prod_count; t.bat = 0; t.split = 0;
         t.c_off = k.c_off; t.a_row = 0; t.b_row = 0;
     }
     return t;
@@ -364,8 +367,14 @@ __device__ __forceinline__ void issue_step(int n16, uint32_t tmem, uint64_t a, u
     else issue_planes<16, NK>(tmem, a, b, fresh);
 }
 
+// Where a tile's values go: the output, or a split tile's part of its scratch.
+template <int MODE>
+__device__ __forceinline__ int64_t out_pitch(const Tile& t) { return MODE == 0 && t.split ? t.n : t.ldc; }
 template <int MODE>
 __device__ __forceinline__ double* out_ptr(const FxArgs& g, const Tile& t) {
+    if (MODE == 0 && t.split)
+        return g.split + (int64_t)t.bat * g.split_elems + g.split_tiles[t.split >> 9].off +
+               (int64_t)((t.split >> 5) & 15) * t.m * t.n;
     if constexpr (MODE == 0)
         return (g.to_y ? static_cast<double*>(const_cast<void*>(g.y.p[t.bat]))
                        : g.C + (int64_t)(g.b0 + t.bat) * g.c_batch_elems) + t.c_off;
@@ -399,6 +408,7 @@ __device__ __forceinline__ bool fp64_tile(const FxArgs& g, const Tile& t, double
     double (*Bs)[65] = As + 8;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     double* C = out_ptr<MODE>(g, t);
+    const int64_t ldc = out_pitch<MODE>(t);
     for (int half = 0; half < t.m; half += 64) {
         const int m = t.m - half < 64 ? t.m - half : 64;
         double acc[4][4] = {};
@@ -438,7 +448,7 @@ __device__ __forceinline__ bool fp64_tile(const FxArgs& g, const Tile& t, double
                 const int c = tx * 4 + j;
                 const double v = c < t.n ? acc[i][j] : 0.0;
                 if (r < m && c < t.n + t.n_zero) {
-                    double* cp = C + (int64_t)(half + r) * t.ldc + c;
+                    double* cp = C + (int64_t)(half + r) * ldc + c;
                     if (MODE == 0) *cp = v;
                     else *cp = g.accumulate ? *cp + scale * v : scale * v;
                 }
@@ -632,7 +642,8 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                 const int* es = escale + b * (FM + FN);
                 const int er = es[q * 32 + lane] - 2112;
                 const int rows = t.m - q * 32 < 32 ? t.m - q * 32 : 32;
-                double* C = out_ptr<MODE>(g, t) + (int64_t)(q * 32) * t.ldc;
+                const int64_t ldc = out_pitch<MODE>(t);
+                double* C = out_ptr<MODE>(g, t) + (int64_t)(q * 32) * ldc;
                 const int ncols = t.n + t.n_zero;
                 int code = 0;
 #pragma unroll
@@ -654,7 +665,7 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                         const int c = lane & 7;
                         for (int r = lane >> 3; r < rows; r += 4)
                             if (col0 + c < ncols) {
-                                double* cp = C + (int64_t)r * t.ldc + col0 + c;
+                                double* cp = C + (int64_t)r * ldc + col0 + c;
                                 const double v = tr[r * 9 + c];
                                 *cp = MODE == 1 && g.accumulate ? *cp + v : v;
                             }
@@ -845,6 +856,11 @@ int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbat
             g.a_batch_rows = p->rows_t;
             for (int b = 0; b < g.nbatch; ++b) g.y.p[b] = y[b0 + b];
             g.to_y = 1;
+            if (p->kchunk) {
+                g.split = reinterpret_cast<double*>(w + p->off_split);
+                g.split_tiles = gl.d_split;
+                g.split_elems = gl.split_elems;
+            }
             if (codes) {
                 g.ea = e_t;
                 g.ea_rows = t_rows;
@@ -853,6 +869,7 @@ int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbat
             }
         }
         int rc = launch_fx<0>(g, p->num_sms > 0 ? p->num_sms : 148, static_cast<cudaStream_t>(stream));
+        if (!rc && which == 2 && p->kchunk) rc = launch_sum_parts(p, gl, ws, y + b0, g.nbatch, stream);
         if (rc) return rc;
     }
     return HEFF_OK;

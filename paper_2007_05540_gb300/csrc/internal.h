@@ -81,8 +81,16 @@ struct GemmTask {
     int32_t n_zero;         // columns [n, n + n_zero) of the tile are written as 0 (padding)
     int32_t seg_begin, seg_count;
     int32_t ktotal;         // sum of the segments' klen (padded contraction length)
-    int32_t pad_;
+    int32_t split;          // 0, or one of several parts of the tile's contraction (split_code)
 };
+// A tile whose contraction is split over several tasks: group (of the list), part, number of parts.
+// Each part leaves its sum in the group's scratch, and sum_parts_kernel adds them in order.
+struct SplitTile {
+    int64_t c_off, off;     // tile origin in y; the group's scratch (parts x m x n elements)
+    int32_t ldc, m, n, parts;
+};
+constexpr int SPLIT_MAX = 16;
+inline int32_t split_code(int group, int part, int parts) { return group << 9 | part << 5 | parts; }
 struct KSeg {
     int32_t k0, klen;       // column range shared by A and B (klen multiple of KPAD)
 };
@@ -178,6 +186,10 @@ struct GemmList {
     int cl = 1;             // CTAs per entry: 2 = tasks 2e, 2e + 1 share their B tile (cluster pair)
     double flops = 0;       // executed (valid m, n; padded K)
     double useful = 0;      // valid m, n and unpadded K
+    // split tiles, one per group, and the elements of their scratch
+    std::vector<SplitTile> split;
+    SplitTile* d_split = nullptr;
+    int64_t split_elems = 0;
     // host only, one entry per task: output left sector a' and the task's flop counts
     std::vector<int32_t> owner;
     std::vector<double> task_flops, task_useful;
@@ -241,6 +253,13 @@ struct heff_plan {
     // FP64 plans: exponent codes of the operand arrays, [column / KPAD][row]; they come last in the
     // workspace (ws_min: its size without them, when every tile runs in FP64 arithmetic)
     size_t off_ex = 0, off_elw = 0, off_et = 0, off_erw = 0, ws_min = 0;
+    // split tiles of GEMM 2: chunk of the contraction (in KPAD units; 0: no limit) and their scratch in
+    // the workspace (after ws_min too).
+    // sp2, sp2_alt: the N = 256 and N = 128 lists of GEMM 2 with their long tiles split (g2 and g2_alt
+    // describe them whole); an FP64 plan's fx2 is split itself
+    heff::GemmList sp2, sp2_alt;
+    int kchunk = 0;
+    size_t off_split = 0;
     int64_t stats[24] = {0};
     // tensor-map cache for the tensor-core path: two entries keyed by workspace pointer
     // (two streams alternating workspaces reuse their maps), replaced round-robin
@@ -259,16 +278,22 @@ struct heff_plan {
 
 namespace heff {
 // launchers (apply.cu)
-// (codes: FP64 plans keep the operands' exponent codes in the workspace)
+// (codes: the workspace holds all of ws_bytes: the operands' exponent codes of an FP64 plan, and the
+// scratch of split tiles; false: ws_min, every tile in FP64 arithmetic or whole)
 int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, bool codes, void* stream);
 int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R,
                void* ws, bool codes, void* stream);
 int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream);
+// y's split tiles from their parts (batch entries [0, nbatch), scratch copies of split_elems)
+int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, int nbatch, void* stream);
 int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream);
 // one apply in the first `bytes` of ws, which may hold less than ws_bytes but at least ws_min
 int apply_in(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, const void* x, void* y,
              void* ws, size_t bytes, void* stream);
 void lpt_schedule(GemmList& G, int units, bool tc, bool first);
+// KPAD units per part of GEMM 2's contractions that balances the list over the units (0: as is)
+int split_chunk(const GemmList& G, int units, bool tc, int least);
+void split_tasks(GemmList& G, int chunk);
 // clusters of two tensor-core CTAs resident at once (tc_gemm.cu; num_sms / 2 without a device)
 int tc_pair_clusters(int num_sms, int precision);
 // one block waiting at the SVD sweeps' grid barrier set up for two (svd.cu; wait self-test)

@@ -98,6 +98,73 @@ bool check_index(const IndexDesc& a, const IndexDesc& b, int flow_a) {
 
 }  // namespace
 
+// A list of few long tiles leaves SMs idle behind its longest one (GEMM 2 at m = 1024, k = 14: 130 tiles,
+// the longest three times the average SM's work).  Such lists are cut along the contraction, at
+// multiples of one chunk for the whole plan, into parts of at most half the average SM's work:
+// shorter parts cost more in partial sums (each is written once and read once) than they balance.
+int heff::split_chunk(const GemmList& G, int units, bool tc, int least) {
+    double total = 0, longest = 0;
+    int kmax = 0, wmax = 1;
+    for (const GemmTask& k : G.tasks) {
+        const int w = tc ? (int)tile_width_cost(k.m, k.n, HEFF_TILE_COST_G2) : k.n + 32;
+        const double c = (double)(k.ktotal / KPAD + 4) * w;
+        total += c;
+        longest = std::max(longest, c);
+        kmax = std::max(kmax, k.ktotal / KPAD);
+        wmax = std::max(wmax, w);
+    }
+    const double avg = total / units;
+    if (longest <= 1.3 * avg || kmax <= least) return 0;
+    int chunk = std::max(least, (int)(avg / 2 / wmax) - 4);
+    chunk = std::max(chunk, (kmax + SPLIT_MAX - 1) / SPLIT_MAX);
+    return chunk < kmax ? chunk : 0;
+}
+
+void heff::split_tasks(GemmList& G, int chunk) {
+    GemmList s;
+    for (size_t i = 0; i < G.tasks.size(); ++i) {
+        const GemmTask& k = G.tasks[i];
+        const int parts = (k.ktotal / KPAD + chunk - 1) / chunk;
+        if (parts < 2) {
+            s.tasks.push_back(k);
+            s.owner.push_back(G.owner[i]);
+            s.task_flops.push_back(G.task_flops[i]);
+            s.task_useful.push_back(G.task_useful[i]);
+            continue;
+        }
+        const int group = (int)G.split.size();
+        G.split.push_back({k.c_off, G.split_elems, k.ldc, k.m, k.n, parts});
+        G.split_elems += (int64_t)parts * k.m * k.n;
+        int seg = 0, at = 0;                          // segment and columns of it used
+        for (int part = 0; part < parts; ++part) {
+            GemmTask t = k;
+            t.split = split_code(group, part, parts);
+            t.seg_begin = (int32_t)G.segs.size();
+            t.seg_count = 0;
+            t.ktotal = 0;
+            int left = chunk * KPAD;
+            while (left > 0 && seg < k.seg_count) {
+                const KSeg sg = G.segs[k.seg_begin + seg];
+                const int len = std::min(left, sg.klen - at);
+                G.segs.push_back({sg.k0 + at, len});
+                ++t.seg_count;
+                t.ktotal += len;
+                left -= len;
+                at += len;
+                if (at == sg.klen) { ++seg; at = 0; }
+            }
+            s.tasks.push_back(t);
+            s.owner.push_back(G.owner[i]);
+            s.task_flops.push_back(G.task_flops[i] * t.ktotal / k.ktotal);
+            s.task_useful.push_back(G.task_useful[i] * t.ktotal / k.ktotal);
+        }
+    }
+    G.tasks.swap(s.tasks);
+    G.owner.swap(s.owner);
+    G.task_flops.swap(s.task_flops);
+    G.task_useful.swap(s.task_useful);
+}
+
 // Static schedule of the persistent kernels: CTA c of a grid of min(units, entries) runs the
 // entries c, c + grid, c + 2 grid, ...  The entries are assigned by longest-processing-time (each to
 // the least loaded CTA, longest first; a tile's time ~ (K blocks + a fixed overhead) x its width
@@ -776,8 +843,71 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
             if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) ncl = heff::tc_pair_clusters(nsm, opts->precision);
             cudaGetLastError();
         }
+        // ---- workspace layout
+        size_t end = 0;
+        {
+            auto al = [](size_t v) { return (v + 255) / 256 * 256; };
+            const size_t e = (size_t)P->esize * P->planes;
+            P->off_xt = end; end = al(end + e * (size_t)opts->max_batch * P->rows_x * P->ld_x);
+            P->off_lw = end; end = al(end + e * (size_t)P->rows_lw * P->ld_x);
+            P->off_t = end;  end = al(end + e * (size_t)opts->max_batch * P->rows_t * P->ld_t);
+            P->off_rw = end; end = al(end + e * (size_t)P->rows_rw * P->ld_t);
+            P->off_flags = end; end = al(end + 256);
+            P->ws_min = end;
+            if (!tc) {
+                const size_t kx = (size_t)(P->ld_x / KPAD) * sizeof(uint16_t);
+                const size_t kt = (size_t)(P->ld_t / KPAD) * sizeof(uint16_t);
+                P->off_ex = end;  end = al(end + kx * opts->max_batch * P->rows_x);
+                P->off_elw = end; end = al(end + kx * P->rows_lw);
+                P->off_et = end;  end = al(end + kt * opts->max_batch * P->rows_t);
+                P->off_erw = end; end = al(end + kt * P->rows_rw);
+            }
+        }
+        // ---- split contractions of GEMM 2 (single-CTA tiles; the accumulation chunks of every other
+        // variant and of batched launches follow the same cuts, so that the sums' bits agree)
+        {
+            // the TF32 split's own chunk is 512 elements (16 KPAD units)
+            const bool tf32 = opts->precision == HEFF_PREC_TF32X3;
+            // (FP64 tiles cost 15-20 us each beside their contraction: split, m = 1024, 587 against 577 us)
+            int chunk = tc ? heff::split_chunk(P->g2, nsm, tc, 16) : 0;
+            if (tf32 && chunk) chunk = std::max(16, std::min(chunk, 16));
+            if (tf32 && chunk && P->g2.tasks.size()) {
+                int kmax = 0;
+                for (const auto& k : P->g2.tasks) kmax = std::max(kmax, k.ktotal / KPAD);
+                if (kmax > 16 * heff::SPLIT_MAX) chunk = 0;
+            }
+            if (chunk) {
+                const heff::GemmList whole = P->fx2;
+                heff::GemmList* split[3] = {&P->sp2, &P->sp2_alt, &P->fx2};
+                if (tc) {
+                    P->sp2 = P->g2;
+                    P->sp2_alt = P->g2_alt;
+                }
+                int64_t elems = 0;
+                for (int k = 0; k < 3; ++k) {
+                    if (tc == (k == 2)) continue;
+                    heff::split_tasks(*split[k], chunk);
+                    elems = std::max(elems, split[k]->split_elems);
+                }
+                // one scratch per batch entry where batched launches split too (FP64)
+                const size_t bytes = tc ? 4 * (size_t)elems : 8 * (size_t)opts->max_batch * (size_t)elems;
+                // not at the price of the built-in workspace, which would otherwise hold the plan, nor of
+                // a tenth of the workspace
+                if ((P->ws_min <= HEFF_NOALLOC_WORKSPACE_BYTES && end + bytes + 256 > HEFF_NOALLOC_WORKSPACE_BYTES) ||
+                    bytes > end / 10 + ((size_t)1 << 20)) {
+                    P->sp2 = P->sp2_alt = heff::GemmList{};
+                    P->fx2 = whole;
+                } else {
+                    P->kchunk = chunk;
+                    P->off_split = end;
+                    end = (end + bytes + 255) / 256 * 256;
+                }
+            }
+            P->ws_bytes = end;
+        }
         if (HEFF_LPT_SCHEDULE) {
-            for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->g1_pair, &P->g2_pair, &P->fx1, &P->fx2}) {
+            for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->g1_pair, &P->g2_pair, &P->sp2,
+                                      &P->sp2_alt, &P->fx1, &P->fx2}) {
                 if (!tc && (G == &P->g1 || G == &P->g2)) continue;    // 64 x 64 tiles: only described, not run
                 const bool first = G == &P->g1 || G == &P->g1_alt || G == &P->g1_pair;
                 heff::lpt_schedule(*G, G->cl == 2 ? ncl : nsm, tc, first);
@@ -785,24 +915,6 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
         }
         for (int i = 0; i < na; ++i) if (owned[i]) P->shard_sectors.push_back(i);
         const int TM = P->g1.tm, TN = P->g1.tn;
-        // ---- workspace layout
-        auto al = [](size_t v) { return (v + 255) / 256 * 256; };
-        const size_t e = (size_t)P->esize * P->planes;
-        size_t off = 0;
-        P->off_xt = off; off = al(off + e * (size_t)opts->max_batch * P->rows_x * P->ld_x);
-        P->off_lw = off; off = al(off + e * (size_t)P->rows_lw * P->ld_x);
-        P->off_t = off;  off = al(off + e * (size_t)opts->max_batch * P->rows_t * P->ld_t);
-        P->off_rw = off; off = al(off + e * (size_t)P->rows_rw * P->ld_t);
-        P->off_flags = off; off = al(off + 256);
-        P->ws_min = off;
-        if (!tc) {
-            const size_t kx = (size_t)(P->ld_x / KPAD) * sizeof(uint16_t), kt = (size_t)(P->ld_t / KPAD) * sizeof(uint16_t);
-            P->off_ex = off;  off = al(off + kx * opts->max_batch * P->rows_x);
-            P->off_elw = off; off = al(off + kx * P->rows_lw);
-            P->off_et = off;  off = al(off + kt * opts->max_batch * P->rows_t);
-            P->off_erw = off; off = al(off + kt * P->rows_rw);
-        }
-        P->ws_bytes = off;
         int64_t* st = P->stats;
         st[0] = (int64_t)Q.size(); st[1] = (int64_t)rgs.size(); st[2] = (int64_t)rws.size();
         st[3] = (int64_t)P->g1.tasks.size(); st[4] = (int64_t)P->g2.tasks.size();

@@ -244,6 +244,8 @@ struct TcArgs {
     int b0;                               // first batch entry of this launch
     int* err;                             // sticky error flag in the workspace
     Merge mg;                             // merged items
+    float* split;                         // scratch of the split tiles
+    const SplitTile* split_tiles;
 };
 
 // A work item: the task, its first batch entry (of the launch) and their number, the slot width
@@ -712,6 +714,12 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                             *reinterpret_cast<uint4*>(lo + o) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
                         }
                     }
+                } else if (!MG && CL == 1 && t.split) {
+                    // a part of a split tile: its sum goes to the part's scratch
+                    float* sp = g.split + g.split_tiles[t.split >> 9].off +
+                                (int64_t)((t.split >> 5) & 15) * t.m * t.n + (int64_t)row0 * t.n + c;
+                    if (c < t.n)
+                        for (int r = 0; r < rows; ++r) sp[(int64_t)r * t.n] = stage[r * 32 + (lane ^ r)];
                 } else if (c < t.n) {
                     // chunk 0 stores, later chunks add (same thread, same order: deterministic);
                     // the previous values of 8 rows are loaded before their stores so the
@@ -926,7 +934,8 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
         if (rc) return rc;
         p->tmap_ws[slot] = ws;
     }
-    const GemmList& gl = which == 1 ? p->g1 : p->g2;
+    const bool split = which == 2 && p->kchunk && CL == 1 && !MG && nbatch == 1;
+    const GemmList& gl = split ? (TN_TC == 256 ? p->sp2 : p->sp2_alt) : which == 1 ? p->g1 : p->g2;
     const MergeList& ml = which == 1 ? p->mg1 : p->mg2;
     if (gl.tasks.empty()) return HEFF_OK;
     TcMaps maps;
@@ -954,7 +963,12 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
             g.a_batch_rows = p->rows_t; g.b_batch_rows = 0;
             for (int b = 0; b < nb; ++b) g.y.p[b] = y[b0 + b];
             g.mode = 1;
-            g.kchunk = (PREC == HEFF_PREC_TF32X3 ? KCHUNK_TF32 : KCHUNK_BF16) * 64 / SWZ_TC;
+            g.kchunk = p->kchunk ? p->kchunk * (KPAD * (PREC == HEFF_PREC_TF32X3 ? 4 : 2) / SWZ_TC)
+                                 : (PREC == HEFF_PREC_TF32X3 ? KCHUNK_TF32 : KCHUNK_BF16) * 64 / SWZ_TC;
+            if (split) {
+                g.split = reinterpret_cast<float*>(w + p->off_split);
+                g.split_tiles = gl.d_split;
+            }
             g.y_f64 = p->opts.io_dtype == HEFF_DTYPE_F64;
         }
         long total = (long)(g.ntasks / CL) * nb;              // entries (tiles, or pairs of tiles)
@@ -992,7 +1006,7 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "tc_gemm launch: %s", cudaGetErrorString(e));
-    return HEFF_OK;
+    return split ? launch_sum_parts(p, gl, ws, y, 1, st) : HEFF_OK;
 }
 
 }  // namespace
