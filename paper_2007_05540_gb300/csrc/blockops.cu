@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <type_traits>
 
 #include "convert.cuh"
@@ -76,10 +77,7 @@ void BList::retile(int tm, int tn) {
 }
 
 int blist_upload(BList& b) {
-    b.d_tiles = nullptr;
-    b.d_prods = nullptr;
-    b.d_rows = nullptr;
-    b.d_codes = nullptr;
+    b.d_tables = nullptr;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&b.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -89,22 +87,32 @@ int blist_upload(BList& b) {
         std::stable_sort(b.tiles.begin(), b.tiles.end(), [](const BTile& x, const BTile& y) {
             return (int64_t)x.steps * (x.n + 32) > (int64_t)y.steps * (y.n + 32);
         });
-    auto up = [](const auto& v, auto** d) {
-        return v.empty() || (cudaMalloc((void**)d, v.size() * sizeof(v[0])) == cudaSuccess &&
-                             cudaMemcpy(*d, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice) == cudaSuccess);
-    };
-    if (!up(b.tiles, &b.d_tiles) || !up(b.prods, &b.d_prods) || !up(b.rows, &b.d_rows))
+    // one allocation for the tables and the codes
+    auto al = [](size_t v) { return (v + 255) / 256 * 256; };
+    const size_t nt = b.tiles.size() * sizeof(BTile), np = b.prods.size() * sizeof(BProd), nr = b.rows.size() * sizeof(FxRows);
+    const size_t op = al(nt), orow = op + al(np), oc = orow + al(nr);
+    if (oc + b.ncodes == 0) return HEFF_OK;
+    std::vector<char> host(oc);
+    if (nt) std::memcpy(host.data(), b.tiles.data(), nt);
+    if (np) std::memcpy(host.data() + op, b.prods.data(), np);
+    if (nr) std::memcpy(host.data() + orow, b.rows.data(), nr);
+    char* d = nullptr;
+    if (cudaMalloc((void**)&d, oc + b.ncodes * sizeof(uint16_t)) != cudaSuccess ||
+        cudaMemcpy(d, host.data(), oc, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaFree(d);
         return fail(HEFF_ERR_CUDA, "block list upload failed");
-    if (b.ncodes && cudaMalloc((void**)&b.d_codes, b.ncodes * sizeof(uint16_t)) != cudaSuccess)
-        return fail(HEFF_ERR_CUDA, "block list upload failed");
+    }
+    b.d_tables = d;
+    b.d_tiles = reinterpret_cast<BTile*>(d);
+    b.d_prods = reinterpret_cast<BProd*>(d + op);
+    b.d_rows = reinterpret_cast<FxRows*>(d + orow);
+    b.d_codes = reinterpret_cast<uint16_t*>(d + oc);
     return HEFF_OK;
 }
 
 void blist_free(BList& b) {
-    cudaFree(b.d_tiles);
-    cudaFree(b.d_prods);
-    cudaFree(b.d_rows);
-    cudaFree(b.d_codes);
+    cudaFree(b.d_tables);
+    b.d_tables = nullptr;
     b.d_tiles = nullptr;
     b.d_prods = nullptr;
     b.d_rows = nullptr;

@@ -46,6 +46,7 @@ struct heff_env_plan {
     bool dense = true;
     std::vector<GemmTask> blocks1, blocks2;
     std::vector<heff::KSeg> segs1, segs2;
+    std::vector<std::tuple<int, int64_t, int, std::vector<heff::KSeg>>> units;   // array, row, rows, segments
     std::vector<heff::PackTile> pack;
     std::vector<heff::MixTile> mix;
     std::vector<heff::MixTerm> terms;
@@ -116,6 +117,8 @@ void build_dense(heff_env_plan* P, const heff_layout* env_old, const heff_layout
                 P->mix.push_back({sp_row[j], c0, mj, mi, pad, r0, std::min(32, mj - r0), tb, 1, 1});
         }
     }
+    for (int j = 0; j < nj; ++j)
+        if (width[j]) P->units.push_back({1, sp_row[j], (int)out.dims[j], {{0, width[j]}}});
     P->rows_sp = std::max<int64_t>(rows, 1);
     P->ld = KPAD;
     for (int j = 0; j < nj; ++j) P->ld = std::max<int64_t>(P->ld, width[j]);
@@ -169,7 +172,8 @@ void build_dense(heff_env_plan* P, const heff_layout* env_old, const heff_layout
             if (it == groups.end()) continue;
             Group& g = it->second;
             const int mip = in.dims[ip], pad = (int)pad_up(mip, KPAD);
-            if (g.row < 0) {
+            const bool fresh = g.row < 0;
+            if (fresh) {
                 g.row = lw_rows;
                 lw_rows += mip;
                 for (auto& kv : g.segs) {
@@ -198,11 +202,15 @@ void build_dense(heff_env_plan* P, const heff_layout* env_old, const heff_layout
                 g1.ktotal += len;
             }
             g1.seg_count = (int32_t)P->segs1.size() - g1.seg_begin;
+            if (fresh)
+                P->units.push_back({0, g.row, mip, std::vector<heff::KSeg>(P->segs1.begin() + g1.seg_begin,
+                                                                           P->segs1.end())});
             P->blocks1.push_back(g1);
             P->segs2.push_back({c0, pad});
             g2.ktotal += pad;
         }
         g2.seg_count = (int32_t)P->segs2.size() - g2.seg_begin;
+        P->units.push_back({2, t_rows, mj, std::vector<heff::KSeg>(P->segs2.begin() + g2.seg_begin, P->segs2.end())});
         P->blocks2.push_back(g2);
         t_rows += mj;
     }
@@ -229,7 +237,20 @@ size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
         o_ex = off;  off = al(off + kb * P->rows_sp);
         o_elw = off; off = al(off + kb * P->rows_lw);
         o_et = off;  off = al(off + kb * P->rows_t);
-        if (p) { p->off_ex = o_ex; p->off_elw = o_elw; p->off_et = o_et; p->off_erw = o_et; }
+        heff_plan size_only;
+        heff_plan* f = p ? p : &size_only;
+        f->off_ex = o_ex; f->off_elw = o_elw; f->off_et = o_et; f->off_erw = o_et;
+        f->ws_codes = off;
+        const struct { int64_t rows; bool a; size_t src, codes; } ops[3] = {
+            {P->rows_lw, false, o_lw, o_elw}, {P->rows_sp, true, o_sp, o_ex}, {P->rows_t, false, o_t, o_et}};
+        for (int o = 0; o < 3; ++o) {
+            f->fxo[o].ld = P->ld;
+            f->fxo[o].rows = ops[o].rows;
+            f->fxo[o].a_side = ops[o].a;
+            f->fxo[o].off_src = ops[o].src;
+            f->fxo[o].off_codes = ops[o].codes;
+        }
+        off = heff::plane_layout(f, off);
     }
     if (p) p->ws_bytes = off;
     return off;
@@ -252,6 +273,8 @@ int ensure_plan(heff_env_plan* P) {
         p->rows_x = P->rows_sp; p->ld_x = P->ld; p->rows_lw = P->rows_lw;
         p->rows_t = P->rows_t; p->ld_t = P->ld; p->rows_rw = 0;
         dense_bytes(P, P->precision, p.get());
+        if (!tc)
+            for (const auto& u : P->units) p->fxo[std::get<0>(u)].add(std::get<1>(u), std::get<2>(u), std::get<3>(u));
         p->pack = P->pack;
         p->mix = P->mix;
         p->terms = P->terms;
@@ -514,10 +537,14 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
         const void* xs[1] = {site};
         void* ys[1] = {env_new};
         // the mix tiles read env_old as L with W as W1, and (side 1) the site tensor as R
-        if ((rc = heff::launch_mix(p, env_old, W, W, site, ws, true, stream))) return rc;
-        if ((rc = heff::launch_pack_batch(p, xs, 1, ws, true, stream))) return rc;
-        if ((rc = heff::launch_gemm(p, 1, ws, ys, 1, true, stream))) return rc;
-        return heff::launch_gemm(p, 2, ws, ys, 1, true, stream);
+        const int level = heff::fx_level(p, workspace_bytes);
+        if ((rc = heff::launch_mix(p, env_old, W, W, site, ws, level, stream))) return rc;
+        if ((rc = heff::launch_pack_batch(p, xs, 1, ws, level, stream))) return rc;
+        if (level == 2 && plan->precision == HEFF_PREC_FP64)
+            for (int array : {1, 0})
+                if ((rc = heff::launch_digits(p, array, ws, 1, stream))) return rc;
+        if ((rc = heff::launch_gemm(p, 1, ws, ys, 1, level, stream))) return rc;
+        return heff::launch_gemm(p, 2, ws, ys, 1, level, stream);
     }
     int* err = reinterpret_cast<int*>(ws);
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), static_cast<cudaStream_t>(stream));

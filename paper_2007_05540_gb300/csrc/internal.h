@@ -124,6 +124,7 @@ constexpr int FX_TILE_M = 128, FX_TILE_N = 64;
 struct BList {
     std::vector<BTile> tiles;
     std::vector<BProd> prods;
+    char* d_tables = nullptr;  // the device tables' one allocation
     BTile* d_tiles = nullptr;
     BProd* d_prods = nullptr;
     double flops = 0;
@@ -203,6 +204,33 @@ struct MergeList {
     int first[7] = {0, 0, 0, 0, 0, 0, 0};
 };
 
+// An FP64 plan's operand array as digit planes (fx_planes.cu).  Units: up to 8 rows that share their
+// column segments (the ones that are written and read).
+struct FxUnit {
+    int64_t row0;
+    int32_t nrows, seg_begin, seg_count;
+};
+struct FxOperand {
+    std::vector<FxUnit> units;
+    std::vector<KSeg> segs;
+    FxUnit* d_units = nullptr;
+    KSeg* d_segs = nullptr;
+    int64_t ld = 0, rows = 0, batch_rows = 0;     // rows: of all batch entries; 0 batch_rows: shared by them
+    bool a_side = false;
+    int code_cols = KPAD;           // columns per exponent code
+    size_t off_src = 0, off_codes = 0, off_planes = 0, off_scale = 0;    // in the workspace
+    // rows [row0, row0 + n) over the given segments
+    void add(int64_t row0, int n, const std::vector<KSeg>& s) {
+        const int32_t sb = (int32_t)segs.size();
+        segs.insert(segs.end(), s.begin(), s.end());
+        for (int r = 0; r < n; r += 8) units.push_back({row0 + r, n - r < 8 ? n - r : 8, sb, (int32_t)s.size()});
+    }
+};
+// the largest workspace with digit planes (16 bytes per operand element beside 8)
+constexpr size_t FX_PLANES_MAX = (size_t)64 << 30;
+// columns per exponent code of T where fx_planes.cu writes it (eight columns go through its drain at a time)
+constexpr int FX_T_CODE_COLS = 8;
+
 }  // namespace heff
 
 struct heff_layout {
@@ -231,7 +259,8 @@ struct heff_plan {
     size_t off_xt = 0, off_lw = 0, off_t = 0, off_rw = 0, off_flags = 0, ws_bytes = 0;
     double flops_canonical = 0;
     std::vector<int32_t> shard_sectors;   // left sectors a' of y this plan computes
-    // device tables
+    // device tables: one allocation, the pointers below into it
+    void* d_tables = nullptr;
     std::vector<heff::PackTile> pack;
     std::vector<heff::MixTile> mix;
     std::vector<heff::MixTerm> terms;
@@ -260,6 +289,14 @@ struct heff_plan {
     heff::GemmList sp2, sp2_alt;
     int kchunk = 0;
     size_t off_split = 0;
+    // FP64 plans: LW, XT, T, RW as digit planes, after ws_codes in the workspace (planes: whether they
+    // are there; ws_codes: its size without them), and their tensor maps for the last two workspaces
+    heff::FxOperand fxo[4];
+    bool planes_ok = false;
+    size_t ws_codes = 0;
+    void* fx_ws[2] = {nullptr, nullptr};
+    int fx_next = 0;
+    alignas(64) unsigned char fx_maps[2][4][4 * 128];
     int64_t stats[24] = {0};
     // tensor-map cache for the tensor-core path: two entries keyed by workspace pointer
     // (two streams alternating workspaces reuse their maps), replaced round-robin
@@ -278,12 +315,18 @@ struct heff_plan {
 
 namespace heff {
 // launchers (apply.cu)
-// (codes: the workspace holds all of ws_bytes: the operands' exponent codes of an FP64 plan, and the
-// scratch of split tiles; false: ws_min, every tile in FP64 arithmetic or whole)
-int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, bool codes, void* stream);
+// level: what an FP64 plan's call has in its workspace: 2 digit planes, 1 the operands' exponent codes, 0
+// the FP64 operands alone (every tile in FP64 arithmetic)
+int fx_level(const heff_plan* p, size_t ws_bytes);
+int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, int level, void* stream);
 int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R,
-               void* ws, bool codes, void* stream);
-int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream);
+               void* ws, int level, void* stream);
+int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, int level, void* stream);
+int launch_digits(heff_plan* p, int array, void* ws, int nbatch, void* stream);
+int launch_fx_planes(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
+// workspace of the digit planes from `end` on (offsets set); returns the new end, or `end` when the
+// planes would pass FX_PLANES_MAX
+size_t plane_layout(heff_plan* p, size_t end);
 // y's split tiles from their parts (batch entries [0, nbatch), scratch copies of split_elems)
 int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, int nbatch, void* stream);
 int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream);

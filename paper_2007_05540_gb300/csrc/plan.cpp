@@ -98,6 +98,21 @@ bool check_index(const IndexDesc& a, const IndexDesc& b, int flow_a) {
 
 }  // namespace
 
+size_t heff::plane_layout(heff_plan* p, size_t end) {
+    auto al = [](size_t v) { return (v + 255) / 256 * 256; };
+    size_t o = end;
+    for (FxOperand& f : p->fxo) {
+        f.off_planes = o; o = al(o + 16 * (size_t)f.ld * (size_t)f.rows);
+        f.off_scale = o;  o = al(o + sizeof(int32_t) * (size_t)f.rows);
+    }
+    // T's exponent codes, finer than those that fx_gemm.cu writes
+    FxOperand& t = p->fxo[2];
+    t.code_cols = FX_T_CODE_COLS;
+    t.off_codes = o; o = al(o + sizeof(uint16_t) * (size_t)(t.ld / FX_T_CODE_COLS) * (size_t)t.rows);
+    p->planes_ok = o <= FX_PLANES_MAX;
+    return p->planes_ok ? o : end;
+}
+
 // A list of few long tiles leaves SMs idle behind its longest one (GEMM 2 at m = 1024, k = 14: 130 tiles,
 // the longest three times the average SM's work).  Such lists are cut along the contraction, at
 // multiples of one chunk for the whole plan, into parts of at most half the average SM's work:
@@ -868,8 +883,7 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
         {
             // the TF32 split's own chunk is 512 elements (16 KPAD units)
             const bool tf32 = opts->precision == HEFF_PREC_TF32X3;
-            // (FP64 tiles cost 15-20 us each beside their contraction: split, m = 1024, 587 against 577 us)
-            int chunk = tc ? heff::split_chunk(P->g2, nsm, tc, 16) : 0;
+            int chunk = heff::split_chunk(tc ? P->g2 : P->fx2, nsm, tc, tc ? 16 : 8);
             if (tf32 && chunk) chunk = std::max(16, std::min(chunk, 16));
             if (tf32 && chunk && P->g2.tasks.size()) {
                 int kmax = 0;
@@ -903,7 +917,55 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
                     end = (end + bytes + 255) / 256 * 256;
                 }
             }
-            P->ws_bytes = end;
+            P->ws_codes = P->ws_bytes = end;
+        }
+        if (!tc) {
+            // operand units for the digit planes
+            auto pad = [](int v) { return (int32_t)pad_up(v, KPAD); };
+            for (auto& rg : rgs) {
+                if (!owned[rg.ip]) continue;
+                std::vector<heff::KSeg> sg;
+                for (auto& s : rg.segs) sg.push_back({Q[rg.q].cg[s.cg].col, pad(Q[rg.q].cg[s.cg].dim)});
+                P->fxo[0].add(rg.lw_row0, alpha.dims[rg.ip], sg);
+            }
+            for (int q = 0; q < (int)Q.size(); ++q) {
+                const QSec& qs = Q[q];
+                P->fxo[1].add(qs.xt_row0, qs.nrows, {{0, qs.kc}});
+                for (auto& gc : qs.cg) {
+                    if (!owned[gc.sec]) continue;
+                    std::vector<heff::KSeg> sg;
+                    for (auto& kv : qs.toff) {
+                        const int qsrc = q_minus_m[(size_t)q * km + kv.first.first];
+                        if (!present_tab[((size_t)qsrc * d1 + gc.s) * km + kv.first.first]) continue;
+                        sg.push_back({kv.second, pad(Q[qsrc].eg[kv.first.second].dim)});
+                    }
+                    P->fxo[2].add(qs.t_row0 + gc.row, gc.dim, sg);
+                }
+            }
+            for (auto& rw : rws) {
+                const QSec& qs = Q[rw.q];
+                std::vector<heff::KSeg> sg;
+                for (auto& s : rw.segs) {
+                    auto it = qs.toff.find({s.wm, s.eg_src});
+                    if (it != qs.toff.end()) sg.push_back({it->second, pad(Q[s.q_src].eg[s.eg_src].dim)});
+                }
+                P->fxo[3].add(qs.rw_row0 + qs.eg[rw.eg].row, qs.eg[rw.eg].dim, sg);
+            }
+            const struct { int64_t ld, rows, batch; bool a; size_t src, codes; } ops[4] = {
+                {P->ld_x, P->rows_lw, 0, true, P->off_lw, P->off_elw},
+                {P->ld_x, P->rows_x, P->rows_x, false, P->off_xt, P->off_ex},
+                {P->ld_t, P->rows_t, P->rows_t, true, P->off_t, P->off_et},
+                {P->ld_t, P->rows_rw, 0, false, P->off_rw, P->off_erw}};
+            for (int o = 0; o < 4; ++o) {
+                heff::FxOperand& f = P->fxo[o];
+                f.ld = ops[o].ld;
+                f.rows = ops[o].batch ? opts->max_batch * ops[o].rows : ops[o].rows;
+                f.batch_rows = ops[o].batch;
+                f.a_side = ops[o].a;
+                f.off_src = ops[o].src;
+                f.off_codes = ops[o].codes;
+            }
+            P->ws_bytes = heff::plane_layout(P, P->ws_codes);
         }
         if (HEFF_LPT_SCHEDULE) {
             for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->g1_pair, &P->g2_pair, &P->sp2,
