@@ -9,6 +9,11 @@
 //                    written per element: bound by HBM or L2)
 //   fx_plane_kernel  multiplies planes: a persistent CTA per SM, 128 x 64 tiles, one thread issuing TMA
 //                    loads, one issuing MMAs, eight drain warps
+// Prepared matvec, m = 1024, k = 14: 577 us from fx_gemm.cu, 400 us here (GEMM 1 163, GEMM 2 124, planes of T
+// 45, of x 7); environment update m = 1024 309 -> 253 us.  Bound by the drain (74 us of GEMM 1's 163 go when it is
+// left out) and the loads' latency on contractions of two to ten K blocks; the MMAs are 45 us of it.  128 x 32
+// tiles with two accumulator sets drain under the next tile's MMAs, but read A twice as often: 151 and
+// 160 us.
 // The planes take 16 bytes per operand element, so plans whose workspace would pass FX_PLANES_MAX and
 // calls on a smaller workspace (heff_apply_noalloc) use fx_gemm.cu.
 //
