@@ -122,14 +122,29 @@ void blist_free(BList& b) {
 namespace {
 
 // one CTA per dot: partial[d] = <X[x_off..], Y[y_off..]>, accumulated in the element type
-// (FP32 vectors come from the tensor-core products, whose values carry ~1e-5 anyway)
+// (FP32 vectors come from the tensor-core products, whose values carry ~1e-5 anyway).  Bound by the
+// latency of its loads: four of each vector are issued before the first product.
 template <typename T>
 __global__ void __launch_bounds__(256) block_dot_kernel(const BDot* __restrict__ dots, const T* __restrict__ X,
                                                         const T* __restrict__ Y, double* __restrict__ partial) {
     __shared__ T sh[8];
     const BDot d = dots[blockIdx.x];
-    T a = 0;
-    for (int64_t i = threadIdx.x; i < d.len; i += blockDim.x) a = fma(X[d.x_off + i], Y[d.y_off + i], a);
+    const T* x = X + d.x_off;
+    const T* y = Y + d.y_off;
+    T a4[4] = {0, 0, 0, 0};
+    int64_t i = threadIdx.x;
+    for (; i + 3 * 256 < d.len; i += 4 * 256) {
+        T u[4], v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            u[j] = x[i + j * 256];
+            v[j] = y[i + j * 256];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a4[j] = fma(u[j], v[j], a4[j]);
+    }
+    for (; i < d.len; i += 256) a4[0] = fma(x[i], y[i], a4[0]);
+    T a = (a4[0] + a4[1]) + (a4[2] + a4[3]);
     for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
     __syncthreads();
@@ -141,14 +156,18 @@ __global__ void __launch_bounds__(256) block_dot_kernel(const BDot* __restrict__
     }
 }
 
-// out[j] = scale * sum of partial[d] for d in [off[j], off[j+1]) (dots sorted by output;
-// fixed order, deterministic)
-__global__ void gather_dots_kernel(const int32_t* __restrict__ off, const double* __restrict__ partial,
-                                   double* __restrict__ out, int nout, double scale, int accumulate) {
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nout; j += gridDim.x * blockDim.x) {
+// out[j] = scale * sum of partial[d] for d in [off[j], off[j+1]) (dots sorted by output), a warp per
+// output: each lane sums every 32nd partial, then the lanes in a fixed tree (deterministic)
+__global__ void __launch_bounds__(256) gather_dots_kernel(const int32_t* __restrict__ off,
+                                                          const double* __restrict__ partial,
+                                                          double* __restrict__ out, int nout, double scale,
+                                                          int accumulate) {
+    const int lane = threadIdx.x & 31, nw = gridDim.x * (blockDim.x >> 5);
+    for (int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < nout; j += nw) {
         double s = 0.0;
-        for (int d = off[j]; d < off[j + 1]; ++d) s += partial[d];
-        out[j] = accumulate ? out[j] + scale * s : scale * s;
+        for (int d = off[j] + lane; d < off[j + 1]; d += 32) s += partial[d];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) out[j] = accumulate ? out[j] + scale * s : scale * s;
     }
 }
 
@@ -162,7 +181,7 @@ static int block_dots_t(const BDot* d_dots, int ndots, const int32_t* d_off, con
         block_dot_kernel<T><<<ndots, 256, 0, st>>>(d_dots, X, Y, scratch);
         count_launches(1);
     }
-    gather_dots_kernel<<<(nout + 255) / 256, 256, 0, st>>>(d_off, scratch, out, nout, scale, accumulate ? 1 : 0);
+    gather_dots_kernel<<<(nout + 7) / 8, 256, 0, st>>>(d_off, scratch, out, nout, scale, accumulate ? 1 : 0);
     count_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "block dots launch: %s", cudaGetErrorString(e));

@@ -222,10 +222,13 @@ extern "C" int heff_grad_plan_create(const heff_layout* L, const heff_layout* W1
         }
         // Chunks of consecutive left sectors whose U and T1 fit the limit (0: one chunk)
         auto al = [](int64_t v) { return (v + 31) / 32 * 32; };
-        const int64_t CH = 1 << 16;
-        const int64_t nxd = (x->nelem + CH - 1) / CH;
         int64_t total_g = 0;
         for (auto& kv : cnt) total_g += kv.second.first * kv.second.second;
+        // x in pieces for <x, x> and <x, y>, one block each: of 4096 elements, as far as the partial sums fit
+        // the slots that the G dots need anyway (the workspace size stays)
+        const int64_t slots = std::min<int64_t>(2048, std::max<int64_t>(total_g, (x->nelem + 65535) / 65536));
+        const int64_t CH = std::max<int64_t>(4096, slots > 0 ? (x->nelem + slots - 1) / slots : 4096);
+        const int64_t nxd = (x->nelem + CH - 1) / CH;
         const int64_t fixed = 2 * al(g->ng) + 32 + al(std::max<int64_t>(total_g, nxd));
         std::vector<int> chunk_of(nsa, 0);
         int nchunk = 1;
