@@ -87,51 +87,60 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // instruction writes two full 32-column row pieces of a half (hi or lo).
 constexpr int PACK_WARPS = 4;
 
-template <typename In, int PREC>
-__global__ void __launch_bounds__(32 * PACK_WARPS) pack_kernel(const PackTile* __restrict__ tiles, int ntiles,
-                                                               PtrBatch xs, char* __restrict__ xt, int64_t ld,
-                                                               int64_t batch_elems, uint16_t* __restrict__ codes,
-                                                               int64_t code_rows, int64_t batch_rows) {
+struct PackArgs {
+    const PackTile* tiles;
+    int ntiles;
+    PtrBatch xs;
+    char* xt;
+    int64_t ld, batch_elems;
+    uint16_t* codes;             // FP64: exponent codes, or null
+    int64_t code_rows, batch_rows;
+};
+
+template <int PREC> using PackAcc = typename std::conditional<PREC == HEFF_PREC_FP64, double, float>::type;
+
+// G: rows of x whose loads are issued before the first conversion
+template <typename In, int PREC, int G>
+__device__ __forceinline__ void pack_tile(const PackArgs& g, int ti, int bz, PackAcc<PREC> (*sw)[33]) {
     using E = typename Plane<PREC>::T;
     constexpr bool SPLIT = PREC != HEFF_PREC_FP64;
     constexpr int KB = 64 / (int)sizeof(E);          // elements per K block of one half
-    const int64_t pitch = SPLIT ? 2 * ld : ld;
-    using Acc = typename std::conditional<PREC == HEFF_PREC_FP64, double, float>::type;
-    __shared__ Acc s[PACK_WARPS][32][33];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ti = blockIdx.x * PACK_WARPS + warp;
-    if (ti >= ntiles) return;                       // warp-uniform; the block never synchronises
-    const PackTile t = tiles[ti];
-    const int bz = blockIdx.y;
-    Acc (*sw)[33] = s[warp];
+    const int64_t pitch = SPLIT ? 2 * g.ld : g.ld;
+    using Acc = PackAcc<PREC>;
+    const int lane = threadIdx.x & 31;
+    const PackTile t = g.tiles[ti];
     pdl_wait();                                     // x may come from the previous kernel
     pdl_trigger();
     {
-        const In* x = static_cast<const In*>(xs.p[bz]) + t.x_off;
+        const In* x = static_cast<const In*>(g.xs.p[bz]) + t.x_off;
         const int b = t.b0 + lane;
         const bool bv = b < t.m_b;
         const int na = t.m_a - t.a0;                // rows of x left in this tile (may be <= 0)
-        // all 32 rows' loads are issued before the first conversion: converting an FP64 element
+        // a group's loads are all issued before its first conversion: converting an FP64 element
         // takes branches, which kept the loads from overlapping (m = 1024, FP64 vectors to BF16x3:
-        // 21 us a call; with the loads first, 5 us)
-        In v[32];
+        // 21 us a call; with all 32 loads first, 6.8 us)
+#pragma unroll 1
+        for (int r0 = 0; r0 < 32; r0 += G) {
+            In v[G];
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = (bv && r < na) ? x[(int64_t)(t.a0 + r) * t.m_b + b] : (In)0;
+            for (int r = 0; r < G; ++r)
+                v[r] = (bv && r0 + r < na) ? x[(int64_t)(t.a0 + r0 + r) * t.m_b + b] : (In)0;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) sw[r][lane] = to_acc<Acc>(v[r]);
+            for (int r = 0; r < G; ++r) sw[r0 + r][lane] = to_acc<Acc>(v[r]);
+        }
     }
     __syncwarp();
     if constexpr (!SPLIT) {
         // exponent codes of the tile's XT rows (lane = row) over these 32 columns
-        if (codes && t.b0 + lane < t.m_b) {
+        if (g.codes && t.b0 + lane < t.m_b) {
             int e = 0;
 #pragma unroll
             for (int r = 0; r < 32; ++r)
                 e = max(e, fx::exp_code((uint32_t)__double2hiint(sw[r][lane]), (uint32_t)__double2loint(sw[r][lane])));
-            codes[(t.xt_col0 + t.a0) / KPAD * code_rows + bz * batch_rows + t.xt_row0 + t.b0 + lane] = (uint16_t)e;
+            g.codes[(t.xt_col0 + t.a0) / KPAD * g.code_rows + bz * g.batch_rows + t.xt_row0 + t.b0 + lane] = (uint16_t)e;
         }
     }
-    E* base = reinterpret_cast<E*>(xt) + (int64_t)bz * batch_elems;
+    E* base = reinterpret_cast<E*>(g.xt) + (int64_t)bz * g.batch_elems;
     const int c = 2 * (lane & 15), h = lane >> 4;
     const int nb = t.m_b - t.b0;                    // XT rows of this tile
     const int64_t col = t.xt_col0 + t.a0 + c;       // even: both columns in one K block
@@ -146,6 +155,14 @@ __global__ void __launch_bounds__(32 * PACK_WARPS) pack_kernel(const PackTile* _
         Plane<PREC>::store2(base + o, h0, h1);
         if (SPLIT) Plane<PREC>::store2(base + o + KB, l0, l1);
     }
+}
+
+template <typename In, int PREC>
+__global__ void __launch_bounds__(32 * PACK_WARPS) pack_kernel(const __grid_constant__ PackArgs g) {
+    __shared__ PackAcc<PREC> s[PACK_WARPS][32][33];
+    const int warp = threadIdx.x >> 5, ti = blockIdx.x * PACK_WARPS + warp;
+    if (ti >= g.ntiles) return;                     // warp-uniform; the block never synchronises
+    pack_tile<In, PREC, 32>(g, ti, blockIdx.y, s[warp]);
 }
 
 // ------------------------------------------------------------------ LW / RW preparation
@@ -291,6 +308,22 @@ __global__ void __launch_bounds__(256, HEFF_MIX_MINB) mix_kernel(MixArgs a) {
     mix_tile<In, PREC>(a.tiles[blockIdx.x], a);
 }
 
+// The preparation and the packing of one apply in one launch (they are independent): the first blocks pack,
+// eight tiles each, the others mix.
+template <typename In, int PREC>
+__global__ void __launch_bounds__(256, HEFF_MIX_MINB) mix_pack_kernel(MixArgs a, const __grid_constant__ PackArgs p,
+                                                                      int pack_blocks, int nbatch) {
+    if ((int)blockIdx.x < pack_blocks) {
+        __shared__ PackAcc<PREC> s[8][32][33];
+        const int warp = threadIdx.x >> 5, per = pack_blocks / nbatch;
+        const int ti = ((int)blockIdx.x % per) * 8 + warp;
+        if (ti < p.ntiles) pack_tile<In, PREC, 8>(p, ti, (int)blockIdx.x / per, s[warp]);
+        return;
+    }
+    pdl_trigger();
+    mix_tile<In, PREC>(a.tiles[blockIdx.x - pack_blocks], a);
+}
+
 // ------------------------------------------------------------------ host side
 #define CK(call)                                                                        \
     do {                                                                                \
@@ -372,6 +405,11 @@ void plan_free_device(heff_plan* p) {
     p->d_tables = nullptr;
 }
 
+static PackArgs pack_args(heff_plan* p, const PtrBatch& xs, char* ws, uint16_t* codes) {
+    return PackArgs{p->d_pack, (int)p->pack.size(), xs, ws + p->off_xt, p->ld_x,
+                    (int64_t)p->planes * p->rows_x * p->ld_x, codes, p->opts.max_batch * p->rows_x, p->rows_x};
+}
+
 template <typename In, int PREC>
 static void launch_pack_t(heff_plan* p, const PtrBatch& xs, int nb, char* ws, uint16_t* codes, cudaStream_t st) {
     const int nt = (int)p->pack.size();
@@ -384,9 +422,7 @@ static void launch_pack_t(heff_plan* p, const PtrBatch& xs, int nb, char* ws, ui
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = HEFF_PDL ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, pack_kernel<In, PREC>, static_cast<const PackTile*>(p->d_pack), nt, xs,
-                       ws + p->off_xt, p->ld_x, (int64_t)p->planes * p->rows_x * p->ld_x, codes,
-                       p->opts.max_batch * p->rows_x, p->rows_x);
+    cudaLaunchKernelEx(&cfg, pack_kernel<In, PREC>, pack_args(p, xs, ws, codes));
 }
 
 int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, int level, void* stream) {
@@ -518,6 +554,37 @@ int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, 
     return HEFF_OK;
 }
 
+// Mixing and packing in one launch: split precisions (an FP64 tile needs twice the shared memory), up to
+// MAXB vectors, where all blocks are resident at once.  A small apply is a chain of launches, one less here
+// (m = 32: 20.4 -> 16.4 us); with many waves of mixing blocks the shared memory that packing needs takes
+// L1 from all of them (m = 4096: 549 us in two launches, 562 in one).  Returns whether it ran.
+template <typename In, int PREC>
+static void launch_mix_pack_t(heff_plan* p, const MixArgs& m, const PtrBatch& xs, int nb, char* ws, cudaStream_t st) {
+    const int per = ((int)p->pack.size() + 7) / 8;
+    mix_pack_kernel<In, PREC><<<(unsigned)(per * nb + p->mix.size()), 256, 0, st>>>(m, pack_args(p, xs, ws, nullptr),
+                                                                                  per * nb, nb);
+}
+static bool launch_mix_pack(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R,
+                            const void* const* x, int nbatch, void* ws, cudaStream_t st) {
+    if (p->opts.precision == HEFF_PREC_FP64 || p->timing || p->mix.empty() || p->pack.empty() || nbatch > MAXB)
+        return false;
+    if ((p->pack.size() + 7) / 8 * nbatch + p->mix.size() > (size_t)HEFF_MIX_MINB * p->num_sms) return false;
+    PtrBatch xs{};
+    for (int b = 0; b < nbatch; ++b) xs.p[b] = x[b];
+    char* w = static_cast<char*>(ws);
+    const MixArgs m = mix_args(p, L, W1, W2, R, w, false);
+    const bool f32 = p->opts.io_dtype == HEFF_DTYPE_F32;
+    if (p->opts.precision == HEFF_PREC_BF16X3) {
+        if (f32) launch_mix_pack_t<float, HEFF_PREC_BF16X3>(p, m, xs, nbatch, w, st);
+        else launch_mix_pack_t<double, HEFF_PREC_BF16X3>(p, m, xs, nbatch, w, st);
+    } else {
+        if (f32) launch_mix_pack_t<float, HEFF_PREC_TF32X3>(p, m, xs, nbatch, w, st);
+        else launch_mix_pack_t<double, HEFF_PREC_TF32X3>(p, m, xs, nbatch, w, st);
+    }
+    count_launches(1);
+    return true;
+}
+
 int launch_tc_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
 
 int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, int level, void* stream) {
@@ -598,6 +665,10 @@ static int do_matvec(heff_plan* plan, const void* const* x, void* const* y, int 
 static int do_apply(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
                     const void* const* x, void* const* y, int nbatch, void* workspace, int level, void* stream) {
     plan->ev_prepare = true;
+    if (heff::launch_mix_pack(plan, L, W1, W2, R, x, nbatch, workspace, static_cast<cudaStream_t>(stream))) {
+        CK(cudaGetLastError());
+        return do_gemms(plan, y, nbatch, workspace, level, stream);
+    }
     int rc = do_prepare(plan, L, W1, W2, R, workspace, level, stream);
     return rc ? rc : do_matvec(plan, x, y, nbatch, workspace, level, stream);
 }
