@@ -28,7 +28,6 @@
 #include <new>
 #include <numeric>
 #include <tuple>
-#include <type_traits>
 
 #include "barrier.cuh"
 #include "internal.h"
@@ -152,12 +151,11 @@ __global__ void svd_copy_w_kernel(const SvdSector* __restrict__ secs, double* __
         ws[s.j_off + e] = ws[s.w_off + e];
 }
 
-// One sweep (all rounds) as one cooperative launch: the warps of the grid take the
+// A sweep (all rounds) inside one cooperative launch: the warps of the grid take the
 // (sector, pair) items of a round from a flattened list (pair_off: prefix sums of each
 // sector's pair count), rotate, and meet at a grid barrier before the next round.  The
 // barrier is a counter and a generation word in global memory; its wait is bounded (about a
-// second), after which the kernel sets err and returns.  Each block writes the largest
-// off-diagonal measure it saw to block_max[blockIdx.x].
+// second), after which the kernel sets err and returns.  The phase's further sweeps follow in the same launch.
 //
 // Column norms are carried instead of recomputed per pair (as in the standard one-sided
 // Jacobi codes): the sweep starts by computing every column's squared norm into nrm
@@ -167,143 +165,223 @@ __global__ void svd_copy_w_kernel(const SvdSector* __restrict__ secs, double* __
 // three.  The updates change a norm by t g, tiny once the columns are nearly orthogonal, and
 // the norms are recomputed at the start of every sweep, so the rounding drift stays at a
 // few ulps of the column's norm.
+//
+// Bound by the SM's FP64 unit (two lanes a clock: a warp's instruction holds it 16 cycles) and by the
+// latency of a round.  So the pairs go to blocks first and warps second, which spreads them over every SM
+// (472 pairs on 59 SMs: 2.45 ms a sweep); the first SVD_PIECES * 32 rows of both columns of J and V are
+// loaded at once and stay in registers from the dot product to the rotation; and a rotation takes three
+// multiply-adds per element pair, as the shears u -= p v, v += s u, u -= p v with p = tan(theta / 2), or
+// two where the cosine rounds to one, instead of two products and two multiply-adds: 1.42 ms a sweep.  The
+// shears have determinant one whatever p and s round to; with a cosine that rounds to one the columns grew
+// with every rotation (sum of s^2 over |x|^2 - 1 at m = 512: 1.2e-14, now 6e-16).
 constexpr int SVD_SWEEP_NT = 256;
-#ifndef SVD_UNROLL
-#define SVD_UNROLL 8        // column pieces per lane loaded together in a pair's loops
-#endif
+constexpr int SVD_PIECES = 16;
 using heff::grid_barrier;
 
-template <typename T>
-__device__ __forceinline__ T warp_sum_t(T v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// The sweeps of a phase are one launch: they end when a sweep's largest off-diagonal measure is below stop.
+struct Sweeps {
+    int limit;
+    float stop;
+    int* seen;                   // [3]: a sweep's largest measure (float bits), zero before the launch
+    int* count;                  // sweeps run
+};
+
+// Whether to run another sweep after number `sweep`, in which this block saw `mine` (float bits, >= 0).  A
+// slot is cleared while the sweep before it runs, two barriers after it was last read.
+__device__ __forceinline__ bool sweep_goes_on(const Sweeps& sw, int sweep, int mine, unsigned int* bar, int* err) {
+    if (threadIdx.x == 0) {
+        atomicMax(sw.seen + sweep % 3, mine);
+        if (blockIdx.x == 0) {
+            sw.seen[(sweep + 1) % 3] = 0;
+            *sw.count = sweep + 1;
+        }
+    }
+    if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return false;
+    return !(__int_as_float(*(volatile int*)(sw.seen + sweep % 3)) < sw.stop);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(SVD_SWEEP_NT) svd_sweep_kernel(const SvdSector* __restrict__ secs, int nsec,
-                                                                 const int* __restrict__ pair_off, int kk_all,
-                                                                 T* __restrict__ base, T* __restrict__ nrm,
-                                                                 int ncols_all, float* __restrict__ block_max,
-                                                                 unsigned int* __restrict__ bar, int* __restrict__ err) {
-    constexpr bool F32 = sizeof(T) == 4;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int warps = SVD_SWEEP_NT / 32;
-    const int gw = blockIdx.x * warps + w, nw = gridDim.x * warps;
-    const int npairs = pair_off[nsec];
-    float mymax = 0.f;
-    constexpr int UJ = SVD_UNROLL;
-    // squared column norms (one warp per column; the sectors' s_off are prefix sums of k)
-    bool go = true;
-    if (ncols_all > 0) {
-        for (int item = gw; item < ncols_all; item += nw) {
-            int lo = 0, hi = nsec;                       // sector: s_off[lo] <= item < s_off[lo + 1]
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (secs[mid].s_off <= item) lo = mid; else hi = mid;
-            }
-            const SvdSector s = secs[lo];
-            const T* c = base + (F32 ? s.j32_off : s.j_off) + (int64_t)(item - s.s_off) * s.r;
-            T a = 0;
-            for (int i0 = lane; i0 < s.r; i0 += 32 * UJ) {
-                T u[UJ];
-#pragma unroll
-                for (int t = 0; t < UJ; ++t) u[t] = i0 + 32 * t < s.r ? c[i0 + 32 * t] : (T)0;
-#pragma unroll
-                for (int t = 0; t < UJ; ++t) a = fma(u[t], u[t], a);
-            }
-            a = warp_sum_t(a);
-            if (lane == 0) nrm[item] = a;
-        }
-        go = grid_barrier(bar, bar + 1, gridDim.x, err);
+struct Rotation {
+    double p, s;                 // tan(theta / 2), sin(theta)
+};
+
+// tan(theta) = t -> p, s.  Below 1e-3 by the first terms of their series in t (the next are under 1e-18).
+__device__ __forceinline__ Rotation make_rotation(double t) {
+    const double t2 = t * t;
+    if (fabs(t) < 1e-3)
+        return {t * fma(t2, fma(t2, 0.0625, -0.125), 0.5), t * fma(t2, fma(t2, 0.375, -0.5), 1.0)};
+    const double c = 1.0 / sqrt(1.0 + t2), s = c * t;
+    return {s / (1.0 + c), s};
+}
+
+template <bool TINY>
+__device__ __forceinline__ void rotate(const Rotation& r, double& u, double& v) {
+    if (TINY) {
+        const double u0 = u;
+        u = fma(-r.s, v, u0);
+        v = fma(r.s, u0, v);
+    } else {
+        u = fma(-r.p, v, u);
+        v = fma(r.s, u, v);
+        u = fma(-r.p, v, u);
     }
-    for (int round = 0; go && round < kk_all - 1; ++round) {
-        for (int item = gw; item < npairs; item += nw) {
-            int lo = 0, hi = nsec;                       // sector: pair_off[lo] <= item < pair_off[lo + 1]
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (pair_off[mid] <= item) lo = mid; else hi = mid;
+}
+
+// Rotates the columns cp, cq of n rows, whose first SVD_PIECES * 32 rows are in u, v.
+template <bool TINY>
+__device__ __forceinline__ void rotate_columns(const Rotation& rot, double* cp, double* cq, int n, int lane,
+                                               double (&u)[SVD_PIECES], double (&v)[SVD_PIECES]) {
+#pragma unroll
+    for (int t = 0; t < SVD_PIECES; ++t)
+        if (32 * t < n) {                                // uniform: no FP64 work past the last row
+            rotate<TINY>(rot, u[t], v[t]);
+            const int i = lane + 32 * t;
+            if (i < n) {
+                cp[i] = u[t];
+                cq[i] = v[t];
             }
-            const SvdSector s = secs[lo];
+        }
+    for (int i0 = lane + 32 * SVD_PIECES; i0 < n; i0 += 32 * 4) {
+        double a[4], b[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int i = i0 + 32 * t;
+            a[t] = i < n ? cp[i] : 0.0;
+            b[t] = i < n ? cq[i] : 0.0;
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int i = i0 + 32 * t;
+            if (i < n) {
+                rotate<TINY>(rot, a[t], b[t]);
+                cp[i] = a[t];
+                cq[i] = b[t];
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(SVD_SWEEP_NT, 1) svd_sweep_kernel(const SvdSector* __restrict__ secs, int nsec,
+                                                                 const int* __restrict__ pair_off, int kk_all,
+                                                                 double* __restrict__ base, double* __restrict__ nrm,
+                                                                 int ncols_all, Sweeps sw,
+                                                                 unsigned int* __restrict__ bar, int* __restrict__ err) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int warps = SVD_SWEEP_NT / 32;
+    const int gw = w * gridDim.x + blockIdx.x, nw = gridDim.x * warps;
+    const int npairs = pair_off[nsec];
+    // (a warp's first item is the same in every round: its sector is looked up once, since a barrier
+    // empties L1 and each step of the search then waits for L2)
+    SvdSector s{};
+    int pair = 0;
+    auto find = [&](int item) {
+        int lo = 0, hi = nsec;                           // sector: pair_off[lo] <= item < pair_off[lo + 1]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (pair_off[mid] <= item) lo = mid; else hi = mid;
+        }
+        s = secs[lo];
+        pair = item - pair_off[lo];
+    };
+    const bool several = npairs > nw;
+    if (gw < npairs) find(gw);
+    __shared__ int mx;
+    for (int sweep = 0; sweep < sw.limit; ++sweep) {
+    if (threadIdx.x == 0) mx = 0;
+    float mymax = 0.f;
+    // squared column norms (one warp per column; the sectors' s_off are prefix sums of k)
+    for (int item = gw; item < ncols_all; item += nw) {
+        int lo = 0, hi = nsec;                           // sector: s_off[lo] <= item < s_off[lo + 1]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (secs[mid].s_off <= item) lo = mid; else hi = mid;
+        }
+        const SvdSector cs = secs[lo];
+        const int n = cs.r;
+        const double* c = base + cs.j_off + (int64_t)(item - cs.s_off) * n;
+        double a = 0;
+        for (int i0 = lane; i0 < n; i0 += 32 * 8) {
+            double u[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) u[t] = i0 + 32 * t < n ? c[i0 + 32 * t] : 0.0;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) a = fma(u[t], u[t], a);
+        }
+        a = warp_sum(a);
+        if (lane == 0) nrm[item] = a;
+    }
+    if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return;
+    for (int round = 0; round < kk_all - 1; ++round) {
+        for (int item = gw; item < npairs; item += nw) {
+            if (several) find(item);
             const int kk = s.k + (s.k & 1);
             if (round >= kk - 1) continue;
-            const int pair = item - pair_off[lo];
             auto pos = [&](int j) { return j == 0 ? 0 : 1 + (j - 1 + round) % (kk - 1); };
             int p = pos(pair), q = pos(kk - 1 - pair);
             if (p >= s.k || q >= s.k) continue;          // pair with the dummy column
             if (p > q) { const int t = p; p = q; q = t; }
-            T* J = base + (F32 ? s.j32_off : s.j_off);
-            T* cp = J + (int64_t)p * s.r;
-            T* cq = J + (int64_t)q * s.r;
-            // (the column pieces of UJ iterations are loaded together: the pair's loops are
-            // bound by L2 latency; each lane's sums keep their order)
-            T* np = nrm + s.s_off + p;
-            T* nq = nrm + s.s_off + q;
-            const T a = *np, b = *nq;
-            T g = 0;
-            for (int i0 = lane; i0 < s.r; i0 += 32 * UJ) {
-                T u[UJ], v[UJ];
+            double* cp = base + s.j_off + (int64_t)p * s.r;
+            double* cq = base + s.j_off + (int64_t)q * s.r;
+            double* vp = base + s.v_off + (int64_t)p * s.k;
+            double* vq = base + s.v_off + (int64_t)q * s.k;
+            double* np = nrm + s.s_off + p;
+            double* nq = nrm + s.s_off + q;
+            const double a = *np, b = *nq;
+            double u[SVD_PIECES], v[SVD_PIECES], x[SVD_PIECES], y[SVD_PIECES];
 #pragma unroll
-                for (int t = 0; t < UJ; ++t) {
+            for (int t = 0; t < SVD_PIECES; ++t) {
+                const int i = lane + 32 * t;
+                u[t] = i < s.r ? cp[i] : 0.0;
+                v[t] = i < s.r ? cq[i] : 0.0;
+            }
+#pragma unroll
+            for (int t = 0; t < SVD_PIECES; ++t) {
+                const int i = lane + 32 * t;
+                x[t] = i < s.k ? vp[i] : 0.0;
+                y[t] = i < s.k ? vq[i] : 0.0;
+            }
+            double g4[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int t = 0; t < SVD_PIECES; ++t)
+                if (32 * t < s.r) g4[t & 3] = fma(u[t], v[t], g4[t & 3]);
+            for (int i0 = lane + 32 * SVD_PIECES; i0 < s.r; i0 += 32 * 4) {
+                double c[4], d[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
                     const int i = i0 + 32 * t;
-                    u[t] = i < s.r ? cp[i] : (T)0;
-                    v[t] = i < s.r ? cq[i] : (T)0;
+                    c[t] = i < s.r ? cp[i] : 0.0;
+                    d[t] = i < s.r ? cq[i] : 0.0;
                 }
 #pragma unroll
-                for (int t = 0; t < UJ; ++t) g = fma(u[t], v[t], g);
+                for (int t = 0; t < 4; ++t) g4[t] = fma(c[t], d[t], g4[t]);
             }
-            g = warp_sum_t(g);
-            if (g == (T)0 || a == (T)0 || b == (T)0) continue;
-            const double da = a, db = b, dg = g;
-            const double meas = fabs(dg) / sqrt(da * db);
+            const double g = warp_sum((g4[0] + g4[1]) + (g4[2] + g4[3]));
+            if (g == 0.0 || a == 0.0 || b == 0.0) continue;
+            const double meas = fabs(g) / sqrt(a * b);
             mymax = fmaxf(mymax, (float)meas);
-            if (meas < (F32 ? 1e-7 : 1e-15)) continue;
-            const double zeta = (db - da) / (2.0 * dg);
-            const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-            const double cd = 1.0 / sqrt(1.0 + t * t);
-            const T c = (T)cd, sn = (T)(cd * t);
+            if (meas < 1e-15) continue;
+            const double zeta = (b - a) / (2.0 * g);
+            // (from 2^27 on, 1 + zeta^2 rounds to zeta^2)
+            const double t = fabs(zeta) > 134217728.0 ? 0.5 / zeta
+                                                      : copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
             if (lane == 0) {                             // the rotated columns' squared norms
-                *np = (T)(da - t * dg);
-                *nq = (T)(db + t * dg);
+                *np = a - t * g;
+                *nq = b + t * g;
             }
-            // rotate the two columns of J and of V in one loop (both only need c, sn)
-            T* V = base + (F32 ? s.v32_off : s.v_off);
-            T* vp = V + (int64_t)p * s.k;
-            T* vq = V + (int64_t)q * s.k;
-            constexpr int UR = SVD_UNROLL / 2;
-            for (int i0 = lane; i0 < s.r; i0 += 32 * UR) {       // s.k <= s.r
-                T u[UR], v[UR], x[UR], y[UR];
-#pragma unroll
-                for (int t = 0; t < UR; ++t) {
-                    const int i = i0 + 32 * t;
-                    u[t] = i < s.r ? cp[i] : (T)0;
-                    v[t] = i < s.r ? cq[i] : (T)0;
-                    x[t] = i < s.k ? vp[i] : (T)0;
-                    y[t] = i < s.k ? vq[i] : (T)0;
-                }
-#pragma unroll
-                for (int t = 0; t < UR; ++t) {
-                    const int i = i0 + 32 * t;
-                    if (i < s.r) {
-                        cp[i] = c * u[t] - sn * v[t];
-                        cq[i] = sn * u[t] + c * v[t];
-                    }
-                    if (i < s.k) {
-                        vp[i] = c * x[t] - sn * y[t];
-                        vq[i] = sn * x[t] + c * y[t];
-                    }
-                }
+            const Rotation rot = make_rotation(t);
+            if (fabs(t) < 7.4505805969238281e-9) {       // 2^-27: the cosine, 1 - t^2 / 2, rounds to 1
+                rotate_columns<true>(rot, cp, cq, s.r, lane, u, v);
+                rotate_columns<true>(rot, vp, vq, s.k, lane, x, y);
+            } else {
+                rotate_columns<false>(rot, cp, cq, s.r, lane, u, v);
+                rotate_columns<false>(rot, vp, vq, s.k, lane, x, y);
             }
         }
-        if (!grid_barrier(bar, bar + 1, gridDim.x, err)) break;
+        if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return;
     }
-    __shared__ float wm[SVD_SWEEP_NT / 32];
     for (int o = 16; o > 0; o >>= 1) mymax = fmaxf(mymax, __shfl_xor_sync(0xffffffffu, mymax, o));
-    if (lane == 0) wm[w] = mymax;
+    if (lane == 0) atomicMax(&mx, __float_as_int(mymax));
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float m = 0.f;
-        for (int i = 0; i < warps; ++i) m = fmaxf(m, wm[i]);
-        block_max[blockIdx.x] = m;
+    if (!sweep_goes_on(sw, sweep, mx, bar, err)) return;
     }
 }
 
@@ -311,20 +389,51 @@ __global__ void __launch_bounds__(SVD_SWEEP_NT) svd_sweep_kernel(const SvdSector
 // sector are grouped into blocks of SVD_BW; a round pairs the blocks round-robin (a block
 // left without a partner, or the only block, is processed alone), and one thread block
 // takes one block pair: it forms the Gram matrix G = P^T P of the pair's <= 2 SVD_BW columns
-// (64-row tiles through shared memory), runs one cyclic Jacobi sweep on G (disjoint
+// (its columns in shared memory), runs one cyclic Jacobi sweep on G (disjoint
 // rotations in parallel; each is the rotation the one-sided method would apply to that
 // column pair), accumulates the rotations in W, and updates the columns of J and V by
 // P <- P W.  One round per block pair instead of one per column pair: ~SVD_BW times fewer
-// grid barriers per sweep, and the work is in small dense products.  Each block writes the
-// largest off-diagonal ratio |G_ab| / sqrt(G_aa G_bb) it saw to block_max.
+// grid barriers per sweep, and the work is in small dense products.  The sweep's
+// measure is the largest off-diagonal ratio |G_ab| / sqrt(G_aa G_bb).
+//
+// Bound by the latency of its steps (a pair of 216 + 179 rows, cycles a round: Gram matrix 5300, rotations
+// 10400, update 8700, copies 2200, barrier 6000).  A sweep of m = 512 (942 columns in 19 sectors) went from
+// 371 to 195 us: 31 rounds of rotations from 24000 cycles to 10400, the rest from columns resident in shared
+// memory and 16-byte loads.
 constexpr int SVD_BW = 16, SVD_PC = 2 * SVD_BW;
 #ifndef SVD_TR_ROWS
 #define SVD_TR_ROWS 128
 #endif
 constexpr int SVD_TR = SVD_TR_ROWS;
-#ifndef HEFF_SVD_BLOCK
-#define HEFF_SVD_BLOCK 1    // FP32 phase by block sweeps (0: column-pair sweeps)
-#endif
+
+// row pitches: of G even, for 8-byte loads, with the 2 x 2 blocks on the diagonal in different banks; of W for
+// 16-byte loads
+constexpr int SVD_GLD = SVD_PC + 2, SVD_WLD = SVD_PC + 4;
+
+// cosine and sine of the rotation that zeroes gab, in FP32 (the block sweeps only precondition).  The rounds
+// of a block pair wait for one another through this chain, so it is written with two dependent reciprocal
+// roots and no division.
+__device__ __forceinline__ float2 pair_rotation(float gab, float gaa, float gbb) {
+    // |gab| against 1e-7 of the columns' norms
+    float n;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(n) : "f"(gaa * gbb));
+    const bool turn = gab != 0.f && gaa > 0.f && gbb > 0.f && fabsf(gab) > 1e-7f * n;
+    // scaled by a power of two so that the larger square lies in [1, 2)
+    // (to [2, 4) at the top of the range, where the reciprocal would be subnormal)
+    const float scale = __int_as_float(max(0x7f000000 - (__float_as_int(fmaxf(gaa, gbb)) & 0x7f800000), 0x00800000));
+    const float d = (gbb - gaa) * scale, g = gab * scale;
+    // cos(2 theta) = |d| / h, sin(2 theta) = 2 g / h, h^2 = d^2 + 4 g^2, |theta| <= pi / 4
+    const float rh = rsqrtf(fmaf(d, d, 4.f * g * g));
+    const float c2 = fmaf(0.5f * fabsf(d), rh, 0.5f), rc = rsqrtf(c2);
+    float c = c2 * rc, sn = copysignf(1.f, d) * (g * rh * rc);
+    // The approximate roots leave c^2 + s^2 a few ulps from one, always to the same side, and a column goes
+    // through k rotations a sweep: a Newton step to unit length.  (Without it V32 was too far from orthonormal
+    // for the two Newton-Schulz steps at k = 2450: V^T V - 1 ended at 8e-11, with it at 1e-14.)
+    const float e = 0.5f * fmaf(-sn, sn, fmaf(-c, c, 1.f));
+    c = fmaf(c, e, c);
+    sn = fmaf(sn, e, sn);
+    return turn ? make_float2(c, sn) : make_float2(1.f, 0.f);
+}
 
 __device__ __forceinline__ int rr_pos(int j, int round, int n) { return j == 0 ? 0 : 1 + (j - 1 + round) % (n - 1); }
 
@@ -332,30 +441,45 @@ __device__ __forceinline__ int rr_pos(int j, int round, int n) { return j == 0 ?
 #define SVD_BT_THREADS 512
 #endif
 constexpr int SVD_BT = SVD_BT_THREADS;    // threads of a block-pair CTA
+// RES: the pair's columns of J and V are copied to shared memory once (rows_j + rows_v rows of SVD_TLD
+// floats), V's while G is formed and turned; else they pass through one tile of SVD_TR rows, twice for J.
+// (row pitch: 8 rows of four consecutive columns lie in 32 different banks)
+constexpr int SVD_TLD = SVD_PC + 4;
+constexpr size_t SVD_RES_BYTES = 208 << 10;          // with 18 KB of static shared memory within the SM's 227
+template <bool RES>
 __global__ void __launch_bounds__(SVD_BT) svd_block_sweep_kernel(const SvdSector* __restrict__ secs, int nsec,
                                                               const int* __restrict__ bpair_off, int nbb_all,
-                                                              float* __restrict__ base, float* __restrict__ block_max,
-                                                              unsigned int* __restrict__ bar, int* __restrict__ err) {
-    __shared__ float tile[SVD_TR][SVD_PC + 1];
-    __shared__ float G[SVD_PC][SVD_PC + 1];
-    __shared__ float W[SVD_PC][SVD_PC + 1];
-    __shared__ float rc[SVD_PC / 2], rs[SVD_PC / 2];
+                                                              float* __restrict__ base, Sweeps sw,
+                                                              unsigned int* __restrict__ bar, int* __restrict__ err,
+                                                              int rows_j) {
+    extern __shared__ __align__(16) float dyn[];
+    float* const sj = dyn;
+    float* const sv = RES ? dyn + (int64_t)rows_j * SVD_TLD : dyn;
+    __shared__ __align__(16) float G[2][SVD_PC][SVD_GLD], W[2][SVD_PC][SVD_WLD];
     __shared__ int col[SVD_PC];
-    __shared__ float bmax;
+    __shared__ int bmax;
     const int tid = threadIdx.x;
     const int npairs = bpair_off[nsec];
-    if (tid == 0) bmax = 0.f;
+    SvdSector sc{};
+    int pair = 0;
+    auto find = [&](int item) {                          // bpair_off[lo] <= item < bpair_off[lo + 1]
+        int lo = 0, hi = nsec;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (bpair_off[mid] <= item) lo = mid; else hi = mid;
+        }
+        sc = secs[lo];
+        pair = item - bpair_off[lo];
+    };
+    const bool several = npairs > (int)gridDim.x;        // (a block's only item is looked up once)
+    if ((int)blockIdx.x < npairs) find(blockIdx.x);
+    for (int sweep = 0; sweep < sw.limit; ++sweep) {
+    if (tid == 0) bmax = 0;                              // (the pairs synchronise before they use it)
     for (int round = 0; round < nbb_all - 1; ++round) {
         for (int item = blockIdx.x; item < npairs; item += gridDim.x) {
-            int lo = 0, hi = nsec;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (bpair_off[mid] <= item) lo = mid; else hi = mid;
-            }
-            const SvdSector sc = secs[lo];
+            if (several) find(item);
             const int nb = (sc.k + SVD_BW - 1) / SVD_BW, nbb = nb + (nb & 1);
             if (round >= (nbb > 1 ? nbb - 1 : 1)) continue;                 // block-uniform
-            const int pair = item - bpair_off[lo];
             int bp = nbb > 1 ? rr_pos(pair, round, nbb) : 0;
             int bq = nbb > 1 ? rr_pos(nbb - 1 - pair, round, nbb) : nbb;
             if (bp >= nb) { const int t = bp; bp = bq; bq = t; }              // the real block first
@@ -367,10 +491,30 @@ __global__ void __launch_bounds__(SVD_BT) svd_block_sweep_kernel(const SvdSector
             float* J = base + sc.j32_off;
             float* V = base + sc.v32_off;
             __syncthreads();
+            // (a column that is not there, and the rows up to the next multiple of 8, are zeros)
+            auto copy_columns = [&](float* dst, const float* M, int rows) {
+                const int a = 4 * ((tid >> 5) & 7) + ((tid >> 3) & 3), cidx = col[a];
+                const float* src = M + (int64_t)max(cidx, 0) * rows;
+#pragma unroll 4
+                for (int rr = 8 * (tid >> 8) + (tid & 7); rr < (rows + 7) / 8 * 8; rr += 16) {
+                    const bool in = cidx >= 0 && rr < rows;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(dst + rr * SVD_TLD + a)),
+                                 "l"(in ? src + rr : src), "r"(in ? 4 : 0)
+                                 : "memory");
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            if (RES) {
+                copy_columns(sj, J, sc.r);
+                copy_columns(sv, V, sc.k);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+                __syncthreads();
+            }
             // 1. G = P^T P, register-tiled: thread t takes the 4 x 4 block blk = t / 8 of G
             //    (rows 4 (blk / 8) .., columns 4 (blk % 8) ..) over the tile rows g, g + 8, ...
             //    (g = t % 8), and the 8 partial sums of a block (8 consecutive lanes) are added
-            //    by shuffles: 8 shared-memory loads per 16 FMAs
+            //    by shuffles: two 16-byte shared-memory loads per 16 FMAs
             static_assert(SVD_PC == 32 && SVD_BT == 512 && SVD_TR % 8 == 0, "Gram tiling assumes 32 columns");
             const int gblk = tid >> 3, gg = tid & 7;
             const int ga0 = 4 * (gblk >> 3), gb0 = 4 * (gblk & 7);
@@ -386,7 +530,7 @@ __global__ void __launch_bounds__(SVD_BT) svd_block_sweep_kernel(const SvdSector
             auto load_tile = [&](const float* M, int rows, int r0) {
 #pragma unroll
                 for (int u = 0; u < TE; ++u) {
-                    const int e = tid + SVD_BT * u, a = e / SVD_TR, rr = e % SVD_TR;
+                    const int e = tid + SVD_BT * u, a = ((e >> 3) & 3) + 4 * ((e >> 5) & 7), rr = (e & 7) + 8 * (e >> 8);
                     const int cidx = col[a];
                     nxt[u] = (cidx >= 0 && r0 + rr < rows) ? M[(int64_t)cidx * rows + r0 + rr] : 0.f;
                 }
@@ -394,26 +538,30 @@ __global__ void __launch_bounds__(SVD_BT) svd_block_sweep_kernel(const SvdSector
             auto stage_tile = [&]() {
 #pragma unroll
                 for (int u = 0; u < TE; ++u) {
-                    const int e = tid + SVD_BT * u;
-                    tile[e % SVD_TR][e / SVD_TR] = nxt[u];
+                    const int e = tid + SVD_BT * u, a = ((e >> 3) & 3) + 4 * ((e >> 5) & 7), rr = (e & 7) + 8 * (e >> 8);
+                    sj[rr * SVD_TLD + a] = nxt[u];
                 }
             };
-            load_tile(J, sc.r, 0);
+            if (!RES) load_tile(J, sc.r, 0);
             for (int r0 = 0; r0 < sc.r; r0 += SVD_TR) {
-                stage_tile();
-                __syncthreads();
-                if (r0 + SVD_TR < sc.r) load_tile(J, sc.r, r0 + SVD_TR);
+                if (!RES) {
+                    stage_tile();
+                    __syncthreads();
+                    if (r0 + SVD_TR < sc.r) load_tile(J, sc.r, r0 + SVD_TR);
+                }
+                const float* tile = RES ? sj + r0 * SVD_TLD : sj;
+                const int end = RES ? min(SVD_TR, (sc.r - r0 + 7) / 8 * 8) : SVD_TR;
 #pragma unroll 4
-                for (int rr = gg; rr < SVD_TR; rr += 8) {
-                    float xa[4], xb[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { xa[i] = tile[rr][ga0 + i]; xb[i] = tile[rr][gb0 + i]; }
+                for (int rr = gg; rr < end; rr += 8) {
+                    const float4 fa = *reinterpret_cast<const float4*>(tile + rr * SVD_TLD + ga0);
+                    const float4 fb = *reinterpret_cast<const float4*>(tile + rr * SVD_TLD + gb0);
+                    const float xa[4] = {fa.x, fa.y, fa.z, fa.w}, xb[4] = {fb.x, fb.y, fb.z, fb.w};
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
                         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xa[i], xb[j], acc[i][j]);
                 }
-                __syncthreads();
+                if (!RES) __syncthreads();
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -427,10 +575,10 @@ __global__ void __launch_bounds__(SVD_BT) svd_block_sweep_kernel(const SvdSector
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const int a = ga0 + i, b = gb0 + j;
-                        G[a][b] = (a < nc && b < nc) ? acc[i][j] : (a == b ? 1.f : 0.f);
+                        G[0][a][b] = a == b && a >= nc ? 1.f : acc[i][j];          // (an absent column: 1)
                     }
             }
-            for (int e = tid; e < SVD_PC * SVD_PC; e += SVD_BT) W[e / SVD_PC][e % SVD_PC] = (e / SVD_PC == e % SVD_PC);
+            for (int e = tid; e < SVD_PC * SVD_PC; e += SVD_BT) W[0][e / SVD_PC][e % SVD_PC] = (e / SVD_PC == e % SVD_PC);
             __syncthreads();
             // off-diagonal measure before the rotations (thread t: row t / 16, columns 2 (t % 16) + u)
             {
@@ -440,126 +588,144 @@ __global__ void __launch_bounds__(SVD_BT) svd_block_sweep_kernel(const SvdSector
                 for (int u = 0; u < 2; ++u) {
                     const int b = gbp + u;
                     if (ga < b && b < nc) {
-                        const float d = sqrtf(G[ga][ga] * G[b][b]);
-                        if (d > 0.f) m = fmaxf(m, fabsf(G[ga][b]) / d);
+                        const float d = sqrtf(G[0][ga][ga] * G[0][b][b]);
+                        if (d > 0.f) m = fmaxf(m, fabsf(G[0][ga][b]) / d);
                     }
                 }
                 for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                if ((tid & 31) == 0) atomicMax(reinterpret_cast<int*>(&bmax), __float_as_int(m));
+                if ((tid & 31) == 0) atomicMax(&bmax, __float_as_int(m));
             }
-            // 2. one cyclic Jacobi sweep on G: SVD_PC - 1 rounds of SVD_PC / 2 disjoint rotations
-            for (int jr = 0; jr < SVD_PC - 1; ++jr) {
-                if (tid < SVD_PC / 2) {
-                    int a = rr_pos(tid, jr, SVD_PC), b = rr_pos(SVD_PC - 1 - tid, jr, SVD_PC);
-                    if (a > b) { const int t = a; a = b; b = t; }
-                    const float gab = G[a][b], gaa = G[a][a], gbb = G[b][b];
-                    float c = 1.f, sn = 0.f;
-                    if (gab != 0.f && gaa > 0.f && gbb > 0.f && fabsf(gab) > 1e-7f * sqrtf(gaa * gbb)) {
-                        // the rotation in FP32 (this phase only preconditions; FP64 arithmetic
-                        // runs at GB300's much lower FP64 rate): a zeta too large to square
-                        // gives t = 0, the limit of the formula
-                        const float zeta = (gbb - gaa) / (2.f * gab);
-                        const float t = copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
-                        c = rsqrtf(fmaf(t, t, 1.f));
-                        sn = c * t;
+            // 2. one cyclic Jacobi sweep on G: SVD_PC - 1 rounds of SVD_PC / 2 disjoint rotations, each waiting
+            //    for the one before.  The columns move instead of the pairs: pair j always lies in the places
+            //    2 j, 2 j + 1, and a round writes what it turned to the places of the next (the tournament's
+            //    step; after all rounds every column is back), so no address changes from round to round.
+            //    Each lane l works out the rotation of pair l % 16; thread (i, j) of the first half takes
+            //    the 2 x 2 block of the pairs i and j from one copy of G to the other, the second half two
+            //    rows each of W.
+            {
+                const int j = tid & 15, i = (tid >> 4) & 15;
+                // tournament position t (pairs t, 31 - t) <-> place; the column at position t moves to t - 1
+                auto place = [](int t) { return t < 16 ? 2 * t : 2 * (SVD_PC - 1 - t) + 1; };
+                auto next = [&](int t) { return place(t == 0 ? 0 : (t == 1 ? SVD_PC - 1 : t - 1)); };
+                const int na = next(j), nb2 = next(SVD_PC - 1 - j);
+                if (tid < 256) {
+                    const int nc2 = next(i), nd = next(SVD_PC - 1 - i);
+                    const int rd_j = 2 * j * SVD_GLD + 2 * j, rd_b = 2 * i * SVD_GLD + 2 * j;
+                    const int wca = nc2 * SVD_GLD + na, wcb = nc2 * SVD_GLD + nb2;
+                    const int wda = nd * SVD_GLD + na, wdb = nd * SVD_GLD + nb2;
+                    auto step = [&](const float* Gc, float* Gn) {
+                        const float2 g0 = *reinterpret_cast<const float2*>(Gc + rd_j);
+                        const float gbb = Gc[rd_j + SVD_GLD + 1];
+                        const float2 cv = *reinterpret_cast<const float2*>(Gc + rd_b);
+                        const float2 dv = *reinterpret_cast<const float2*>(Gc + rd_b + SVD_GLD);
+                        const float2 cs = pair_rotation(g0.y, g0.x, gbb);
+                        const float rx = __shfl_sync(0xffffffffu, cs.x, i), ry = __shfl_sync(0xffffffffu, cs.y, i);
+                        const float p0 = cs.x * cv.x - cs.y * cv.y, p1 = cs.y * cv.x + cs.x * cv.y;      // columns
+                        const float q0 = cs.x * dv.x - cs.y * dv.y, q1 = cs.y * dv.x + cs.x * dv.y;
+                        Gn[wca] = rx * p0 - ry * q0;                                                    // rows
+                        Gn[wcb] = rx * p1 - ry * q1;
+                        Gn[wda] = ry * p0 + rx * q0;
+                        Gn[wdb] = ry * p1 + rx * q1;
+                    };
+                    for (int jr = 0; jr < SVD_PC - 2; jr += 2) {
+                        step(&G[0][0][0], &G[1][0][0]);
+                        __syncthreads();
+                        step(&G[1][0][0], &G[0][0][0]);
+                        __syncthreads();
                     }
-                    rc[tid] = c;
-                    rs[tid] = sn;
-                }
-                __syncthreads();
-                // columns: G <- G R, W <- W R (item: pair j = idx / SVD_PC, row x = idx % SVD_PC)
-                for (int idx = tid; idx < (SVD_PC / 2) * SVD_PC; idx += SVD_BT) {
-                    const int j = idx / SVD_PC, x = idx % SVD_PC;
-                    int a = rr_pos(j, jr, SVD_PC), b = rr_pos(SVD_PC - 1 - j, jr, SVD_PC);
-                    if (a > b) { const int t = a; a = b; b = t; }
-                    const float c = rc[j], sn = rs[j];
-                    if (sn != 0.f) {
-                        const float ga_ = G[x][a], gb_ = G[x][b];
-                        G[x][a] = c * ga_ - sn * gb_;
-                        G[x][b] = sn * ga_ + c * gb_;
-                        const float wa = W[x][a], wb = W[x][b];
-                        W[x][a] = c * wa - sn * wb;
-                        W[x][b] = sn * wa + c * wb;
+                } else {
+                    const int rd_j = 2 * j * SVD_GLD + 2 * j;
+                    auto step = [&](const float* Gc, const float* Wc, float* Wn) {
+                        const float2 g0 = *reinterpret_cast<const float2*>(Gc + rd_j);
+                        const float gbb = Gc[rd_j + SVD_GLD + 1];
+                        const float2 u = *reinterpret_cast<const float2*>(Wc + i * SVD_WLD + 2 * j);
+                        const float2 v = *reinterpret_cast<const float2*>(Wc + (i + 16) * SVD_WLD + 2 * j);
+                        const float2 cs = pair_rotation(g0.y, g0.x, gbb);
+                        Wn[i * SVD_WLD + na] = cs.x * u.x - cs.y * u.y;
+                        Wn[i * SVD_WLD + nb2] = cs.y * u.x + cs.x * u.y;
+                        Wn[(i + 16) * SVD_WLD + na] = cs.x * v.x - cs.y * v.y;
+                        Wn[(i + 16) * SVD_WLD + nb2] = cs.y * v.x + cs.x * v.y;
+                    };
+                    for (int jr = 0; jr < SVD_PC - 2; jr += 2) {
+                        step(&G[0][0][0], &W[0][0][0], &W[1][0][0]);
+                        __syncthreads();
+                        step(&G[1][0][0], &W[1][0][0], &W[0][0][0]);
+                        __syncthreads();
                     }
+                    step(&G[0][0][0], &W[0][0][0], &W[1][0][0]);
                 }
-                __syncthreads();
-                // rows: G <- R^T G
-                for (int idx = tid; idx < (SVD_PC / 2) * SVD_PC; idx += SVD_BT) {
-                    const int j = idx / SVD_PC, x = idx % SVD_PC;
-                    int a = rr_pos(j, jr, SVD_PC), b = rr_pos(SVD_PC - 1 - j, jr, SVD_PC);
-                    if (a > b) { const int t = a; a = b; b = t; }
-                    const float c = rc[j], sn = rs[j];
-                    if (sn != 0.f) {
-                        const float ga_ = G[a][x], gb_ = G[b][x];
-                        G[a][x] = c * ga_ - sn * gb_;
-                        G[b][x] = sn * ga_ + c * gb_;
-                    }
-                }
-                __syncthreads();
             }
-            // 3. P <- P W for the columns of J (r rows) and of V (k rows), 128-row tiles,
-            //    register-tiled: warp w takes the output columns 2w, 2w + 1 (their W columns
-            //    held in registers), lane l the tile rows l, l + 32, l + 64, l + 96: 32 shared-
-            //    memory loads per 64 FMAs, coalesced column stores
-            static_assert(SVD_BT / 32 == SVD_PC / 2 && SVD_TR == 128, "update tiling: one warp per column pair");
-            const int ua = 2 * (tid >> 5), ul = tid & 31;
-            float w0[SVD_PC], w1[SVD_PC];
+            if (RES) asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+            // 3. P <- P W for the columns of J (r rows) and of V (k rows): a warp takes eight output columns of
+            //    32 UR rows, UR rows a lane: 2 UR + 8 (broadcast) 16-byte shared-memory loads per 32 UR FMAs
+            //    of four inner columns, coalesced column stores
+            constexpr int UR = RES ? 2 : 1;
+            const int ul = tid & 31, uw = tid >> 5;
+            auto update = [&](const float* tile, float* M, int rows, int r0, int c8) {
+                // rows r0 .. of M (tile: their first), output columns c8 .. c8 + 7
+                float o[UR][8];
 #pragma unroll
-            for (int bb = 0; bb < SVD_PC; ++bb) { w0[bb] = W[bb][ua]; w1[bb] = W[bb][ua + 1]; }
-            for (int pass = 0; pass < 2; ++pass) {
-                float* M = pass == 0 ? J : V;
-                const int rows = pass == 0 ? sc.r : sc.k;
-                load_tile(M, rows, 0);
-                for (int r0 = 0; r0 < rows; r0 += SVD_TR) {
-                    stage_tile();
-                    __syncthreads();
-                    if (r0 + SVD_TR < rows) load_tile(M, rows, r0 + SVD_TR);
-                    float o0[4], o1[4];
+                for (int u = 0; u < UR; ++u)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int rr = ul + 32 * i;
-                        float v0 = 0.f, v1 = 0.f;
+                    for (int c = 0; c < 8; ++c) o[u][c] = 0.f;
+#pragma unroll 2
+                for (int b4 = 0; b4 < SVD_PC; b4 += 4) {
+                    float t[UR][4];
 #pragma unroll
-                        for (int bb = 0; bb < SVD_PC; ++bb) {
-                            const float t = tile[rr][bb];
-                            v0 = fmaf(t, w0[bb], v0);
-                            v1 = fmaf(t, w1[bb], v1);
-                        }
-                        o0[i] = v0;
-                        o1[i] = v1;
+                    for (int u = 0; u < UR; ++u) {
+                        const float4 f = *reinterpret_cast<const float4*>(tile + (ul + 32 * u) * SVD_TLD + b4);
+                        t[u][0] = f.x; t[u][1] = f.y; t[u][2] = f.z; t[u][3] = f.w;
                     }
-                    __syncthreads();
-                    const int c0 = col[ua], c1 = col[ua + 1];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int rr = ul + 32 * i;
-                        if (r0 + rr < rows) {
-                            if (c0 >= 0) M[(int64_t)c0 * rows + r0 + rr] = o0[i];
-                            if (c1 >= 0) M[(int64_t)c1 * rows + r0 + rr] = o1[i];
-                        }
+                    for (int bb = 0; bb < 4; ++bb) {
+                        const float4 wa = *reinterpret_cast<const float4*>(&W[1][b4 + bb][c8]);
+                        const float4 wb = *reinterpret_cast<const float4*>(&W[1][b4 + bb][c8 + 4]);
+                        const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+                        for (int u = 0; u < UR; ++u)
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) o[u][c] = fmaf(t[u][bb], wv[c], o[u][c]);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const int cidx = col[c8 + c];
+                    if (cidx < 0) continue;
+#pragma unroll
+                    for (int u = 0; u < UR; ++u)
+                        if (r0 + ul + 32 * u < rows) M[(int64_t)cidx * rows + r0 + ul + 32 * u] = o[u][c];
+                }
+            };
+            if (RES) {
+                const int nj = (sc.r + 63) / 64, nv = (sc.k + 63) / 64;
+                for (int unit = uw; unit < 4 * (nj + nv); unit += SVD_BT / 32) {
+                    const int g = unit >> 2, c8 = 8 * (unit & 3);
+                    if (g < nj) update(sj + 64 * g * SVD_TLD, J, sc.r, 64 * g, c8);
+                    else update(sv + 64 * (g - nj) * SVD_TLD, V, sc.k, 64 * (g - nj), c8);
+                }
+            } else {
+                static_assert(SVD_TR == 128 && SVD_BT == 512, "one unit of 32 rows and 8 columns per warp");
+                for (int pass = 0; pass < 2; ++pass) {
+                    float* M = pass == 0 ? J : V;
+                    const int rows = pass == 0 ? sc.r : sc.k;
+                    load_tile(M, rows, 0);
+                    for (int r0 = 0; r0 < rows; r0 += SVD_TR) {
+                        stage_tile();
+                        __syncthreads();
+                        if (r0 + SVD_TR < rows) load_tile(M, rows, r0 + SVD_TR);
+                        const int rr = 32 * (uw >> 2);
+                        if (r0 + rr < rows) update(sj + rr * SVD_TLD, M, rows, r0 + rr, 8 * (uw & 3));
+                        __syncthreads();
                     }
                 }
             }
             __syncthreads();
         }
-        if (!grid_barrier(bar, bar + 1, gridDim.x, err)) break;
+        if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return;
     }
-    __syncthreads();
-    if (tid == 0) block_max[blockIdx.x] = bmax;
-}
-
-// largest slot value -> out[0] (one block; fixed order)
-__global__ void __launch_bounds__(256) svd_offmax_kernel(const float* __restrict__ off, int n, float* __restrict__ out) {
-    __shared__ float sh[256];
-    float m = 0.f;
-    for (int i = threadIdx.x; i < n; i += 256) m = fmaxf(m, off[i]);
-    sh[threadIdx.x] = m;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] = fmaxf(sh[threadIdx.x], sh[threadIdx.x + w]);
-        __syncthreads();
+    if (!sweep_goes_on(sw, sweep, bmax, bar, err)) return;
     }
-    if (threadIdx.x == 0) out[0] = sh[0];
 }
 
 // column norms of J = singular values
@@ -775,8 +941,7 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
         if (rc) return rc;
         S->lists_uploaded = true;
     }
-    // Jacobi sweeps until the largest off-diagonal measure is below tol: one cooperative
-    // launch per sweep (all rounds, grid barrier between rounds)
+    // Jacobi sweeps until the largest off-diagonal measure is below a limit: one cooperative launch per phase
     const int kk_all = S->max_k + (S->max_k & 1);
     if (S->pair_off.empty()) {
         S->pair_off.push_back(0);
@@ -788,90 +953,58 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
     SVD_CK(cudaMemcpyAsync(d_pair_off, S->pair_off.data(), S->pair_off.size() * sizeof(int), cudaMemcpyHostToDevice,
                            st));
     SVD_CK(cudaMemsetAsync(d_bar, 0, 3 * sizeof(unsigned int), st));
-    // stop_below: a sweep whose largest off-diagonal measure (taken before its rotations) is
-    // below this ends the loop; for the FP64 phase it is sqrt(tol): Jacobi sweeps converge
-    // quadratically, so that sweep's rotations leave the measure near tol, and a further
-    // sweep would only confirm it
-    auto sweeps = [&](auto* base, float stop_below, int max_sweeps, int& out) -> int {
-        using T = typename std::remove_pointer<decltype(base)>::type;
-        out = 0;
-        if (kk_all < 2) return HEFF_OK;
-        int dev = 0, nsm = 0, per_sm = 0;
-        SVD_CK(cudaGetDevice(&dev));
-        SVD_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-        SVD_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, svd_sweep_kernel<T>, SVD_SWEEP_NT, 0));
-        const int npairs = S->pair_off.back();
-        int grid = std::max(1, std::min(nsm * std::max(per_sm, 1), (npairs + 7) / 8));
-        grid = std::min<int>(grid, (int)S->nslots);
-        const SvdSector* secs = S->d_sec;
-        int nsec_i = nsec, kk_i = kk_all;
-        T* base_t = base;
-        T* nrm_t = reinterpret_cast<T*>(sv);             // the singular-value slots, free until the end
-        int ncols_i = (int)S->s_total;
-        while (out < max_sweeps) {
-            void* args[] = {(void*)&secs, (void*)&nsec_i, (void*)&d_pair_off, (void*)&kk_i, (void*)&base_t,
-                            (void*)&nrm_t, (void*)&ncols_i, (void*)&slots, (void*)&d_bar, (void*)&d_err};
-            SVD_CK(cudaLaunchCooperativeKernel((const void*)svd_sweep_kernel<T>, dim3(grid), dim3(SVD_SWEEP_NT),
-                                               args, 0, st));
-            svd_offmax_kernel<<<1, 256, 0, st>>>(slots, grid, offmax);
-            heff::count_launches(2);
-            float m = 0.f;
-            int e = 0;
-            SVD_CK(cudaMemcpyAsync(&m, offmax, sizeof(float), cudaMemcpyDeviceToHost, st));
-            SVD_CK(cudaMemcpyAsync(&e, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-            SVD_CK(cudaStreamSynchronize(st));
-            if (e) return fail(HEFF_ERR_TIMEOUT, "SVD sweep: grid barrier timed out");
-            ++out;
-            if (m < stop_below) break;
-        }
+    int* seen = reinterpret_cast<int*>(slots + S->nslots);          // FP32 [0, 3), FP64 [3, 6); sweeps run [6, 8)
+    SVD_CK(cudaMemsetAsync(seen, 0, 8 * sizeof(int), st));
+    int dev = 0, nsm = 0;
+    SVD_CK(cudaGetDevice(&dev));
+    SVD_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const SvdSector* secs = S->d_sec;
+    int nsec_i = nsec;
+    auto sweeps = [&](double* base, Sweeps sw) -> int {
+        int per_sm = 0, kk_i = kk_all, ncols_i = (int)S->s_total;
+        SVD_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, svd_sweep_kernel, SVD_SWEEP_NT, 0));
+        // a pair to a block while SMs are free
+        const int grid = std::max(1, std::min(nsm * std::max(per_sm, 1), S->pair_off.back()));
+        double* nrm = sv;                                // the singular-value slots, free until the end
+        void* args[] = {(void*)&secs, (void*)&nsec_i, (void*)&d_pair_off, (void*)&kk_i, (void*)&base,
+                        (void*)&nrm, (void*)&ncols_i, (void*)&sw, (void*)&d_bar, (void*)&d_err};
+        SVD_CK(cudaLaunchCooperativeKernel((const void*)svd_sweep_kernel, dim3(grid), dim3(SVD_SWEEP_NT), args, 0, st));
+        heff::count_launches(1);
         return HEFF_OK;
     };
     // FP32 block sweeps: the same convergence test on the block pairs' Gram matrices
-    auto block_sweeps = [&](float* base, float tol, int max_sweeps, int& out) -> int {
-        out = 0;
+    auto block_sweeps = [&](float* base, Sweeps sw) -> int {
         std::vector<int> boff(1, 0);
-        int nbb_all = 2;
+        int nbb_all = 2, max_r = 0, per_sm = 0;
         for (const SvdSector& sc : S->sec) {
             const int nb = (sc.k + SVD_BW - 1) / SVD_BW, nbb = nb + (nb & 1);
             boff.push_back(boff.back() + nbb / 2);
             nbb_all = std::max(nbb_all, nbb);
+            max_r = std::max(max_r, (int)sc.r);
         }
         int* d_boff = d_err + 2;
         SVD_CK(cudaMemcpyAsync(d_boff, boff.data(), boff.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-        int dev = 0, nsm = 0, per_sm = 0;
-        SVD_CK(cudaGetDevice(&dev));
-        SVD_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-        SVD_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, svd_block_sweep_kernel, SVD_BT, 0));
-        int grid = std::max(1, std::min(nsm * std::max(per_sm, 1), boff.back()));
-        grid = std::min<int>(grid, (int)S->nslots);
-        const SvdSector* secs = S->d_sec;
-        int nsec_i = nsec, nbb_i = nbb_all;
-        float* base_t = base;
-        while (out < max_sweeps) {
-            void* args[] = {(void*)&secs, (void*)&nsec_i, (void*)&d_boff, (void*)&nbb_i, (void*)&base_t,
-                            (void*)&slots, (void*)&d_bar, (void*)&d_err};
-            SVD_CK(cudaLaunchCooperativeKernel((const void*)svd_block_sweep_kernel, dim3(grid), dim3(SVD_BT), args, 0,
-                                               st));
-            svd_offmax_kernel<<<1, 256, 0, st>>>(slots, grid, offmax);
-            heff::count_launches(2);
-            float m = 0.f;
-            int e = 0;
-            SVD_CK(cudaMemcpyAsync(&m, offmax, sizeof(float), cudaMemcpyDeviceToHost, st));
-            SVD_CK(cudaMemcpyAsync(&e, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-            SVD_CK(cudaStreamSynchronize(st));
-            if (e) return fail(HEFF_ERR_TIMEOUT, "SVD block sweep: grid barrier timed out");
-            ++out;
-            if (m < tol) break;
-        }
+        // shared memory for the columns of a pair, where they fit (rows rounded up to the update's tiles)
+        auto tiles = [](int rows) { return (rows + SVD_TR - 1) / SVD_TR * SVD_TR; };
+        int rows_j = tiles(max_r);
+        size_t smem = (size_t)(rows_j + tiles(S->max_k)) * SVD_TLD * sizeof(float);
+        const bool res = smem <= SVD_RES_BYTES;
+        if (!res) smem = (size_t)SVD_TR * SVD_TLD * sizeof(float);
+        const auto kernel = res ? svd_block_sweep_kernel<true> : svd_block_sweep_kernel<false>;
+        SVD_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    res ? (int)SVD_RES_BYTES : (int)smem));
+        SVD_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, SVD_BT, smem));
+        const int grid = std::max(1, std::min(nsm * std::max(per_sm, 1), boff.back()));
+        void* args[] = {(void*)&secs, (void*)&nsec_i, (void*)&d_boff, (void*)&nbb_all, (void*)&base,
+                        (void*)&sw, (void*)&d_bar, (void*)&d_err, (void*)&rows_j};
+        SVD_CK(cudaLaunchCooperativeKernel((const void*)kernel, dim3(grid), dim3(SVD_BT), args, smem, st));
+        heff::count_launches(1);
         return HEFF_OK;
     };
     int rc;
-    // FP32 preconditioning sweeps (to FP32 accuracy of the dot products)
-    if (HEFF_SVD_BLOCK) {
-        if ((rc = block_sweeps(f32, 1e-5f, 30, S->fp32_sweeps))) return rc;
-    } else if ((rc = sweeps(f32, 1e-5f, 30, S->fp32_sweeps))) {
-        return rc;
-    }
+    // FP32 preconditioning sweeps.  A sweep's measure is taken before its rotations and Jacobi sweeps converge
+    // quadratically: one that saw at most 1e-4 leaves FP32 rounding, and another would only confirm it.
+    if ((rc = block_sweeps(f32, Sweeps{30, 1e-4f, seen, seen + 6}))) return rc;
     // V = orthonormalised double(V32), J = J V
     svd_v_to_f64_kernel<<<dim3(128, nsec), 256, 0, st>>>(S->d_sec, f32, ws);
     heff::count_launches(1);
@@ -886,15 +1019,20 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
     heff::count_launches(1);
     // FP64 sweeps to convergence: off-diagonal measure 1e-14, i.e. stop after the sweep that
     // saw at most 1e-7
-    if ((rc = sweeps(ws, 1e-7f, 40, S->fp64_sweeps))) return rc;
-    const int sweep = S->fp64_sweeps;
+    if (kk_all >= 2 && (rc = sweeps(ws, Sweeps{40, 1e-7f, seen + 3, seen + 7}))) return rc;
     svd_norms_kernel<<<dim3((S->max_k + 3) / 4 + 1, nsec), 128, 0, st>>>(S->d_sec, ws, sv);
     heff::count_launches(1);
     S->s.assign(S->s_total, 0.0);
     SVD_CK(cudaMemcpyAsync(S->s.data(), sv, S->s_total * sizeof(double), cudaMemcpyDeviceToHost, st));
+    int state[8] = {0}, e = 0;
+    SVD_CK(cudaMemcpyAsync(state, seen, sizeof state, cudaMemcpyDeviceToHost, st));
+    SVD_CK(cudaMemcpyAsync(&e, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     SVD_CK(cudaStreamSynchronize(st));
     SVD_CK(cudaGetLastError());
-    if (sweeps_out) *sweeps_out = sweep;
+    if (e) return fail(HEFF_ERR_TIMEOUT, "SVD sweep: grid barrier timed out");
+    S->fp32_sweeps = state[6];
+    S->fp64_sweeps = state[7];
+    if (sweeps_out) *sweeps_out = S->fp64_sweeps;
     S->computed = true;
     S->kept.clear();
     return HEFF_OK;
