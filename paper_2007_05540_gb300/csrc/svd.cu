@@ -204,13 +204,38 @@ struct Rotation {
     double p, s;                 // tan(theta / 2), sin(theta)
 };
 
-// tan(theta) = t -> p, s.  Below 1e-3 by the first terms of their series in t (the next are under 1e-18).
-__device__ __forceinline__ Rotation make_rotation(double t) {
-    const double t2 = t * t;
-    if (fabs(t) < 1e-3)
-        return {t * fma(t2, fma(t2, 0.0625, -0.125), 0.5), t * fma(t2, fma(t2, 0.375, -0.5), 1.0)};
-    const double c = 1.0 / sqrt(1.0 + t2), s = c * t;
-    return {s / (1.0 + c), s};
+// |g| / sqrt(a b) for a, b > 0.  It steers the sweeps, so FP32 will do: the three numbers, over the larger
+// square's power of two, get their FP32 forms from their upper words, 20 bits of mantissa each, without an
+// FP64 instruction (a root and a division in FP64 cost as much as rotating 180 rows).
+__device__ __forceinline__ float off_diagonal(double g, double a, double b) {
+    const int ha = __double2hiint(a), hb = __double2hiint(b), hg = __double2hiint(g) & 0x7fffffff;
+    const int e = max(ha, hb) >> 20;                     // biased exponent of the larger square
+    auto scaled = [&](int h) {
+        const int x = (h >> 20) - e + 127;
+        return x > 0 && x < 255 ? __int_as_float((x << 23) | ((h & 0xfffff) << 3)) : 0.f;
+    };
+    const float ab = scaled(ha) * scaled(hb);
+    if (e > 64 && e < 2047 && ab > 1e-36f) return scaled(hg) * rsqrtf(ab);
+    return (float)(fabs(g) / sqrt(a * b));
+}
+
+// tan(theta) of the rotation that makes columns of squared norms a, b and inner product g orthogonal, and
+// its shears.  With w = 2 g / (b - a) = tan(2 theta) under 1e-3 by the first terms of their series in w (the
+// next are under 3e-19): one division instead of three and two roots.
+__device__ __forceinline__ double rotation(double g, double a, double b, Rotation& r) {
+    const double d = b - a, g2 = 2.0 * g;
+    if (fabs(g2) < 1e-3 * fabs(d)) {
+        const double w = g2 / d, w2 = w * w;
+        r.p = w * fma(w2, fma(w2, 23.0 / 512.0, -5.0 / 64.0), 0.25);
+        r.s = w * fma(w2, fma(w2, 31.0 / 256.0, -3.0 / 16.0), 0.5);
+        return w * fma(w2, fma(w2, 0.0625, -0.125), 0.5);
+    }
+    const double zeta = d / g2;
+    const double t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+    const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
+    r.p = s / (1.0 + c);
+    r.s = s;
+    return t;
 }
 
 template <bool TINY>
@@ -356,18 +381,15 @@ __global__ void __launch_bounds__(SVD_SWEEP_NT, 1) svd_sweep_kernel(const SvdSec
             }
             const double g = warp_sum((g4[0] + g4[1]) + (g4[2] + g4[3]));
             if (g == 0.0 || a == 0.0 || b == 0.0) continue;
-            const double meas = fabs(g) / sqrt(a * b);
-            mymax = fmaxf(mymax, (float)meas);
-            if (meas < 1e-15) continue;
-            const double zeta = (b - a) / (2.0 * g);
-            // (from 2^27 on, 1 + zeta^2 rounds to zeta^2)
-            const double t = fabs(zeta) > 134217728.0 ? 0.5 / zeta
-                                                      : copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+            const float meas = off_diagonal(g, a, b);
+            mymax = fmaxf(mymax, meas);
+            if (meas < 1e-15f) continue;
+            Rotation rot;
+            const double t = rotation(g, a, b, rot);
             if (lane == 0) {                             // the rotated columns' squared norms
                 *np = a - t * g;
                 *nq = b + t * g;
             }
-            const Rotation rot = make_rotation(t);
             if (fabs(t) < 7.4505805969238281e-9) {       // 2^-27: the cosine, 1 - t^2 / 2, rounds to 1
                 rotate_columns<true>(rot, cp, cq, s.r, lane, u, v);
                 rotate_columns<true>(rot, vp, vq, s.k, lane, x, y);
