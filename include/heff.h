@@ -357,6 +357,7 @@ int heff_env_status(const heff_env_plan* plan, void* workspace, size_t workspace
  * A and B have flows (+1, +1, -1) and share the bond c; x is the (a, s1, s2, b) layout of
  * the bond's problem (flows +1, +1, +1, -1).  heff_two_site_apply writes every x block
  * (zeros where no (A, B) block pair matches); device doubles, asynchronous on `stream`.
+ * If a bounded device-side wait expires, x is NaN.
  * Errors: INVALID_ARG, CHARGE_MISMATCH (indices disagree), UNSUPPORTED (plan made
  * without a device), CUDA.
  */

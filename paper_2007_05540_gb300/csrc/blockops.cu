@@ -87,12 +87,12 @@ int blist_upload(BList& b) {
         std::stable_sort(b.tiles.begin(), b.tiles.end(), [](const BTile& x, const BTile& y) {
             return (int64_t)x.steps * (x.n + 32) > (int64_t)y.steps * (y.n + 32);
         });
-    // one allocation for the tables and the codes
+    // one allocation for the tables, an error flag (zero) and the codes
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t nt = b.tiles.size() * sizeof(BTile), np = b.prods.size() * sizeof(BProd), nr = b.rows.size() * sizeof(FxRows);
-    const size_t op = al(nt), orow = op + al(np), oc = orow + al(nr);
-    if (oc + b.ncodes == 0) return HEFF_OK;
-    std::vector<char> host(oc);
+    const size_t op = al(nt), orow = op + al(np), oe = orow + al(nr), oc = oe + 256;
+    if (nt + np + nr == 0) return HEFF_OK;
+    std::vector<char> host(oc, 0);
     if (nt) std::memcpy(host.data(), b.tiles.data(), nt);
     if (np) std::memcpy(host.data() + op, b.prods.data(), np);
     if (nr) std::memcpy(host.data() + orow, b.rows.data(), nr);
@@ -106,6 +106,7 @@ int blist_upload(BList& b) {
     b.d_tiles = reinterpret_cast<BTile*>(d);
     b.d_prods = reinterpret_cast<BProd*>(d + op);
     b.d_rows = reinterpret_cast<FxRows*>(d + orow);
+    b.d_err = reinterpret_cast<int*>(d + oe);
     b.d_codes = reinterpret_cast<uint16_t*>(d + oc);
     return HEFF_OK;
 }
@@ -116,6 +117,7 @@ void blist_free(BList& b) {
     b.d_tiles = nullptr;
     b.d_prods = nullptr;
     b.d_rows = nullptr;
+    b.d_err = nullptr;
     b.d_codes = nullptr;
 }
 

@@ -627,8 +627,23 @@ extern "C" void heff_env_plan_destroy(heff_env_plan* plan) {
 struct heff_two_site {
     BList prods;
     bool uploaded = false;
-    int* err = nullptr;        // host memory mapped to the device: a bounded wait expired
+    int64_t nx = 0;
 };
+
+namespace {
+
+// A bounded wait of the products expired: x is not the product; it becomes NaN and the flag zero again.
+// (One block; a flag that the host can read would cost 330 us of pinning per plan, and a plan lives for one
+// bond.)
+__global__ void __launch_bounds__(1024) two_site_check_kernel(int* __restrict__ err, double* __restrict__ x, int64_t n) {
+    const int e = *err;
+    __syncthreads();
+    if (e == 0) return;
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) x[i] = nan("");
+    if (threadIdx.x == 0) *err = 0;
+}
+
+}  // namespace
 
 extern "C" int heff_two_site_create(const heff_layout* A, const heff_layout* B, const heff_layout* x,
                                     heff_two_site** out) {
@@ -646,6 +661,7 @@ extern "C" int heff_two_site_create(const heff_layout* A, const heff_layout* B, 
         return fail(HEFF_ERR_CHARGE_MISMATCH, "A (a, s1, c), B (c, s2, b) and x (a, s1, s2, b) indices disagree");
     heff_two_site* P = new (std::nothrow) heff_two_site();
     if (!P) return fail(HEFF_ERR_OOM, "out of host memory");
+    P->nx = x->nelem;
     try {
         std::map<std::pair<int, int>, std::vector<std::pair<int, int64_t>>> a_by;   // (a, s1) -> (c, offset)
         for (size_t k = 0; k < A->offsets.size(); ++k)
@@ -675,14 +691,11 @@ extern "C" int heff_two_site_create(const heff_layout* A, const heff_layout* B, 
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) {
         int rc = heff::blist_upload(P->prods);
-        if (!rc && cudaHostAlloc((void**)&P->err, sizeof(int), cudaHostAllocMapped) != cudaSuccess)
-            rc = fail(HEFF_ERR_OOM, "heff_two_site_create: host allocation failed");
         if (rc) {
             heff::blist_free(P->prods);
             delete P;
             return rc;
         }
-        *P->err = 0;
         P->uploaded = true;
     } else {
         cudaGetLastError();
@@ -695,16 +708,16 @@ extern "C" int heff_two_site_apply(heff_two_site* P, const double* A, const doub
     heff::clear_error();
     if (!P || !A || !B || !x) return fail(HEFF_ERR_INVALID_ARG, "heff_two_site_apply: null argument");
     if (!P->uploaded) return fail(HEFF_ERR_UNSUPPORTED, "two-site plan was created without a CUDA device");
-    if (*static_cast<volatile int*>(P->err)) {
-        *P->err = 0;
-        return fail(HEFF_ERR_TIMEOUT, "heff_two_site_apply: a bounded device-side wait of an earlier call expired");
-    }
-    return heff::launch_bgemm(P->prods, A, B, x, nullptr, nullptr, 1.0, stream, P->err);
+    const int rc = heff::launch_bgemm(P->prods, A, B, x, nullptr, nullptr, 1.0, stream, P->prods.d_err);
+    if (rc || !P->prods.d_err) return rc;
+    two_site_check_kernel<<<1, 1024, 0, static_cast<cudaStream_t>(stream)>>>(P->prods.d_err, x, P->nx);
+    heff::count_launches(1);
+    if (cudaGetLastError() != cudaSuccess) return fail(HEFF_ERR_CUDA, "heff_two_site_apply: launch failed");
+    return HEFF_OK;
 }
 
 extern "C" void heff_two_site_destroy(heff_two_site* P) {
     if (!P) return;
     heff::blist_free(P->prods);
-    cudaFreeHost(P->err);
     delete P;
 }

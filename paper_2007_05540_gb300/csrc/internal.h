@@ -136,6 +136,7 @@ struct BList {
     std::vector<FxRows> rows;
     FxRows* d_rows = nullptr;
     uint16_t* d_codes = nullptr;
+    int* d_err = nullptr;      // a flag for launches that have none elsewhere, zero after the upload
     int32_t ncodes = 0;
     std::map<std::array<int64_t, 6>, int32_t> views;
     int num_sms = 0;
