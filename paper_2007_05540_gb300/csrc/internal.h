@@ -303,7 +303,7 @@ struct heff_plan {
     // (two streams alternating workspaces reuse their maps), replaced round-robin
     void* tmap_ws[2] = {nullptr, nullptr};
     int tmap_next = 0;
-    alignas(64) unsigned char tmaps[2][17][128];
+    alignas(64) unsigned char tmaps[2][24][128];
     heff::MergeList mg1, mg2;  // max_batch > 1, split precisions: the N = 256 tasks by merge class
     int device = 0;
     int num_sms = 0;

@@ -91,6 +91,11 @@ struct TcMaps {
     CUtensorMap c;      // T store map: 32 x 32 boxes (GEMM 1 only)
     CUtensorMap bq;     // B operand, 32-row box (a CTA pair's half of a narrow B tile, merged items)
     CUtensorMap aq;     // A operand, 32-row box (merged items)
+    CUtensorMap m3[5];  // merged items: the slots of all their entries, slot x entries 128 x 2, 64 x 4, 32 x 8 (256
+                        // tile columns), 64 x 2, 32 x 4 (128 tile rows).  The producer's time is the number
+                        // of loads it issues: with one per entry a batch of 16 took 1296 us, with one
+                        // for all entries 1187 (blocks of 10-60); lower boxes for the rows that are
+                        // there, half the bytes, changed nothing.
 };
 
 // Merged items of a batched launch: the batch entries of one task that share a tile, entry e in
@@ -118,6 +123,13 @@ __device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* map, uint
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(su32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(su32(bar)), "r"(x), "r"(y)
+        : "memory");
+}
+// the same from a 3-D map: z counts batch entries
+__device__ __forceinline__ void tma_load3(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y, int z) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(su32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(su32(bar)), "r"(x), "r"(y), "r"(z)
         : "memory");
 }
 
@@ -372,18 +384,19 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
             const CUtensorMap* mh = hb == 0 ? &maps.bq : &maps.b[hb - 1];
             uint32_t bytes = CL == 1 ? 2u * (uint32_t)((64 << ia) + (64 << ib)) * SWZ
                                      : (uint32_t)CL * 2u * (uint32_t)(128 + (32 << hb)) * SWZ;
-            // merged: cnt slots of the B tile (GEMM 1) or of the A tile (GEMM 2), one box each
+            // merged: the entries' slots of the B tile (GEMM 1) or of the A tile (GEMM 2, transposed) in one box
+            // (entries past the batch are other vectors' rows or zeros, for accumulator slots nobody reads)
             const int slot = w.slot;
             const CUtensorMap *ms = nullptr, *ml = nullptr;
             if (MG && slot) {
-                ms = g.mode == 0 ? (slot == 128 ? &maps.b[1] : (slot == 64 ? &maps.b[0] : &maps.bq))
-                                 : (slot == 64 ? &maps.a[0] : &maps.aq);
+                const bool cols = g.mode == 0 && !w.swap;             // the slots are tile columns
+                ms = &maps.m3[cols ? (slot == 128 ? 0 : (slot == 64 ? 1 : 2)) : (slot == 64 ? 3 : 4)];
                 int other = g.mode == 0 ? 64 << ia : 64 << ib;        // rows of the shared operand
                 if (w.swap) {
                     other = t.m <= 32 ? 32 : other;
                     ml = other == 32 ? &maps.aq : ma;
                 }
-                bytes = 2u * (uint32_t)(w.cnt * slot + other) * SWZ;
+                bytes = 2u * (uint32_t)((cols ? 256 : 128) + other) * SWZ;
             }
             // a K block at column k of the rows starts at element 2 k of the interleaved rows
             KSeg sn = t.seg_count > 0 ? g.segs[t.seg_begin] : KSeg{};
@@ -399,17 +412,13 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs g) {
                             tma_load(base, ma, &full[st], 2 * k, ar);
                             tma_load(base + S::A_BYTES, mb, &full[st], 2 * k, br);
                         } else if (w.swap) {
-                            for (int e = 0; e < w.cnt; ++e)
-                                tma_load(base + e * slot * 2 * SWZ, ms, &full[st], 2 * k, br + e * (int)g.b_batch_rows);
+                            tma_load3(base, ms, &full[st], 2 * k, t.b_row, b);
                             tma_load(base + S::A_BYTES, ml, &full[st], 2 * k, ar);
                         } else if (g.mode == 0) {
                             tma_load(base, ma, &full[st], 2 * k, ar);
-                            for (int e = 0; e < w.cnt; ++e)
-                                tma_load(base + S::A_BYTES + e * slot * 2 * SWZ, ms, &full[st], 2 * k,
-                                         br + e * (int)g.b_batch_rows);
+                            tma_load3(base + S::A_BYTES, ms, &full[st], 2 * k, t.b_row, b);
                         } else {
-                            for (int e = 0; e < w.cnt; ++e)
-                                tma_load(base + e * slot * 2 * SWZ, ms, &full[st], 2 * k, ar + e * (int)g.a_batch_rows);
+                            tma_load3(base, ms, &full[st], 2 * k, t.a_row, b);
                             tma_load(base + S::A_BYTES, mb, &full[st], 2 * k, br);
                         }
                     } else {
@@ -800,16 +809,18 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 // A 2-D map over rows of `pitch` elements whose boxes are box_rows x swz bytes (the
 // operand arrays: 128-byte boxes, a K block of the hi half and the same of the lo half).
-int make_map(CUtensorMap* m, void* base, int prec, uint64_t rows, uint64_t pitch, uint32_t box_rows, int swz) {
+// With batch > 1: a 3-D map whose boxes take box_rows rows of each of `entries` consecutive batch entries.
+int make_map(CUtensorMap* m, void* base, int prec, uint64_t rows, uint64_t pitch, uint32_t box_rows, int swz,
+             uint64_t batch = 1, uint32_t entries = 1) {
     auto fn = encode_fn();
     if (!fn) return fail(HEFF_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");
     const bool bf = prec == HEFF_PREC_BF16X3;
     const uint32_t es = bf ? 2 : 4;
-    cuuint64_t dims[2] = {pitch, rows};
-    cuuint64_t strides[1] = {pitch * es};
-    cuuint32_t box[2] = {(cuuint32_t)swz / es, box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(m, bf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims,
+    cuuint64_t dims[3] = {pitch, rows, batch};
+    cuuint64_t strides[2] = {pitch * es, rows * pitch * es};
+    cuuint32_t box[3] = {(cuuint32_t)swz / es, box_rows, entries};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(m, bf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, batch > 1 ? 3 : 2, base, dims,
                     strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                     swz == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                : (swz == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B),
@@ -937,6 +948,16 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
         int rc = make_map(&m[16], w + p->off_t, PREC, (uint64_t)(B * p->rows_t), (uint64_t)(2 * p->ld_t), 32u,
                           2 * SWZ_TC);
         if (rc) return rc;
+        // [17 ..): merged items, XT (GEMM 1) and T (GEMM 2; from the fourth on, as 128 rows are one tile)
+        constexpr int SLOTS[5][2] = {{128, 2}, {64, 4}, {32, 8}, {64, 2}, {32, 4}};
+        for (int k = 0; k < 7 && B > 1 && !p->env; ++k) {
+            const bool x = k < 5;
+            const int* sl = SLOTS[x ? k : k - 2];
+            if ((rc = make_map(&m[17 + k], w + (x ? p->off_xt : p->off_t), PREC, (uint64_t)(x ? p->rows_x : p->rows_t),
+                               (uint64_t)(2 * (x ? p->ld_x : p->ld_t)), (uint32_t)sl[0], 2 * SWZ_TC, (uint64_t)B,
+                               (uint32_t)sl[1])))
+                return rc;
+        }
         p->tmap_ws[slot] = ws;
     }
     const bool split = which == 2 && p->kchunk && CL == 1 && !MG && nbatch == 1;
@@ -949,6 +970,8 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
     maps.aq = ma[0]; maps.a[0] = ma[1]; maps.a[1] = ma[2];
     maps.bq = mb[0]; maps.b[0] = mb[1]; maps.b[1] = mb[2]; maps.b[2] = mb[3];
     maps.c = m[16];
+    if (MG)
+        for (int k = 0; k < 5; ++k) maps.m3[k] = which == 1 ? m[17 + k] : m[17 + 5 + (k < 3 ? 0 : k - 3)];
     for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
         const int nb = nbatch - b0 < MAXB ? nbatch - b0 : MAXB;
         TcArgs g{};
