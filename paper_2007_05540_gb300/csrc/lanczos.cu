@@ -208,8 +208,12 @@ __global__ void __launch_bounds__(RT) normalize_kernel(const double* __restrict_
 // The cooperative kernels run at most one block of LT threads per SM; block b owns the
 // elements [b chunk, (b + 1) chunk) of every vector, and its piece of w lives in shared memory
 // when it fits (LW_MAX doubles), else in place.
-constexpr int LT = 512, LWARPS = LT / 32;
+constexpr int LTS = 512, LTL = 1024;     // threads of a block: short and long vectors
 constexpr int LW_MAX = 25600;
+// elements per block from which it has LTL threads: twice the loads in flight (m = 4096, 39k elements a block,
+// 30 steps: 34.5 ms with 512 threads, 28.3 with 1024; m = 1024, 1.5k elements, 20 steps: 2.376 and
+// 2.360), while fewer elements leave the added warps only reductions (m = 48, 20 steps: 0.70 and 0.76)
+constexpr int LT_WIDE = 1280;
 
 struct LzArgs {
     Lz z;
@@ -223,20 +227,21 @@ struct LzArgs {
 
 struct LzBlock {
     double* h;              // [NVMAX + 1] sums over all blocks, shared memory
-    double* red;            // [LWARPS * 2]
+    double* red;            // [2 * LTL / 32]
     int64_t beg;
     int len;
 };
 
 // Sum over the block, for thread 0 (a warp's FP64 addition takes 16 cycles of the SM's FP64 unit:
 // only one warp adds the warps' sums).
+template <int LT>
 __device__ __forceinline__ double lz_block_sum(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x < 32) {
-        v = threadIdx.x < LWARPS ? red[threadIdx.x] : 0.0;
-        for (int o = LWARPS / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        v = threadIdx.x < LT / 32 ? red[threadIdx.x] : 0.0;
+        for (int o = LT / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     }
     __syncthreads();
     return v;
@@ -254,9 +259,10 @@ __device__ __forceinline__ bool lz_barrier(const LzArgs& a) {
 
 // out[j] = sum over the blocks of part[j0 + j][block], j < nv: one warp per quantity, every block
 // the same sums in the same order.
+template <int LT>
 __device__ __forceinline__ void lz_gather(const LzArgs& a, int j0, int nv, double* out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int j = warp; j < nv; j += LWARPS) {
+    for (int j = warp; j < nv; j += (LT / 32)) {
         double v = 0.0;
         for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(a.z.part + (int64_t)(j0 + j) * RB + b);
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -267,11 +273,12 @@ __device__ __forceinline__ void lz_gather(const LzArgs& a, int j0, int nv, doubl
 
 // part[j][this block] = V_j . w over the block's elements, j < nv, and part[nv] = w . w.  A warp
 // takes one vector over one of `seg` pieces of the chunk (all warps busy also for few vectors).
+template <int LT>
 __device__ __forceinline__ void lz_dots(const LzArgs& a, const LzBlock& b, const double* w, int nv) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int q = nv + 1, seg = q >= LWARPS ? 1 : LWARPS / q;
+    const int q = nv + 1, seg = q >= (LT / 32) ? 1 : (LT / 32) / q;
     const int piece = ((b.len + seg - 1) / seg + 31) & ~31;
-    for (int item = warp; item < q * seg; item += LWARPS) {
+    for (int item = warp; item < q * seg; item += (LT / 32)) {
         const int j = item / seg, s = item % seg;
         const double* v = j < nv ? a.z.V + (int64_t)j * a.z.n + b.beg : w;
         const int end = (s + 1) * piece < b.len ? (s + 1) * piece : b.len;
@@ -302,6 +309,7 @@ __device__ __forceinline__ void lz_dots(const LzArgs& a, const LzBlock& b, const
 }
 
 // w -= sum_{j < nv} h_j V_j over the block's elements; returns the block's new w . w
+template <int LT>
 __device__ __forceinline__ double lz_subtract(const LzArgs& a, const LzBlock& b, double* w, int nv) {
     double sq = 0.0;
     for (int i = threadIdx.x; i < b.len; i += LT) {
@@ -313,7 +321,7 @@ __device__ __forceinline__ double lz_subtract(const LzArgs& a, const LzBlock& b,
         w[i] = y;
         sq = fma(y, y, sq);
     }
-    return lz_block_sum(sq, b.red);
+    return lz_block_sum<LT>(sq, b.red);
 }
 
 __device__ __forceinline__ LzBlock lz_block(const LzArgs& a, double* h, double* red) {
@@ -325,9 +333,10 @@ __device__ __forceinline__ LzBlock lz_block(const LzArgs& a, double* h, double* 
 
 // One Lanczos step on w = H v_k (in the workspace): recurrence, one or two Gram-Schmidt passes,
 // alpha_k, beta_k and v_{k+1}.
+template <int LT>
 __global__ void __launch_bounds__(LT, 1) lz_step_kernel(LzArgs a) {
     extern __shared__ double dyn[];
-    __shared__ double h[NVMAX + 1], red[LWARPS * 2];
+    __shared__ double h[NVMAX + 1], red[2 * LTL / 32];
     double* state = a.z.state;
     if (state[1] == 0.0) return;                       // the same for every block: no barrier is left open
     const LzBlock b = lz_block(a, h, red);
@@ -346,25 +355,25 @@ __global__ void __launch_bounds__(LT, 1) lz_step_kernel(LzArgs a) {
     }
     // slots NVMAX (||w||^2 after a pass) and NVMAX + 1 (a) are their own: no block still reads a
     // slot that another writes, with one barrier per sum
-    acc = lz_block_sum(acc, red);
+    acc = lz_block_sum<LT>(acc, red);
     if (threadIdx.x == 0) a.z.part[(int64_t)(NVMAX + 1) * RB + blockIdx.x] = acc;
     if (!lz_barrier(a)) return;
-    lz_gather(a, NVMAX + 1, 1, h);
+    lz_gather<LT>(a, NVMAX + 1, 1, h);
     double alpha = h[0];
     for (int i = threadIdx.x; i < b.len; i += LT) w[i] -= alpha * vk[i];
     __syncthreads();
     // Gram-Schmidt against v_0 .. v_k; again when less than half of ||w||^2 is left
     double sq = 0.0;
     for (int pass = 0; pass < 2; ++pass) {
-        lz_dots(a, b, w, k + 1);
+        lz_dots<LT>(a, b, w, k + 1);
         if (!lz_barrier(a)) return;
-        lz_gather(a, 0, k + 2, h);
+        lz_gather<LT>(a, 0, k + 2, h);
         const double before = h[k + 1];
         alpha += h[k];
-        const double mine = lz_subtract(a, b, w, k + 1);
+        const double mine = lz_subtract<LT>(a, b, w, k + 1);
         if (threadIdx.x == 0) a.z.part[(int64_t)NVMAX * RB + blockIdx.x] = mine;
         if (!lz_barrier(a)) return;
-        lz_gather(a, NVMAX, 1, h);
+        lz_gather<LT>(a, NVMAX, 1, h);
         sq = h[0];
         __syncthreads();
         if (!(sq < 0.5 * before)) break;
@@ -385,16 +394,17 @@ __global__ void __launch_bounds__(LT, 1) lz_step_kernel(LzArgs a) {
 }
 
 // v_0 = x0 / ||x0||; a zero x0 leaves the iteration inactive
+template <int LT>
 __global__ void __launch_bounds__(LT, 1) lz_start_kernel(LzArgs a) {
-    __shared__ double h[NVMAX + 1], red[LWARPS * 2];
+    __shared__ double h[NVMAX + 1], red[2 * LTL / 32];
     const LzBlock b = lz_block(a, h, red);
     const double* x = a.x0 + b.beg;
     double acc = 0.0;
     for (int i = threadIdx.x; i < b.len; i += LT) acc = fma(x[i], x[i], acc);
-    acc = lz_block_sum(acc, red);
+    acc = lz_block_sum<LT>(acc, red);
     if (threadIdx.x == 0) a.z.part[blockIdx.x] = acc;
     if (!lz_barrier(a)) return;
-    lz_gather(a, 0, 1, h);
+    lz_gather<LT>(a, 0, 1, h);
     const double r = sqrt(h[0]);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.z.state[0] = 0.0;
@@ -550,8 +560,9 @@ __device__ double lz_tridiag(const double* al, const double* be, int n, double* 
 
 // The lowest Ritz pair: theta, the residual estimate |beta_{n-1} s_{n-1}|, x = V s normalised, and
 // the result record.
+template <int LT>
 __global__ void __launch_bounds__(LT, 1) lz_finish_kernel(LzArgs a) {
-    __shared__ double h[NVMAX + 1], red[LWARPS * 2], al[NVMAX], be[NVMAX], work[5 * NVMAX];
+    __shared__ double h[NVMAX + 1], red[2 * LTL / 32], al[NVMAX], be[NVMAX], work[5 * NVMAX];
     const LzBlock b = lz_block(a, h, red);
     double* state = a.z.state;
     const int n = (int)state[0], nmax = a.z.nmax;
@@ -591,10 +602,10 @@ __global__ void __launch_bounds__(LT, 1) lz_finish_kernel(LzArgs a) {
         x[i] = s;
         acc = fma(s, s, acc);
     }
-    acc = lz_block_sum(acc, red);
+    acc = lz_block_sum<LT>(acc, red);
     if (threadIdx.x == 0) a.z.part[blockIdx.x] = acc;
     if (!lz_barrier(a)) return;
-    lz_gather(a, 0, 1, h);
+    lz_gather<LT>(a, 0, 1, h);
     const double r = sqrt(h[0]);
     if (!(r > 0.0)) return;
     const double inv = 1.0 / r;
@@ -751,29 +762,34 @@ int lanczos_core(heff_plan* plan, const double* x0, int32_t n_iter, double* x_ou
              reinterpret_cast<int*>(static_cast<char*>(apply_ws) + plan->off_flags)};
     a.w_shared = a.chunk <= LW_MAX;
     const size_t smem = a.w_shared ? (size_t)a.chunk * sizeof(double) : 0;
+    const bool wide = a.chunk >= LT_WIDE;
+    const unsigned threads = wide ? LTL : LTS;
     static bool attr = false;
     cudaError_t e = cudaSuccess;
     if (!attr) {
-        e = cudaFuncSetAttribute(lz_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(lz_step_kernel<LTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  LW_MAX * (int)sizeof(double));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(lz_step_kernel<LTL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     LW_MAX * (int)sizeof(double));
         attr = e == cudaSuccess;
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(z.bar, 0, 3 * sizeof(unsigned int), st);
     void* args[] = {&a};
     auto launch = [&](const void* kernel, size_t bytes) {
         if (e == cudaSuccess)
-            e = cudaLaunchCooperativeKernel(kernel, dim3((unsigned)blocks), dim3(LT), args, bytes, st);
+            e = cudaLaunchCooperativeKernel(kernel, dim3((unsigned)blocks), dim3(threads), args, bytes, st);
         count_launches(1);
     };
-    launch((const void*)lz_start_kernel, 0);
+    launch((const void*)(wide ? lz_start_kernel<LTL> : lz_start_kernel<LTS>), 0);
     for (int k = 0; k < n_iter && e == cudaSuccess; ++k) {
         // w = H v_k (skipped work is harmless after breakdown: the result is not used)
         int rc = heff_apply_prepared(plan, z.V + (int64_t)k * n, z.w(), apply_ws, apply_ws_bytes, st);
         if (rc) return rc;
         a.k = k;
-        launch((const void*)lz_step_kernel, smem);
+        launch((const void*)(wide ? lz_step_kernel<LTL> : lz_step_kernel<LTS>), smem);
     }
-    launch((const void*)lz_finish_kernel, 0);
+    launch((const void*)(wide ? lz_finish_kernel<LTL> : lz_finish_kernel<LTS>), 0);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "heff_lanczos: %s", cudaGetErrorString(e));
     return HEFF_OK;
