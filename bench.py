@@ -558,7 +558,7 @@ def env_update_timing(w, dev, stream, precs=("fp64", "bf16x3")):
     old = old_l.assemble(lambda k: w.L_block(k))
     plan = heff.heff_env_plan_create(old_l.handle, site_l.handle, W_l.handle, new_l.handle, Wv, "left")
     out = {"m_old": m_new, "m_new": m_new,
-           "note": "left environment L[a',w,a] extended by one site; fp64: FP64 block products on CUDA cores, "
+           "note": "left environment L[a',w,a] extended by one site; fp64: FP64 accuracy from fixed-point digits on the tensor cores, "
                    "bf16x3: the same products on the tensor cores (BF16 hi/lo split, FP32 accumulation); "
                    "rel_err_bf16x3: norm-wise against the FP64 result"}
     try:
@@ -877,9 +877,9 @@ def run_ours(args):
     dom = max(g_ms, key=g_ms.get)
     useful = float(st[18] if dom == "gemm1" else st[19])
     if prec == "fp64":
-        # FP64 on CUDA cores: the GB300 FP64 rate (nominal 1.25 TFLOP/s) bounds it
-        roof = {"bound": "alu", "unit": "TFLOP/s", "peak": 1.25,
-                "peak_source": "nominal GB300 FP64 rate (no measured FP64 peak)",
+        # FP64 accuracy from eight digits an element: 36 FP16 products per useful multiply-add
+        roof = {"bound": "tensor", "unit": "TFLOP/s", "peak": peaks["bf16_tflops"] / 36,
+                "peak_source": "bf16 burst / 36 digit products, " + peak_src,
                 "achieved": useful / (g_ms[dom] * 1e-3) / 1e12}
         roof["frac"] = roof["achieved"] / roof["peak"]
     else:

@@ -1,11 +1,13 @@
 // Packing, operator preparation, and the C-ABI compute entry points of the two-site H_eff
 // matvec (Section II-C / Fig. 1d).
 //
-// One apply is four launches on the caller's stream:
+// One apply is four launches on the caller's stream (the first two are one for small plans; FP64 adds the
+// operands' digit planes, split GEMM 2 tiles a sum over their parts):
 //   mix_kernel   LW = L.W1 and RW = W2.R into the workspace (operator preparation)
 //   pack_kernel  x -> XT (per charge sector, transposed so the contraction index is
 //                contiguous; hi/lo split for the tensor-core precisions)
-//   GEMM 1       T = LW . XT^T              (split precisions: tc_gemm.cu; FP64: fx_gemm.cu)
+//   GEMM 1       T = LW . XT^T              (split precisions: tc_gemm.cu; FP64: fx_planes.cu, or
+//                                            fx_gemm.cu where the workspace has no room for planes)
 //   GEMM 2       y = T . RW^T               (written straight into y's block layout)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -556,7 +558,7 @@ int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, 
 
 // Mixing and packing in one launch: split precisions (an FP64 tile needs twice the shared memory), up to
 // MAXB vectors, where all blocks are resident at once.  A small apply is a chain of launches, one less here
-// (m = 32: 20.4 -> 16.4 us); with many waves of mixing blocks the shared memory that packing needs takes
+// (m = 100: 20.4 -> 16.4 us); with many waves of mixing blocks the shared memory that packing needs takes
 // L1 from all of them (m = 4096: 549 us in two launches, 562 in one).  Returns whether it ran.
 template <typename In, int PREC>
 static void launch_mix_pack_t(heff_plan* p, const MixArgs& m, const PtrBatch& xs, int nb, char* ws, cudaStream_t st) {

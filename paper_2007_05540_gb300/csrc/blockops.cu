@@ -1,6 +1,6 @@
 // Block-product engine: lists of strided dense block products summed into output tiles (run by
-// fx_gemm.cu in FP64 accuracy, or by blockops_tc.cu in BF16x3), and block dot products.  Used by the environment update and the Rayleigh-quotient
-// gradients (the block-pair contractions of Algorithm 2 with charge-matched blocks, each
+// fx_gemm.cu in FP64 accuracy, or by blockops_tc.cu in BF16x3), and block dot products.  Used by the environment update,
+// the two-site tensor, the SVD and the Rayleigh-quotient gradients (the block-pair contractions of Algorithm 2 with charge-matched blocks, each
 // product a small dense GEMM, Section IV "list" algorithm).
 #include <cuda_runtime.h>
 

@@ -8,7 +8,7 @@
 //   LW[(n, t, i', j) a', (s, i) a] = sum_u c(u, t, s, n) env_old[i', u, i]                  (mix)
 // so the update is one operator preparation and two grouped GEMMs over workspace operands with
 // the contraction index contiguous: the kernels of the H_eff matvec (apply.cu, tc_gemm.cu,
-// fx_gemm.cu) run it from tables of the same form (heff_plan with env set).  W enters with the
+// fx_planes.cu) run it from tables of the same form (heff_plan with env set).  W enters with the
 // environment, before the GEMMs: a product per entry of W, as in the list form below, contracts the
 // same site block with up to k blocks that differ by a coefficient.
 //

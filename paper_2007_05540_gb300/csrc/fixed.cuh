@@ -1,5 +1,5 @@
 // FP64 values as 64-bit fixed-point numbers of eight signed 8-bit digits, and back: the
-// arithmetic of the FP64 products on the FP16 tensor pipe (fx_gemm.cu).
+// arithmetic of the FP64 products on the FP16 tensor pipe (fx_gemm.cu, fx_planes.cu).
 //
 // A row of an operand shares one exponent code E (|v| < 2^(E - 1022) for every v of the row),
 // and v is held as q = trunc(v 2^(1084 - E)), |q| < 2^62, written in balanced base 256:

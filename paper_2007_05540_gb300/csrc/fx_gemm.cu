@@ -19,9 +19,10 @@
 // Rows that the scale cannot hold (infinities, NaNs, magnitudes beyond 2^+-400) make their tile
 // run in FP64 arithmetic on the CUDA cores inside the same kernel.
 //
-// Two sources of work share the kernel: the matvec's task lists over the workspace operands
-// (MODE 0; K contiguous, one pitch) and the block-product lists with arbitrary strides and
-// scalar coefficients (MODE 1).
+// Two sources of work share the kernel: the block-product lists with arbitrary strides and scalar
+// coefficients (MODE 1: gradients, two-site tensor, the SVD's products), and the matvec's task lists over
+// the workspace operands (MODE 0; K contiguous, one pitch) where the workspace has no room for the digit
+// planes that fx_planes.cu multiplies.
 //
 // One persistent CTA per SM, 128 x 64 output tiles, 20 warps:
 //   warps 0-7    producers: load 128 + 64 rows x 16 K of FP64, convert to digits, write the FP16
@@ -35,8 +36,8 @@
 //
 // Bound by the 36 digit products: 1.9 PFLOP/s of FP16 / 36 = 53 TFLOP/s, less the ragged tiles and
 // the drain of the accumulators every 256 steps.  Against the FP64 units (64 x 64 tiles on the
-// CUDA cores), whole calls: prepared matvec m = 1024, k = 14, 6.24 -> 0.65 ms; environment update
-// m = 1024, 4.9 -> 0.59 ms; gradients m = 320, 9.2 -> 1.46 ms.
+// CUDA cores), whole calls: prepared matvec m = 1024, k = 14, 6.24 -> 0.58 ms (0.40 from planes); gradients
+// m = 320, 9.2 -> 1.23 ms.
 // Every mbarrier wait is bounded; on expiry the CTA raises the error flag, stops issuing work,
 // waits (bounded) for its MMAs in flight, frees its tensor memory and returns.
 #include <cuda_fp16.h>

@@ -119,7 +119,7 @@ struct FxRows {
     int32_t out;            // first code
     int32_t which;          // 0: A, 1: B
 };
-// output tile of the FP64 products (fx_gemm.cu)
+// output tile of the FP64 products (fx_gemm.cu, fx_planes.cu)
 constexpr int FX_TILE_M = 128, FX_TILE_N = 64;
 struct BList {
     std::vector<BTile> tiles;
@@ -280,8 +280,8 @@ struct heff_plan {
     // there is no RW, and which = 1 mix tiles fill XT
     bool env = false;
     heff::GemmList fx1, fx2;          // FP64 plans: the task lists that run (FX_TILE_M x FX_TILE_N tiles)
-    // FP64 plans: exponent codes of the operand arrays, [column / KPAD][row]; they come last in the
-    // workspace (ws_min: its size without them, when every tile runs in FP64 arithmetic)
+    // FP64 plans: exponent codes of the operand arrays, [column / KPAD][row], after the arrays and the
+    // flags (ws_min: the workspace up to here, when every tile runs in FP64 arithmetic)
     size_t off_ex = 0, off_elw = 0, off_et = 0, off_erw = 0, ws_min = 0;
     // split tiles of GEMM 2: chunk of the contraction (in KPAD units; 0: no limit) and their scratch in
     // the workspace (after ws_min too).

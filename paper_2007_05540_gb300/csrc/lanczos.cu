@@ -24,7 +24,7 @@
 // Reductions are two-stage with a fixed order, so results are deterministic.
 //
 // One step's vector work was twelve launches whose kernels ran 3-16 us each; at m = 1024 (n =
-// 232k) they took 120 us of a 216 us step.  In one kernel the phases meet at grid barriers (about
+// 406k) they took 120 us of a 216 us step.  In one kernel the phases meet at grid barriers (about
 // 2 us each) and w stays in shared memory between them.
 #include <cuda_runtime.h>
 
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(RT) normalize_kernel(const double* __restrict_
 constexpr int LTS = 512, LTL = 1024;     // threads of a block: short and long vectors
 constexpr int LW_MAX = 25600;
 // elements per block from which it has LTL threads: twice the loads in flight (m = 4096, 39k elements a block,
-// 30 steps: 34.5 ms with 512 threads, 28.3 with 1024; m = 1024, 1.5k elements, 20 steps: 2.376 and
+// 30 steps: 34.5 ms with 512 threads, 28.3 with 1024; m = 1024, 2.7k elements, 20 steps: 2.376 and
 // 2.360), while fewer elements leave the added warps only reductions (m = 48, 20 steps: 0.70 and 0.76)
 constexpr int LT_WIDE = 1280;
 

@@ -166,12 +166,14 @@ __global__ void svd_copy_w_kernel(const SvdSector* __restrict__ secs, double* __
 // the norms are recomputed at the start of every sweep, so the rounding drift stays at a
 // few ulps of the column's norm.
 //
-// Bound by the SM's FP64 unit (two lanes a clock: a warp's instruction holds it 16 cycles) and by the
-// latency of a round.  So the pairs go to blocks first and warps second, which spreads them over every SM
+// Bound by the latency of a round (grid barrier 2 us, a trip to L2, the dot product's and the angle's chains),
+// which FP64 work lengthens where several pairs share an SM's FP64 unit (two lanes a clock: a warp's
+// instruction holds it 16 cycles).  So the pairs go to blocks first and warps second, which spreads them over every SM
 // (472 pairs on 59 SMs: 2.45 ms a sweep); the first SVD_PIECES * 32 rows of both columns of J and V are
 // loaded at once and stay in registers from the dot product to the rotation; and a rotation takes three
 // multiply-adds per element pair, as the shears u -= p v, v += s u, u -= p v with p = tan(theta / 2), or
-// two where the cosine rounds to one, instead of two products and two multiply-adds: 1.42 ms a sweep.  The
+// two where the cosine rounds to one, instead of two products and two multiply-adds; and an angle takes one
+// division: 0.82 ms a sweep (942 columns in 19 sectors; 0.11 ms of it is FP64 multiply-adds at 0.6 T/s).  The
 // shears have determinant one whatever p and s round to; with a cosine that rounds to one the columns grew
 // with every rotation (sum of s^2 over |x|^2 - 1 at m = 512: 1.2e-14, now 6e-16).
 constexpr int SVD_SWEEP_NT = 256;

@@ -1096,7 +1096,7 @@ extern "C" int heff_wait_selftest(const heff_plan* plan, void* workspace, size_t
     if (!plan || !workspace || (kind != 0 && kind != 1))
         return fail(HEFF_ERR_INVALID_ARG, "heff_wait_selftest: null plan/workspace or kind not 0/1");
     if (plan->opts.precision == HEFF_PREC_FP64)
-        return fail(HEFF_ERR_INVALID_ARG, "heff_wait_selftest: FP64 plans have no device-side waits");
+        return fail(HEFF_ERR_INVALID_ARG, "heff_wait_selftest: not available for FP64 plans");
     if (workspace_bytes < plan->off_flags + 256)
         return fail(HEFF_ERR_WORKSPACE, "heff_wait_selftest: workspace smaller than the plan's");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
