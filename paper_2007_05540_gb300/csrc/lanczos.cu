@@ -72,7 +72,7 @@ struct Lz {
     double* state;   // n_eff, active, theta, resid, -, ..., alpha[nmax], beta[nmax]
     double* s;       // eigenvector of the tridiagonal matrix
     double* part;    // partial sums, [quantity][block]
-    unsigned int* bar;   // grid barrier: counter, generation, error
+    unsigned int* bar;   // grid barrier: counter, -, error
     double* V;       // (nmax) basis vectors, then w
     int64_t n;
     int nmax;
@@ -252,7 +252,7 @@ __device__ __forceinline__ bool lz_barrier(const LzArgs& a) {
         __syncthreads();
         return true;
     }
-    const bool ok = grid_barrier(a.z.bar, a.z.bar + 1, gridDim.x, reinterpret_cast<int*>(a.z.bar + 2));
+    const bool ok = grid_barrier(a.z.bar, gridDim.x, reinterpret_cast<int*>(a.z.bar + 2));
     if (!ok && threadIdx.x == 0) atomicExch(a.apply_err, 1);
     return ok;
 }

@@ -154,7 +154,7 @@ __global__ void svd_copy_w_kernel(const SvdSector* __restrict__ secs, double* __
 // A sweep (all rounds) inside one cooperative launch: the warps of the grid take the
 // (sector, pair) items of a round from a flattened list (pair_off: prefix sums of each
 // sector's pair count), rotate, and meet at a grid barrier before the next round.  The
-// barrier is a counter and a generation word in global memory; its wait is bounded (about a
+// barrier is a counter word in global memory; its wait is bounded (about a
 // second), after which the kernel sets err and returns.  The phase's further sweeps follow in the same launch.
 //
 // Column norms are carried instead of recomputed per pair (as in the standard one-sided
@@ -198,7 +198,7 @@ __device__ __forceinline__ bool sweep_goes_on(const Sweeps& sw, int sweep, int m
             *sw.count = sweep + 1;
         }
     }
-    if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return false;
+    if (!grid_barrier(bar, gridDim.x, err)) return false;
     return !(__int_as_float(*(volatile int*)(sw.seen + sweep % 3)) < sw.stop);
 }
 
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(SVD_SWEEP_NT, 1) svd_sweep_kernel(const SvdSec
         a = warp_sum(a);
         if (lane == 0) nrm[item] = a;
     }
-    if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return;
+    if (!grid_barrier(bar, gridDim.x, err)) return;
     for (int round = 0; round < kk_all - 1; ++round) {
         for (int item = gw; item < npairs; item += nw) {
             if (several) find(item);
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(SVD_SWEEP_NT, 1) svd_sweep_kernel(const SvdSec
                 rotate_columns<false>(rot, vp, vq, s.k, lane, x, y);
             }
         }
-        if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return;
+        if (!grid_barrier(bar, gridDim.x, err)) return;
     }
     for (int o = 16; o > 0; o >>= 1) mymax = fmaxf(mymax, __shfl_xor_sync(0xffffffffu, mymax, o));
     if (lane == 0) atomicMax(&mx, __float_as_int(mymax));
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(SVD_BT) svd_block_sweep_kernel(const SvdSector
             }
             __syncthreads();
         }
-        if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return;
+        if (!grid_barrier(bar, gridDim.x, err)) return;
     }
     if (!sweep_goes_on(sw, sweep, bmax, bar, err)) return;
     }
@@ -800,7 +800,7 @@ __global__ void svd_write_kernel(const SvdSector* __restrict__ secs, const Write
 
 // One block meets the sweeps' grid barrier set up for two blocks: its wait must give up,
 // set err and return.
-__global__ void barrier_selftest_kernel(unsigned int* bar, int* err) { grid_barrier(bar, bar + 1, 2u, err); }
+__global__ void barrier_selftest_kernel(unsigned int* bar, int* err) { grid_barrier(bar, 2u, err); }
 
 }  // namespace
 

@@ -1105,7 +1105,7 @@ extern "C" int heff_wait_selftest(const heff_plan* plan, void* workspace, size_t
     cudaEvent_t ev[2] = {nullptr, nullptr};
     cudaError_t e = cudaEventCreate(&ev[0]);
     if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
-    // error flag at byte 0 of the flag area; the barrier's counter and generation at 64, 68
+    // error flag at byte 0 of the flag area; the barrier's counter at 64
     if (e == cudaSuccess) e = cudaMemsetAsync(f, 0, 128, st);
     if (e == cudaSuccess) e = cudaEventRecord(ev[0], st);
     if (e == cudaSuccess) {
