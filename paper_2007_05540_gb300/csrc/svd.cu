@@ -91,6 +91,10 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// blocks per tensor block of the kernels that copy between the tensors and J, V (m = 512, 70 tensor blocks: one
+// each took 26 and 40 us)
+constexpr int COPY_SPLIT = 8;
+
 // scatter x blocks into column-major J (or J^T layout for wide sectors)
 __global__ void svd_load_kernel(const SvdSector* __restrict__ secs, const int64_t* __restrict__ tab, int ntab,
                                 const double* __restrict__ x, double* __restrict__ ws) {
@@ -101,7 +105,7 @@ __global__ void svd_load_kernel(const SvdSector* __restrict__ secs, const int64_
         const int64_t xo = t[1];
         const int mr = (int)t[2], nc = (int)t[3], r0 = (int)t[4], c0 = (int)t[5];
         double* J = ws + s.j_off;
-        for (int e = threadIdx.x; e < mr * nc; e += blockDim.x) {
+        for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < mr * nc; e += gridDim.y * blockDim.x) {
             const int a = e / nc, c = e % nc;
             const int R = r0 + a, Cc = c0 + c;         // position in M_Q
             const double v = x[xo + e];
@@ -777,7 +781,7 @@ __global__ void svd_write_kernel(const SvdSector* __restrict__ secs, const Write
     const SvdSector s = secs[e.sec];
     const double* J = ws + s.j_off;
     const double* V = ws + s.v_off;
-    for (int idx = threadIdx.x; idx < e.rows * e.cols; idx += blockDim.x) {
+    for (int idx = blockIdx.y * blockDim.x + threadIdx.x; idx < e.rows * e.cols; idx += gridDim.y * blockDim.x) {
         const int r = idx / e.cols, c = idx % e.cols;
         double v;
         if (e.left) {
@@ -955,7 +959,7 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
     SVD_CK(cudaMemcpyAsync(d_tab, tab.data(), tab.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     const int ntab = (int)(tab.size() / 6);
     float* f32 = reinterpret_cast<float*>(static_cast<char*>(workspace) + S->off_f32);
-    if (ntab) svd_load_kernel<<<std::min(ntab, 4096), 256, 0, st>>>(S->d_sec, d_tab, ntab, x, ws);
+    if (ntab) svd_load_kernel<<<dim3(std::min(ntab, 4096), COPY_SPLIT), 256, 0, st>>>(S->d_sec, d_tab, ntab, x, ws);
     svd_to_f32_kernel<<<dim3(128, nsec), 256, 0, st>>>(S->d_sec, ws, f32);
     heff::count_launches(2);
     if (!S->lists_uploaded) {
@@ -1198,7 +1202,7 @@ extern "C" int heff_svd_write(heff_svd* S, const heff_layout* A_layout, const he
     SVD_CK(cudaMemcpyAsync(d_ent, ents.data(), ents.size() * sizeof(WriteEntry), cudaMemcpyHostToDevice, st));
     SVD_CK(cudaMemcpyAsync(d_kept, keptflat.data(), keptflat.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     if (!ents.empty())
-        svd_write_kernel<<<(unsigned)ents.size(), 256, 0, st>>>(S->d_sec, d_ent, d_kept, ws, sv, A, B, absorb_right);
+        svd_write_kernel<<<dim3((unsigned)ents.size(), COPY_SPLIT), 256, 0, st>>>(S->d_sec, d_ent, d_kept, ws, sv, A, B, absorb_right);
     heff::count_launches(1);
     SVD_CK(cudaStreamSynchronize(st));
     cudaFree(d_ent);
