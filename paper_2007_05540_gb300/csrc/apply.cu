@@ -495,25 +495,25 @@ int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, cons
 }
 
 // ------------------------------------------------------------------ split tiles
-// y of the split tiles: the parts of a tile added in order (block: 8 rows of a tile; lanes along the
-// columns).  Adding them in the GEMM, by whichever CTA finishes a tile last, leaves the additions to a
+// y of the split tiles: the parts of a tile added in order (block: SUM_ELEMS elements of a tile).  Adding them in the GEMM, by whichever CTA finishes a tile last, leaves the additions to a
 // few warps and their load latency: apply m = 1024, TF32x3, 85 us of GEMM 2 unsplit, 110 us that way.
+// Bound by the latency of its loads, all parts of an element at once.  Blocks of eight rows with lanes along the
+// columns left most of a block without work at 31 x 44 elements a tile: m = 1024, 60 tiles, 16 us; now 9.
+constexpr int SUM_ELEMS = 512;
 template <typename P, typename Y>
-__global__ void __launch_bounds__(256) sum_parts_kernel(const SplitTile* __restrict__ tiles, int row_blocks,
+__global__ void __launch_bounds__(256) sum_parts_kernel(const SplitTile* __restrict__ tiles, int blocks,
                                                         const P* __restrict__ scratch, int64_t scratch_elems,
                                                         PtrBatch ys) {
-    const SplitTile t = tiles[blockIdx.x / row_blocks];
-    const int r = (int)(blockIdx.x % row_blocks) * 8 + (threadIdx.x >> 5);
+    const SplitTile t = tiles[blockIdx.x / blocks];
+    const int part = t.m * t.n, e0 = (int)(blockIdx.x % blocks) * SUM_ELEMS;
     pdl_wait();
     pdl_trigger();
-    if (r >= t.m) return;
-    const P* sp = scratch + (int64_t)blockIdx.y * scratch_elems + t.off + (int64_t)r * t.n;
-    Y* y = static_cast<Y*>(const_cast<void*>(ys.p[blockIdx.y])) + t.c_off + (int64_t)r * t.ldc;
-    const int64_t part = (int64_t)t.m * t.n;
-    for (int c = threadIdx.x & 31; c < t.n; c += 32) {
+    const P* sp = scratch + (int64_t)blockIdx.y * scratch_elems + t.off;
+    Y* y = static_cast<Y*>(const_cast<void*>(ys.p[blockIdx.y])) + t.c_off;
+    for (int e = e0 + (int)threadIdx.x; e < e0 + SUM_ELEMS && e < part; e += 256) {
         P v[SPLIT_MAX];
 #pragma unroll
-        for (int k = 0; k < SPLIT_MAX; ++k) v[k] = k < t.parts ? sp[k * part + c] : (P)0;
+        for (int k = 0; k < SPLIT_MAX; ++k) v[k] = k < t.parts ? sp[(int64_t)k * part + e] : (P)0;
         auto wide = [](P f) {
             if constexpr (std::is_same<P, float>::value && std::is_same<Y, double>::value) return f32_to_f64(f);
             else return (Y)f;
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const SplitTile* __restr
 #pragma unroll
         for (int k = 1; k < SPLIT_MAX; ++k)
             if (k < t.parts) a += wide(v[k]);
-        y[c] = a;
+        y[(int64_t)(e / t.n) * t.ldc + e % t.n] = a;
     }
 }
 
@@ -530,12 +530,14 @@ int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, 
     if (g.split.empty()) return HEFF_OK;
     PtrBatch ys{};
     for (int b = 0; b < nbatch; ++b) ys.p[b] = y[b];
-    const int row_blocks = (g.tm + 7) / 8;
+    int most = 1;
+    for (const SplitTile& t : g.split) most = std::max(most, (int)(t.m * t.n));
+    const int blocks = (most + SUM_ELEMS - 1) / SUM_ELEMS;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)(g.split.size() * row_blocks), (unsigned)nbatch);
+    cfg.gridDim = dim3((unsigned)(g.split.size() * blocks), (unsigned)nbatch);
     cfg.blockDim = dim3(256);
     cfg.stream = static_cast<cudaStream_t>(stream);
     cfg.attrs = at;
@@ -543,13 +545,13 @@ int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, 
     const char* w = static_cast<const char*>(ws) + p->off_split;
     const SplitTile* t = g.d_split;
     if (p->opts.precision == HEFF_PREC_FP64)
-        cudaLaunchKernelEx(&cfg, sum_parts_kernel<double, double>, t, row_blocks, reinterpret_cast<const double*>(w),
+        cudaLaunchKernelEx(&cfg, sum_parts_kernel<double, double>, t, blocks, reinterpret_cast<const double*>(w),
                            g.split_elems, ys);
     else if (p->opts.io_dtype == HEFF_DTYPE_F64)
-        cudaLaunchKernelEx(&cfg, sum_parts_kernel<float, double>, t, row_blocks, reinterpret_cast<const float*>(w),
+        cudaLaunchKernelEx(&cfg, sum_parts_kernel<float, double>, t, blocks, reinterpret_cast<const float*>(w),
                            g.split_elems, ys);
     else
-        cudaLaunchKernelEx(&cfg, sum_parts_kernel<float, float>, t, row_blocks, reinterpret_cast<const float*>(w),
+        cudaLaunchKernelEx(&cfg, sum_parts_kernel<float, float>, t, blocks, reinterpret_cast<const float*>(w),
                            g.split_elems, ys);
     count_launches(1);
     CK(cudaGetLastError());
