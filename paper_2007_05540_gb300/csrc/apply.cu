@@ -495,8 +495,9 @@ int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, cons
 }
 
 // ------------------------------------------------------------------ split tiles
-// y of the split tiles: the parts of a tile added in order (block: SUM_ELEMS elements of a tile).  Adding them in the GEMM, by whichever CTA finishes a tile last, leaves the additions to a
-// few warps and their load latency: apply m = 1024, TF32x3, 85 us of GEMM 2 unsplit, 110 us that way.
+// y of the split tiles: the parts of a tile added in order (block: SUM_ELEMS elements of a tile).
+// Adding them in the GEMM, by whichever CTA finishes a tile last, leaves the additions to a few
+// warps and their load latency: apply m = 1024, TF32x3, 85 us of GEMM 2 unsplit, 110 us that way.
 // Bound by the latency of its loads, all parts of an element at once.  Blocks of eight rows with lanes along the
 // columns left most of a block without work at 31 x 44 elements a tile: m = 1024, 60 tiles, 16 us; now 9.
 constexpr int SUM_ELEMS = 512;
