@@ -61,7 +61,9 @@ extern "C" {
 #define HEFF_ERR_WORKSPACE -7       /* workspace too small or misaligned (256 B)     */
 
 /* ---- precisions and element types ----------------------------------------- */
-#define HEFF_PREC_FP64 0   /* FP64 accuracy: 62-bit fixed-point digits, exact sums      */
+/* FP64: every element of a product within a small multiple (up to 5) of the bound of a running FP64 sum,
+ * n 2^-53 sum |a||b| over its n terms, whatever the operands' scales and gradings. */
+#define HEFF_PREC_FP64 0
 #define HEFF_PREC_BF16X3 1 /* tcgen05 BF16 hi/lo split, 3 products, FP32 accumulate   */
 #define HEFF_PREC_TF32X3 2 /* tcgen05 TF32 hi/lo split, 3 products, FP32 accumulate   */
 
@@ -334,7 +336,7 @@ void heff_env_plan_destroy(heff_env_plan* plan);
 
 /*
  * Arithmetic of the environment update's block products.  HEFF_PREC_FP64 (the default):
- * FP64 accuracy, from fixed-point digits.  HEFF_PREC_BF16X3: on the tensor cores, each operand element split
+ * FP64 accuracy (as HEFF_PREC_FP64 above).  HEFF_PREC_BF16X3: on the tensor cores, each operand element split
  * into bf16 hi + lo and three products per K block, FP32 accumulation (about 1e-5 relative
  * per product); the tensors stay FP64 buffers (the update converts env_old and the site
  * tensor to FP32 copies in the workspace, whose size covers both precisions) and the call

@@ -7,7 +7,7 @@
 //   pack_kernel  x -> XT (per charge sector, transposed so the contraction index is
 //                contiguous; hi/lo split for the tensor-core precisions)
 //   GEMM 1       T = LW . XT^T              (split precisions: tc_gemm.cu; FP64: fx_planes.cu, or
-//                                            fx_gemm.cu where the workspace has no room for planes)
+//                                            below where the workspace has no room for digit planes)
 //   GEMM 2       y = T . RW^T               (written straight into y's block layout)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -328,6 +328,65 @@ __global__ void __launch_bounds__(256, HEFF_MIX_MINB) mix_pack_kernel(MixArgs a,
     mix_tile<In, PREC>(a.tiles[blockIdx.x - pack_blocks], a);
 }
 
+// ------------------------------------------------------------------ FP64 CUDA-core GEMM
+// FP64 plans whose workspace has no room for digit planes (fx_planes.cu): C[m x n] = sum_seg A[a_row + r, k]
+// B[b_row + c, k], 64 rows of a tile a block (blockIdx.z: which), 4 x 4 outputs a thread.  Bound by the FP64
+// units, 1.2 TFLOP/s of the chip.
+struct GemmArgs {
+    const GemmTask* tasks;
+    const KSeg* segs;
+    const double* A; int64_t a_batch_rows;  // operand arrays and their per-batch row offsets
+    const double* B; int64_t b_batch_rows;
+    int64_t ld;                             // shared row pitch of A and B
+    double* C; int64_t c_batch_elems;       // GEMM 1 output (T) and per-batch offset
+    PtrBatch y;                             // GEMM 2 outputs (one per batch entry)
+    int to_y;
+};
+
+__global__ void __launch_bounds__(256) gemm_fp64_kernel(const __grid_constant__ GemmArgs g) {
+    __shared__ double As[16][64 + 1];
+    __shared__ double Bs[16][64 + 1];
+    const GemmTask t = g.tasks[blockIdx.x];
+    const int bz = blockIdx.y, r0 = 64 * (int)blockIdx.z, m = min(64, t.m - r0);
+    if (m <= 0) return;
+    const double* A = g.A + (t.a_row + r0 + (int64_t)bz * g.a_batch_rows) * g.ld;
+    const double* B = g.B + (t.b_row + (int64_t)bz * g.b_batch_rows) * g.ld;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    double acc[4][4] = {};
+    for (int s = 0; s < t.seg_count; ++s) {
+        const KSeg sg = g.segs[t.seg_begin + s];
+        for (int k0 = sg.k0; k0 < sg.k0 + sg.klen; k0 += 16) {
+            for (int l = 0; l < 4; ++l) {
+                const int idx = tid + 256 * l, row = idx >> 4, kk = idx & 15;
+                As[kk][row] = row < m ? A[row * g.ld + k0 + kk] : 0.0;
+                Bs[kk][row] = row < t.n ? B[row * g.ld + k0 + kk] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int kk = 0; kk < 16; ++kk) {
+                double a[4], b[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty * 4 + i]; b[i] = Bs[kk][tx * 4 + i]; }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            }
+            __syncthreads();
+        }
+    }
+    double* C = (g.to_y ? static_cast<double*>(const_cast<void*>(g.y.p[bz])) : g.C + (int64_t)bz * g.c_batch_elems) +
+                t.c_off + (int64_t)r0 * t.ldc;
+    for (int i = 0; i < 4; ++i) {
+        const int r = ty * 4 + i;
+        if (r >= m) continue;
+        for (int j = 0; j < 4; ++j) {
+            const int c = tx * 4 + j;
+            if (c < t.n + t.n_zero) C[(int64_t)r * t.ldc + c] = c < t.n ? acc[i][j] : 0.0;
+        }
+    }
+}
+
 // ------------------------------------------------------------------ host side
 #define CK(call)                                                                        \
     do {                                                                                \
@@ -375,12 +434,11 @@ int plan_upload(heff_plan* p) {
     a.add(p->pack, &p->d_pack);
     a.add(p->mix, &p->d_mix);
     a.add(p->terms, &p->d_terms);
-    for (GemmList* g : {&p->g1, &p->g2, &p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->sp2, &p->sp2_alt, &p->fx1,
-                        &p->fx2}) {
-        if (p->opts.precision == HEFF_PREC_FP64 && (g == &p->g1 || g == &p->g2)) continue;   // fx1, fx2 run
+    for (GemmList* g : {&p->g1, &p->g2, &p->g1_alt, &p->g2_alt, &p->g1_pair, &p->g2_pair, &p->sp2, &p->sp2_alt}) {
         a.add(g->tasks, &g->d_tasks);
         a.add(g->segs, &g->d_segs);
         a.add(g->split, &g->d_split);
+        a.add(g->fp64_at, &g->d_fp64_at);
     }
     for (FxOperand& o : p->fxo)
         if (p->planes_ok) {
@@ -429,8 +487,7 @@ static void launch_pack_t(heff_plan* p, const PtrBatch& xs, int nb, char* ws, ui
     cudaLaunchKernelEx(&cfg, pack_kernel<In, PREC>, pack_args(p, xs, ws, codes));
 }
 
-int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, int level, void* stream) {
-    const bool codes = level >= 1;
+int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, bool planes, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (p->pack.empty()) return HEFF_OK;
     for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
@@ -439,8 +496,8 @@ int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, 
         for (int b = 0; b < nb; ++b) xs.p[b] = x[b0 + b];
         char* w = static_cast<char*>(ws) + (size_t)b0 * p->rows_x * p->ld_x * p->esize * p->planes;
         const bool f32 = p->opts.io_dtype == HEFF_DTYPE_F32;
-        uint16_t* e = codes && p->opts.precision == HEFF_PREC_FP64 ? reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + p->off_ex) + (int64_t)b0 * p->rows_x
-                            : nullptr;
+        uint16_t* e = planes ? reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + p->off_ex) + (int64_t)b0 * p->rows_x
+                             : nullptr;
         switch (p->opts.precision) {
             case HEFF_PREC_FP64: launch_pack_t<double, HEFF_PREC_FP64>(p, xs, nb, w, e, st); break;
             case HEFF_PREC_BF16X3:
@@ -475,14 +532,13 @@ static void launch_mix_t(heff_plan* p, const void* L, const void* W1, const void
 }
 
 int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, void* ws,
-               int level, void* stream) {
-    const bool codes = level >= 1;
+               bool planes, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (p->mix.empty()) return HEFF_OK;
     char* w = static_cast<char*>(ws);
     const bool f32 = p->opts.io_dtype == HEFF_DTYPE_F32;
     switch (p->opts.precision) {
-        case HEFF_PREC_FP64: launch_mix_t<double, HEFF_PREC_FP64>(p, L, W1, W2, R, w, st, codes); break;
+        case HEFF_PREC_FP64: launch_mix_t<double, HEFF_PREC_FP64>(p, L, W1, W2, R, w, st, planes); break;
         case HEFF_PREC_BF16X3:
             if (f32) launch_mix_t<float, HEFF_PREC_BF16X3>(p, L, W1, W2, R, w, st);
             else launch_mix_t<double, HEFF_PREC_BF16X3>(p, L, W1, W2, R, w, st);
@@ -602,15 +658,47 @@ static bool launch_mix_pack(heff_plan* p, const void* L, const void* W1, const v
 
 int launch_tc_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
 
-int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, int level, void* stream) {
+int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool planes, void* stream) {
     if (p->opts.precision != HEFF_PREC_FP64) return launch_tc_gemm(p, which, ws, y, nbatch, stream);
-    return level == 2 ? launch_fx_planes(p, which, ws, y, nbatch, stream)
-                      : launch_fx_matvec(p, which, ws, y, nbatch, level >= 1, stream);
+    if (planes) return launch_fx_planes(p, which, ws, y, nbatch, stream);
+    const GemmList& gl = which == 1 ? p->g1 : p->g2;
+    if (gl.tasks.empty()) return HEFF_OK;
+    char* w = static_cast<char*>(ws);
+    for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
+        const int nb = nbatch - b0 < MAXB ? nbatch - b0 : MAXB;
+        const double* T = reinterpret_cast<const double*>(w + p->off_t) + (int64_t)b0 * p->rows_t * p->ld_t;
+        const double* XT = reinterpret_cast<const double*>(w + p->off_xt) + (int64_t)b0 * p->rows_x * p->ld_x;
+        const double* LW = reinterpret_cast<const double*>(w + p->off_lw);
+        GemmArgs g{};
+        g.tasks = gl.d_tasks;
+        g.segs = gl.d_segs;
+        g.ld = which == 1 ? p->ld_x : p->ld_t;
+        if (p->env) {                               // one vector; A: the site tensor, B: LW, then T
+            g.A = XT;
+            g.B = which == 1 ? LW : T;
+        } else if (which == 1) {
+            g.A = LW;
+            g.B = XT;
+            g.b_batch_rows = p->rows_x;
+        } else {
+            g.A = T;
+            g.a_batch_rows = p->rows_t;
+            g.B = reinterpret_cast<const double*>(w + p->off_rw);
+        }
+        g.C = const_cast<double*>(T);
+        g.c_batch_elems = p->rows_t * p->ld_t;
+        g.to_y = which == 2;
+        for (int b = 0; b < nb && g.to_y; ++b) g.y.p[b] = y[b0 + b];
+        gemm_fp64_kernel<<<dim3((unsigned)gl.tasks.size(), nb, (unsigned)(gl.tm / 64)), 256, 0,
+                           static_cast<cudaStream_t>(stream)>>>(g);
+        count_launches(1);
+    }
+    CK(cudaGetLastError());
+    return HEFF_OK;
 }
 
-int fx_level(const heff_plan* p, size_t ws_bytes) {
-    if (ws_bytes >= p->ws_bytes) return p->planes_ok ? 2 : 1;
-    return ws_bytes >= p->ws_codes ? 1 : 0;
+bool has_planes(const heff_plan* p, size_t ws_bytes) {
+    return p->opts.precision == HEFF_PREC_FP64 && p->planes_ok && ws_bytes >= p->ws_bytes;
 }
 
 }  // namespace heff
@@ -648,51 +736,51 @@ static int fresh_workspace(heff_plan* p, void* ws, void* stream) {
 }
 
 static int do_prepare(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
-                      void* workspace, int level, void* stream) {
+                      void* workspace, bool planes, void* stream) {
     heff::record_phase(plan, 0, stream);
-    int rc = heff::launch_mix(plan, L, W1, W2, R, workspace, level, stream);
-    if (level == 2)
+    int rc = heff::launch_mix(plan, L, W1, W2, R, workspace, planes, stream);
+    if (planes)
         for (int array : {0, 3})
             if (!rc) rc = heff::launch_digits(plan, array, workspace, 1, stream);
     heff::record_phase(plan, 1, stream);
     return rc;
 }
 
-static int do_gemms(heff_plan* plan, void* const* y, int nbatch, void* workspace, int level, void* stream) {
+static int do_gemms(heff_plan* plan, void* const* y, int nbatch, void* workspace, bool planes, void* stream) {
     int rc;
-    if ((rc = heff::launch_gemm(plan, 1, workspace, y, nbatch, level, stream))) return rc;
+    if ((rc = heff::launch_gemm(plan, 1, workspace, y, nbatch, planes, stream))) return rc;
     heff::record_phase(plan, 3, stream);
-    if ((rc = heff::launch_gemm(plan, 2, workspace, y, nbatch, level, stream))) return rc;
+    if ((rc = heff::launch_gemm(plan, 2, workspace, y, nbatch, planes, stream))) return rc;
     heff::record_phase(plan, 4, stream);
     return HEFF_OK;
 }
 
 static int do_matvec(heff_plan* plan, const void* const* x, void* const* y, int nbatch, void* workspace,
-                     int level, void* stream) {
+                     bool planes, void* stream) {
     int rc;
     if ((rc = fresh_workspace(plan, workspace, stream))) return rc;
-    if ((rc = heff::launch_pack_batch(plan, x, nbatch, workspace, level, stream))) return rc;
-    if (level == 2 && (rc = heff::launch_digits(plan, 1, workspace, nbatch, stream))) return rc;
+    if ((rc = heff::launch_pack_batch(plan, x, nbatch, workspace, planes, stream))) return rc;
+    if (planes && (rc = heff::launch_digits(plan, 1, workspace, nbatch, stream))) return rc;
     heff::record_phase(plan, 2, stream);
-    return do_gemms(plan, y, nbatch, workspace, level, stream);
+    return do_gemms(plan, y, nbatch, workspace, planes, stream);
 }
 
 static int do_apply(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
-                    const void* const* x, void* const* y, int nbatch, void* workspace, int level, void* stream) {
+                    const void* const* x, void* const* y, int nbatch, void* workspace, bool planes, void* stream) {
     plan->ev_prepare = true;
     if (heff::launch_mix_pack(plan, L, W1, W2, R, x, nbatch, workspace, static_cast<cudaStream_t>(stream))) {
         CK(cudaGetLastError());
-        return do_gemms(plan, y, nbatch, workspace, level, stream);
+        return do_gemms(plan, y, nbatch, workspace, planes, stream);
     }
-    int rc = do_prepare(plan, L, W1, W2, R, workspace, level, stream);
-    return rc ? rc : do_matvec(plan, x, y, nbatch, workspace, level, stream);
+    int rc = do_prepare(plan, L, W1, W2, R, workspace, planes, stream);
+    return rc ? rc : do_matvec(plan, x, y, nbatch, workspace, planes, stream);
 }
 
 int heff::apply_in(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, const void* x,
                    void* y, void* ws, size_t bytes, void* stream) {
     const void* xs[1] = {x};
     void* ys[1] = {y};
-    return do_apply(p, L, W1, W2, R, xs, ys, 1, ws, fx_level(p, bytes), stream);
+    return do_apply(p, L, W1, W2, R, xs, ys, 1, ws, has_planes(p, bytes), stream);
 }
 
 extern "C" int heff_prepare(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
@@ -702,7 +790,7 @@ extern "C" int heff_prepare(heff_plan* plan, const void* L, const void* W1, cons
     int rc = check_ws(plan, workspace, workspace_bytes);
     if (rc) return rc;
     plan->ev_prepare = true;
-    return do_prepare(plan, L, W1, W2, R, workspace, heff::fx_level(plan, workspace_bytes), stream);
+    return do_prepare(plan, L, W1, W2, R, workspace, heff::has_planes(plan, workspace_bytes), stream);
 }
 
 extern "C" int heff_apply_prepared(heff_plan* plan, const void* x, void* y, void* workspace,
@@ -717,7 +805,7 @@ extern "C" int heff_apply_prepared(heff_plan* plan, const void* x, void* y, void
     void* ys[1] = {y};
     plan->ev_prepare = false;
     heff::record_phase(plan, 1, stream);
-    return do_matvec(plan, xs, ys, 1, workspace, heff::fx_level(plan, workspace_bytes), stream);
+    return do_matvec(plan, xs, ys, 1, workspace, heff::has_planes(plan, workspace_bytes), stream);
 }
 
 extern "C" int heff_apply(heff_plan* plan, const void* L, const void* W1, const void* W2, const void* R,
@@ -798,7 +886,7 @@ extern "C" int heff_apply_batched(heff_plan* plan, const void* L, const void* W1
     int rc = check_ws(plan, workspace, workspace_bytes);
     if (rc) return rc;
     plan->ev_prepare = true;
-    return do_apply(plan, L, W1, W2, R, x, y, nbatch, workspace, heff::fx_level(plan, workspace_bytes), stream);
+    return do_apply(plan, L, W1, W2, R, x, y, nbatch, workspace, heff::has_planes(plan, workspace_bytes), stream);
 }
 
 // Tile-shape autotuner: time each GEMM with every task list the plan built (N = 256, N = 128,
@@ -835,8 +923,8 @@ extern "C" int heff_plan_autotune(heff_plan* plan, const void* L, const void* W1
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         const void* xs[1] = {x};
         void* ys[1] = {y};
-        if ((rc = heff::launch_mix(plan, L, W1, W2, R, workspace, true, stream))) return rc;
-        if ((rc = heff::launch_pack_batch(plan, xs, 1, workspace, true, stream))) return rc;
+        if ((rc = heff::launch_mix(plan, L, W1, W2, R, workspace, false, stream))) return rc;
+        if ((rc = heff::launch_pack_batch(plan, xs, 1, workspace, false, stream))) return rc;
         // each candidate: one warm-up launch, then the median of 5 separately timed launches
         cudaEvent_t e[6];
         for (auto& ev : e) CK(cudaEventCreate(&ev));
@@ -849,10 +937,10 @@ extern "C" int heff_plan_autotune(heff_plan* plan, const void* L, const void* W1
                 ms[c] = 0.f;
                 if (v[c]->tasks.empty() && !v[0]->tasks.empty()) continue;
                 std::swap(*v[0], *v[c]);
-                rc = heff::launch_gemm(plan, which, workspace, ys, 1, true, stream);
+                rc = heff::launch_gemm(plan, which, workspace, ys, 1, false, stream);
                 CK(cudaEventRecord(e[0], st));
                 for (int r = 0; r < 5 && !rc; ++r) {
-                    rc = heff::launch_gemm(plan, which, workspace, ys, 1, true, stream);
+                    rc = heff::launch_gemm(plan, which, workspace, ys, 1, false, stream);
                     CK(cudaEventRecord(e[r + 1], st));
                 }
                 if (!rc) {

@@ -17,11 +17,11 @@ void BList::add_block(int64_t c_off, int32_t ldc, int32_t m, int32_t n, const st
     blocks.push_back(Block{c_off, ldc, m, n, (int32_t)block_prods.size(), (int32_t)ps.size()});
     block_prods.insert(block_prods.end(), ps.begin(), ps.end());
     const bool fx = tile_n == FX_TILE_N;
-    std::vector<std::pair<int32_t, int32_t>> codes(ps.size());
+    std::vector<std::pair<View, View>> v(ps.size());
     int32_t steps = 0;
     for (size_t i = 0; fx && i < ps.size(); ++i) {
         const BProd& p = ps[i];
-        codes[i] = {view_codes(0, p.a_off, p.a_rs, p.a_cs, m, p.K), view_codes(1, p.b_off, p.b_cs, p.b_rs, n, p.K)};
+        v[i] = {view(0, p.a_off, p.a_rs, p.a_cs, m, p.K), view(1, p.b_off, p.b_cs, p.b_rs, n, p.K)};
         steps += (p.K + 15) / 16;
     }
     for (int r0 = 0; r0 < m; r0 += tile_m)
@@ -34,11 +34,17 @@ void BList::add_block(int64_t c_off, int32_t ldc, int32_t m, int32_t n, const st
             t.prod_begin = (int32_t)prods.size();
             t.prod_count = (int32_t)ps.size();
             t.steps = steps;
+            t.fp64_at = nfp64;
+            if (fx) nfp64 += t.m * ((t.n + 31) / 32);
             for (size_t i = 0; i < ps.size(); ++i) {
                 const BProd& p = ps[i];
                 BProd q = p;
-                q.ea = codes[i].first + r0;
-                q.eb = codes[i].second + c0;
+                q.ea = v[i].first.code + r0;
+                q.eb = v[i].second.code + c0;
+                q.za = v[i].first.word + r0;
+                q.zb = v[i].second.word + c0;
+                q.na = m;
+                q.nb = n;
                 q.a_off += (int64_t)r0 * p.a_rs;
                 q.b_off += (int64_t)c0 * p.b_cs;
                 prods.push_back(q);
@@ -48,12 +54,13 @@ void BList::add_block(int64_t c_off, int32_t ldc, int32_t m, int32_t n, const st
         }
 }
 
-int32_t BList::view_codes(int which, int64_t off, int32_t rs, int32_t ks, int32_t n, int32_t K) {
-    auto ins = views.insert({{which, off, rs, ks, n, K}, ncodes});
+BList::View BList::view(int which, int64_t off, int32_t rs, int32_t ks, int32_t n, int32_t K) {
+    auto ins = views.insert({{which, off, rs, ks, n, K}, {ncodes, nwords}});
     if (ins.second) {
         for (int32_t r = 0; r < n; r += 32)
-            rows.push_back({off + (int64_t)r * rs, rs, ks, n - r < 32 ? n - r : 32, K, ncodes + r, which});
+            rows.push_back({off + (int64_t)r * rs, rs, ks, n - r < 32 ? n - r : 32, K, ncodes + r, which, nwords + r, n});
         ncodes += n;
+        nwords += (K + 31) / 32 * n;
     }
     return ins.first->second;
 }
@@ -67,7 +74,7 @@ void BList::retile(int tm, int tn) {
     prods.clear();
     rows.clear();
     views.clear();
-    ncodes = 0;
+    ncodes = nwords = nfp64 = 0;
     flops = 0;
     tile_m = tm;
     tile_n = tn;
@@ -87,17 +94,19 @@ int blist_upload(BList& b) {
         std::stable_sort(b.tiles.begin(), b.tiles.end(), [](const BTile& x, const BTile& y) {
             return (int64_t)x.steps * (x.n + 32) > (int64_t)y.steps * (y.n + 32);
         });
-    // one allocation for the tables, an error flag (zero) and the codes
+    // one allocation for the tables, an error flag (zero), the codes, words, sums and bits
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t nt = b.tiles.size() * sizeof(BTile), np = b.prods.size() * sizeof(BProd), nr = b.rows.size() * sizeof(FxRows);
     const size_t op = al(nt), orow = op + al(np), oe = orow + al(nr), oc = oe + 256;
+    const size_t ow = oc + al(b.ncodes * sizeof(uint16_t)), os = ow + al(b.nwords * sizeof(uint32_t));
+    const size_t of = os + al(b.ncodes * sizeof(float));
     if (nt + np + nr == 0) return HEFF_OK;
     std::vector<char> host(oc, 0);
     if (nt) std::memcpy(host.data(), b.tiles.data(), nt);
     if (np) std::memcpy(host.data() + op, b.prods.data(), np);
     if (nr) std::memcpy(host.data() + orow, b.rows.data(), nr);
     char* d = nullptr;
-    if (cudaMalloc((void**)&d, oc + b.ncodes * sizeof(uint16_t)) != cudaSuccess ||
+    if (cudaMalloc((void**)&d, of + b.nfp64 * sizeof(uint32_t)) != cudaSuccess ||
         cudaMemcpy(d, host.data(), oc, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaFree(d);
         return fail(HEFF_ERR_CUDA, "block list upload failed");
@@ -108,6 +117,9 @@ int blist_upload(BList& b) {
     b.d_rows = reinterpret_cast<FxRows*>(d + orow);
     b.d_err = reinterpret_cast<int*>(d + oe);
     b.d_codes = reinterpret_cast<uint16_t*>(d + oc);
+    b.d_words = reinterpret_cast<uint32_t*>(d + ow);
+    b.d_sums = reinterpret_cast<float*>(d + os);
+    b.d_fp64 = reinterpret_cast<uint32_t*>(d + of);
     return HEFF_OK;
 }
 
@@ -119,6 +131,9 @@ void blist_free(BList& b) {
     b.d_rows = nullptr;
     b.d_err = nullptr;
     b.d_codes = nullptr;
+    b.d_words = nullptr;
+    b.d_sums = nullptr;
+    b.d_fp64 = nullptr;
 }
 
 namespace {

@@ -228,6 +228,7 @@ size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
     o_lw = off; off = al(off + e * P->rows_lw);
     o_t = off;  off = al(off + e * P->rows_t);
     o_f = off;  off = al(off + 256);
+    const size_t least = off;
     if (p) {
         p->off_xt = o_sp; p->off_lw = o_lw; p->off_t = o_t; p->off_rw = o_t; p->off_flags = o_f;
         p->ws_min = off;
@@ -240,7 +241,6 @@ size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
         heff_plan size_only;
         heff_plan* f = p ? p : &size_only;
         f->off_ex = o_ex; f->off_elw = o_elw; f->off_et = o_et; f->off_erw = o_et;
-        f->ws_codes = off;
         const struct { int64_t rows; bool a; size_t src, codes; } ops[3] = {
             {P->rows_lw, false, o_lw, o_elw}, {P->rows_sp, true, o_sp, o_ex}, {P->rows_t, false, o_t, o_et}};
         for (int o = 0; o < 3; ++o) {
@@ -250,7 +250,12 @@ size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
             f->fxo[o].off_src = ops[o].src;
             f->fxo[o].off_codes = ops[o].codes;
         }
-        off = heff::plane_layout(f, off);
+        // (bits for FP64 outputs: a word per row and 32 columns, GEMM 1's, then GEMM 2's)
+        int64_t words[2] = {0, 0};
+        for (int g = 0; g < 2; ++g)
+            for (const GemmTask& k : g == 0 ? P->blocks1 : P->blocks2)
+                words[g] += (int64_t)k.m * ((k.n + 31) / 32);
+        off = heff::plane_layout(f, off, std::max(words[0], words[1]), least);
     }
     if (p) p->ws_bytes = off;
     return off;
@@ -305,9 +310,10 @@ int ensure_plan(heff_env_plan* P) {
             G.task_flops.assign(G.tasks.size(), 0.0);
             G.task_useful.assign(G.tasks.size(), 0.0);
             heff::lpt_schedule(G, nsm, tc, first);
+            if (!tc) G.count_fp64();
         };
-        cut(P->blocks1, P->segs1, tc ? p->g1 : p->fx1, true);
-        cut(P->blocks2, P->segs2, tc ? p->g2 : p->fx2, false);
+        cut(P->blocks1, P->segs1, p->g1, true);
+        cut(P->blocks2, P->segs2, p->g2, false);
         if ((rc = heff::plan_upload(p.get())) != HEFF_OK) {
             heff::plan_free_device(p.get());
             return rc;
@@ -537,14 +543,14 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
         const void* xs[1] = {site};
         void* ys[1] = {env_new};
         // the mix tiles read env_old as L with W as W1, and (side 1) the site tensor as R
-        const int level = heff::fx_level(p, workspace_bytes);
-        if ((rc = heff::launch_mix(p, env_old, W, W, site, ws, level, stream))) return rc;
-        if ((rc = heff::launch_pack_batch(p, xs, 1, ws, level, stream))) return rc;
-        if (level == 2 && plan->precision == HEFF_PREC_FP64)
+        const bool planes = heff::has_planes(p, workspace_bytes);
+        if ((rc = heff::launch_mix(p, env_old, W, W, site, ws, planes, stream))) return rc;
+        if ((rc = heff::launch_pack_batch(p, xs, 1, ws, planes, stream))) return rc;
+        if (planes)
             for (int array : {1, 0})
                 if ((rc = heff::launch_digits(p, array, ws, 1, stream))) return rc;
-        if ((rc = heff::launch_gemm(p, 1, ws, ys, 1, level, stream))) return rc;
-        return heff::launch_gemm(p, 2, ws, ys, 1, level, stream);
+        if ((rc = heff::launch_gemm(p, 1, ws, ys, 1, planes, stream))) return rc;
+        return heff::launch_gemm(p, 2, ws, ys, 1, planes, stream);
     }
     int* err = reinterpret_cast<int*>(ws);
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), static_cast<cudaStream_t>(stream));

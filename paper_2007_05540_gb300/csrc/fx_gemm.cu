@@ -11,18 +11,19 @@
 // K step land in 8 accumulators (one per g) in tensor memory.  All sums that matter at FP64
 // precision are exact: a digit product is at most 2^14, and a chunk of 256 contraction steps
 // keeps the accumulators g <= 4 below 2^24, where FP32 adds integers exactly; the later ones
-// weigh 2^-40 and less.  After each chunk the accumulators are added into 96-bit integers, and
+// weigh 2^-40 and less (5 and 6 leave FP32's integers only where the digits of a whole chunk are alike and near
+// their largest value).  After each chunk the accumulators are added into 96-bit integers, and
 // the sum is rounded to FP64 once at the end.  What is dropped is the part of an element below
-// 2^-62 of the largest in its row, and the digit products g >= 8: together about
-// 2^-61 K max|a row| max|b column|, against 2^-53 per addition of a running FP64 sum.
+// 2^-62 of its row's scale, and the digit products g >= 8: in all under 9 2^-62 K of the two scales' product, a
+// bound by the largest elements of the row and the column.  Outputs whose terms are so small against the scales that
+// this is more than the error of a running FP64 sum are found and computed in FP64 (fx_check.cuh).
 //
 // Rows that the scale cannot hold (infinities, NaNs, magnitudes beyond 2^+-400) make their tile
 // run in FP64 arithmetic on the CUDA cores inside the same kernel.
 //
-// Two sources of work share the kernel: the block-product lists with arbitrary strides and scalar
-// coefficients (MODE 1: gradients, two-site tensor, the SVD's products), and the matvec's task lists over
-// the workspace operands (MODE 0; K contiguous, one pitch) where the workspace has no room for the digit
-// planes that fx_planes.cu multiplies.
+// The work is lists of block products with arbitrary strides and scalar coefficients: gradients, two-site
+// tensor, the SVD's products.  (The matvec's and the environment update's operands are converted once:
+// fx_planes.cu.)
 //
 // One persistent CTA per SM, 128 x 64 output tiles, 20 warps:
 //   warps 0-7    producers: load 128 + 64 rows x 16 K of FP64, convert to digits, write the FP16
@@ -34,16 +35,16 @@
 //                i .. 7, which lie one after another in tensor memory
 // Registers are moved from the other warps to the drain warps (96 integers a thread).
 //
-// Bound by the 36 digit products: 1.9 PFLOP/s of FP16 / 36 = 53 TFLOP/s, less the ragged tiles and
-// the drain of the accumulators every 256 steps.  Against the FP64 units (64 x 64 tiles on the
-// CUDA cores), whole calls: prepared matvec m = 1024, k = 14, 6.24 -> 0.58 ms (0.40 from planes); gradients
-// m = 320, 9.2 -> 1.23 ms.
+// Bound by the producers' conversions (1.9 us per step of 16 contraction elements, where the tensor pipe needs
+// 0.6).  Against the FP64 units (64 x 64 tiles on the CUDA cores): gradients m = 320, 9.2 -> 1.44 ms a call, 0.14 of
+// it for weak_list_kernel.
 // Every mbarrier wait is bounded; on expiry the CTA raises the error flag, stops issuing work,
 // waits (bounded) for its MMAs in flight, frees its tensor memory and returns.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "fixed.cuh"
+#include "fx_check.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
 
@@ -76,134 +77,141 @@ constexpr int R_ALL = 96, R_PROD = 80, R_DRAIN = 136, R_MMA = 48;
 static_assert(2 * R_PROD + 2 * R_DRAIN + R_MMA <= 5 * R_ALL, "registers of a partition");
 
 struct FxArgs {
-    // MODE 0
-    const GemmTask* tasks;
-    const KSeg* segs;
-    int64_t ld, a_batch_rows, b_batch_rows;
-    const uint16_t *ea, *eb;             // exponent codes [column / 32][row]; null: all tiles in FP64
-    int64_t ea_rows, eb_rows;
-    uint16_t* et;                        // codes of the output T (null for y)
-    int64_t et_rows, c_batch_rows, c_batch_elems;
-    PtrBatch y;                          // outputs (mode y), or y.p[0] unused
-    int nbatch, b0, to_y;
-    double* split;                       // scratch of the split tiles, split_elems per batch entry
-    const SplitTile* split_tiles;
-    int64_t split_elems;
-    // MODE 1
     const BTile* tiles;
     const BProd* prods;
     const uint16_t* e;                   // exponent codes per operand row (BProd.ea, eb)
+    const float* sums;                   // sum of its magnitudes over the code's power of two
+    const uint32_t* words;               // and words of its nonzero elements (BProd.za, zb)
+    uint32_t* fp64;                      // outputs computed in FP64 (BTile.fp64_at)
     const double *coef1, *coef2, *inv_scale;
     double scale;
     int accumulate;
-    // both
     int ntiles;
     const double *A, *B;
     double* C;
     int* err;
 };
 
-struct Tile {
-    int m, n, n_zero, ldc, steps, pbeg, pcnt, bat, split;
-    int64_t c_off, a_row, b_row;
-};
-
-template <int MODE>
-__device__ __forceinline__ Tile get_tile(const FxArgs& g, long item) {
-    Tile t;
-    if constexpr (MODE == 0) {
-        const int b = (int)(item % g.nbatch);
-        const GemmTask k = g.tasks[item / g.nbatch];
-        t.m = k.m; t.n = k.n; t.n_zero = k.n_zero; t.ldc = k.ldc; t.steps = k.ktotal / FKS;
-        t.pbeg = k.seg_begin; t.pcnt = k.seg_count; t.bat = b; t.split = k.split;
-        t.c_off = k.c_off;
-        t.a_row = k.a_row + (g.b0 + b) * g.a_batch_rows;
-        t.b_row = k.b_row + (g.b0 + b) * g.b_batch_rows;
-    } else {
-        const BTile k = g.tiles[item];
-        t.m = k.m; t.n = k.n; t.n_zero = 0; t.ldc = k.ldc; t.steps = k.steps;
-        t.pbeg = k.prod_begin; t.pcnt = k.prod_count; t.bat = 0; t.split = 0;
-        t.c_off = k.c_off; t.a_row = 0; t.b_row = 0;
-    }
-    return t;
-}
-
-// round i of this CTA: block lists run in a snake over the sorted tiles; task lists are laid
-// out for a plain round robin by the planner
-template <int MODE>
+// round i of this CTA: a snake over the sorted tiles
 __device__ __forceinline__ long item_of(long i) {
     const long G = gridDim.x, c = blockIdx.x;
-    return MODE == 0 ? i * G + c : i * G + ((i & 1) ? G - 1 - c : c);
+    return i * G + ((i & 1) ? G - 1 - c : c);
 }
 
 __device__ __forceinline__ double prod_coef(const FxArgs& g, const BProd& p) {
     return (p.c1 < 0 ? 1.0 : g.coef1[p.c1]) * (p.c2 < 0 ? 1.0 : g.coef2[p.c2]);
 }
 
-// One product (a contraction segment) of a tile: element (r, k) of A at a[r ars + k acs], column
-// c's element k of B at b[c bcs + k brs].
-struct Prod {
-    const double *a, *b;
-    int64_t ars, bcs;
-    int acs, brs, K;
-    double coef;
-};
-
-template <int MODE>
-__device__ __forceinline__ Prod get_prod(const FxArgs& g, const Tile& t, int i) {
-    Prod p;
-    if constexpr (MODE == 0) {
-        const KSeg s = g.segs[t.pbeg + i];
-        p.a = g.A + t.a_row * g.ld + s.k0;
-        p.b = g.B + t.b_row * g.ld + s.k0;
-        p.ars = p.bcs = g.ld;
-        p.acs = p.brs = 1;
-        p.K = s.klen;
-        p.coef = 1.0;
-    } else {
-        const BProd q = g.prods[t.pbeg + i];
-        p.a = g.A + q.a_off;
-        p.b = g.B + q.b_off;
-        p.ars = q.a_rs; p.acs = q.a_cs;
-        p.bcs = q.b_cs; p.brs = q.b_rs;
-        p.K = q.K;
-        p.coef = prod_coef(g, q);
-    }
-    return p;
-}
-
 // Scale of row r of A (side 0) or column r of B (side 1) over the tile's products; ok: cleared
 // when the row needs FP64.
-template <int MODE>
-__device__ __forceinline__ int row_scale(const FxArgs& g, const Tile& t, int side, int r, bool& ok) {
+__device__ __forceinline__ int row_scale(const FxArgs& g, const BTile& t, int side, int r, bool& ok) {
     int E = 0;
-    if constexpr (MODE == 0) {
-        const uint16_t* e = side ? g.eb : g.ea;
-        const int64_t rows = side ? g.eb_rows : g.ea_rows;
-        if (!e) { ok = false; return fx::E_ZERO; }
-        e += (side ? t.b_row : t.a_row) + r;
-        for (int s = 0; s < t.pcnt; ++s) {
-            const KSeg sg = g.segs[t.pbeg + s];
-            const int kb0 = sg.k0 / KPAD, nkb = sg.klen / KPAD;
-#pragma unroll 4
-            for (int j = 0; j < nkb; ++j) E = max(E, (int)e[(kb0 + j) * rows]);
+    for (int s = 0; s < t.prod_count; ++s) {
+        const BProd& p = g.prods[t.prod_begin + s];
+        int v = g.e[(side ? p.eb : p.ea) + r];
+        if (side == 0 && (p.c1 >= 0 || p.c2 >= 0)) {
+            const double c = prod_coef(g, p);
+            const int ec = fx::exp_code((uint32_t)__double2hiint(c), (uint32_t)__double2loint(c));
+            if (ec == 0x7ff) ok = false;
+            // |c v| < 2^(ec - 1022) 2^(v - 1022)
+            v = (v == 0 || ec == 0) && v != 0x7ff ? 0 : (v == 0x7ff ? v : max(v + ec - 1022, 1));
         }
-    } else {
-        for (int s = 0; s < t.pcnt; ++s) {
-            const BProd& p = g.prods[t.pbeg + s];
-            int v = g.e[(side ? p.eb : p.ea) + r];
-            if (side == 0 && (p.c1 >= 0 || p.c2 >= 0)) {
-                const double c = prod_coef(g, p);
-                const int ec = fx::exp_code((uint32_t)__double2hiint(c), (uint32_t)__double2loint(c));
-                if (ec == 0x7ff) ok = false;
-                // |c v| < 2^(ec - 1022) 2^(v - 1022)
-                v = (v == 0 || ec == 0) && v != 0x7ff ? 0 : (v == 0x7ff ? v : max(v + ec - 1022, 1));
-            }
-            E = max(E, v);
-        }
+        E = max(E, v);
     }
     if (!fx::exp_plain(E)) ok = false;
     return E ? E : fx::E_ZERO;
+}
+
+// A patch of a tile, as fx_check.cuh reads it: one piece per product.
+struct ListSrc {
+    static constexpr bool DENSE = false;
+    const FxArgs& g;
+    const BTile& t;
+    int r0, c0;                          // the patch's first row and column in the tile
+    bool rowed, coled;                   // whether there is a row, a column `lane`
+    double scale;
+    __device__ __forceinline__ int lane() const { return threadIdx.x & 31; }
+    __device__ __forceinline__ const BProd& prod(int i) const { return g.prods[t.prod_begin + i]; }
+    __device__ __forceinline__ int pieces() const { return t.prod_count; }
+    __device__ __forceinline__ fx::Piece piece(int i, int r) const {
+        const BProd& q = prod(i);
+        return {g.A + q.a_off + (int64_t)(r0 + r) * q.a_rs, g.B + q.b_off + (int64_t)c0 * q.b_cs, q.b_cs, q.a_cs, q.b_rs,
+                q.K, prod_coef(g, q)};
+    }
+    __device__ __forceinline__ int bias(int i) const {
+        const BProd& q = prod(i);
+        if (q.c1 < 0 && q.c2 < 0) return 0;
+        const double c = prod_coef(g, q);
+        const int ec = fx::exp_code((uint32_t)__double2hiint(c), (uint32_t)__double2loint(c));
+        return ec > 1 ? ec - 1023 : fx::NO_TERM;
+    }
+    __device__ __forceinline__ void words(int i, int j, uint32_t& x, uint32_t& y) const {
+        const BProd& q = prod(i);
+        x = rowed ? g.words[q.za + (int64_t)j * q.na + r0 + lane()] : 0u;
+        y = coled ? g.words[q.zb + (int64_t)j * q.nb + c0 + lane()] : 0u;
+    }
+    __device__ __forceinline__ void store(int c, double v) const {
+        double* o = g.C + t.c_off + (int64_t)(r0 + lane()) * t.ldc + c0 + c;
+        *o = g.accumulate ? *o + scale * v : scale * v;
+    }
+};
+
+// The outputs that the digits do not resolve (fx_check.cuh): a block per tile, a warp per patch.
+constexpr int WEAK_WARPS = 4;
+__global__ void __launch_bounds__(32 * WEAK_WARPS) weak_list_kernel(const __grid_constant__ FxArgs g) {
+    const BTile t = g.tiles[blockIdx.x];
+    const int lane = threadIdx.x & 31, wpr = (t.n + 31) / 32, patches = (t.m + 31) / 32 * wpr;
+    const double scale = g.inv_scale ? g.scale / g.inv_scale[0] : g.scale;
+    auto power = [](int e) { return e >= -126 ? __int_as_float((127 + e) << 23) : 0.f; };
+    for (int p = threadIdx.x >> 5; p < patches; p += WEAK_WARPS) {
+        const int row0 = p / wpr * 32, col0 = p % wpr * 32, r = row0 + lane, c = col0 + lane;
+        const int rows = min(t.m - row0, 32), cols = min(t.n - col0, 32);
+        const ListSrc src{g, t, row0, col0, lane < rows, lane < cols, scale};
+        const uint32_t valid = 0xffffffffu >> (32 - cols);
+        bool plain = true;                               // (other tiles run in FP64 as a whole)
+        const int er = src.rowed ? row_scale(g, t, 0, r, plain) : fx::E_ZERO;
+        const int ec = src.coled ? row_scale(g, t, 1, c, plain) : fx::E_ZERO;
+        uint32_t need = 0;
+        if (__all_sync(0xffffffffu, plain) && t.steps > 0) {
+            // nonzero elements and sums of the rows and columns, where counting them is cheap; else the contraction length
+            const int most = max(t.steps * FKS - (FKS - 1) * t.prod_count, 1);
+            int fewest = most;
+            float sr = (float)most, sc = sr;
+            uint32_t mr = most, mc = most;
+            if (t.steps <= 64 && t.prod_count <= 4) {
+                int nr = 0, nc = 0;
+                sr = sc = 0.f;
+                for (int i = 0; i < t.prod_count; ++i) {
+                    const BProd& q = src.prod(i);
+                    for (int j = 0; j < (q.K + 31) / 32; ++j) {
+                        uint32_t x, y;
+                        src.words(i, j, x, y);
+                        nr += __popc(x);
+                        nc += __popc(y);
+                    }
+                    const int bias = src.bias(i);
+                    if (src.rowed && bias != fx::NO_TERM) sr += 2.f * g.sums[q.ea + r] * power(g.e[q.ea + r] + bias - er);
+                    if (src.coled) sc += g.sums[q.eb + c] * power(g.e[q.eb + c] - ec);
+                }
+                mr = __reduce_max_sync(0xffffffffu, nr);
+                mc = __reduce_max_sync(0xffffffffu, nc);
+                fewest = (int)(__reduce_min_sync(0xffffffffu, min((uint32_t)nr - 1u, (uint32_t)nc - 1u)) + 1u);   // (zeros last)
+                sr = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sr)));
+                sc = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sc)));
+            }
+            if (mr <= 2 || mc <= 2) {
+                need = src.rowed ? valid : 0u;
+                if (mr <= 2) fx::sparse_outputs<true, 16>(src, src.rowed, cols);
+                else fx::sparse_outputs<false, 16>(src, src.rowed, cols);
+            } else {
+                need = fx::weak_outputs(src, rows, cols, __ballot_sync(0xffffffffu, src.rowed),
+                                        __ballot_sync(0xffffffffu, src.coled), er, ec, fx::least_sum((float)fewest, sr, sc));
+                need = src.rowed ? need & valid : 0u;
+                if (__any_sync(0xffffffffu, need != 0)) fx::fp64_outputs(src, src.rowed, cols, need, false);
+            }
+        }
+        if (src.rowed) g.fp64[t.fp64_at + r * wpr + col0 / 32] = need;
+    }
 }
 
 // byte offset of the 8-element chunk h of row r in a plane, on the even steps of the ring (the
@@ -214,10 +222,10 @@ __device__ __forceinline__ uint32_t chunk_off(int r, int h) {
 
 // A producer thread's walk over one operand of a tile: its row, and the eight K values of each
 // step that it loads and converts.  SIDE 0: A, SIDE 1: B.
-template <int MODE, int SIDE>
+template <int SIDE>
 struct Walk {
     const double* p;        // this thread's first element of the step
-    int ks;                 // stride along K (MODE 0: 1)
+    int ks;                 // stride along K
     int left;               // elements of the product from there on (beyond them: zeros)
     int i, end;             // product, and the elements of it that the step's first half starts at
     int h;                  // which 8 of the step's 16 elements
@@ -230,46 +238,36 @@ struct Walk {
         E = es[SIDE * FM + r];
     }
     // the first step of product n
-    __device__ __forceinline__ void set(const FxArgs& g, const Tile& t, const int* es, int n) {
+    __device__ __forceinline__ void set(const FxArgs& g, const BTile& t, const int* es, int n) {
         i = n;
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         // K contiguous: 16 rows x 2 halves a warp, in an order that spreads its stores over the
         // banks; rows contiguous: 32 rows, one half
         const int rl = ((lane >> 1) & 1) | ((lane >> 2) & 1) << 2 | ((lane >> 3) & 1) << 1 | ((lane >> 4) & 1) << 3;
-        if constexpr (MODE == 0) {
-            const KSeg s = g.segs[t.pbeg + n];
-            end = s.klen;
+        const BProd& q = g.prods[t.prod_begin + n];
+        end = q.K;
+        ks = SIDE ? q.b_rs : q.a_cs;
+        const int w = SIDE ? warp & 3 : warp;
+        int r;
+        if (ks == 1) {
+            r = w * 16 + rl;
             h = lane & 1;
-            const int r = (SIDE ? warp & 3 : warp) * 16 + rl;
-            p = (SIDE ? g.B : g.A) + ((SIDE ? t.b_row : t.a_row) + r) * g.ld + s.k0 + 8 * h;
-            ks = 1;
-            place(r, SIDE ? t.n : t.m, es);
         } else {
-            const BProd& q = g.prods[t.pbeg + n];
-            end = q.K;
-            ks = SIDE ? q.b_rs : q.a_cs;
-            const int w = SIDE ? warp & 3 : warp;
-            int r;
-            if (ks == 1) {
-                r = w * 16 + rl;
-                h = lane & 1;
-            } else {
-                r = (SIDE ? w & 1 : w & 3) * 32 + lane;
-                h = SIDE ? w >> 1 : w >> 2;
-            }
-            p = (SIDE ? g.B + q.b_off : g.A + q.a_off) + (int64_t)r * (SIDE ? q.b_cs : q.a_rs) + (int64_t)8 * h * ks;
-            if (SIDE == 0) coef = prod_coef(g, q);
-            place(r, SIDE ? t.n : t.m, es);
+            r = (SIDE ? w & 1 : w & 3) * 32 + lane;
+            h = SIDE ? w >> 1 : w >> 2;
         }
+        p = (SIDE ? g.B + q.b_off : g.A + q.a_off) + (int64_t)r * (SIDE ? q.b_cs : q.a_rs) + (int64_t)8 * h * ks;
+        if (SIDE == 0) coef = prod_coef(g, q);
+        place(r, SIDE ? t.n : t.m, es);
         left = off != ~0u ? end - 8 * h : 0;
     }
-    // the next step (pcnt products in all)
-    __device__ __forceinline__ void next(const FxArgs& g, const Tile& t, const int* es) {
+    // the next step
+    __device__ __forceinline__ void next(const FxArgs& g, const BTile& t, const int* es) {
         end -= FKS;
         if (end > 0) {
-            p += MODE == 0 ? (int64_t)FKS : (int64_t)FKS * ks;
+            p += (int64_t)FKS * ks;
             left -= FKS;
-        } else if (i + 1 < t.pcnt) {
+        } else if (i + 1 < t.prod_count) {
             set(g, t, es, i + 1);
         } else {
             left = 0;
@@ -277,7 +275,7 @@ struct Walk {
     }
     __device__ __forceinline__ void load(double (&v)[8]) const {
         if (left >= 8) {
-            if (MODE == 0 || (ks == 1 && (reinterpret_cast<uintptr_t>(p) & 15) == 0)) {
+            if (ks == 1 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
                 const double2* q = reinterpret_cast<const double2*>(p);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -368,26 +366,6 @@ __device__ __forceinline__ void issue_step(int n16, uint32_t tmem, uint64_t a, u
     else issue_planes<16, NK>(tmem, a, b, fresh);
 }
 
-// Where a tile's values go: the output, or a split tile's part of its scratch.
-template <int MODE>
-__device__ __forceinline__ int64_t out_pitch(const Tile& t) { return MODE == 0 && t.split ? t.n : t.ldc; }
-template <int MODE>
-__device__ __forceinline__ double* out_ptr(const FxArgs& g, const Tile& t) {
-    if (MODE == 0 && t.split)
-        return g.split + (int64_t)t.bat * g.split_elems + g.split_tiles[t.split >> 9].off +
-               (int64_t)((t.split >> 5) & 15) * t.m * t.n;
-    if constexpr (MODE == 0)
-        return (g.to_y ? static_cast<double*>(const_cast<void*>(g.y.p[t.bat]))
-                       : g.C + (int64_t)(g.b0 + t.bat) * g.c_batch_elems) + t.c_off;
-    return g.C + t.c_off;
-}
-
-// exponent codes of T: the 32-column block of column c (of the tile) in row r (of the tile)
-__device__ __forceinline__ uint16_t* code_ptr(const FxArgs& g, const Tile& t, int r, int c) {
-    const int64_t row = t.c_off / t.ldc + r + (int64_t)(g.b0 + t.bat) * g.c_batch_rows;
-    return g.et + ((t.c_off % t.ldc + c) / KPAD) * g.et_rows + row;
-}
-
 // Producer warps meet (bounded, so that a CTA that gives up does not hang here).
 struct PSync {
     uint64_t* bar;
@@ -403,70 +381,58 @@ struct PSync {
 
 // A tile in FP64 arithmetic on the producer warps (256 threads, 4 x 4 outputs each, two halves
 // of 64 rows).
-template <int MODE>
-__device__ __forceinline__ bool fp64_tile(const FxArgs& g, const Tile& t, double* sh, PSync& psync, double scale) {
+__device__ __forceinline__ bool fp64_tile(const FxArgs& g, const BTile& t, double* sh, PSync& psync, double scale) {
     double (*As)[65] = reinterpret_cast<double (*)[65]>(sh);
     double (*Bs)[65] = As + 8;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    double* C = out_ptr<MODE>(g, t);
-    const int64_t ldc = out_pitch<MODE>(t);
+    double* C = g.C + t.c_off;
     for (int half = 0; half < t.m; half += 64) {
         const int m = t.m - half < 64 ? t.m - half : 64;
         double acc[4][4] = {};
-        for (int s = 0; s < t.pcnt; ++s) {
-            const Prod p = get_prod<MODE>(g, t, s);
+        for (int s = 0; s < t.prod_count; ++s) {
+            const BProd& p = g.prods[t.prod_begin + s];
+            const double* a = g.A + p.a_off;
+            const double* b = g.B + p.b_off;
+            const double coef = prod_coef(g, p);
             for (int k0 = 0; k0 < p.K; k0 += 8) {
                 for (int l = 0; l < 2; ++l) {
                     const int idx = tid + 256 * l;
                     int r, k;
-                    if (p.acs == 1) { r = idx >> 3; k = idx & 7; } else { r = idx & 63; k = idx >> 6; }
+                    if (p.a_cs == 1) { r = idx >> 3; k = idx & 7; } else { r = idx & 63; k = idx >> 6; }
                     As[k][r] = r < m && k0 + k < p.K
-                                   ? p.coef * p.a[(int64_t)(half + r) * p.ars + (int64_t)(k0 + k) * p.acs] : 0.0;
-                    if (p.brs == 1) { r = idx >> 3; k = idx & 7; } else { r = idx & 63; k = idx >> 6; }
+                                   ? coef * a[(int64_t)(half + r) * p.a_rs + (int64_t)(k0 + k) * p.a_cs] : 0.0;
+                    if (p.b_rs == 1) { r = idx >> 3; k = idx & 7; } else { r = idx & 63; k = idx >> 6; }
                     Bs[k][r] = r < t.n && k0 + k < p.K
-                                   ? p.b[(int64_t)r * p.bcs + (int64_t)(k0 + k) * p.brs] : 0.0;
+                                   ? b[(int64_t)r * p.b_cs + (int64_t)(k0 + k) * p.b_rs] : 0.0;
                 }
                 if (!psync()) return false;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    double a[4], b[4];
+                    double av[4], bv[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) { a[i] = As[k][ty * 4 + i]; b[i] = Bs[k][tx * 4 + i]; }
+                    for (int i = 0; i < 4; ++i) { av[i] = As[k][ty * 4 + i]; bv[i] = Bs[k][tx * 4 + i]; }
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                        for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
                 }
                 if (!psync()) return false;
             }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = ty * 4 + i;
-            int code = 0;
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int c = tx * 4 + j;
-                const double v = c < t.n ? acc[i][j] : 0.0;
-                if (r < m && c < t.n + t.n_zero) {
-                    double* cp = C + (int64_t)(half + r) * ldc + c;
-                    if (MODE == 0) *cp = v;
-                    else *cp = g.accumulate ? *cp + scale * v : scale * v;
+                const int r = ty * 4 + i, c = tx * 4 + j;
+                if (r < m && c < t.n) {
+                    double* cp = C + (int64_t)(half + r) * t.ldc + c;
+                    *cp = g.accumulate ? *cp + scale * acc[i][j] : scale * acc[i][j];
                 }
-                code = max(code, fx::exp_code((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v)));
             }
-            if (MODE == 0 && !g.to_y && g.et) {
-                // eight lanes hold one row's 32 columns
-                for (int o = 1; o < 8; o <<= 1) code = max(code, __shfl_xor_sync(0xffffffffu, code, o));
-                if ((tx & 7) == 0 && r < m && tx * 4 < t.n + t.n_zero)
-                    *code_ptr(g, t, half + r, tx * 4) = (uint16_t)code;
-            }
-        }
     }
     return true;
 }
 
-template <int MODE>
 __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_constant__ FxArgs g) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -502,20 +468,20 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
     const uint32_t base = su32(smem);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long total = (long)g.ntiles * (MODE == 0 ? g.nbatch : 1);
+    const long total = g.ntiles;
     const long rounds = (total + gridDim.x - 1) / gridDim.x;
 
     if (warp < PW) {
         // ------------------------------------------------ producers
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_PROD));
         PSync psync{pbar, 0, abort_flag, g.err};
-        const double scale = MODE == 1 ? (g.inv_scale ? g.scale / g.inv_scale[0] : g.scale) : 1.0;
+        const double scale = g.inv_scale ? g.scale / g.inv_scale[0] : g.scale;
         uint32_t step = 0, tcount = 0;
         bool ok = true;
         for (long i = 0; i < rounds && ok; ++i) {
-            const long item = item_of<MODE>(i);
+            const long item = item_of(i);
             if (item >= total) continue;
-            const Tile t = get_tile<MODE>(g, item);
+            const BTile t = g.tiles[item];
             if (t.m == 0) continue;
             const int b = tcount & 1;
             if (!(ok = mbar_wait(&edone[b], ((tcount >> 1) & 1) ^ 1, abort_flag, g.err))) break;
@@ -526,7 +492,7 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                 const int side = threadIdx.x >= FM, r = side ? threadIdx.x - FM : threadIdx.x;
                 bool plain = true;
                 if (threadIdx.x < FM + FN)
-                    es[threadIdx.x] = r < (side ? t.n : t.m) ? row_scale<MODE>(g, t, side, r, plain) : fx::E_ZERO;
+                    es[threadIdx.x] = r < (side ? t.n : t.m) ? row_scale(g, t, side, r, plain) : fx::E_ZERO;
                 const bool bad = __any_sync(0xffffffffu, !plain);
                 if (lane == 0) ebad[b * PW + warp] = bad;
             }
@@ -536,7 +502,7 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
 #pragma unroll
             for (int w = 0; w < PW; ++w) bad |= ebad[b * PW + w] != 0;
             if (bad) {
-                ok = fp64_tile<MODE>(g, t, reinterpret_cast<double*>(smem + OFF_DF), psync, scale);
+                ok = fp64_tile(g, t, reinterpret_cast<double*>(smem + OFF_DF), psync, scale);
                 continue;
             }
             if (t.steps == 0) continue;
@@ -544,8 +510,8 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
             // warp w converts 16 (or half of 32) rows of A on every step; B has half as many rows:
             // warps 0-3 convert it on even steps, warps 4-7 on odd steps.  The loads of the next
             // item are issued before an item is converted.
-            Walk<MODE, 0> wa;
-            Walk<MODE, 1> wb;
+            Walk<0> wa;
+            Walk<1> wb;
             double va[8], vb[8];
             wa.set(g, t, es, 0);
             wa.load(va);
@@ -559,12 +525,10 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                 for (int e = 0; e < 8; ++e) cur[e] = va[e];
                 const int E = wa.E;
                 const uint32_t off = wa.off, odd = 32 * (st & 1);
-                if (MODE == 1) {
-                    const double coef = wa.coef;
-                    if (coef != 1.0) {
+                const double coef = wa.coef;
+                if (coef != 1.0) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) cur[e] *= coef;
-                    }
+                    for (int e = 0; e < 8; ++e) cur[e] *= coef;
                 }
                 wa.next(g, t, es);
                 wa.load(va);
@@ -585,15 +549,15 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
     } else if (warp < PW + EW) {
         // ------------------------------------------------ drain
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_DRAIN));
-        const double scale = MODE == 1 ? (g.inv_scale ? g.scale / g.inv_scale[0] : g.scale) : 1.0;
+        const double scale = g.inv_scale ? g.scale / g.inv_scale[0] : g.scale;
         const int q = warp & 3, h = (warp - PW) >> 2;       // tensor-memory lanes, column half
         double* tr = reinterpret_cast<double*>(smem + OFF_TR + (warp - PW) * TR_WARP);
         uint32_t ccount = 0, tcount = 0;
         bool ok = true;
         for (long i = 0; i < rounds && ok; ++i) {
-            const long item = item_of<MODE>(i);
+            const long item = item_of(i);
             if (item >= total) continue;
-            const Tile t = get_tile<MODE>(g, item);
+            const BTile t = g.tiles[item];
             if (t.m == 0) continue;
             const int b = tcount & 1;
             if (!(ok = mbar_wait(&tready[b], (tcount >> 1) & 1, abort_flag, g.err))) break;
@@ -603,6 +567,13 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
             for (int w = 0; w < PW; ++w) bad |= ebad[b * PW + w] != 0;
             if (!bad) {
                 const int n16 = (t.n + 15) & ~15;
+                const int* es = escale + b * (FM + FN);
+                const int rows = t.m - q * 32 < 32 ? t.m - q * 32 : 32, ncol = t.n - 32 * h < 32 ? t.n - 32 * h : 32;
+                // outputs that are there already (weak_list_kernel); `whole`: all of the patch
+                const bool rowed = lane < rows && ncol > 0;
+                const uint32_t valid = ncol > 0 ? 0xffffffffu >> (32 - ncol) : 0u;
+                const uint32_t need = rowed ? g.fp64[t.fp64_at + (q * 32 + lane) * ((t.n + 31) / 32) + h] : 0u;
+                const bool whole = __all_sync(0xffffffffu, !rowed || need == valid);
                 uint32_t w0[32], w1[32], w2[32];
 #pragma unroll
                 for (int c = 0; c < 32; ++c) { w0[c] = 0; w1[c] = 0; w2[c] = 0; }
@@ -613,7 +584,7 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                     const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + 32 * h;
 #pragma unroll
                     for (int c = 0; c < 32; c += 2) {
-                        if (32 * h + c < n16) {
+                        if (32 * h + c < n16 && !whole) {
                             uint32_t d[FD][2];
 #pragma unroll
                             for (int e = 0; e < FD; ++e) tmem_ld2(ta + e * n16 + c, d[e][0], d[e][1]);
@@ -640,41 +611,34 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
                 }
                 if (!ok) break;
                 // round to FP64 and store, 8 columns at a time
-                const int* es = escale + b * (FM + FN);
                 const int er = es[q * 32 + lane] - 2112;
-                const int rows = t.m - q * 32 < 32 ? t.m - q * 32 : 32;
-                const int64_t ldc = out_pitch<MODE>(t);
-                double* C = out_ptr<MODE>(g, t) + (int64_t)(q * 32) * ldc;
-                const int ncols = t.n + t.n_zero;
-                int code = 0;
+                double* C = g.C + t.c_off + (int64_t)(q * 32) * t.ldc;
 #pragma unroll
                 for (int c0 = 0; c0 < 32; c0 += 8) {
                     const int col0 = 32 * h + c0;
-                    if (col0 < ncols && rows > 0) {
+                    if (col0 < t.n && rows > 0) {
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
                             double v = 0.0;
-                            if (col0 + c < t.n) {
+                            if ((need >> (c0 + c)) & 1u) {
+                                if (!g.accumulate) v = C[(int64_t)lane * t.ldc + col0 + c];
+                            } else if (col0 + c < t.n) {
                                 v = fx::from_fixed(w2[c0 + c], w1[c0 + c], w0[c0 + c], er + es[FM + col0 + c]);
-                                if (MODE == 1 && scale != 1.0) v *= scale;
+                                if (scale != 1.0) v *= scale;
                             }
-                            if (MODE == 0)
-                                code = max(code, fx::exp_code((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v)));
                             tr[lane * 9 + c] = v;
                         }
                         __syncwarp();
                         const int c = lane & 7;
                         for (int r = lane >> 3; r < rows; r += 4)
-                            if (col0 + c < ncols) {
-                                double* cp = C + (int64_t)r * ldc + col0 + c;
+                            if (col0 + c < t.n) {
+                                double* cp = C + (int64_t)r * t.ldc + col0 + c;
                                 const double v = tr[r * 9 + c];
-                                *cp = MODE == 1 && g.accumulate ? *cp + v : v;
+                                *cp = g.accumulate ? *cp + v : v;
                             }
                         __syncwarp();
                     }
                 }
-                if (MODE == 0 && !g.to_y && lane < rows && 32 * h < ncols)
-                    *code_ptr(g, t, q * 32 + lane, 32 * h) = (uint16_t)code;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&edone[b]);
@@ -686,9 +650,9 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
             uint32_t step = 0, ccount = 0, tcount = 0;
             bool ok = true;
             for (long i = 0; i < rounds && ok; ++i) {
-                const long item = item_of<MODE>(i);
+                const long item = item_of(i);
                 if (item >= total) continue;
-                const Tile t = get_tile<MODE>(g, item);
+                const BTile t = g.tiles[item];
                 if (t.m == 0) continue;
                 const int b = tcount & 1;
                 if (!(ok = mbar_wait(&tready[b], (tcount >> 1) & 1, abort_flag, g.err))) break;
@@ -739,65 +703,103 @@ __global__ void __launch_bounds__(FTHREADS, 1) fx_gemm_kernel(const __grid_const
 }
 
 // Exponent codes of operand rows: unit u covers up to 32 rows of one operand view, element
-// (r, k) at off + r rs + k ks; out[r] = the largest code of row r.
+// (r, k) at off + r rs + k ks; out[r] = the largest code E of row r, sums[r] = the sum of its magnitudes over
+// 2^(E - 1022).  And which of its elements are not zero, 32 to a word.
 __global__ void __launch_bounds__(256) row_code_kernel(const FxRows* __restrict__ units, const double* __restrict__ A,
-                                                       const double* __restrict__ B, uint16_t* __restrict__ out) {
+                                                       const double* __restrict__ B, uint16_t* __restrict__ out,
+                                                       uint32_t* __restrict__ words, float* __restrict__ sums) {
     __shared__ int part[8][32];
+    __shared__ float fpart[8][32];
     const FxRows u = units[blockIdx.x];
     const double* src = (u.which ? B : A) + u.off;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a running sum for the largest code so far
+    auto add = [](int& e, float& f, int e2, float f2) {
+        const int d = e2 - e, s = d > 0 ? d : -d;
+        const float down = s < 126 ? __int_as_float((127 - s) << 23) : 0.f;
+        f = d > 0 ? fmaf(f, down, f2) : fmaf(f2, down, f);
+        e = max(e, e2);
+    };
+    // (the mantissa's upper bits over the code's power of two; subnormals count as the largest)
+    auto part_of = [](double v, int c) {
+        return c ? (c == 1 ? 1.f : __int_as_float(0x3f000000 | ((__double2hiint(v) & 0xfffff) << 3))) : 0.f;
+    };
     auto code = [](double v) { return fx::exp_code((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v)); };
     if (u.ks == 1) {
         // lanes along K; each warp four rows, loads of the four in flight together
         int e[4] = {0, 0, 0, 0};
-        for (int k = lane; k < u.K; k += 32)
+        float f[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int k = lane; k - lane < u.K; k += 32) {
+            double v[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int r = warp + 8 * j;
-                if (r < u.rows) e[j] = max(e[j], code(src[(int64_t)r * u.rs + k]));
+                v[j] = r < u.rows && k < u.K ? src[(int64_t)r * u.rs + k] : 0.0;
             }
 #pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int r = warp + 8 * j, c = code(v[j]);
+                add(e[j], f[j], c, part_of(v[j], c));
+                const uint32_t bits = __ballot_sync(0xffffffffu, c != 0);
+                if (lane == 0 && r < u.rows) words[u.word + (int64_t)(k / 32) * u.all + r] = bits;
+            }
+        }
+#pragma unroll
         for (int j = 0; j < 4; ++j) {
-            for (int o = 16; o > 0; o >>= 1) e[j] = max(e[j], __shfl_xor_sync(0xffffffffu, e[j], o));
-            if (lane == 0 && warp + 8 * j < u.rows) out[u.out + warp + 8 * j] = (uint16_t)e[j];
+            for (int o = 16; o > 0; o >>= 1)
+                add(e[j], f[j], __shfl_xor_sync(0xffffffffu, e[j], o), __shfl_xor_sync(0xffffffffu, f[j], o));
+            if (lane == 0 && warp + 8 * j < u.rows) {
+                out[u.out + warp + 8 * j] = (uint16_t)e[j];
+                sums[u.out + warp + 8 * j] = f[j] * 1.001f;
+            }
         }
     } else {
         // lanes along the rows, warps along K
         int e = 0;
+        float f = 0.f;
         if (lane < u.rows) {
-#pragma unroll 4
-            for (int k = warp; k < u.K; k += 8) e = max(e, code(src[(int64_t)lane * u.rs + (int64_t)k * u.ks]));
+            for (int b = warp; 32 * b < u.K; b += 8) {
+                uint32_t bits = 0;
+#pragma unroll 8
+                for (int k = 0; k < 32; ++k) {
+                    const double v = 32 * b + k < u.K ? src[(int64_t)lane * u.rs + (int64_t)(32 * b + k) * u.ks] : 0.0;
+                    const int c = code(v);
+                    add(e, f, c, part_of(v, c));
+                    bits |= (c ? 1u : 0u) << k;
+                }
+                words[u.word + (int64_t)b * u.all + lane] = bits;
+            }
         }
         part[warp][lane] = e;
+        fpart[warp][lane] = f;
         __syncthreads();
         if (warp == 0 && lane < u.rows) {
 #pragma unroll
-            for (int w = 1; w < 8; ++w) e = max(e, part[w][lane]);
+            for (int w = 1; w < 8; ++w) add(e, f, part[w][lane], fpart[w][lane]);
             out[u.out + lane] = (uint16_t)e;
+            sums[u.out + lane] = f * 1.001f;
         }
     }
 }
 
-template <int MODE>
 int launch_fx(const FxArgs& g, int num_sms, cudaStream_t st) {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(fx_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
+        cudaError_t e = cudaFuncSetAttribute(fx_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
         if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
         attr = true;
     }
-    const long total = (long)g.ntiles * (MODE == 0 ? g.nbatch : 1);
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)(total < num_sms ? total : num_sms));
+    cfg.gridDim = dim3((unsigned)(g.ntiles < num_sms ? g.ntiles : num_sms));
     cfg.blockDim = dim3(FTHREADS);
     cfg.dynamicSmemBytes = FSMEM;
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = HEFF_PDL ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, fx_gemm_kernel<MODE>, g);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fx_gemm_kernel, g);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "fx_gemm launch: %s", cudaGetErrorString(e));
     count_launches(1);
@@ -806,76 +808,6 @@ int launch_fx(const FxArgs& g, int num_sms, cudaStream_t st) {
 
 }  // namespace
 
-int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream) {
-    const GemmList& gl = which == 1 ? p->fx1 : p->fx2;
-    if (gl.tasks.empty()) return HEFF_OK;
-    char* w = static_cast<char*>(ws);
-    for (int b0 = 0; b0 < nbatch; b0 += MAXB) {
-        FxArgs g{};
-        g.tasks = gl.d_tasks;
-        g.segs = gl.d_segs;
-        g.ntiles = (int)gl.tasks.size();
-        g.nbatch = nbatch - b0 < MAXB ? nbatch - b0 : MAXB;
-        g.b0 = b0;
-        g.err = reinterpret_cast<int*>(w + p->off_flags);
-        uint16_t* e_t = reinterpret_cast<uint16_t*>(w + p->off_et);
-        const int64_t t_rows = p->opts.max_batch * p->rows_t;
-        if (p->env) {
-            // A: XT in both; B: LW into T, then T into y
-            g.A = reinterpret_cast<const double*>(w + p->off_xt);
-            g.B = reinterpret_cast<const double*>(w + (which == 1 ? p->off_lw : p->off_t));
-            g.ld = p->ld_x;
-            g.C = reinterpret_cast<double*>(w + p->off_t);
-            g.y.p[0] = y[b0];
-            g.to_y = which == 2;
-            g.ea = reinterpret_cast<const uint16_t*>(w + p->off_ex);
-            g.ea_rows = p->rows_x;
-            g.eb = which == 1 ? reinterpret_cast<const uint16_t*>(w + p->off_elw) : e_t;
-            g.eb_rows = which == 1 ? p->rows_lw : t_rows;
-            g.et = which == 1 ? e_t : nullptr;
-            g.et_rows = t_rows;
-        } else if (which == 1) {
-            g.A = reinterpret_cast<const double*>(w + p->off_lw);
-            g.B = reinterpret_cast<const double*>(w + p->off_xt);
-            g.ld = p->ld_x;
-            g.b_batch_rows = p->rows_x;
-            g.C = reinterpret_cast<double*>(w + p->off_t);
-            g.c_batch_elems = p->rows_t * p->ld_t;
-            g.c_batch_rows = p->rows_t;
-            if (codes) {
-                g.ea = reinterpret_cast<const uint16_t*>(w + p->off_elw);
-                g.ea_rows = p->rows_lw;
-                g.eb = reinterpret_cast<const uint16_t*>(w + p->off_ex);
-                g.eb_rows = p->opts.max_batch * p->rows_x;
-                g.et = e_t;
-                g.et_rows = t_rows;
-            }
-        } else {
-            g.A = reinterpret_cast<const double*>(w + p->off_t);
-            g.B = reinterpret_cast<const double*>(w + p->off_rw);
-            g.ld = p->ld_t;
-            g.a_batch_rows = p->rows_t;
-            for (int b = 0; b < g.nbatch; ++b) g.y.p[b] = y[b0 + b];
-            g.to_y = 1;
-            if (p->kchunk) {
-                g.split = reinterpret_cast<double*>(w + p->off_split);
-                g.split_tiles = gl.d_split;
-                g.split_elems = gl.split_elems;
-            }
-            if (codes) {
-                g.ea = e_t;
-                g.ea_rows = t_rows;
-                g.eb = reinterpret_cast<const uint16_t*>(w + p->off_erw);
-                g.eb_rows = p->rows_rw;
-            }
-        }
-        int rc = launch_fx<0>(g, p->num_sms > 0 ? p->num_sms : 148, static_cast<cudaStream_t>(stream));
-        if (!rc && which == 2 && p->kchunk) rc = launch_sum_parts(p, gl, ws, y + b0, g.nbatch, stream);
-        if (rc) return rc;
-    }
-    return HEFF_OK;
-}
-
 int launch_bgemm(const BList& b, const double* A, const double* B, double* C, const double* coef1,
                  const double* coef2, double scale, void* stream, int* err, const double* inv_scale) {
     if (b.tiles.empty()) return HEFF_OK;
@@ -883,13 +815,16 @@ int launch_bgemm(const BList& b, const double* A, const double* B, double* C, co
         return fail(HEFF_ERR_INVALID_ARG, "FP64 block products need %d x %d tiles", FM, FN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!b.rows.empty()) {
-        row_code_kernel<<<(unsigned)b.rows.size(), 256, 0, st>>>(b.d_rows, A, B, b.d_codes);
+        row_code_kernel<<<(unsigned)b.rows.size(), 256, 0, st>>>(b.d_rows, A, B, b.d_codes, b.d_words, b.d_sums);
         count_launches(1);
     }
     FxArgs g{};
     g.tiles = b.d_tiles;
     g.prods = b.d_prods;
     g.e = b.d_codes;
+    g.words = b.d_words;
+    g.sums = b.d_sums;
+    g.fp64 = b.d_fp64;
     g.coef1 = coef1;
     g.coef2 = coef2;
     g.inv_scale = inv_scale;
@@ -900,7 +835,9 @@ int launch_bgemm(const BList& b, const double* A, const double* B, double* C, co
     g.B = B;
     g.C = C;
     g.err = err;
-    return launch_fx<1>(g, b.num_sms > 0 ? b.num_sms : 148, st);
+    weak_list_kernel<<<(unsigned)b.tiles.size(), 32 * WEAK_WARPS, 0, st>>>(g);
+    count_launches(1);
+    return launch_fx(g, b.num_sms > 0 ? b.num_sms : 148, st);
 }
 
 }  // namespace heff

@@ -9,13 +9,14 @@
 //                    written per element: bound by HBM or L2)
 //   fx_plane_kernel  multiplies planes: a persistent CTA per SM, 128 x 64 tiles, one thread issuing TMA
 //                    loads, one issuing MMAs, eight drain warps
-// Prepared matvec, m = 1024, k = 14: 577 us from fx_gemm.cu, 400 us here (GEMM 1 163, GEMM 2 124, planes of T
-// 45, of x 7); environment update m = 1024 309 -> 253 us.  Bound by the drain (74 us of GEMM 1's 163 go when it is
+//   weak_plane_kernel  finds the outputs that digits do not resolve and computes them in FP64 (fx_check.cuh)
+// Prepared matvec, m = 1024, k = 14: 577 us with the conversion in every tile, 400 us here (GEMM 1 163, GEMM 2 124,
+// planes of T 45, of x 7) and 464 with the check; environment update m = 1024 309, 253 and 314 us.  Bound by the drain (74 us of GEMM 1's 163 go when it is
 // left out) and the loads' latency on contractions of two to ten K blocks; the MMAs are 45 us of it.  128 x 32
 // tiles with two accumulator sets drain under the next tile's MMAs, but read A twice as often: 151 and
 // 160 us.
-// The planes take 16 bytes per operand element, so plans whose workspace would pass FX_PLANES_MAX and
-// calls on a smaller workspace (heff_apply_noalloc) use fx_gemm.cu.
+// The planes take 16 bytes per operand element: plans whose workspace would pass FX_PLANES_MAX and calls on a
+// smaller workspace (heff_apply_noalloc) run on the FP64 units (apply.cu).
 //
 // Plane layout.  A virtual row is one row's K block of 32 elements, numbered kb R + row (R rows in the
 // array): the rows of a K block lie one after another, so a TMA box is one contiguous piece.
@@ -32,6 +33,7 @@
 #include <cstring>
 
 #include "fixed.cuh"
+#include "fx_check.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
 
@@ -74,6 +76,8 @@ struct DigitArgs {
     int code_cols;
     char* planes;
     int32_t* scale;          // per row
+    uint32_t* nonzero;       // per virtual row: which elements are not zero
+    uint2* total;            // per row: its elements' sum over the scale (a float, rounded up), nonzero elements
     int64_t rows;            // rows of the array (all batch entries): stride of codes and virtual rows
     int64_t batch_rows;
     int a_side;              // plane layout: A (pairs) or B
@@ -83,6 +87,7 @@ struct DigitArgs {
 // rows' exponent codes, then a warp per K block converts 8 rows x 32 elements.
 __global__ void __launch_bounds__(256) digit_kernel(DigitArgs g) {
     __shared__ int es[8];
+    __shared__ unsigned int sum[8], count[8];            // (integers: the same whatever the order of the warps)
     const FxUnit u = g.units[blockIdx.x];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row0 = u.row0 + (int64_t)blockIdx.y * g.batch_rows;
@@ -101,6 +106,7 @@ __global__ void __launch_bounds__(256) digit_kernel(DigitArgs g) {
         if (lane == 0) {
             const int E = fx::exp_plain(e) ? (e ? e : fx::E_ZERO) : E_BAD;
             es[warp] = E < 0 ? fx::E_ZERO : E;           // a bad row's digits are not used
+            sum[warp] = count[warp] = 0;
             if (warp < u.nrows) g.scale[row0 + warp] = E;
         }
     }
@@ -126,6 +132,25 @@ __global__ void __launch_bounds__(256) digit_kernel(DigitArgs g) {
             for (int e = 0; e < 8; ++e)
                 q[e] = fx::to_fixed((uint32_t)__double2hiint(v[e]), (uint32_t)__double2loint(v[e]), E);
             const int64_t vr = (int64_t)k * g.rows + row0 + r;
+            // eight elements a lane, four lanes a row
+            uint32_t nz = 0;
+            float f = 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                f += __uint_as_float(fx::magnitude(v[e], fx::magnitude_base(E)));
+                nz |= (code_of(v[e]) ? 1u : 0u) << (8 * c + e);
+            }
+            const unsigned lanes = 0xffffffffu >> (32 - 4 * u.nrows);
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                nz |= __shfl_xor_sync(lanes, nz, o);
+                f += __shfl_xor_sync(lanes, f, o);
+            }
+            if (c == 0) {
+                g.nonzero[vr] = nz;
+                atomicAdd(&sum[r], (unsigned int)(f * 16384.f) + 2u);
+                atomicAdd(&count[r], (unsigned int)__popc(nz));
+            }
             const __half2 bias = __half2half2(__ushort_as_half((unsigned short)0x6480));
 #pragma unroll
             for (int d = 0; d < FD; ++d) {
@@ -148,6 +173,9 @@ __global__ void __launch_bounds__(256) digit_kernel(DigitArgs g) {
             }
         }
     }
+    __syncthreads();
+    if ((int)threadIdx.x < u.nrows)
+        g.total[row0 + threadIdx.x] = make_uint2(__float_as_uint((float)sum[threadIdx.x] * (1.f / 16384)), count[threadIdx.x]);
 }
 
 // ------------------------------------------------------------------ plane products
@@ -160,7 +188,12 @@ struct PlaneArgs {
     int64_t ld, a_rows, b_rows;          // operand pitch; rows of the arrays
     int64_t a_batch_rows, b_batch_rows;
     const int32_t *ea, *eb;              // row scales
-    const double *A, *B;                 // FP64 operands (rows that need FP64 arithmetic)
+    const uint32_t *za, *zb;             // nonzero elements of the virtual rows, and totals of the rows
+    const uint2 *ta, *tb;
+    uint32_t* fp64;                      // outputs computed in FP64: a bit each, [batch entry][fp64_at[task] + row * words + word]
+    const int32_t* fp64_at;
+    int64_t fp64_words;                  // of a batch entry
+    const double *A, *B;                 // FP64 operands (outputs that need FP64 arithmetic)
     double* C;
     int64_t c_batch_elems, c_batch_rows;
     uint16_t* et;                        // exponent codes of T, per CODE_COLS columns
@@ -238,6 +271,105 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&d)[FD][4]) {
     }
 }
 
+// A patch of a tile, as fx_check.cuh reads it: one piece per segment.
+struct PlaneSrc {
+    static constexpr bool DENSE = true;
+    const KSeg* segs;
+    int nseg;
+    bool rowed, coled;                   // whether there is a row, a column `lane`
+    const double *a, *b;                 // the patch's first row and column
+    int64_t ld;
+    const uint32_t *za, *zb;             // of row `lane`, of column `lane`
+    int64_t a_rows, b_rows;
+    double* out;                         // row `lane` of the output
+    __device__ __forceinline__ int pieces() const { return nseg; }
+    __device__ __forceinline__ fx::Piece piece(int i, int r) const {
+        const KSeg s = segs[i];
+        return {a + r * ld + s.k0, b + s.k0, ld, 1, 1, s.klen, 1.0};
+    }
+    __device__ __forceinline__ int bias(int) const { return 0; }
+    __device__ __forceinline__ void words(int i, int j, uint32_t& x, uint32_t& y) const {
+        const int64_t kb = segs[i].k0 / KPAD + j;
+        x = rowed ? za[kb * a_rows] : 0u;
+        y = coled ? zb[kb * b_rows] : 0u;
+    }
+    __device__ __forceinline__ void store(int c, double v) const { out[c] = v; }
+};
+
+// where a task's values go: T, y, or a split tile's part of its scratch (bat: batch entry of the launch)
+__device__ __forceinline__ double* task_out(const PlaneArgs& g, const GemmTask& t, int bat, int64_t& ldc) {
+    ldc = t.ldc;
+    if (t.split) {
+        ldc = t.n;
+        return g.split + (int64_t)bat * g.split_elems + g.split_tiles[t.split >> 9].off +
+               (int64_t)((t.split >> 5) & 15) * t.m * t.n;
+    }
+    return (g.to_y ? static_cast<double*>(const_cast<void*>(g.y.p[bat])) : g.C + (int64_t)(g.b0 + bat) * g.c_batch_elems) +
+           t.c_off;
+}
+
+// The outputs of a patch (rows x cols from row0, col0 of the tile; C: its first row, column col0 of the output)
+// that the digits do not resolve, computed in FP64: their bits in this lane's row.
+__device__ __forceinline__ uint32_t check_patch(const PlaneArgs& g, const GemmTask& t, int b, int row0, int col0, int rows,
+                                                int cols, double* C, int64_t ldc) {
+    if (t.seg_count == 0) return 0;
+    const int lane = threadIdx.x & 31;
+    const int64_t a_row = t.a_row + b * g.a_batch_rows, b_row = t.b_row + b * g.b_batch_rows;
+    rows = min(rows, 32);
+    const bool rowed = lane < rows, coled = lane < cols;
+    const int er = rowed ? g.ea[a_row + row0 + lane] : fx::E_ZERO;
+    const int ec = coled ? g.eb[b_row + col0 + lane] : fx::E_ZERO;
+    const uint2 rt = rowed ? g.ta[a_row + row0 + lane] : make_uint2(0, 0);
+    const uint2 ct = coled ? g.tb[b_row + col0 + lane] : make_uint2(0, 0);
+    auto patch = [&](int seg_begin, int seg_count) {
+        return PlaneSrc{g.segs + seg_begin, seg_count, rowed, coled, g.A + (a_row + row0) * g.ld,
+                        g.B + (b_row + col0) * g.ld, g.ld, g.za + a_row + row0 + lane, g.zb + b_row + col0 + lane,
+                        g.a_rows, g.b_rows, C + (int64_t)lane * ldc};
+    };
+    const PlaneSrc src = patch(t.seg_begin, t.seg_count);
+    const uint32_t valid = 0xffffffffu >> (32 - cols);
+    const uint32_t bad_cols = __ballot_sync(0xffffffffu, ec < 0);
+    const bool any_bad = __any_sync(0xffffffffu, er < 0) || bad_cols;
+    const uint32_t mr = __reduce_max_sync(0xffffffffu, rt.y), mc = __reduce_max_sync(0xffffffffu, ct.y);
+    if (!any_bad && (mr <= 2 || mc <= 2)) {
+        if (mr <= 2) fx::sparse_outputs<true, 16>(src, rowed, cols);
+        else fx::sparse_outputs<false, 16>(src, rowed, cols);
+        return rowed ? valid : 0u;
+    }
+    const uint32_t fewest = __reduce_min_sync(0xffffffffu, min(rt.y - 1, ct.y - 1)) + 1;     // (zeros last)
+    const float least = fx::least_sum((float)fewest, __uint_as_float(__reduce_max_sync(0xffffffffu, rt.x)),
+                                      __uint_as_float(__reduce_max_sync(0xffffffffu, ct.x)));
+    // (a part of a split tile decides on the whole contraction, whose rows' scales it has)
+    const SplitTile* whole = t.split ? &g.split_tiles[t.split >> 9] : nullptr;
+    uint32_t need = fx::weak_outputs(whole ? patch(whole->seg_begin, whole->seg_count) : src, rows, cols,
+                                     __ballot_sync(0xffffffffu, rt.y != 0), __ballot_sync(0xffffffffu, ct.y != 0),
+                                     max(er, 0), max(ec, 0), least);
+    need = rowed ? (need | bad_cols | (er < 0 ? 0xffffffffu : 0u)) & valid : 0u;
+    if (__any_sync(0xffffffffu, need != 0)) fx::fp64_outputs(src, rowed, cols, need, any_bad);
+    return need;
+}
+
+// The same for all patches of a task and batch entry, a block each, a warp per patch.
+constexpr int WEAK_WARPS = 4;
+__global__ void __launch_bounds__(32 * WEAK_WARPS) weak_plane_kernel(const __grid_constant__ PlaneArgs g) {
+    const GemmTask t = g.tasks[blockIdx.x];
+    const int lane = threadIdx.x & 31, bat = blockIdx.y;
+    const int wpr = (t.n + 31) / 32, patches = (t.m + 31) / 32 * wpr;
+    int64_t ldc;
+    double* const C = task_out(g, t, bat, ldc);
+    uint32_t* const bits = g.fp64 + bat * g.fp64_words + g.fp64_at[blockIdx.x];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int p = threadIdx.x >> 5; p < patches; p += WEAK_WARPS) {
+        const int row0 = p / wpr * 32, col0 = p % wpr * 32;
+        const uint32_t need = check_patch(g, t, g.b0 + bat, row0, col0, t.m - row0, min(t.n - col0, 32),
+                                          C + (int64_t)row0 * ldc + col0, ldc);
+        if (lane < t.m - row0) bits[(row0 + lane) * wpr + col0 / 32] = need;
+    }
+}
+
+// CHECK: with the check in the drain warps; else weak_plane_kernel has run.
+template <bool CHECK>
 __global__ void __launch_bounds__(PTHREADS, 1) fx_plane_kernel(const __grid_constant__ PlaneArgs g) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -389,10 +521,26 @@ __global__ void __launch_bounds__(PTHREADS, 1) fx_plane_kernel(const __grid_cons
             const int row0 = 32 * (rep == 4 ? 0 : (rep == 2 ? q & 1 : q));            // this warp's rows
             const int wc = 32 / rep, colb = wc * (rep == 4 ? 2 * q + h : (rep == 2 ? 2 * (q >> 1) + h : h));   // and columns
             const int rows = t.m - row0 < 32 ? t.m - row0 : 32;                        // may be <= 0
+            int64_t ldc;
+            double* C = task_out(g, t, bat, ldc);
+            C += (int64_t)row0 * ldc;
+            const int ncols = t.n + t.n_zero;
             // scales of this lane's row and of this lane's column
-            const int er = lane < rows ? g.ea[a_row + row0 + lane] : 0;
-            const int ec = lane < wc && colb + lane < t.n ? g.eb[b_row + colb + lane] : 0;
-            const bool bad = __any_sync(0xffffffffu, er < 0 || ec < 0);
+            const int ncol = min(wc, t.n - colb);                                       // may be <= 0
+            const bool rowed = lane < rows && ncol > 0, coled = lane < ncol && rows > 0;
+            const int er = rowed ? g.ea[a_row + row0 + lane] : fx::E_ZERO;
+            const int ec = coled ? g.eb[b_row + colb + lane] : fx::E_ZERO;
+            // outputs that are there already (check_patch); `whole`: all of the patch, whose sums are left alone
+            double* const out = C + (int64_t)lane * ldc + colb;
+            const uint32_t valid = ncol > 0 ? 0xffffffffu >> (32 - ncol) : 0u;
+            uint32_t need = 0;
+            if (CHECK) {
+                if (rows > 0 && ncol > 0) need = check_patch(g, t, b, row0, colb, rows, ncol, C + colb, ldc);
+            } else if (rowed) {
+                need = g.fp64[bat * g.fp64_words + g.fp64_at[item / g.nbatch] + (row0 + lane) * ((t.n + 31) / 32) + colb / 32] >>
+                       (colb % 32) & valid;
+            }
+            const bool whole = __all_sync(0xffffffffu, !rowed || need == valid);
             uint32_t w0[32], w1[32], w2[32];
 #pragma unroll
             for (int c = 0; c < 32; ++c) { w0[c] = 0; w1[c] = 0; w2[c] = 0; }
@@ -403,7 +551,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) fx_plane_kernel(const __grid_cons
                 const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + colb;
 #pragma unroll
                 for (int c = 0; c < 32; c += 4) {
-                    if (c < wc && colb + c < n16 && rows > 0) {
+                    if (c < wc && colb + c < n16 && rows > 0 && !whole) {
                         uint32_t d[FD][4];
 #pragma unroll
                         for (int e = 0; e < FD; ++e) tmem_ld4(ta + e * n16 + c, d[e]);
@@ -430,70 +578,30 @@ __global__ void __launch_bounds__(PTHREADS, 1) fx_plane_kernel(const __grid_cons
             }
             if (!ok) break;
             if (rows <= 0) continue;
-            // where the tile's values go: T, y, or a split tile's part of its scratch
-            double* C;
-            int64_t ldc = t.ldc;
-            if (t.split) {
-                ldc = t.n;
-                C = g.split + (int64_t)bat * g.split_elems + g.split_tiles[t.split >> 9].off +
-                    (int64_t)((t.split >> 5) & 15) * t.m * t.n;
-            } else {
-                C = (g.to_y ? static_cast<double*>(const_cast<void*>(g.y.p[bat]))
-                            : g.C + (int64_t)b * g.c_batch_elems) + t.c_off;
-            }
-            C += (int64_t)row0 * ldc;
-            const int ncols = t.n + t.n_zero;
             // exponent codes of T: this lane's row, per 8 columns
             uint16_t* et = !g.to_y ? g.et + (t.c_off % t.ldc) / CODE_COLS * g.et_rows + t.c_off / t.ldc + row0 + lane +
                                          (int64_t)b * g.c_batch_rows : nullptr;
             // 8 columns at a time: FP64 values into the transpose, then row pieces of 64 bytes
-            auto put = [&](int col0, const double (&v)[8]) {
-                int code = 0;
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    code = max(code, code_of(v[c]));
-                    tr[lane * 9 + c] = v[c];
-                }
-                if (et && lane < rows) et[col0 / CODE_COLS * g.et_rows] = (uint16_t)code;
-                __syncwarp();
-                const int c = lane & 7;
-                if (col0 + c < ncols)
-                    for (int r = lane >> 3; r < rows; r += 4) C[(int64_t)r * ldc + col0 + c] = tr[r * 9 + c];
-                __syncwarp();
-            };
-            if (!bad) {
+            for (int c0 = 0; c0 < 32; c0 += 8) {
+                const int col0 = colb + c0;
+                if (c0 < wc && col0 < ncols) {
+                    int code = 0;
 #pragma unroll
-                for (int c0 = 0; c0 < 32; c0 += 8) {
-                    const int col0 = colb + c0;
-                    if (c0 < wc && col0 < ncols) {
-                        double v[8];
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const int e = __shfl_sync(0xffffffffu, ec, c0 + c);
-                            v[c] = col0 + c < t.n
-                                       ? fx::from_fixed(w2[c0 + c], w1[c0 + c], w0[c0 + c], er + e - 2112) : 0.0;
-                        }
-                        put(col0, v);
+                    for (int c = 0; c < 8; ++c) {
+                        const int e = __shfl_sync(0xffffffffu, ec, c0 + c);
+                        double v = 0.0;
+                        if ((need >> (c0 + c)) & 1u) v = out[c0 + c];
+                        else if (col0 + c < t.n) v = fx::from_fixed(w2[c0 + c], w1[c0 + c], w0[c0 + c], er + e - 2112);
+                        code = max(code, code_of(v));
+                        tr[lane * 9 + c] = v;
                     }
-                }
-            } else {
-                // a row or column that the scales do not hold: this warp's values in FP64, lane = row
-                for (int c0 = 0; c0 < wc; c0 += 8) {
-                    const int col0 = colb + c0;
-                    if (col0 >= ncols) break;
-                    double v[8] = {};
-                    const double* ap = g.A + (a_row + row0 + (lane < rows ? lane : 0)) * g.ld;
-                    const double* bp = g.B + b_row * g.ld;
-                    for (int s = 0; s < t.seg_count; ++s) {
-                        const KSeg sg = g.segs[t.seg_begin + s];
-                        for (int k = sg.k0; k < sg.k0 + sg.klen; ++k) {
-                            const double x = ap[k];
-#pragma unroll
-                            for (int c = 0; c < 8; ++c)
-                                if (col0 + c < t.n) v[c] = fma(x, bp[(int64_t)(col0 + c) * g.ld + k], v[c]);
-                        }
-                    }
-                    put(col0, v);
+                    if (et && lane < rows) et[col0 / CODE_COLS * g.et_rows] = (uint16_t)code;
+                    __syncwarp();
+                    const int c = lane & 7;
+                    if (col0 + c < ncols)
+                        for (int r = lane >> 3; r < rows; r += 4) C[(int64_t)r * ldc + col0 + c] = tr[r * 9 + c];
+                    __syncwarp();
                 }
             }
         }
@@ -551,6 +659,8 @@ int launch_digits(heff_plan* p, int array, void* ws, int nbatch, void* stream) {
     g.rows = o.rows;
     g.batch_rows = o.batch_rows;
     g.a_side = o.a_side;
+    g.nonzero = reinterpret_cast<uint32_t*>(w + o.off_nonzero);
+    g.total = reinterpret_cast<uint2*>(w + o.off_total);
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -568,11 +678,13 @@ int launch_digits(heff_plan* p, int array, void* ws, int nbatch, void* stream) {
 }
 
 int launch_fx_planes(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream) {
-    const GemmList& gl = which == 1 ? p->fx1 : p->fx2;
+    const GemmList& gl = which == 1 ? p->g1 : (p->kchunk ? p->sp2 : p->g2);
     if (gl.tasks.empty()) return HEFF_OK;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(fx_plane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
+        cudaError_t e = cudaFuncSetAttribute(fx_plane_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fx_plane_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
         if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
         attr = true;
     }
@@ -614,8 +726,15 @@ int launch_fx_planes(heff_plan* p, int which, void* ws, void* const* y, int nbat
     g.b_batch_rows = B.batch_rows;
     g.ea = reinterpret_cast<const int32_t*>(w + A.off_scale);
     g.eb = reinterpret_cast<const int32_t*>(w + B.off_scale);
+    g.za = reinterpret_cast<const uint32_t*>(w + A.off_nonzero);
+    g.zb = reinterpret_cast<const uint32_t*>(w + B.off_nonzero);
+    g.ta = reinterpret_cast<const uint2*>(w + A.off_total);
+    g.tb = reinterpret_cast<const uint2*>(w + B.off_total);
     g.A = reinterpret_cast<const double*>(w + A.off_src);
     g.B = reinterpret_cast<const double*>(w + B.off_src);
+    g.fp64 = reinterpret_cast<uint32_t*>(w + p->off_fp64);
+    g.fp64_at = gl.d_fp64_at;
+    g.fp64_words = gl.fp64_words();
     g.err = reinterpret_cast<int*>(w + p->off_flags);
     if (which == 1) {
         g.C = reinterpret_cast<double*>(w + T.off_src);
@@ -648,7 +767,19 @@ int launch_fx_planes(heff_plan* p, int which, void* ws, void* const* y, int nbat
         cfg.stream = static_cast<cudaStream_t>(stream);
         cfg.attrs = at;
         cfg.numAttrs = HEFF_PDL ? 1 : 0;
-        cudaError_t e = cudaLaunchKernelEx(&cfg, fx_plane_kernel, g);
+        // one tile a CTA: the check while its first loads arrive; more: in a launch of its own (m = 48, 10 Lanczos
+        // steps: 683 and 749 us; apply m = 1024: 539 and 457)
+        const bool inline_check = total <= nsm;
+        cudaError_t e = cudaSuccess;
+        if (!inline_check) {
+            cudaLaunchConfig_t weak = cfg;
+            weak.gridDim = dim3((unsigned)g.ntasks, (unsigned)g.nbatch);
+            weak.blockDim = dim3(32 * WEAK_WARPS);
+            weak.dynamicSmemBytes = 0;
+            e = cudaLaunchKernelEx(&weak, weak_plane_kernel, g);
+            count_launches(1);
+        }
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, inline_check ? fx_plane_kernel<true> : fx_plane_kernel<false>, g);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "fx_plane launch: %s", cudaGetErrorString(e));
         count_launches(1);

@@ -88,6 +88,7 @@ struct GemmTask {
 struct SplitTile {
     int64_t c_off, off;     // tile origin in y; the group's scratch (parts x m x n elements)
     int32_t ldc, m, n, parts;
+    int32_t seg_begin, seg_count;   // segments of the whole contraction
 };
 constexpr int SPLIT_MAX = 16;
 inline int32_t split_code(int group, int part, int parts) { return group << 9 | part << 5 | parts; }
@@ -105,19 +106,22 @@ struct BProd {
     int32_t K;
     int32_t c1, c2;
     int32_t ea, eb;         // FP64 lists: exponent codes of the A rows and of the B columns
+    int32_t za, zb, na, nb; // and words of nonzero elements, and rows of a view
 };
 struct BTile {
     int64_t c_off;
     int32_t ldc, m, n;
     int32_t prod_begin, prod_count;
     int32_t steps;          // FP64 lists: steps of 16 contraction elements, each product rounded up
+    int32_t fp64_at;        // FP64 lists: first word of the bits for outputs computed in FP64
 };
-// up to 32 rows of one operand view whose exponent codes an FP64 list needs
+// up to 32 rows of one operand view whose exponent codes and nonzero elements an FP64 list needs
 struct FxRows {
     int64_t off;
     int32_t rs, ks, rows, K;
     int32_t out;            // first code
     int32_t which;          // 0: A, 1: B
+    int32_t word, all;      // first word of nonzero elements, and rows of the view
 };
 // output tile of the FP64 products (fx_gemm.cu, fx_planes.cu)
 constexpr int FX_TILE_M = 128, FX_TILE_N = 64;
@@ -136,11 +140,16 @@ struct BList {
     std::vector<FxRows> rows;
     FxRows* d_rows = nullptr;
     uint16_t* d_codes = nullptr;
+    float* d_sums = nullptr;        // of a row's magnitudes, over its scale, rounded up
+    uint32_t* d_fp64 = nullptr;     // outputs computed in FP64: a word per row and 32 columns of a tile
+    int32_t nfp64 = 0;
     int* d_err = nullptr;      // a flag for launches that have none elsewhere, zero after the upload
-    int32_t ncodes = 0;
-    std::map<std::array<int64_t, 6>, int32_t> views;
+    uint32_t* d_words = nullptr;    // nonzero elements, [32 elements][row] of a view
+    int32_t ncodes = 0, nwords = 0;
+    struct View { int32_t code, word; };
+    std::map<std::array<int64_t, 6>, View> views;
     int num_sms = 0;
-    int32_t view_codes(int which, int64_t off, int32_t rs, int32_t ks, int32_t n, int32_t K);
+    View view(int which, int64_t off, int32_t rs, int32_t ks, int32_t n, int32_t K);
     // the output blocks as added (products given for the block origin), kept for re-tiling
     struct Block { int64_t c_off; int32_t ldc, m, n, prod_begin, prod_count; };
     std::vector<Block> blocks;
@@ -192,6 +201,14 @@ struct GemmList {
     std::vector<SplitTile> split;
     SplitTile* d_split = nullptr;
     int64_t split_elems = 0;
+    // FP64 lists: first word of each task's bits for outputs computed in FP64 (a word per row and 32 columns)
+    std::vector<int32_t> fp64_at;
+    int32_t* d_fp64_at = nullptr;
+    void count_fp64() {
+        fp64_at.assign(1, 0);
+        for (const GemmTask& t : tasks) fp64_at.push_back(fp64_at.back() + t.m * ((t.n + 31) / 32));
+    }
+    int64_t fp64_words() const { return fp64_at.empty() ? 0 : fp64_at.back(); }
     // host only, one entry per task: output left sector a' and the task's flop counts
     std::vector<int32_t> owner;
     std::vector<double> task_flops, task_useful;
@@ -219,7 +236,7 @@ struct FxOperand {
     int64_t ld = 0, rows = 0, batch_rows = 0;     // rows: of all batch entries; 0 batch_rows: shared by them
     bool a_side = false;
     int code_cols = KPAD;           // columns per exponent code
-    size_t off_src = 0, off_codes = 0, off_planes = 0, off_scale = 0;    // in the workspace
+    size_t off_src = 0, off_codes = 0, off_planes = 0, off_scale = 0, off_nonzero = 0, off_total = 0;    // in the workspace
     // rows [row0, row0 + n) over the given segments
     void add(int64_t row0, int n, const std::vector<KSeg>& s) {
         const int32_t sb = (int32_t)segs.size();
@@ -279,22 +296,21 @@ struct heff_plan {
     // the environment update's plan (env.cu): GEMM 1 contracts XT with LW into T, GEMM 2 XT with T;
     // there is no RW, and which = 1 mix tiles fill XT
     bool env = false;
-    heff::GemmList fx1, fx2;          // FP64 plans: the task lists that run (FX_TILE_M x FX_TILE_N tiles)
     // FP64 plans: exponent codes of the operand arrays, [column / KPAD][row], after the arrays and the
-    // flags (ws_min: the workspace up to here, when every tile runs in FP64 arithmetic)
+    // flags (ws_min: the workspace up to here, enough without digit planes)
     size_t off_ex = 0, off_elw = 0, off_et = 0, off_erw = 0, ws_min = 0;
     // split tiles of GEMM 2: chunk of the contraction (in KPAD units; 0: no limit) and their scratch in
     // the workspace (after ws_min too).
-    // sp2, sp2_alt: the N = 256 and N = 128 lists of GEMM 2 with their long tiles split (g2 and g2_alt
-    // describe them whole); an FP64 plan's fx2 is split itself
+    // sp2, sp2_alt: the N = 256 (FP64: FX_TILE_N) and N = 128 lists of GEMM 2 with their long tiles split (g2
+    // and g2_alt describe them whole)
     heff::GemmList sp2, sp2_alt;
     int kchunk = 0;
     size_t off_split = 0;
-    // FP64 plans: LW, XT, T, RW as digit planes, after ws_codes in the workspace (planes: whether they
-    // are there; ws_codes: its size without them), and their tensor maps for the last two workspaces
+    // FP64 plans: LW, XT, T, RW as digit planes, last in the workspace (planes_ok: whether it has them), and
+    // their tensor maps for the last two workspaces
     heff::FxOperand fxo[4];
     bool planes_ok = false;
-    size_t ws_codes = 0;
+    size_t off_fp64 = 0;
     void* fx_ws[2] = {nullptr, nullptr};
     int fx_next = 0;
     alignas(64) unsigned char fx_maps[2][4][4 * 128];
@@ -316,21 +332,20 @@ struct heff_plan {
 
 namespace heff {
 // launchers (apply.cu)
-// level: what an FP64 plan's call has in its workspace: 2 digit planes, 1 the operands' exponent codes, 0
-// the FP64 operands alone (every tile in FP64 arithmetic)
-int fx_level(const heff_plan* p, size_t ws_bytes);
-int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, int level, void* stream);
+// planes: an FP64 plan's call has the digit planes and the operands' exponent codes in its workspace; without
+// them its products run on the FP64 units
+bool has_planes(const heff_plan* p, size_t ws_bytes);
+int launch_pack_batch(heff_plan* p, const void* const* x, int nbatch, void* ws, bool planes, void* stream);
 int launch_mix(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R,
-               void* ws, int level, void* stream);
-int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, int level, void* stream);
+               void* ws, bool planes, void* stream);
+int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool planes, void* stream);
 int launch_digits(heff_plan* p, int array, void* ws, int nbatch, void* stream);
 int launch_fx_planes(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
-// workspace of the digit planes from `end` on (offsets set); returns the new end, or `end` when the
-// planes would pass FX_PLANES_MAX
-size_t plane_layout(heff_plan* p, size_t end);
+// workspace of the digit planes from `end` on, and of fp64_words words of bits for FP64 outputs (offsets set);
+// returns the new end, or `without` when the planes would pass FX_PLANES_MAX
+size_t plane_layout(heff_plan* p, size_t end, int64_t fp64_words, size_t without);
 // y's split tiles from their parts (batch entries [0, nbatch), scratch copies of split_elems)
 int launch_sum_parts(heff_plan* p, const GemmList& g, void* ws, void* const* y, int nbatch, void* stream);
-int launch_fx_matvec(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool codes, void* stream);
 // one apply in the first `bytes` of ws, which may hold less than ws_bytes but at least ws_min
 int apply_in(heff_plan* p, const void* L, const void* W1, const void* W2, const void* R, const void* x, void* y,
              void* ws, size_t bytes, void* stream);

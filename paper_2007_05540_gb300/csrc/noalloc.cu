@@ -45,8 +45,7 @@ extern "C" int heff_apply_noalloc(heff_plan* plan, const void* L, const void* W1
                                   const void* R, const void* x, void* y, void* stream) {
     heff::clear_error();
     if (!plan) return fail(HEFF_ERR_INVALID_ARG, "heff_apply_noalloc: null plan");
-    // an FP64 plan also fits without the room for its operands' exponent codes (it then runs every
-    // tile in FP64 arithmetic)
+    // an FP64 plan also fits without the room for its digit planes (its products then run on the FP64 units)
     const size_t need = plan->ws_min;
     if (need > (size_t)HEFF_NOALLOC_WORKSPACE_BYTES)
         return fail(HEFF_ERR_WORKSPACE,

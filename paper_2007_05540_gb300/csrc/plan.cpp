@@ -98,19 +98,22 @@ bool check_index(const IndexDesc& a, const IndexDesc& b, int flow_a) {
 
 }  // namespace
 
-size_t heff::plane_layout(heff_plan* p, size_t end) {
+size_t heff::plane_layout(heff_plan* p, size_t end, int64_t fp64_words, size_t without) {
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     size_t o = end;
     for (FxOperand& f : p->fxo) {
         f.off_planes = o; o = al(o + 16 * (size_t)f.ld * (size_t)f.rows);
         f.off_scale = o;  o = al(o + sizeof(int32_t) * (size_t)f.rows);
+        f.off_nonzero = o; o = al(o + 4 * (size_t)(f.ld / KPAD) * (size_t)f.rows);
+        f.off_total = o;  o = al(o + 8 * (size_t)f.rows);
     }
     // T's exponent codes, finer than those that fx_gemm.cu writes
     FxOperand& t = p->fxo[2];
     t.code_cols = FX_T_CODE_COLS;
     t.off_codes = o; o = al(o + sizeof(uint16_t) * (size_t)(t.ld / FX_T_CODE_COLS) * (size_t)t.rows);
+    p->off_fp64 = o; o = al(o + sizeof(uint32_t) * (size_t)fp64_words);
     p->planes_ok = o <= FX_PLANES_MAX;
-    return p->planes_ok ? o : end;
+    return p->planes_ok ? o : without;
 }
 
 // A list of few long tiles leaves SMs idle behind its longest one (GEMM 2 at m = 1024, k = 14: 130 tiles,
@@ -148,7 +151,7 @@ void heff::split_tasks(GemmList& G, int chunk) {
             continue;
         }
         const int group = (int)G.split.size();
-        G.split.push_back({k.c_off, G.split_elems, k.ldc, k.m, k.n, parts});
+        G.split.push_back({k.c_off, G.split_elems, k.ldc, k.m, k.n, parts, k.seg_begin, k.seg_count});
         G.split_elems += (int64_t)parts * k.m * k.n;
         int seg = 0, at = 0;                          // segment and columns of it used
         for (int part = 0; part < parts; ++part) {
@@ -738,9 +741,8 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
             for (size_t t = 0; t < G.tasks.size(); ++t) { G.flops += G.task_flops[t]; G.useful += G.task_useful[t]; }
         };
         const bool tc = opts->precision != HEFF_PREC_FP64;
-        if (!build_lists(tc ? 128 : 64, tc ? 256 : 64, P->g1, P->g2) ||
-            (tc ? !build_lists(128, 128, P->g1_alt, P->g2_alt)
-                : !build_lists(heff::FX_TILE_M, heff::FX_TILE_N, P->fx1, P->fx2))) {
+        if (!build_lists(tc ? 128 : heff::FX_TILE_M, tc ? 256 : heff::FX_TILE_N, P->g1, P->g2) ||
+            (tc && !build_lists(128, 128, P->g1_alt, P->g2_alt))) {
             delete P;
             return fail(HEFF_ERR_CHARGE_MISMATCH, "internal: y block missing");
         }
@@ -774,7 +776,7 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
             P->stats[16] = (int64_t)c1;
             P->stats[17] = (int64_t)c2;
         }
-        for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->fx1, &P->fx2}) keep_owned(*G, owned);
+        for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt}) keep_owned(*G, owned);
         // ---- merge classes (batched launches; defined in tc_gemm.cu): the narrowest slot that holds
         // the tile, so that as many batch entries as possible fill one tile; T's columns come in
         // blocks of 32
@@ -883,7 +885,7 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
         {
             // the TF32 split's own chunk is 512 elements (16 KPAD units)
             const bool tf32 = opts->precision == HEFF_PREC_TF32X3;
-            int chunk = heff::split_chunk(tc ? P->g2 : P->fx2, nsm, tc, tc ? 16 : 8);
+            int chunk = heff::split_chunk(P->g2, nsm, tc, tc ? 16 : 8);
             if (tf32 && chunk) chunk = std::max(16, std::min(chunk, 16));
             if (tf32 && chunk && P->g2.tasks.size()) {
                 int kmax = 0;
@@ -891,17 +893,12 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
                 if (kmax > 16 * heff::SPLIT_MAX) chunk = 0;
             }
             if (chunk) {
-                const heff::GemmList whole = P->fx2;
-                heff::GemmList* split[3] = {&P->sp2, &P->sp2_alt, &P->fx2};
-                if (tc) {
-                    P->sp2 = P->g2;
-                    P->sp2_alt = P->g2_alt;
-                }
+                P->sp2 = P->g2;
+                P->sp2_alt = P->g2_alt;
                 int64_t elems = 0;
-                for (int k = 0; k < 3; ++k) {
-                    if (tc == (k == 2)) continue;
-                    heff::split_tasks(*split[k], chunk);
-                    elems = std::max(elems, split[k]->split_elems);
+                for (heff::GemmList* G : {&P->sp2, &P->sp2_alt}) {
+                    heff::split_tasks(*G, chunk);
+                    elems = std::max(elems, G->split_elems);
                 }
                 // one scratch per batch entry where batched launches split too (FP64)
                 const size_t bytes = tc ? 4 * (size_t)elems : 8 * (size_t)opts->max_batch * (size_t)elems;
@@ -910,14 +907,13 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
                 if ((P->ws_min <= HEFF_NOALLOC_WORKSPACE_BYTES && end + bytes + 256 > HEFF_NOALLOC_WORKSPACE_BYTES) ||
                     bytes > end / 10 + ((size_t)1 << 20)) {
                     P->sp2 = P->sp2_alt = heff::GemmList{};
-                    P->fx2 = whole;
                 } else {
                     P->kchunk = chunk;
                     P->off_split = end;
                     end = (end + bytes + 255) / 256 * 256;
                 }
             }
-            P->ws_codes = P->ws_bytes = end;
+            P->ws_bytes = end;
         }
         if (!tc) {
             // operand units for the digit planes
@@ -965,14 +961,25 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
                 f.off_src = ops[o].src;
                 f.off_codes = ops[o].codes;
             }
-            P->ws_bytes = heff::plane_layout(P, P->ws_codes);
+            // bits for outputs computed in FP64, of the batch entries of a launch (GEMM 1's, then GEMM 2's)
+            int64_t words = 0;
+            for (heff::GemmList* G : {&P->g1, &P->g2, &P->sp2}) {
+                G->count_fp64();
+                words = std::max(words, G->fp64_words());
+            }
+            words *= std::min<int64_t>(opts->max_batch, heff::MAXB);
+            P->ws_bytes = heff::plane_layout(P, P->ws_bytes, words, P->ws_min);
+            if (!P->planes_ok) {
+                P->kchunk = 0;
+                P->sp2 = heff::GemmList{};
+            }
         }
         if (HEFF_LPT_SCHEDULE) {
             for (heff::GemmList* G : {&P->g1, &P->g2, &P->g1_alt, &P->g2_alt, &P->g1_pair, &P->g2_pair, &P->sp2,
-                                      &P->sp2_alt, &P->fx1, &P->fx2}) {
-                if (!tc && (G == &P->g1 || G == &P->g2)) continue;    // 64 x 64 tiles: only described, not run
+                                      &P->sp2_alt}) {
                 const bool first = G == &P->g1 || G == &P->g1_alt || G == &P->g1_pair;
                 heff::lpt_schedule(*G, G->cl == 2 ? ncl : nsm, tc, first);
+                if (!tc) G->count_fp64();
             }
         }
         for (int i = 0; i < na; ++i) if (owned[i]) P->shard_sectors.push_back(i);

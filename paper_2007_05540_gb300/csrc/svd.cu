@@ -139,12 +139,19 @@ __global__ void svd_v_to_f64_kernel(const SvdSector* __restrict__ secs, const fl
         ws[s.v_off + e] = (double)f32[s.v32_off + e];
 }
 
-// Newton-Schulz combine: V = 1.5 V + W, with W = -0.5 V G already formed
+// G = V^T V - 1: what is left of the identity is all of one size (products with G itself would round to its ones)
+__global__ void svd_residual_kernel(const SvdSector* __restrict__ secs, double* __restrict__ ws) {
+    const SvdSector s = secs[blockIdx.y];
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < s.k; e += gridDim.x * blockDim.x)
+        ws[s.g_off + (int64_t)e * (s.k + 1)] -= 1.0;
+}
+
+// Newton-Schulz combine: V (3 - V^T V) / 2 = V + W, with W = -0.5 V (V^T V - 1) already formed
 __global__ void svd_ns_kernel(const SvdSector* __restrict__ secs, double* __restrict__ ws) {
     const SvdSector s = secs[blockIdx.y];
     const int64_t nv = (int64_t)s.k * s.k;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nv; e += (int64_t)gridDim.x * blockDim.x)
-        ws[s.v_off + e] = 1.5 * ws[s.v_off + e] + ws[s.w_off + e];
+        ws[s.v_off + e] += ws[s.w_off + e];
 }
 
 // J = W (the product J V)
@@ -1038,6 +1045,8 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
     heff::count_launches(1);
     for (int it = 0; it < 2; ++it) {
         if ((rc = heff::launch_bgemm(S->gram, ws, ws, ws, nullptr, nullptr, 1.0, stream, d_err))) return rc;
+        svd_residual_kernel<<<dim3(4, nsec), 256, 0, st>>>(S->d_sec, ws);
+        heff::count_launches(1);
         if ((rc = heff::launch_bgemm(S->vg, ws, ws, ws, nullptr, nullptr, -0.5, stream, d_err))) return rc;
         svd_ns_kernel<<<dim3(128, nsec), 256, 0, st>>>(S->d_sec, ws);
         heff::count_launches(1);

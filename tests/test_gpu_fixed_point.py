@@ -1,10 +1,9 @@
-"""FP64 block products as fixed-point digits on the tensor cores (csrc/fx_gemm.cu).
+"""FP64 products as fixed-point digits on the tensor cores (csrc/fx_gemm.cu, csrc/fx_planes.cu).
 
 One charge sector and one local state turn the two-site product x[a, b] = sum_c A[a, c] B[c, b]
-into a plain matrix product, so tile edges, contraction remainders and special values can be
-set directly.  Bound per element: the operands keep 61 bits below their row's (column's) largest
-element, the dropped digit products and the FP32 roundings of the low accumulators stay below
-2^-50 K of the two largest elements' product, and the sum is rounded to FP64 once.
+into a plain matrix product, and the matvec into y = L x R^T, so tile edges, contraction remainders
+and special values can be set directly.  The bound is that of a running FP64 sum, element by element:
+K 2^-53 sum |a||b|, whose factor is 1.2 where digits are used (csrc/fx_check.cuh), and one rounding.
 """
 import numpy as np
 import pytest
@@ -35,9 +34,8 @@ def _product(a, b):
     return out[32:32 + m * n].reshape(m, n)
 
 
-def _bound(a, b, c):
-    k = a.shape[1]
-    return 2.0 ** -50 * k * np.outer(np.abs(a).max(1), np.abs(b).max(0)) + 2.0 ** -52 * np.abs(c)
+def _bound(a, b):
+    return (1.2 * a.shape[1] + 2) * 2.0 ** -53 * (np.abs(a) @ np.abs(b))
 
 
 @pytest.mark.parametrize("m,k,n", [(1, 1, 1), (127, 15, 63), (128, 16, 64), (129, 17, 65), (5, 255, 16), (64, 256, 17),
@@ -57,7 +55,16 @@ def test_product_within_the_fixed_point_bound(m, k, n, fill):
         a[rng.integers(m)] = 0.0
     ref = np.asarray(a.astype(np.longdouble) @ b.astype(np.longdouble))
     got = _product(a, b)
-    assert (np.abs(got - ref) <= _bound(a, b, ref.astype(np.float64))).all()
+    assert (np.abs(got - ref) <= _bound(a, b)).all()
+
+
+@pytest.mark.parametrize("m,k,n", [(1, 1, 1), (127, 15, 63), (130, 96, 70), (33, 513, 48), (300, 1100, 140)])
+@pytest.mark.parametrize("fill", ["opposite", "gauge", "spike", "sparse", "mixed", "coherent"])
+def test_product_of_operands_whose_large_elements_do_not_meet(m, k, n, fill):
+    a, b = _operands(fill, m, k, n, np.random.default_rng([m, k, n]))
+    for u, v in ((a, b), (b.T, a.T)):
+        ref = u.astype(np.longdouble) @ v.astype(np.longdouble)
+        assert (np.abs(_product(u, v) - ref) <= _bound(u, v)).all()
 
 
 def test_integers_are_exact():
@@ -106,3 +113,67 @@ def test_matvec_is_homogeneous_over_the_exponent_range(power):
     heff.heff_apply(plan.handle, d["L"], d["W1"], d["W2"], d["R"], x * 2.0 ** power, ys, ws)
     assert heff.heff_workspace_status(plan.handle, ws) == 0
     assert float((ys * 2.0 ** -power - y).norm() / y.norm()) < 1e-14
+
+
+# ------------------------------------------------------------------ the matvec
+def _matvec(L, x, R):
+    """y = L x R^T by a plan with one sector, one local state and one MPO channel."""
+    import torch
+    from paper_2007_05540_gb300 import heff
+    m, n = x.shape
+    q, one = np.zeros((1, 1), dtype=np.int32), np.zeros((1, 1), dtype=np.int32)
+    lays = heff.heff_layouts((q, np.array([m], dtype=np.int32)), (q, np.array([n], dtype=np.int32)), one, q, q, q)
+    w = np.ones(1)
+    plan = heff.Plan(*lays, w, w, "fp64", "f64")
+    t = [torch.from_numpy(np.ascontiguousarray(v).reshape(-1)).cuda() for v in (L, w, w, R, x)]
+    y, ws = torch.full((m * n,), float("nan"), dtype=torch.float64, device="cuda"), plan.workspace()
+    heff.heff_apply(plan.handle, *t, y, ws)
+    assert heff.heff_workspace_status(plan.handle, ws) == 0
+    return y.cpu().numpy().reshape(m, n)
+
+
+def _operands(fill, m, k, n, rng):
+    """(m x k, k x n) whose large elements do not meet."""
+    a, b = rng.standard_normal((m, k)), rng.standard_normal((k, n))
+    if fill == "opposite":                    # a falls off along the contraction index, b rises
+        w = np.exp(-40.0 * np.arange(k) / k)
+        a, b = a * w, b / w[:, None]
+    elif fill == "gauge":                     # D and its inverse between the operands
+        d = 2.0 ** rng.integers(-40, 41, k)
+        a, b = a * d, b / d[:, None]
+    elif fill == "spike":                     # the row's largest element meets a zero
+        a[:, :-1] *= 1e-20
+        b[-1] = 0.0
+    elif fill == "sparse":                    # one element a row, graded columns
+        a = np.eye(m, k) * 2.0 ** rng.integers(-3, 4, (m, 1))
+        b = b * np.exp(-60.0 * rng.random((k, 1)))
+    elif fill == "mixed":                     # a few such rows and columns among others
+        a[::7] *= np.exp(-40.0 * np.arange(k) / k)
+        b[:, ::5] *= np.exp(40.0 * np.arange(k) / k)[:, None]
+    elif fill == "coherent":                  # low digits all alike below a single large element: the
+        v = (0x007f7f7f7f7f7f7f + 0.0) / 2.0 ** 62   # low accumulators pass 2^24
+        a, b = np.full((m, k), v), np.full((k, n), v)
+        a[:, 0], b[-1] = 0.9, 0.9
+    return a, b
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (17, 5), (33, 70), (64, 31), (130, 96), (300, 70), (520, 33)])
+@pytest.mark.parametrize("fill", ["opposite", "gauge", "spike", "sparse", "mixed", "coherent"])
+def test_matvec_within_the_bound_of_an_fp64_sum(m, n, fill):
+    rng = np.random.default_rng([m, n])
+    # both contractions: L x with R = 1, and x R^T with L = 1
+    L, x = _operands(fill, m, m, n, rng)
+    one = np.eye(n)
+    ld = lambda v: v.astype(np.longdouble)
+    err = np.abs(_matvec(L, x, one) - ld(L) @ ld(x))
+    assert (err <= _bound(L, x)).all()
+    x, rt = _operands(fill, n, m, m, rng)     # n x m by m x m
+    err = np.abs(_matvec(np.eye(n), x, np.ascontiguousarray(rt.T)) - ld(x) @ ld(rt))
+    assert (err <= _bound(x, rt)).all()
+
+
+def test_matvec_with_identities_is_exact():
+    rng = np.random.default_rng(8)
+    x = rng.standard_normal((210, 150)) * np.exp(-50.0 * rng.random((210, 150)))
+    x[rng.random(x.shape) < 0.2] = 0.0
+    assert (_matvec(np.eye(210), x, np.eye(150)) == x).all()

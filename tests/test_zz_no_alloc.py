@@ -29,9 +29,12 @@ TOL = {"fp64": 1e-10, "bf16x3": 1e-3, "tf32x3": 1e-5}
 
 
 def _setup(name, prec):
+    return _problem(wl.workload_by_name(name), prec)
+
+
+def _problem(w, prec):
     io = "f64" if prec == "fp64" else "f32"
     dt = torch.float64 if io == "f64" else torch.float32
-    w = wl.workload_by_name(name)
     lays, bufs = library_problem(w)
     Ll, W1l, W2l, Rl, xl = lays
     plan = heff.Plan(Ll, W1l, W2l, Rl, xl, bufs["W1"], bufs["W2"], prec, io)
@@ -60,6 +63,20 @@ def test_noalloc_matches_apply_on_two_calls(name, prec):
         assert not np.isnan(y).any()
         err = np.linalg.norm(y - ref) / np.linalg.norm(ref)
         assert err < TOL[prec], f"{name} {prec}: rel err {err:.3e}"
+
+
+def test_noalloc_fp64_without_room_for_digit_planes():
+    """An FP64 plan whose operands fit the built-in workspace and whose digit planes do not: its products
+    run on the FP64 units, to a running sum's accuracy."""
+    plan, d = _problem(wl.spin_heff_workload(512, 18, 0, name="spin_m512"), "fp64")
+    assert plan.workspace_bytes > heff.NOALLOC_WORKSPACE_BYTES
+    ws = plan.workspace()
+    ref, y = torch.full_like(d["x"], float("nan")), torch.full_like(d["x"], float("nan"))
+    heff.heff_apply(plan.handle, d["L"], d["W1"], d["W2"], d["R"], d["x"], ref, ws)
+    heff.heff_apply_noalloc(plan.handle, d["L"], d["W1"], d["W2"], d["R"], d["x"], y)
+    torch.cuda.synchronize()
+    assert heff.heff_apply_noalloc_status(plan.handle) == 0
+    assert float((y - ref).norm() / ref.norm()) < 1e-14
 
 
 def test_noalloc_rejects_plans_beyond_the_builtin_workspace():
