@@ -42,7 +42,7 @@ struct heff_env_plan {
     int64_t n_env = 0, n_site = 0;
     bool device = false;              // created with a CUDA device
     const void* last_ws = nullptr;    // workspace of the last update (its error flag is initialised)
-    // dense form: block-level tasks, cut into the precision's tiles when the plan is first used
+    // dense form: block-level tasks, and the tiles and device tables of the current precision
     bool dense = true;
     std::vector<GemmTask> blocks1, blocks2;
     std::vector<heff::KSeg> segs1, segs2;
@@ -261,15 +261,20 @@ size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
     return off;
 }
 
-// The device tables of the current precision.
-int ensure_plan(heff_env_plan* P) {
-    if (P->plan) return HEFF_OK;
+void free_plan(heff_env_plan* P) {
+    if (P->plan) heff::plan_free_device(P->plan.get());
+    P->plan.reset();
+}
+
+// The device tables of a precision, in the place of the plan's.  (At creation and when the precision is set: an
+// update neither allocates nor synchronises, and can be captured.)
+int build_plan(heff_env_plan* P, int precision) {
     int rc;
     try {
         std::unique_ptr<heff_plan> p(new heff_plan());
-        const bool tc = P->precision != HEFF_PREC_FP64;
+        const bool tc = precision != HEFF_PREC_FP64;
         p->env = true;
-        p->opts.precision = P->precision;
+        p->opts.precision = precision;
         p->opts.io_dtype = HEFF_DTYPE_F64;
         p->opts.max_batch = 1;
         p->planes = tc ? 2 : 1;
@@ -277,7 +282,7 @@ int ensure_plan(heff_env_plan* P) {
         p->nelem_x = P->n_site;
         p->rows_x = P->rows_sp; p->ld_x = P->ld; p->rows_lw = P->rows_lw;
         p->rows_t = P->rows_t; p->ld_t = P->ld; p->rows_rw = 0;
-        dense_bytes(P, P->precision, p.get());
+        dense_bytes(P, precision, p.get());
         if (!tc)
             for (const auto& u : P->units) p->fxo[std::get<0>(u)].add(std::get<1>(u), std::get<2>(u), std::get<3>(u));
         p->pack = P->pack;
@@ -318,16 +323,13 @@ int ensure_plan(heff_env_plan* P) {
             heff::plan_free_device(p.get());
             return rc;
         }
+        free_plan(P);
         P->plan = std::move(p);
+        P->precision = precision;
     } catch (const std::bad_alloc&) {
         return fail(HEFF_ERR_OOM, "out of host memory while planning the environment update");
     }
     return HEFF_OK;
-}
-
-void free_plan(heff_env_plan* P) {
-    if (P->plan) heff::plan_free_device(P->plan.get());
-    P->plan.reset();
 }
 
 }  // namespace
@@ -494,7 +496,12 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
     int ndev = 0;
     P->device = cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0;
     cudaGetLastError();
-    if (P->device && !P->dense) {
+    if (P->device && P->dense) {
+        if (const int rc = build_plan(P, P->precision)) {
+            delete P;
+            return rc;
+        }
+    } else if (P->device) {
         int rc;
         if ((rc = heff::blist_upload(P->step1)) || (rc = heff::blist_upload(P->step2))) {
             heff::blist_free(P->step1);
@@ -511,9 +518,7 @@ extern "C" int heff_env_workspace_size(const heff_env_plan* plan, size_t* bytes)
     heff::clear_error();
     if (!plan || !bytes) return fail(HEFF_ERR_INVALID_ARG, "heff_env_workspace_size: null argument");
     *bytes = plan->ws_bytes;
-    // the caller allocates now and updates next: build the device tables of the current precision
-    // here, so that an update neither allocates nor synchronises (stream capture)
-    return plan->dense && plan->device ? ensure_plan(const_cast<heff_env_plan*>(plan)) : HEFF_OK;
+    return HEFF_OK;
 }
 
 extern "C" int heff_env_flops(const heff_env_plan* plan, double* flops) {
@@ -535,7 +540,6 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
     char* ws = static_cast<char*>(workspace);
     int rc;
     if (plan->dense) {
-        if ((rc = ensure_plan(plan))) return rc;
         heff_plan* p = plan->plan.get();
         cudaError_t ez = cudaMemsetAsync(ws + p->off_flags, 0, sizeof(int), static_cast<cudaStream_t>(stream));
         if (ez != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(ez));
@@ -578,7 +582,7 @@ extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precisio
         return fail(HEFF_ERR_UNSUPPORTED, "environment updates run in HEFF_PREC_FP64 or HEFF_PREC_BF16X3");
     if (precision == plan->precision) return HEFF_OK;
     if (plan->dense) {
-        free_plan(plan);
+        if (plan->device) return build_plan(plan, precision);
         plan->precision = precision;
         return HEFF_OK;
     }

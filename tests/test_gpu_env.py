@@ -115,3 +115,31 @@ def test_env_update_precision_switch_back_to_fp64_is_exact():
             heff.heff_env_plan_set_precision(plan, "tf32x3")
     finally:
         heff.heff_env_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "bf16x3"])
+def test_env_update_captured_right_after_the_precision_is_set(prec):
+    """create, workspace size, set_precision, update: the update allocates and synchronises nothing, so it can
+    be the first thing that a graph captures."""
+    old_l, site_l, W_l, new_l, bufs, ref = _env_case("spin_m64", "left", 70, 9)
+    t = [_dev(bufs[k]) for k in ("old", "site", "W")]
+    make = lambda: heff.heff_env_plan_create(old_l.handle, site_l.handle, W_l.handle, new_l.handle, bufs["W"], "left")
+    new = lambda: torch.full((new_l.nelem,), float("nan"), dtype=torch.float64, device="cuda")
+    first, plan = make(), make()
+    try:
+        ws = torch.empty(heff.heff_env_workspace_size(plan), dtype=torch.uint8, device="cuda")
+        want, got = new(), new()
+        heff.heff_env_plan_set_precision(first, prec)
+        heff.heff_env_update(first, *t, want, ws)                   # (the kernels are loaded)
+        heff.heff_env_plan_set_precision(plan, "bf16x3" if prec == "fp64" else "fp64")
+        torch.cuda.synchronize()
+        heff.heff_env_plan_set_precision(plan, prec)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            heff.heff_env_update(plan, *t, got, ws)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
+    finally:
+        heff.heff_env_plan_destroy(first)
+        heff.heff_env_plan_destroy(plan)
