@@ -656,6 +656,15 @@ static bool launch_mix_pack(heff_plan* p, const void* L, const void* W1, const v
     return true;
 }
 
+int raise_smem_limit(PerDevice& done, const void* kernel, int bytes) {
+    int device = -1;
+    CK(cudaGetDevice(&device));
+    return once_per_device(done, device, [&]() -> int {
+        CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        return HEFF_OK;
+    });
+}
+
 int launch_tc_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
 
 int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool planes, void* stream) {

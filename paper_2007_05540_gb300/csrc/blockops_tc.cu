@@ -273,12 +273,8 @@ __global__ void __launch_bounds__(256) convert_f64_f32_kernel(const double* __re
 template <typename TC>
 int launch_t(const BList& b, const float* A, const float* B, void* C, const double* coef1, const double* coef2,
              double scale, cudaStream_t st, const double* inv_scale, int* err) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(bgemm_tc_kernel<TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, BT_SMEM);
-        if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        attr = true;
-    }
+    static PerDevice done;
+    if (int rc = raise_smem_limit(done, (const void*)bgemm_tc_kernel<TC>, BT_SMEM)) return rc;
     BtArgs g{b.d_tiles, b.d_prods, A, B, C, coef1, coef2, scale, inv_scale, b.accumulate ? 1 : 0, err};
     bgemm_tc_kernel<TC><<<(unsigned)b.tiles.size(), BT_THREADS, BT_SMEM, st>>>(g);
     return HEFF_OK;

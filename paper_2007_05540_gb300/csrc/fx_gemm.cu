@@ -783,12 +783,8 @@ __global__ void __launch_bounds__(256) row_code_kernel(const FxRows* __restrict_
 }
 
 int launch_fx(const FxArgs& g, int num_sms, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(fx_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
-        if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        attr = true;
-    }
+    static PerDevice done;
+    if (int rc = raise_smem_limit(done, (const void*)fx_gemm_kernel, FSMEM)) return rc;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -680,24 +680,19 @@ int launch_digits(heff_plan* p, int array, void* ws, int nbatch, void* stream) {
 int launch_fx_planes(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream) {
     const GemmList& gl = which == 1 ? p->g1 : (p->kchunk ? p->sp2 : p->g2);
     if (gl.tasks.empty()) return HEFF_OK;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(fx_plane_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fx_plane_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
-        if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        attr = true;
-    }
+    static PerDevice done[2];
+    int rc = raise_smem_limit(done[0], (const void*)fx_plane_kernel<false>, PSMEM);
+    if (!rc) rc = raise_smem_limit(done[1], (const void*)fx_plane_kernel<true>, PSMEM);
+    if (rc) return rc;
     char* w = static_cast<char*>(ws);
     // operand arrays: LW, XT (the environment update's site tensor), T, RW
     const int ia = p->env ? 1 : (which == 1 ? 0 : 2), ib = p->env ? (which == 1 ? 0 : 2) : (which == 1 ? 1 : 3);
     const FxOperand &A = p->fxo[ia], &B = p->fxo[ib], &T = p->fxo[2];
     if (which == 2) {
-        int rc = launch_digits(p, 2, ws, nbatch, stream);
+        rc = launch_digits(p, 2, ws, nbatch, stream);
         if (rc) return rc;
     }
     PlaneArgs g{};
-    int rc = HEFF_OK;
     // the workspace's tensor maps: encoded once, kept for the last two workspaces
     int slot = p->fx_ws[0] == ws ? 0 : (p->fx_ws[1] == ws ? 1 : -1);
     if (slot < 0) {

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/heff.h"
+#include "per_device.h"
 
 namespace heff {
 
@@ -331,6 +332,8 @@ struct heff_plan {
 };
 
 namespace heff {
+// A kernel's dynamic shared memory limit on the current device (done: the kernel's marks); apply.cu
+int raise_smem_limit(PerDevice& done, const void* kernel, int bytes);
 // launchers (apply.cu)
 // planes: an FP64 plan's call has the digit planes and the operands' exponent codes in its workspace; without
 // them its products run on the FP64 units

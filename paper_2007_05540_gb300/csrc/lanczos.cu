@@ -764,17 +764,11 @@ int lanczos_core(heff_plan* plan, const double* x0, int32_t n_iter, double* x_ou
     const size_t smem = a.w_shared ? (size_t)a.chunk * sizeof(double) : 0;
     const bool wide = a.chunk >= LT_WIDE;
     const unsigned threads = wide ? LTL : LTS;
-    static bool attr = false;
-    cudaError_t e = cudaSuccess;
-    if (!attr) {
-        e = cudaFuncSetAttribute(lz_step_kernel<LTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 LW_MAX * (int)sizeof(double));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(lz_step_kernel<LTL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     LW_MAX * (int)sizeof(double));
-        attr = e == cudaSuccess;
-    }
-    if (e == cudaSuccess) e = cudaMemsetAsync(z.bar, 0, 3 * sizeof(unsigned int), st);
+    static PerDevice done[2];
+    if (int rc = raise_smem_limit(done[wide], wide ? (const void*)lz_step_kernel<LTL> : (const void*)lz_step_kernel<LTS>,
+                                  LW_MAX * (int)sizeof(double)))
+        return rc;
+    cudaError_t e = cudaMemsetAsync(z.bar, 0, 3 * sizeof(unsigned int), st);
     void* args[] = {&a};
     auto launch = [&](const void* kernel, size_t bytes) {
         if (e == cudaSuccess)

@@ -37,6 +37,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <type_traits>
 
@@ -857,15 +858,18 @@ struct TcKernel {
     using S = Smem<TN_TC / CL, STAGES, SWZ_TC>;
     static constexpr auto kern = tc_gemm_kernel<PREC, TN_TC, STAGES, SWZ_TC, CL, MG>;
 
-    // shared-memory opt-in (once) and, for pairs, the clusters that fit on the device at once
+    // shared-memory opt-in and, for pairs, the clusters that fit on the device at once (both once per device)
     static int setup(int num_sms, int* clusters) {
-        static bool done = false;
-        static int ncl = 0;
-        if (!done) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL);
-            if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-            ncl = num_sms / CL;
-            if (CL > 1) {
+        static PerDevice done;
+        static std::atomic<int> fit[64];
+        if (int rc = raise_smem_limit(done, (const void*)kern, S::TOTAL)) return rc;
+        int device = -1, ncl = num_sms / CL;
+        cudaGetDevice(&device);
+        const bool known = device >= 0 && device < 64;
+        if (CL > 1) {
+            if (known && fit[device].load()) {
+                ncl = fit[device].load();
+            } else {
                 cudaLaunchConfig_t cfg{};
                 cudaLaunchAttribute at[1];
                 at[0].id = cudaLaunchAttributeClusterDimension;
@@ -878,8 +882,8 @@ struct TcKernel {
                 int n = 0;
                 if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0 && n < ncl) ncl = n;
                 cudaGetLastError();
+                if (known) fit[device].store(ncl);
             }
-            done = true;
         }
         if (clusters) *clusters = ncl;
         return HEFF_OK;
