@@ -347,8 +347,9 @@ int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precision);
 
 /*
  * Read and clear the sticky error flag of an environment-update workspace: HEFF_ERR_TIMEOUT
- * when a bounded wait of a tensor-core product expired in the last update (its output is
- * then incomplete; the context stays usable), else HEFF_OK.
+ * when a bounded wait of a tensor-core product expired in the last update there (its output is
+ * then incomplete; the context stays usable), whatever other workspaces and precisions the plan
+ * has been used with since, else HEFF_OK (also when no update has run in the workspace).
  * Synchronises `stream`.  Errors: INVALID_ARG, WORKSPACE, CUDA.
  */
 int heff_env_status(const heff_env_plan* plan, void* workspace, size_t workspace_bytes, void* stream);
@@ -542,7 +543,7 @@ int heff_plan_timings(heff_plan* plan, float* ms);
  * tensor memory and returns, so its outputs are incomplete but the context stays usable.
  * A GEMM launch clears the flag when the workspace is not one of the last two the plan
  * used.  Synchronises `stream`.  Returns HEFF_ERR_TIMEOUT if the flag was set (and clears
- * it), else HEFF_OK (also, for an FP64 plan, when no apply has run in this workspace).
+ * it), else HEFF_OK (also when no apply has run in this workspace).
  * workspace: device, at least heff_plan_workspace_size bytes.  Errors: INVALID_ARG,
  * WORKSPACE (too small), CUDA.
  */

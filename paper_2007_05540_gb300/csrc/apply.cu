@@ -665,6 +665,25 @@ int raise_smem_limit(PerDevice& done, const void* kernel, int bytes) {
     });
 }
 
+constexpr int FLAG_CLEAR = 0x5a;                     // every byte of a clear flag
+int reset_flag(void* flag, void* stream) {
+    CK(cudaMemsetAsync(flag, FLAG_CLEAR, FLAG_BYTES, static_cast<cudaStream_t>(stream)));
+    return HEFF_OK;
+}
+
+int read_flag(void* flag, const char* what, void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    unsigned char b[FLAG_BYTES];
+    CK(cudaMemcpyAsync(b, flag, FLAG_BYTES, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    bool clear = true, ours = true;
+    for (size_t i = 0; i < FLAG_BYTES; ++i) (i < sizeof(int) ? clear : ours) &= b[i] == FLAG_CLEAR;
+    if (clear || !ours) return HEFF_OK;
+    if (int rc = reset_flag(flag, stream)) return rc;
+    CK(cudaStreamSynchronize(st));
+    return fail(HEFF_ERR_TIMEOUT, "a bounded device-side wait of %s expired", what);
+}
+
 int launch_tc_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, void* stream);
 
 int launch_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch, bool planes, void* stream) {
@@ -738,7 +757,7 @@ static int check_ws(const heff_plan* p, void* ws, size_t bytes) {
 // contents unknown); the split precisions do this when they encode the workspace's tensor maps
 static int fresh_workspace(heff_plan* p, void* ws, void* stream) {
     if (p->opts.precision != HEFF_PREC_FP64 || p->tmap_ws[0] == ws || p->tmap_ws[1] == ws) return HEFF_OK;
-    CK(cudaMemsetAsync(static_cast<char*>(ws) + p->off_flags, 0, sizeof(int), static_cast<cudaStream_t>(stream)));
+    if (int rc = heff::reset_flag(static_cast<char*>(ws) + p->off_flags, stream)) return rc;
     p->tmap_ws[p->tmap_next] = ws;
     p->tmap_next ^= 1;
     return HEFF_OK;

@@ -41,7 +41,6 @@ struct heff_env_plan {
     size_t ws_bytes = 0;              // covers both precisions
     int64_t n_env = 0, n_site = 0;
     bool device = false;              // created with a CUDA device
-    const void* last_ws = nullptr;    // workspace of the last update (its error flag is initialised)
     // dense form: block-level tasks, and the tiles and device tables of the current precision
     bool dense = true;
     std::vector<GemmTask> blocks1, blocks2;
@@ -223,14 +222,14 @@ size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     const bool tc = precision != HEFF_PREC_FP64;
     const size_t e = (size_t)(tc ? 4 : 8) * P->ld, kb = (size_t)(P->ld / KPAD) * sizeof(uint16_t);
-    size_t off = 0, o_sp, o_lw, o_t, o_f;
+    // the error flag comes first in every precision and form
+    size_t off = 256, o_sp, o_lw, o_t;
     o_sp = off; off = al(off + e * P->rows_sp);
     o_lw = off; off = al(off + e * P->rows_lw);
     o_t = off;  off = al(off + e * P->rows_t);
-    o_f = off;  off = al(off + 256);
     const size_t least = off;
     if (p) {
-        p->off_xt = o_sp; p->off_lw = o_lw; p->off_t = o_t; p->off_rw = o_t; p->off_flags = o_f;
+        p->off_xt = o_sp; p->off_lw = o_lw; p->off_t = o_t; p->off_rw = o_t; p->off_flags = 0;
         p->ws_min = off;
     }
     if (!tc) {
@@ -538,12 +537,10 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
         return fail(HEFF_ERR_WORKSPACE, "environment workspace of %zu bytes, needs %zu (256-byte aligned)",
                     workspace_bytes, plan->ws_bytes);
     char* ws = static_cast<char*>(workspace);
-    int rc;
+    int rc = heff::reset_flag(ws, stream);
+    if (rc) return rc;
     if (plan->dense) {
         heff_plan* p = plan->plan.get();
-        cudaError_t ez = cudaMemsetAsync(ws + p->off_flags, 0, sizeof(int), static_cast<cudaStream_t>(stream));
-        if (ez != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(ez));
-        plan->last_ws = workspace;
         const void* xs[1] = {site};
         void* ys[1] = {env_new};
         // the mix tiles read env_old as L with W as W1, and (side 1) the site tensor as R
@@ -557,9 +554,6 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
         return heff::launch_gemm(p, 2, ws, ys, 1, planes, stream);
     }
     int* err = reinterpret_cast<int*>(ws);
-    cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), static_cast<cudaStream_t>(stream));
-    if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-    plan->last_ws = workspace;
     if (plan->precision == HEFF_PREC_FP64) {
         double* X = reinterpret_cast<double*>(ws + plan->off_x);
         if ((rc = heff::launch_bgemm(plan->step1, env_old, site, X, nullptr, nullptr, 1.0, stream, err))) return rc;
@@ -605,20 +599,8 @@ extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precisio
 extern "C" int heff_env_status(const heff_env_plan* plan, void* workspace, size_t workspace_bytes, void* stream) {
     heff::clear_error();
     if (!plan || !workspace) return fail(HEFF_ERR_INVALID_ARG, "heff_env_status: null argument");
-    // the flag exists once an update has run in this workspace
-    if (workspace != plan->last_ws) return HEFF_OK;
-    if (workspace_bytes < plan->ws_bytes) return fail(HEFF_ERR_WORKSPACE, "heff_env_status: workspace too small");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (plan->dense && !plan->plan) return HEFF_OK;     // nothing has run since the precision was set
-    int* d = reinterpret_cast<int*>(static_cast<char*>(workspace) + (plan->dense ? plan->plan->off_flags : 0));
-    int flag = 0;
-    cudaError_t e = cudaMemcpyAsync(&flag, d, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess && flag) e = cudaMemsetAsync(d, 0, sizeof(int), st);
-    if (e == cudaSuccess && flag) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "heff_env_status: %s", cudaGetErrorString(e));
-    if (flag) return fail(HEFF_ERR_TIMEOUT, "a bounded device-side wait of the environment update expired");
-    return HEFF_OK;
+    if (workspace_bytes < heff::FLAG_BYTES) return fail(HEFF_ERR_WORKSPACE, "heff_env_status: workspace too small");
+    return heff::read_flag(workspace, "the environment update", stream);
 }
 
 extern "C" void heff_env_plan_destroy(heff_env_plan* plan) {

@@ -57,7 +57,6 @@ struct heff_grad_plan {
     int32_t *d_w12_off = nullptr, *d_w12_terms = nullptr;
     int32_t *d_dw1_off = nullptr, *d_dw1_terms = nullptr, *d_dw2_off = nullptr, *d_dw2_terms = nullptr;
     bool uploaded = false;
-    const void* last_ws = nullptr;    // workspace of the last call (its error flag is initialised)
 };
 
 namespace {
@@ -445,11 +444,9 @@ extern "C" int heff_backward(heff_grad_plan* g, heff_plan* plan, const double* L
     float* x32 = reinterpret_cast<float*>(ws + g->off_x32);
     float* L32 = reinterpret_cast<float*>(ws + g->off_L32);
     float* R32 = reinterpret_cast<float*>(ws + g->off_R32);
-    if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess)
-        return fail(HEFF_ERR_CUDA, "heff_backward: memset failed");
-    g->last_ws = grad_ws;
     // y = K x into dx (dx is overwritten by the gradient below)
-    int rc = heff_apply(plan, L, W1, W2, R, x, dx, apply_ws, apply_ws_bytes, stream);
+    int rc = heff::reset_flag(err, stream);
+    if (!rc) rc = heff_apply(plan, L, W1, W2, R, x, dx, apply_ws, apply_ws_bytes, stream);
     if (rc) return rc;
     const int nxd = (int)g->xdots.size();
     if ((rc = heff::launch_block_dots(g->d_xdots, nxd, g->d_xoff, x, x, sc + 0, 1, part, 1.0, stream))) return rc;
@@ -535,19 +532,12 @@ extern "C" int heff_grad_plan_set_precision(heff_grad_plan* g, int32_t precision
 extern "C" int heff_grad_status(const heff_grad_plan* g, void* grad_ws, size_t grad_ws_bytes, void* stream) {
     heff::clear_error();
     if (!g || !grad_ws) return fail(HEFF_ERR_INVALID_ARG, "heff_grad_status: null argument");
-    // an FP64 plan's flag exists once a call has run in this workspace
-    if (g->precision == HEFF_PREC_FP64 && grad_ws != g->last_ws) return HEFF_OK;
-    if (grad_ws_bytes < g->ws_bytes) return fail(HEFF_ERR_WORKSPACE, "heff_grad_status: workspace too small");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int* d = reinterpret_cast<int*>(static_cast<double*>(grad_ws) + g->off_flag);
-    int flag = 0;
-    cudaError_t e = cudaMemcpyAsync(&flag, d, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess && flag) e = cudaMemsetAsync(d, 0, sizeof(int), st);
-    if (e == cudaSuccess && flag) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "heff_grad_status: %s", cudaGetErrorString(e));
-    if (flag) return fail(HEFF_ERR_TIMEOUT, "a bounded device-side wait of the gradient products expired");
-    return HEFF_OK;
+    if (grad_ws_bytes < g->ws_bytes) {
+        // (no FP64 call can have run here)
+        if (g->precision == HEFF_PREC_FP64) return HEFF_OK;
+        return fail(HEFF_ERR_WORKSPACE, "heff_grad_status: workspace too small");
+    }
+    return heff::read_flag(static_cast<double*>(grad_ws) + g->off_flag, "the gradient products", stream);
 }
 
 extern "C" void heff_grad_plan_destroy(heff_grad_plan* g) {

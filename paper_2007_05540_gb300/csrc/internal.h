@@ -334,6 +334,12 @@ struct heff_plan {
 namespace heff {
 // A kernel's dynamic shared memory limit on the current device (done: the kernel's marks); apply.cu
 int raise_smem_limit(PerDevice& done, const void* kernel, int bytes);
+// The error flag of a workspace: an int that a kernel whose bounded wait expires sets to 1, before seven more that
+// show that the flag was ever initialised (a workspace is the caller's memory); apply.cu.
+constexpr size_t FLAG_BYTES = 32;
+int reset_flag(void* flag, void* stream);
+// HEFF_ERR_TIMEOUT where the flag is raised (cleared then), else HEFF_OK; synchronises
+int read_flag(void* flag, const char* what, void* stream);
 // launchers (apply.cu)
 // planes: an FP64 plan's call has the digit planes and the operands' exponent codes in its workspace; without
 // them its products run on the FP64 units
@@ -359,7 +365,7 @@ void split_tasks(GemmList& G, int chunk);
 // clusters of two tensor-core CTAs resident at once (tc_gemm.cu; num_sms / 2 without a device)
 int tc_pair_clusters(int num_sms, int precision);
 // one block waiting at the SVD sweeps' grid barrier set up for two (svd.cu; wait self-test)
-void svd_barrier_selftest(unsigned int* bar, int* err, void* stream);
+void svd_barrier_selftest(unsigned int* bar, int* flag, void* stream);
 int plan_upload(heff_plan* p);
 void plan_free_device(heff_plan* p);
 void record_phase(heff_plan* p, int k, void* stream);

@@ -62,10 +62,8 @@ extern "C" int heff_apply_noalloc(heff_plan* plan, const void* L, const void* W1
     void* ws = nullptr;
     int rc = static_workspace(dev, &ws);
     if (rc) return rc;
-    // the device error flag must start at zero; everything else is written before it is read
-    e = cudaMemsetAsync(static_cast<char*>(ws) + plan->off_flags, 0, 256,
-                        static_cast<cudaStream_t>(stream));
-    if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+    // the device error flag must start clear; everything else is written before it is read
+    if ((rc = heff::reset_flag(static_cast<char*>(ws) + plan->off_flags, stream))) return rc;
     if (plan->ws_bytes > (size_t)HEFF_NOALLOC_WORKSPACE_BYTES && plan->nelem_x > 0) {
         if (!L || !W1 || !W2 || !R || !x || !y) return fail(HEFF_ERR_INVALID_ARG, "heff_apply: null argument");
         if (x == y) return fail(HEFF_ERR_INVALID_ARG, "y must not alias x");

@@ -809,14 +809,16 @@ __global__ void svd_write_kernel(const SvdSector* __restrict__ secs, const Write
     }
 }
 
-// One block meets the sweeps' grid barrier set up for two blocks: its wait must give up,
-// set err and return.
-__global__ void barrier_selftest_kernel(unsigned int* bar, int* err) { grid_barrier(bar, 2u, err); }
+// One block meets the sweeps' grid barrier set up for two blocks (bar: counter, -, its error word): its wait must
+// give up, and the workspace's flag is raised.
+__global__ void barrier_selftest_kernel(unsigned int* bar, int* flag) {
+    if (!grid_barrier(bar, 2u, reinterpret_cast<int*>(bar + 2)) && threadIdx.x == 0) atomicExch(flag, 1);
+}
 
 }  // namespace
 
-void heff::svd_barrier_selftest(unsigned int* bar, int* err, void* stream) {
-    barrier_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(bar, err);
+void heff::svd_barrier_selftest(unsigned int* bar, int* flag, void* stream) {
+    barrier_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(bar, flag);
 }
 
 extern "C" int heff_svd_create(const heff_layout* x, heff_svd** out) {

@@ -934,8 +934,7 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
     CUtensorMap* m = reinterpret_cast<CUtensorMap*>(p->tmaps[slot]);
     if (fresh) {
         // a workspace new to the plan: clear its sticky error flag (caller memory, contents unknown)
-        cudaError_t ez = cudaMemsetAsync(w + p->off_flags, 0, sizeof(int), st);
-        if (ez != cudaSuccess) return fail(HEFF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(ez));
+        if (int rc = reset_flag(w + p->off_flags, st)) return rc;
         // Operand rows interleave the hi and lo halves by K block: 2 ld elements per row, boxes
         // of 128-byte rows (a K block of both halves).
         // [4 o + k]: array o (LW, XT, T, RW) in boxes of 32 << k rows;  [16] T store boxes: 32 rows
@@ -1109,8 +1108,9 @@ extern "C" int heff_wait_selftest(const heff_plan* plan, void* workspace, size_t
     cudaEvent_t ev[2] = {nullptr, nullptr};
     cudaError_t e = cudaEventCreate(&ev[0]);
     if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
-    // error flag at byte 0 of the flag area; the barrier's counter at 64
-    if (e == cudaSuccess) e = cudaMemsetAsync(f, 0, 128, st);
+    // error flag at byte 0 of the flag area; the barrier's words from 64 on
+    if (e == cudaSuccess) e = cudaMemsetAsync(f + 64, 0, 64, st);
+    if (e == cudaSuccess && reset_flag(f, stream)) e = cudaErrorUnknown;
     if (e == cudaSuccess) e = cudaEventRecord(ev[0], st);
     if (e == cudaSuccess) {
         if (kind == 0) mbar_wait_selftest_kernel<<<1, 32, 0, st>>>(err);
@@ -1133,19 +1133,10 @@ extern "C" int heff_workspace_status(const heff_plan* plan, void* workspace, siz
                                      void* stream) {
     using namespace heff;
     if (!plan || !workspace) return fail(HEFF_ERR_INVALID_ARG, "heff_workspace_status: null plan/workspace");
-    // an FP64 plan's flag exists once an apply has run in this workspace
-    if (plan->opts.precision == HEFF_PREC_FP64 && plan->tmap_ws[0] != workspace && plan->tmap_ws[1] != workspace)
-        return HEFF_OK;
-    if (workspace_bytes < plan->off_flags + 256)
+    if (workspace_bytes < plan->off_flags + 256) {
+        // (no apply of an FP64 plan can have run here, and none of its flags been raised)
+        if (plan->opts.precision == HEFF_PREC_FP64) return HEFF_OK;
         return fail(HEFF_ERR_WORKSPACE, "heff_workspace_status: workspace smaller than the plan's");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int* d = reinterpret_cast<int*>(static_cast<char*>(workspace) + plan->off_flags);
-    int flag = 0;
-    cudaError_t e = cudaMemcpyAsync(&flag, d, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess && flag) e = cudaMemsetAsync(d, 0, sizeof(int), st);
-    if (e == cudaSuccess && flag) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return fail(HEFF_ERR_CUDA, "heff_workspace_status: %s", cudaGetErrorString(e));
-    if (flag) return fail(HEFF_ERR_TIMEOUT, "a bounded device-side wait expired (flag %d)", flag);
-    return HEFF_OK;
+    }
+    return read_flag(static_cast<char*>(workspace) + plan->off_flags, "the apply", stream);
 }

@@ -51,3 +51,52 @@ def test_workspace_status_fp64_plan_has_no_waits():
     assert heff.heff_workspace_status(lib.plan.handle, lib.ws) == 0
     with pytest.raises(heff.HeffError):
         heff.heff_wait_selftest(lib.plan.handle, lib.ws, 0)
+
+
+def _raise_flag(ws):
+    """What an expired wait leaves: 1 in the flag, an int before 28 more bytes of its pattern."""
+    head = ws[:ws.numel() // 256 * 256].view(-1, 256)[:, :32]
+    at = (head == 0x5A).all(1).nonzero().flatten()
+    assert len(at) == 1
+    head[int(at[0]), :4] = torch.tensor([1, 0, 0, 0], dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("prec", ["fp64", "bf16x3"])
+def test_status_belongs_to_the_workspace(prec):
+    """Three workspaces of one plan in turn: an expired wait in the first is reported there, after the plan has
+    been used elsewhere; a workspace in which nothing has run has no flag."""
+    w = wl.workload_by_name("spin_m64")
+    lib = Lib(w, prec)
+    lib.apply()
+    _raise_flag(lib.ws)
+    first = lib.ws
+    for _ in range(2):
+        lib.ws = lib.plan.workspace().fill_(0xFF)
+        assert heff.heff_workspace_status(lib.plan.handle, lib.ws) == 0
+        lib.apply()
+        assert heff.heff_workspace_status(lib.plan.handle, lib.ws) == 0
+    assert heff.heff_workspace_status(lib.plan.handle, first) == HEFF_ERR_TIMEOUT
+    assert heff.heff_workspace_status(lib.plan.handle, first) == 0
+
+
+@pytest.mark.parametrize("prec", ["fp64", "bf16x3"])
+def test_environment_status_belongs_to_the_workspace(prec):
+    from tests.test_gpu_env import _dev, _env_case
+    old_l, site_l, W_l, new_l, bufs, _ = _env_case("spin_m64", "left", 70, 9)
+    t = [_dev(bufs[k]) for k in ("old", "site", "W")]
+    plan = heff.heff_env_plan_create(old_l.handle, site_l.handle, W_l.handle, new_l.handle, bufs["W"], "left")
+    try:
+        size = heff.heff_env_workspace_size(plan)
+        a, b = (torch.full((size,), 0xFF, dtype=torch.uint8, device="cuda") for _ in range(2))
+        out = torch.empty(new_l.nelem, dtype=torch.float64, device="cuda")
+        assert heff.heff_env_status(plan, a) == 0                # nothing has run there
+        heff.heff_env_plan_set_precision(plan, prec)
+        heff.heff_env_update(plan, *t, out, a)
+        _raise_flag(a)
+        heff.heff_env_update(plan, *t, out, b)
+        assert heff.heff_env_status(plan, b) == 0
+        heff.heff_env_plan_set_precision(plan, "bf16x3" if prec == "fp64" else "fp64")
+        assert heff.heff_env_status(plan, a) == HEFF_ERR_TIMEOUT
+        assert heff.heff_env_status(plan, a) == 0
+    finally:
+        heff.heff_env_plan_destroy(plan)
