@@ -499,6 +499,8 @@ int heff_apply_noalloc_status(const heff_plan* plan, void* stream);
  *                       on the even CTA's barrier, so B is read once per pair (no multicast
  *                       load is issued)
  * Results are bitwise identical across variants (a tile's K order does not depend on them).
+ * A batched apply whose vectors share tiles (blocks of at most half a tile) runs its own 128 x 256
+ * tiles whatever the variant; one whose blocks are wider runs the plan's.
  */
 #define HEFF_TILE_256 256
 #define HEFF_TILE_128 128

@@ -43,6 +43,7 @@
 
 #include "convert.cuh"
 #include "internal.h"
+#include "merge.h"
 #include "tc_ptx.cuh"
 
 // work order of batched launches: 1 = the batch entries of a task consecutively
@@ -97,22 +98,6 @@ struct TcMaps {
                         // of loads it issues: with one per entry a batch of 16 took 1296 us, with one
                         // for all entries 1187 (blocks of 10-60); lower boxes for the rows that are
                         // there, half the bytes, changed nothing.
-};
-
-// Merged items of a batched launch: the batch entries of one task that share a tile, entry e in
-// slot e.  Merge classes of a task:
-//   0     one entry per item
-//   1-3   GEMM 1: 2, 4 or 8 entries side by side in slots of 128, 64 or 32 columns (the tile's
-//         n fits);  GEMM 2: 2 or 4 entries in slots of 64 or 32 rows (its m fits)
-//   4, 5  GEMM 1, tiles of at most 64 x 64: 2 or 4 entries in slots of 64 or 32 rows of the
-//         transposed tile (A: the vectors, B: the LW rows).  A tile of few LW rows otherwise leaves
-//         all its epilogue to the two warps of its tensor-memory lanes
-// A launch may merge fewer entries than a class allows (its shift is lowered, its slots widen).
-constexpr int MERGE_CLASSES = 6;
-struct Merge {
-    long item0[MERGE_CLASSES + 1];       // first item of each class
-    int task0[MERGE_CLASSES];            // first task
-    int shift[MERGE_CLASSES];            // log2 of the entries per item
 };
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
@@ -890,30 +875,6 @@ struct TcKernel {
     }
 };
 
-// Items of a merged launch over nb batch entries, at most 2^cap entries each.
-Merge merge_items(const MergeList& ml, int nb, int cap) {
-    Merge mg{};
-    long items = 0;
-    for (int c = 0; c < MERGE_CLASSES; ++c) {
-        mg.item0[c] = items;
-        mg.task0[c] = ml.first[c];
-        mg.shift[c] = std::min(c < 4 ? c : c - 3, cap);
-        items += (long)(ml.first[c + 1] - ml.first[c]) * ((nb + (1 << mg.shift[c]) - 1) >> mg.shift[c]);
-    }
-    mg.item0[MERGE_CLASSES] = items;
-    return mg;
-}
-
-// log2 of the most entries per item of a batched launch (0: not merged).  A merged item does the work of up
-// to 2^class items in the time of about one (electron problem, m = 1000, blocks of 10-120, 16
-// vectors: GEMM 1 170k items of 1.0 us), so as many entries are merged as leave every SM two items.
-int merge_cap(const MergeList& ml, int nb, int num_sms) {
-    if (nb < 2 || !ml.d_tasks) return 0;
-    for (int cap = 3; cap >= 1; --cap)
-        if (merge_items(ml, nb, cap).item0[MERGE_CLASSES] >= 2L * num_sms) return cap;
-    return 0;
-}
-
 // merge: log2 of the most batch entries per item (MG, on the N = 256 tiles)
 template <int PREC, int TN_TC, int CL, bool MG = false>
 int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, cudaStream_t st, int merge = 0) {
@@ -1004,7 +965,7 @@ int launch_tc_t(heff_plan* p, int which, void* ws, void* const* y, int nbatch, c
         }
         long total = (long)(g.ntasks / CL) * nb;              // entries (tiles, or pairs of tiles)
         if (MG) {
-            g.mg = merge_items(ml, nb, merge);
+            g.mg = merge_items(ml.first, nb, merge);
             g.tasks = ml.d_tasks;
             total = g.mg.item0[MERGE_CLASSES];
         }
@@ -1049,8 +1010,9 @@ int launch_tc_gemm(heff_plan* p, int which, void* ws, void* const* y, int nbatch
     const bool wide = gl.tn == 256, pair = gl.cl == 2;
     // batched launches whose entries share tiles run the N = 256 tiles whatever variant is active
     // (every variant has the same contraction segments)
-    const int merge = merge_cap(which == 1 ? p->mg1 : p->mg2, nbatch < MAXB ? nbatch : MAXB,
-                                p->num_sms > 0 ? p->num_sms : 148);
+    const MergeList& ml = which == 1 ? p->mg1 : p->mg2;
+    const int merge = ml.d_tasks ? merge_cap(ml.first, nbatch < MAXB ? nbatch : MAXB, p->num_sms > 0 ? p->num_sms : 148)
+                                 : 0;
     if (merge)
         return p->opts.precision == HEFF_PREC_BF16X3
                    ? launch_tc_t<HEFF_PREC_BF16X3, 256, 1, true>(p, which, ws, y, nbatch, st, merge)
