@@ -360,7 +360,7 @@ int apply_in(heff_plan* p, const void* L, const void* W1, const void* W2, const 
              void* ws, size_t bytes, void* stream);
 void lpt_schedule(GemmList& G, int units, bool tc, bool first);
 // KPAD units per part of GEMM 2's contractions that balances the list over the units (0: as is)
-int split_chunk(const GemmList& G, int units, bool tc, int least);
+int split_chunk(const GemmList& G, int units, bool tc, int least, double uneven, int shortest);
 void split_tasks(GemmList& G, int chunk);
 // clusters of two tensor-core CTAs resident at once (tc_gemm.cu; num_sms / 2 without a device)
 int tc_pair_clusters(int num_sms, int precision);

@@ -119,8 +119,9 @@ size_t heff::plane_layout(heff_plan* p, size_t end, int64_t fp64_words, size_t w
 // A list of few long tiles leaves SMs idle behind its longest one (GEMM 2 at m = 1024, k = 14: 130 tiles,
 // the longest three times the average SM's work).  Such lists are cut along the contraction, at
 // multiples of one chunk for the whole plan, into parts of at most half the average SM's work:
-// shorter parts cost more in partial sums (each is written once and read once) than they balance.
-int heff::split_chunk(const GemmList& G, int units, bool tc, int least) {
+// shorter parts cost more in partial sums (each is written once and read once) than they balance.  uneven: longest
+// tile over the average SM's work from which a list is cut; shortest: contraction (KPAD units) that it has then.
+int heff::split_chunk(const GemmList& G, int units, bool tc, int least, double uneven, int shortest) {
     double total = 0, longest = 0;
     int kmax = 0, wmax = 1;
     for (const GemmTask& k : G.tasks) {
@@ -132,7 +133,7 @@ int heff::split_chunk(const GemmList& G, int units, bool tc, int least) {
         wmax = std::max(wmax, w);
     }
     const double avg = total / units;
-    if (longest <= 1.3 * avg || kmax <= least) return 0;
+    if (longest <= uneven * avg || kmax < shortest) return 0;
     int chunk = std::max(least, (int)(avg / 2 / wmax) - 4);
     chunk = std::max(chunk, (kmax + SPLIT_MAX - 1) / SPLIT_MAX);
     return chunk < kmax ? chunk : 0;
@@ -883,14 +884,25 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
         // ---- split contractions of GEMM 2 (single-CTA tiles; the accumulation chunks of every other
         // variant and of batched launches follow the same cuts, so that the sums' bits agree)
         {
-            // the TF32 split's own chunk is 512 elements (16 KPAD units)
-            const bool tf32 = opts->precision == HEFF_PREC_TF32X3;
-            int chunk = heff::split_chunk(P->g2, nsm, tc, tc ? 16 : 8);
-            if (tf32 && chunk) chunk = std::max(16, std::min(chunk, 16));
-            if (tf32 && chunk && P->g2.tasks.size()) {
+            // BF16x3: parts pay from twice the average SM's work on (apply with prepared operators, us whole and split:
+            // m = 2048, k = 14, 1.96 of the average 149 and 147, with FP64 tensors 173 and 157; m = 2558, k = 8, 1.54: 114
+            // and 126, 130 and 143), and with FP32 tensors not for 25 blocks or fewer (m = 1024, k = 5: 33.5 and 34.3).
+            // Plans for batches are not cut: their launches would follow the cuts in the additions to y alone
+            // (8 vectors, m = 1000, k = 14, FP64 tensors: 242 and 352).
+            // TF32x3, whose own chunk is 512 elements (16 KPAD units), has those additions anyway and gains from 1.5
+            // times the average on (m = 2558, k = 8: 263 and 219).
+            // FP64, where every part repeats the check of its outputs: from 26 blocks on (m = 512, k = 8, 24 blocks: 155
+            // and 162; k = 14, 48: 252 and 229), and not for batches either (3 vectors, m = 128, k = 14: 177 and 195).
+            const bool tf32 = opts->precision == HEFF_PREC_TF32X3, bf16 = tc && !tf32;
+            const int least = tc ? 16 : 8;
+            int chunk = 0;
+            if (tf32 || opts->max_batch == 1)
+                chunk = heff::split_chunk(P->g2, nsm, tc, least, bf16 ? 1.8 : 1.3,
+                                          !tc || (bf16 && opts->io_dtype == HEFF_DTYPE_F32) ? 26 : least + 1);
+            if (tf32 && chunk) {
                 int kmax = 0;
                 for (const auto& k : P->g2.tasks) kmax = std::max(kmax, k.ktotal / KPAD);
-                if (kmax > 16 * heff::SPLIT_MAX) chunk = 0;
+                chunk = kmax > 16 * heff::SPLIT_MAX ? 0 : 16;
             }
             if (chunk) {
                 P->sp2 = P->g2;
@@ -900,8 +912,7 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
                     heff::split_tasks(*G, chunk);
                     elems = std::max(elems, G->split_elems);
                 }
-                // one scratch per batch entry where batched launches split too (FP64)
-                const size_t bytes = tc ? 4 * (size_t)elems : 8 * (size_t)opts->max_batch * (size_t)elems;
+                const size_t bytes = (tc ? 4 : 8) * (size_t)elems;
                 // not at the price of the built-in workspace, which would otherwise hold the plan, nor of
                 // a tenth of the workspace
                 if ((P->ws_min <= HEFF_NOALLOC_WORKSPACE_BYTES && end + bytes + 256 > HEFF_NOALLOC_WORKSPACE_BYTES) ||

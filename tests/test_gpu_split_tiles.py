@@ -23,9 +23,10 @@ def _problem(name, prec, io, nb=1):
 
 @pytest.mark.parametrize("prec,io", [("bf16x3", "f32"), ("bf16x3", "f64"), ("tf32x3", "f32"), ("fp64", "f64")])
 @pytest.mark.parametrize("name", ["spin_m1024", "spin_m384"])
-def test_same_bits_on_every_route(name, prec, io):
+@pytest.mark.parametrize("nb", [1, 2])                # plans for batches are not cut (but TF32x3's)
+def test_same_bits_on_every_route(name, prec, io, nb):
     import torch
-    heff, plan, d, x, ws = _problem(name, prec, io, 2)
+    heff, plan, d, x, ws = _problem(name, prec, io, nb)
     y, z = torch.empty_like(x), torch.full_like(x, float("nan"))
     heff.heff_apply(plan.handle, *d, x, y, ws)
     assert heff.heff_workspace_status(plan.handle, ws) == 0
@@ -37,9 +38,9 @@ def test_same_bits_on_every_route(name, prec, io):
         z.fill_(float("nan"))
         heff.heff_apply(plan.handle, *d, x, z, ws)
         assert torch.equal(y, z), tiles
-    zs = [torch.full_like(x, float("nan")) for _ in range(2)]
-    heff.heff_apply_batched(plan.handle, *d, [x, x], zs, ws)
-    assert torch.equal(y, zs[0]) and torch.equal(y, zs[1])
+    zs = [torch.full_like(x, float("nan")) for _ in range(nb)]
+    heff.heff_apply_batched(plan.handle, *d, [x] * nb, zs, ws)
+    assert all(torch.equal(y, z) for z in zs)
     torch.cuda.synchronize()
     g = torch.cuda.CUDAGraph()
     with torch.cuda.graph(g):

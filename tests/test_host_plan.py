@@ -271,6 +271,22 @@ def test_pair_entries_share_b_rows_and_segments(name):
         assert real == sorted(key(t) for t in single if t["m"] > 0)
 
 
+@pytest.mark.parametrize("m,nsec,prec,io,batch,split", [
+    (1024, 30, "bf16x3", "f64", 1, True), (1024, 30, "tf32x3", "f32", 8, True),
+    (1024, 30, "bf16x3", "f64", 2, False),            # batches: only the additions would follow the cuts
+    (2558, 31, "bf16x3", "f32", 1, False)])           # 1.5 times the average SM's work: parts cost more
+def test_long_contractions_are_cut_where_it_pays(m, nsec, prec, io, batch, split):
+    """The scratch of GEMM 2's split tiles follows the operand arrays and the flags in the workspace."""
+    w = wl.spin_heff_workload(m, nsec, 0, name="cut")
+    lays = heff.heff_layouts((w.alpha_q, w.alpha_d), (w.beta_q, w.beta_d), w.phys, w.ql, w.qm, w.qr)
+    W1, W2 = lays[1].assemble(lambda k: w.W1[k]), lays[2].assemble(lambda k: w.W2[k])
+    P = heff.Plan(*lays, W1, W2, prec, io, batch)
+    st, e = P.stats, 4 if prec == "bf16x3" else 8
+    al = lambda v: (v + 255) // 256 * 256
+    whole = sum(al(e * int(n)) for n in (batch * st[8] * st[9], st[10] * st[9], batch * st[11] * st[12], st[13] * st[12])) + 256
+    assert (P.workspace_bytes > whole) == split and P.workspace_bytes >= whole
+
+
 def test_product_state_reaches_total_charge():
     from paper_2007_05540_gb300 import dmrg
     sp = wl.spin_phys()
