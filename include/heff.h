@@ -323,6 +323,11 @@ int heff_davidson(heff_plan* plan, const void* L, const void* W1, const void* W2
  * W_host: host copy of W in its layout; zero entries are dropped from the schedule.
  * heff_env_update: all tensors are device double buffers; env_new is overwritten;
  * workspace >= heff_env_workspace_size bytes, 256-byte aligned.  Asynchronous.
+ * heff_env_workspace_size: what the plan's present precision runs in at full speed.  With
+ * HEFF_PREC_FP64 two thirds of it hold the operands' digit planes (spin, k = 14: 294 MB in all at
+ * m = 1024, 4.4 GB at m = 4096), and it is enough for HEFF_PREC_BF16X3 as well.  The size
+ * with HEFF_PREC_BF16X3 (97 MB, 1.5 GB) is enough for an FP64 update too, which then runs
+ * without the planes on the FP64 units, more slowly.  Smaller ones fail with HEFF_ERR_WORKSPACE.
  */
 typedef struct heff_env_plan heff_env_plan;
 int heff_env_plan_create(const heff_layout* env_old, const heff_layout* site, const heff_layout* W,
@@ -338,10 +343,9 @@ void heff_env_plan_destroy(heff_env_plan* plan);
  * Arithmetic of the environment update's block products.  HEFF_PREC_FP64 (the default):
  * FP64 accuracy (as HEFF_PREC_FP64 above).  HEFF_PREC_BF16X3: on the tensor cores, each operand element split
  * into bf16 hi + lo and three products per K block, FP32 accumulation (about 1e-5 relative
- * per product); the tensors stay FP64 buffers (the update converts env_old and the site
- * tensor to FP32 copies in the workspace, whose size covers both precisions) and the call
- * sequence is unchanged.  Errors:
- * INVALID_ARG, UNSUPPORTED (another precision), CUDA.
+ * per product); the tensors stay FP64 buffers and the call sequence is unchanged.  The device
+ * tables of a precision are made here (a cudaMalloc and a copy), so that the update neither
+ * allocates nor synchronises.  Errors: INVALID_ARG, UNSUPPORTED (another precision), OOM, CUDA.
  */
 int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precision);
 

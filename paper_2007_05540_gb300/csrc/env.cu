@@ -13,7 +13,8 @@
 // same site block with up to k blocks that differ by a coefficient.
 //
 // An update whose dense operands would take more than ENV_DENSE_MAX bytes of workspace runs as lists of
-// block products instead (about a quarter of the memory; blockops.cu):
+// block products instead (blockops.cu; spin, k = 14, m = 4096: 290 MB, where the dense form takes 1.5 GB, and
+// 4.4 GB with the digit planes of FP64):
 //   X[(a', w), (s, b)]  = L[a', w, a] . A[a, s, b],   Lnew[c, v, d] = sum W A[a', t, c]^T . X     (left)
 //   Y[(b', v), (a, s)]  = R[b', v, b] . B[a, s, b]^T, Rnew[c, w, d] = sum W B[c, t, b'] . Y       (right)
 #include <cuda_runtime.h>
@@ -38,7 +39,9 @@ struct heff_env_plan {
     int side = 0;
     int precision = HEFF_PREC_FP64;   // of the block products
     double flops = 0;                 // of the list form (the block pairs of Algorithm 2)
-    size_t ws_bytes = 0;              // covers both precisions
+    // Workspace: what HEFF_PREC_FP64 runs in at full speed, and the least, in which both precisions run (FP64
+    // without digit planes, on the FP64 units: the planes are two thirds of it, and BF16x3 has no use for them).
+    size_t ws_bytes = 0, ws_least = 0;
     int64_t n_env = 0, n_site = 0;
     bool device = false;              // created with a CUDA device
     // dense form: block-level tasks, and the tiles and device tables of the current precision
@@ -217,8 +220,9 @@ void build_dense(heff_env_plan* P, const heff_layout* env_old, const heff_layout
     P->rows_t = std::max<int64_t>(t_rows, 1);
 }
 
-// Workspace of the dense form in a precision; with p, its offsets too.
-size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
+// Workspace of the dense form in a precision (FP64: with its digit planes, unless they are left out); with p, its
+// offsets too.
+size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p, bool digits = true) {
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     const bool tc = precision != HEFF_PREC_FP64;
     const size_t e = (size_t)(tc ? 4 : 8) * P->ld, kb = (size_t)(P->ld / KPAD) * sizeof(uint16_t);
@@ -232,7 +236,7 @@ size_t dense_bytes(const heff_env_plan* P, int precision, heff_plan* p) {
         p->off_xt = o_sp; p->off_lw = o_lw; p->off_t = o_t; p->off_rw = o_t; p->off_flags = 0;
         p->ws_min = off;
     }
-    if (!tc) {
+    if (!tc && digits) {
         size_t o_ex, o_elw, o_et;
         o_ex = off;  off = al(off + kb * P->rows_sp);
         o_elw = off; off = al(off + kb * P->rows_lw);
@@ -379,6 +383,7 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
         build_dense(P, env_old, site, env_new, sa, sp, sb, d, side == 0 ? kw : kv,
                     [&](int u, int t, int s, int n) { return side == 0 ? widx(u, t, s, n) : widx(n, t, s, u); });
         P->ws_bytes = dense_bytes(P, HEFF_PREC_FP64, nullptr);
+        P->ws_least = dense_bytes(P, HEFF_PREC_FP64, nullptr, false);
         P->dense = P->ws_bytes <= ENV_DENSE_MAX;
         if (!P->dense) {
         std::map<std::tuple<int, int, int, int>, int64_t> inter;   // intermediate blocks -> offset
@@ -486,7 +491,7 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
         P->off_env32 = P->off_x + al((size_t)ioff * sizeof(float));
         P->off_site32 = P->off_env32 + al((size_t)P->n_env * sizeof(float));
         const size_t tc_bytes = P->off_site32 + al((size_t)P->n_site * sizeof(float));
-        P->ws_bytes = std::max(fp64_bytes, tc_bytes);
+        P->ws_bytes = P->ws_least = std::max(fp64_bytes, tc_bytes);
         }
     } catch (const std::bad_alloc&) {
         delete P;
@@ -516,7 +521,7 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
 extern "C" int heff_env_workspace_size(const heff_env_plan* plan, size_t* bytes) {
     heff::clear_error();
     if (!plan || !bytes) return fail(HEFF_ERR_INVALID_ARG, "heff_env_workspace_size: null argument");
-    *bytes = plan->ws_bytes;
+    *bytes = plan->precision == HEFF_PREC_FP64 ? plan->ws_bytes : plan->ws_least;
     return HEFF_OK;
 }
 
@@ -533,9 +538,9 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
     if (!plan || !env_old || !site || !W || !env_new)
         return fail(HEFF_ERR_INVALID_ARG, "heff_env_update: null argument");
     if (!plan->device) return fail(HEFF_ERR_UNSUPPORTED, "env plan was created without a CUDA device");
-    if (!workspace || workspace_bytes < plan->ws_bytes || reinterpret_cast<uintptr_t>(workspace) % 256)
+    if (!workspace || workspace_bytes < plan->ws_least || reinterpret_cast<uintptr_t>(workspace) % 256)
         return fail(HEFF_ERR_WORKSPACE, "environment workspace of %zu bytes, needs %zu (256-byte aligned)",
-                    workspace_bytes, plan->ws_bytes);
+                    workspace_bytes, plan->ws_least);
     char* ws = static_cast<char*>(workspace);
     int rc = heff::reset_flag(ws, stream);
     if (rc) return rc;

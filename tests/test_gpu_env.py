@@ -143,3 +143,33 @@ def test_env_update_captured_right_after_the_precision_is_set(prec):
     finally:
         heff.heff_env_plan_destroy(first)
         heff.heff_env_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("side", ["left", "right"])
+@pytest.mark.parametrize("name,new_m,new_nsec", [("spin_m64", 70, 9), ("spin_m1024", 1100, 31)])
+def test_env_update_in_the_workspace_of_bf16x3(name, new_m, new_nsec, side):
+    """The size reported with BF16x3 serves an FP64 update too (on the FP64 units: no digit planes fit); with a
+    byte less both precisions refuse it."""
+    old_l, site_l, W_l, new_l, bufs, ref = _env_case(name, side, new_m, new_nsec)
+    t = [_dev(bufs[k]) for k in ("old", "site", "W")]
+    plan = heff.heff_env_plan_create(old_l.handle, site_l.handle, W_l.handle, new_l.handle, bufs["W"], side)
+    try:
+        full = heff.heff_env_workspace_size(plan)
+        heff.heff_env_plan_set_precision(plan, "bf16x3")
+        size = heff.heff_env_workspace_size(plan)
+        assert size < 0.4 * full
+        ws = torch.full((size,), 0xFF, dtype=torch.uint8, device="cuda")
+        for prec in ("bf16x3", "fp64"):
+            heff.heff_env_plan_set_precision(plan, prec)
+            out = torch.full((new_l.nelem,), float("nan"), dtype=torch.float64, device="cuda")
+            heff.heff_env_update(plan, *t, out, ws)
+            torch.cuda.synchronize()
+            assert heff.heff_env_status(plan, ws) == 0
+            y = out.cpu().numpy()
+            assert np.linalg.norm(y - ref) < TOL[prec] * np.linalg.norm(ref)
+            assert np.abs(y - ref).max() < 20 * TOL[prec] * np.abs(ref).max()
+            with pytest.raises(heff.HeffError) as e:
+                heff.heff_env_update(plan, *t, out, ws[:size - 1])
+            assert e.value.code == -7
+    finally:
+        heff.heff_env_plan_destroy(plan)

@@ -171,6 +171,26 @@ def test_block_product_precision_switch_keeps_the_work():
     heff.heff_env_plan_destroy(P)
 
 
+def test_environment_workspace_without_digits_is_for_both_precisions():
+    """The size with BF16x3 has no room for digit planes: FP64 operands alone, about a third of the size with FP64."""
+    w = wl.workload_by_name("spin_m1024")
+    ones = lambda n: np.ones(n, dtype=np.int32)
+    gq, gd = wl.binomial_sectors(1024, 31, 31, parity=0)
+    site = heff.Layout([(w.alpha_q, w.alpha_d, 1), (w.phys, ones(2), 1), (gq, gd, -1)])
+    Wl = heff.Layout([(w.ql, ones(len(w.ql)), 1), (w.phys, ones(2), 1), (w.phys, ones(2), -1),
+                      (w.qm, ones(len(w.qm)), -1)])
+    old = heff.Layout([(w.alpha_q, w.alpha_d, -1), (w.ql, ones(len(w.ql)), 1), (w.alpha_q, w.alpha_d, 1)])
+    new = heff.Layout([(gq, gd, -1), (w.qm, ones(len(w.qm)), 1), (gq, gd, 1)])
+    P = heff.heff_env_plan_create(old.handle, site.handle, Wl.handle, new.handle, Wl.assemble(lambda k: w.W1[k]),
+                                  "left")
+    full = heff.heff_env_workspace_size(P)
+    heff.heff_env_plan_set_precision(P, "bf16x3")
+    assert 0.3 * full < heff.heff_env_workspace_size(P) < 0.36 * full      # 8 of 8 + 16 + 1/8 bytes an element
+    heff.heff_env_plan_set_precision(P, "fp64")
+    assert heff.heff_env_workspace_size(P) == full
+    heff.heff_env_plan_destroy(P)
+
+
 def _row_block_mask(xl, sectors):
     """Flat mask of the y blocks whose left sector is in `sectors`."""
     mask = np.zeros(xl.nelem, dtype=bool)
