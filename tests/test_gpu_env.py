@@ -173,3 +173,52 @@ def test_env_update_in_the_workspace_of_bf16x3(name, new_m, new_nsec, side):
             assert e.value.code == -7
     finally:
         heff.heff_env_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("side", ["left", "right"])
+def test_env_update_past_the_dense_limit(side):
+    """An update whose dense operands would pass 64 GiB (264 new channels, each with a copy of the environment's
+    4097 rows) while its tensors are small: the block-product lists, in a few MB beside the FP32 copies."""
+    rng = np.random.default_rng(5)
+    ones = lambda n: np.ones(n, dtype=np.int32)
+    ph = np.array([[1], [-1]], dtype=np.int32)
+    old = np.array([[0], [2]], dtype=np.int32), np.array([4097, 35], dtype=np.int32)
+    new = np.array([[-1], [1], [3]], dtype=np.int32), np.array([5, 70, 9], dtype=np.int32)
+    one = np.zeros((1, 1), dtype=np.int32)
+    many = np.repeat(np.array([[0], [2], [-2]], dtype=np.int32), [260, 2, 2], axis=0)
+    (la, ra), (lc, rc) = ((old, new), (one, many)) if side == "left" else ((new, old), (many, one))
+    site_l = heff.Layout([(*la, 1), (ph, ones(2), 1), (*ra, -1)])
+    W_l = heff.Layout([(lc, ones(len(lc)), 1), (ph, ones(2), 1), (ph, ones(2), -1), (rc, ones(len(rc)), -1)])
+    old_l = heff.Layout([(*old, -1), (one, ones(1), 1), (*old, 1)])
+    new_l = heff.Layout([(*new, -1), (many, ones(len(many)), 1), (*new, 1)])
+    bufs = {k: rng.standard_normal(lay.nelem) for k, lay in (("site", site_l), ("W", W_l), ("old", old_l))}
+
+    ix = lambda b: Index(b[0], b[1])
+    views = lambda lay, k: lay.split(bufs[k])
+    W = np.zeros((len(lc), 2, 2, len(rc)))
+    for key, v in views(W_l, "W").items():
+        W[key] = v[0]
+    so, oo = views(site_l, "site"), views(old_l, "old")
+    site_o = BlockTensor.from_fill([ix(la), Index(ph, ones(2)), ix(ra)], (1, 1, -1), np.zeros(1), lambda k: so[k])
+    old_o = BlockTensor.from_fill([ix(old), mpo_index(one), ix(old)], (-1, 1, 1), np.zeros(1), lambda k: oo[k])
+    ref = (oenv.extend_left if side == "left" else oenv.extend_right)(old_o, site_o, W, many)
+    ref = new_l.assemble(lambda k: ref.blocks[k])
+
+    plan = heff.heff_env_plan_create(old_l.handle, site_l.handle, W_l.handle, new_l.handle, bufs["W"], side)
+    try:
+        t = [_dev(bufs[k]) for k in ("old", "site", "W")]
+        size = heff.heff_env_workspace_size(plan)
+        assert size < 1 << 28
+        ws = torch.full((size,), 0xFF, dtype=torch.uint8, device="cuda")
+        for prec in ("fp64", "bf16x3", "fp64"):
+            heff.heff_env_plan_set_precision(plan, prec)
+            assert heff.heff_env_workspace_size(plan) == size
+            out = torch.full((new_l.nelem,), float("nan"), dtype=torch.float64, device="cuda")
+            heff.heff_env_update(plan, *t, out, ws)
+            torch.cuda.synchronize()
+            assert heff.heff_env_status(plan, ws) == 0
+            y = out.cpu().numpy()
+            assert np.linalg.norm(y - ref) < TOL[prec] * np.linalg.norm(ref)
+            assert np.abs(y - ref).max() < 20 * TOL[prec] * np.abs(ref).max()
+    finally:
+        heff.heff_env_plan_destroy(plan)
