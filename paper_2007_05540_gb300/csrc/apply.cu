@@ -421,7 +421,7 @@ struct Arena {
 };
 }  // namespace
 
-int plan_upload(heff_plan* p) {
+int plan_upload(heff_plan* p) try {
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) {
         cudaGetLastError();          // no device: a host-only plan for inspection
@@ -454,6 +454,8 @@ int plan_upload(heff_plan* p) {
     if (int rc = a.upload(&p->d_tables)) return rc;
     p->uploaded = true;
     return HEFF_OK;
+} catch (const std::bad_alloc&) {      // (the callers are C entries)
+    return fail(HEFF_ERR_OOM, "out of host memory for the plan's tables");
 }
 
 void record_phase(heff_plan* p, int k, void* stream) {

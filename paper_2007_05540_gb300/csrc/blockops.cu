@@ -83,7 +83,7 @@ void BList::retile(int tm, int tn) {
                   std::vector<BProd>(bp.begin() + k.prod_begin, bp.begin() + k.prod_begin + k.prod_count));
 }
 
-int blist_upload(BList& b) {
+int blist_upload(BList& b) try {
     b.d_tables = nullptr;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -121,6 +121,8 @@ int blist_upload(BList& b) {
     b.d_sums = reinterpret_cast<float*>(d + os);
     b.d_fp64 = reinterpret_cast<uint32_t*>(d + of);
     return HEFF_OK;
+} catch (const std::bad_alloc&) {      // (the callers are C entries)
+    return fail(HEFF_ERR_OOM, "out of host memory for the block products' tables");
 }
 
 void blist_free(BList& b) {

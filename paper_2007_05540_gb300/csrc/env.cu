@@ -339,7 +339,7 @@ int build_plan(heff_env_plan* P, int precision) {
 
 extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layout* site, const heff_layout* W,
                                     const heff_layout* env_new, const double* W_host, int32_t side,
-                                    heff_env_plan** out) {
+                                    heff_env_plan** out) try {
     heff::clear_error();
     if (!env_old || !site || !W || !env_new || !W_host || !out || (side != 0 && side != 1))
         return fail(HEFF_ERR_INVALID_ARG, "heff_env_plan_create: bad arguments");
@@ -516,6 +516,8 @@ extern "C" int heff_env_plan_create(const heff_layout* env_old, const heff_layou
     }
     *out = P;
     return HEFF_OK;
+} catch (const std::bad_alloc&) {
+    return fail(HEFF_ERR_OOM, "out of host memory while checking the layouts of the environment update");
 }
 
 extern "C" int heff_env_workspace_size(const heff_env_plan* plan, size_t* bytes) {
@@ -574,7 +576,7 @@ extern "C" int heff_env_update(heff_env_plan* plan, const double* env_old, const
     return heff::launch_bgemm_tc(plan->step2, S32, X, env_new, true, W, nullptr, 1.0, stream, nullptr, err);
 }
 
-extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precision) {
+extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precision) try {
     heff::clear_error();
     if (!plan) return fail(HEFF_ERR_INVALID_ARG, "heff_env_plan_set_precision: null plan");
     if (precision != HEFF_PREC_FP64 && precision != HEFF_PREC_BF16X3)
@@ -599,6 +601,9 @@ extern "C" int heff_env_plan_set_precision(heff_env_plan* plan, int32_t precisio
         }
     }
     return HEFF_OK;
+} catch (const std::bad_alloc&) {      // (the lists are not whole)
+    plan->device = false;
+    return fail(HEFF_ERR_OOM, "out of host memory while planning the environment update");
 }
 
 extern "C" int heff_env_status(const heff_env_plan* plan, void* workspace, size_t workspace_bytes, void* stream) {
@@ -643,7 +648,7 @@ __global__ void __launch_bounds__(1024) two_site_check_kernel(int* __restrict__ 
 }  // namespace
 
 extern "C" int heff_two_site_create(const heff_layout* A, const heff_layout* B, const heff_layout* x,
-                                    heff_two_site** out) {
+                                    heff_two_site** out) try {
     heff::clear_error();
     if (!A || !B || !x || !out) return fail(HEFF_ERR_INVALID_ARG, "heff_two_site_create: null argument");
     *out = nullptr;
@@ -699,6 +704,8 @@ extern "C" int heff_two_site_create(const heff_layout* A, const heff_layout* B, 
     }
     *out = P;
     return HEFF_OK;
+} catch (const std::bad_alloc&) {
+    return fail(HEFF_ERR_OOM, "out of host memory while checking the layouts of the two-site tensor");
 }
 
 extern "C" int heff_two_site_apply(heff_two_site* P, const double* A, const double* B, double* x, void* stream) {

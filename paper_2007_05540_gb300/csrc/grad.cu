@@ -113,7 +113,7 @@ void free_all(heff_grad_plan* g) {
 
 extern "C" int heff_grad_plan_create(const heff_layout* L, const heff_layout* W1, const heff_layout* W2,
                                      const heff_layout* R, const heff_layout* x, const double* W1_host,
-                                     const double* W2_host, size_t ws_limit, heff_grad_plan** out) {
+                                     const double* W2_host, size_t ws_limit, heff_grad_plan** out) try {
     heff::clear_error();
     if (!L || !W1 || !W2 || !R || !x || !W1_host || !W2_host || !out)
         return fail(HEFF_ERR_INVALID_ARG, "heff_grad_plan_create: null argument");
@@ -405,6 +405,8 @@ extern "C" int heff_grad_plan_create(const heff_layout* L, const heff_layout* W1
     }
     *out = g;
     return HEFF_OK;
+} catch (const std::bad_alloc&) {
+    return fail(HEFF_ERR_OOM, "out of host memory while checking the layouts of the gradients");
 }
 
 extern "C" int heff_grad_chunks(const heff_grad_plan* g, int32_t* nchunks) {
@@ -509,7 +511,7 @@ extern "C" int heff_backward(heff_grad_plan* g, heff_plan* plan, const double* L
     return HEFF_OK;
 }
 
-extern "C" int heff_grad_plan_set_precision(heff_grad_plan* g, int32_t precision) {
+extern "C" int heff_grad_plan_set_precision(heff_grad_plan* g, int32_t precision) try {
     heff::clear_error();
     if (!g) return fail(HEFF_ERR_INVALID_ARG, "heff_grad_plan_set_precision: null plan");
     if (precision != HEFF_PREC_FP64 && precision != HEFF_PREC_BF16X3)
@@ -527,6 +529,9 @@ extern "C" int heff_grad_plan_set_precision(heff_grad_plan* g, int32_t precision
     g->ws_bytes = precision == HEFF_PREC_FP64 ? g->ws_bytes_fp64 : g->ws_bytes_tc;
     if (rc) g->uploaded = false;
     return rc;
+} catch (const std::bad_alloc&) {      // (the lists are not whole)
+    g->uploaded = false;
+    return fail(HEFF_ERR_OOM, "out of host memory while planning the gradients");
 }
 
 extern "C" int heff_grad_status(const heff_grad_plan* g, void* grad_ws, size_t grad_ws_bytes, void* stream) {

@@ -246,7 +246,7 @@ void heff::lpt_schedule(GemmList& G, int units, bool tc, bool first) {
 
 extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, const heff_layout* W2,
                                 const heff_layout* R, const heff_layout* x, const double* W1_host,
-                                const double* W2_host, const heff_plan_opts* opts, heff_plan** out) {
+                                const double* W2_host, const heff_plan_opts* opts, heff_plan** out) try {
     heff::clear_error();
     if (!L || !W1 || !W2 || !R || !x || !W1_host || !W2_host || !opts || !out)
         return fail(HEFF_ERR_INVALID_ARG, "heff_plan_create: null argument");
@@ -1018,6 +1018,8 @@ extern "C" int heff_plan_create(const heff_layout* L, const heff_layout* W1, con
     }
     *out = P;
     return HEFF_OK;
+} catch (const std::bad_alloc&) {
+    return fail(HEFF_ERR_OOM, "out of host memory while checking the layouts of the plan");
 }
 
 extern "C" int heff_plan_shard_sectors(const heff_plan* plan, int32_t* sectors, int32_t* count) {

@@ -950,7 +950,7 @@ extern "C" int heff_svd_workspace_size(const heff_svd* S, size_t* bytes) {
     } while (0)
 
 extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, size_t workspace_bytes,
-                                void* stream, int32_t* sweeps_out) {
+                                void* stream, int32_t* sweeps_out) try {
     heff::clear_error();
     if (!S || !x) return fail(HEFF_ERR_INVALID_ARG, "heff_svd_compute: null argument");
     if (!workspace || workspace_bytes < S->ws_bytes || reinterpret_cast<uintptr_t>(workspace) % 256)
@@ -1075,6 +1075,8 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
     S->computed = true;
     S->kept.clear();
     return HEFF_OK;
+} catch (const std::bad_alloc&) {
+    return fail(HEFF_ERR_OOM, "out of host memory in heff_svd_compute");
 }
 
 extern "C" int heff_svd_info(const heff_svd* S, int32_t* fp32_sweeps, int32_t* fp64_sweeps) {
