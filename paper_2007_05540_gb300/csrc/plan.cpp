@@ -107,7 +107,7 @@ size_t heff::plane_layout(heff_plan* p, size_t end, int64_t fp64_words, size_t w
         f.off_nonzero = o; o = al(o + 4 * (size_t)(f.ld / KPAD) * (size_t)f.rows);
         f.off_total = o;  o = al(o + 8 * (size_t)f.rows);
     }
-    // T's exponent codes, finer than those that fx_gemm.cu writes
+    // T's exponent codes: GEMM 1's epilogue writes one per FX_T_CODE_COLS columns, finer than the other operands'
     FxOperand& t = p->fxo[2];
     t.code_cols = FX_T_CODE_COLS;
     t.off_codes = o; o = al(o + sizeof(uint16_t) * (size_t)(t.ld / FX_T_CODE_COLS) * (size_t)t.rows);

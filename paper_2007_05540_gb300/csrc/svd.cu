@@ -65,8 +65,9 @@ struct heff_svd {
     std::vector<std::vector<int64_t>> xoff;    // per sector: x block offsets [row group][col group]
     std::vector<int32_t> mrows, ncols;         // M_Q shape
     int64_t ws_doubles = 0;
-    size_t off_slots = 0;                      // byte offset of the per-pair convergence slots
-    int64_t nslots = 0, slot_ld = 0;
+    // byte offset of the sweeps' words: convergence measures and counts (16), the sectors' pair offsets, the grid
+    // barrier and its error word (3), the sectors' block-pair offsets
+    size_t off_words = 0;
     size_t ws_bytes = 0;
     int64_t s_total = 0;
     std::vector<double> s;                     // singular values (per sector, unsorted)
@@ -91,8 +92,9 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// blocks per tensor block of the kernels that copy between the tensors and J, V (m = 512, 70 tensor blocks: one
-// each took 26 and 40 us)
+// Blocks per tensor block of the kernels that copy between the tensors and J, V: bound by latency, and a tensor of
+// few blocks leaves most SMs idle with one each (m = 512, 70 tensor blocks: 26 and 40 us).  Eight is from that size
+// alone.
 constexpr int COPY_SPLIT = 8;
 
 // scatter x blocks into column-major J (or J^T layout for wide sectors)
@@ -922,11 +924,8 @@ extern "C" int heff_svd_create(const heff_layout* x, heff_svd** out) {
         }
         S->xoff.assign(1, tab);   // stash the load table (one entry)
         S->ws_doubles = o + so + 64;
-        const int kk = S->max_k + (S->max_k & 1);
-        S->slot_ld = std::max(1, kk / 2);
-        S->nslots = (int64_t)nsec * S->slot_ld;
-        S->off_slots = ((size_t)S->ws_doubles * sizeof(double) + tab.size() * sizeof(int64_t) + 255) / 256 * 256;
-        S->off_f32 = (S->off_slots + (size_t)(S->nslots + 64 + 2 * nsec + 16) * sizeof(float) + 255) / 256 * 256;
+        S->off_words = ((size_t)S->ws_doubles * sizeof(double) + tab.size() * sizeof(int64_t) + 255) / 256 * 256;
+        S->off_f32 = (S->off_words + (size_t)(16 + 3 + 2 * (nsec + 1)) * sizeof(int) + 255) / 256 * 256;
         S->ws_bytes = S->off_f32 + (size_t)o32 * sizeof(float) + 1024;
     } catch (const std::bad_alloc&) {
         delete S;
@@ -958,8 +957,7 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     double* ws = static_cast<double*>(workspace);
     double* sv = ws + (S->ws_doubles - S->s_total - 64);
-    float* slots = reinterpret_cast<float*>(static_cast<char*>(workspace) + S->off_slots);
-    float* offmax = slots + S->nslots;
+    int* seen = reinterpret_cast<int*>(static_cast<char*>(workspace) + S->off_words);   // FP32 [0, 3), FP64 [3, 6); sweeps run [6, 8)
     const std::vector<int64_t>& tab = S->xoff[0];
     int64_t* d_tab = reinterpret_cast<int64_t*>(ws + S->ws_doubles);
     const int nsec = (int)S->sec.size();
@@ -984,13 +982,12 @@ extern "C" int heff_svd_compute(heff_svd* S, const double* x, void* workspace, s
         S->pair_off.push_back(0);
         for (const SvdSector& sc : S->sec) S->pair_off.push_back(S->pair_off.back() + (sc.k + (sc.k & 1)) / 2);
     }
-    int* d_pair_off = reinterpret_cast<int*>(slots + S->nslots + 16);
+    int* d_pair_off = seen + 16;
     unsigned int* d_bar = reinterpret_cast<unsigned int*>(d_pair_off + S->pair_off.size());
     int* d_err = reinterpret_cast<int*>(d_bar + 2);
     SVD_CK(cudaMemcpyAsync(d_pair_off, S->pair_off.data(), S->pair_off.size() * sizeof(int), cudaMemcpyHostToDevice,
                            st));
     SVD_CK(cudaMemsetAsync(d_bar, 0, 3 * sizeof(unsigned int), st));
-    int* seen = reinterpret_cast<int*>(slots + S->nslots);          // FP32 [0, 3), FP64 [3, 6); sweeps run [6, 8)
     SVD_CK(cudaMemsetAsync(seen, 0, 8 * sizeof(int), st));
     int dev = 0, nsm = 0;
     SVD_CK(cudaGetDevice(&dev));
