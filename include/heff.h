@@ -152,7 +152,12 @@ int heff_plan_check_mpo(const heff_plan* plan, const void* W1, const void* W2, v
  * increasing order; sectors may be NULL to query the count. */
 int heff_plan_shard_sectors(const heff_plan* plan, int32_t* sectors, int32_t* count);
 
-/* Workspace bytes needed by every call on this plan (for nbatch = max_batch). */
+/*
+ * Workspace bytes needed by every call on this plan (for nbatch = max_batch).  Of an FP64 plan's
+ * two thirds hold the operands' digit planes (spin, k = 14: 622 MB at m = 1024, 8.4 GB at m = 4096,
+ * where BF16x3 takes 107 MB and 1.4 GB); plans whose workspace would pass 64 GiB with them do
+ * without, and run on the FP64 units.
+ */
 int heff_plan_workspace_size(const heff_plan* plan, size_t* bytes);
 
 /*
@@ -472,7 +477,8 @@ void heff_svd_destroy(heff_svd* s);
  * into the library; every GPU that loads the library holds one copy until the process
  * exits.  Plans whose heff_plan_workspace_size exceeds that size are rejected with
  * HEFF_ERR_WORKSPACE (for example the m = 1024 spin problem in BF16x3 fits, m = 4096
- * does not).  The first call on a device resolves the array's device address
+ * does not), except FP64 plans that fit without their digit planes: those run on the FP64
+ * units.  The first call on a device resolves the array's device address
  * (cudaGetSymbolAddress) with that device current; make that first call before any
  * stream capture.  All calls share the array and it keeps the last call's contents, so
  * calls that overlap on the GPU (on different streams or from different threads) race

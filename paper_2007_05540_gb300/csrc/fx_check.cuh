@@ -15,8 +15,8 @@
 // outputs and leaves a bit for each, by which the product kernel keeps them.  It adds |a||b| itself, the
 // magnitudes as BF16 rounded down, on mma.sync, 16 contraction elements at a time, until every output has passed: one
 // to three steps for dense operands.  Bound by the latency of a step's loads and, for sparse rows, by the FP64 units.
-// What it costs: apply m = 1024, k = 14, 398 -> 464 us (15000 patches checked and 3000 sparse ones before GEMM 1, 31 us;
-// 4300 before GEMM 2, 39 us), environment update m = 1024 253 -> 314 us, Lanczos m = 48 62 -> 66 us a step.
+// What it costs: apply m = 1024, k = 14, 398 -> 466 us (15000 patches checked and 3000 sparse ones before GEMM 1, 31 us;
+// 4300 before GEMM 2, 41 us), environment update m = 1024 253 -> 315 us, Lanczos m = 48 62 -> 66 us a step.
 // Tried and left: the same in the warps that drain the digit sums (it is on the path of every tile there: GEMM 1
 // of the apply at m = 1024, k = 14, 163 -> 254 us); |a||b| by shuffles and multiply-adds (1000 instructions a step instead of
 // 180); bounds from minima and sums of 32 elements (a thirtieth of S on average).

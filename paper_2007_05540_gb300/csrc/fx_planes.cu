@@ -11,10 +11,10 @@
 //                    loads, one issuing MMAs, eight drain warps
 //   weak_plane_kernel  finds the outputs that digits do not resolve and computes them in FP64 (fx_check.cuh)
 // Prepared matvec, m = 1024, k = 14: 577 us with the conversion in every tile, 400 us here (GEMM 1 163, GEMM 2 124,
-// planes of T 45, of x 7) and 464 with the check; environment update m = 1024 309, 253 and 314 us.  Bound by the drain (74 us of GEMM 1's 163 go when it is
-// left out) and the loads' latency on contractions of two to ten K blocks; the MMAs are 45 us of it.  128 x 32
-// tiles with two accumulator sets drain under the next tile's MMAs, but read A twice as often: 151 and
-// 160 us.
+// planes of T 45, of x 7) and 466 with the check; environment update m = 1024 309, 253 and 315 us.  Bound by the
+// drain, in which the tensor pipe waits (active 27 % of GEMM 1's cycles and 25 % of the environment update's), and by the
+// loads' latency on contractions of two to ten K blocks.  128 x 32 tiles with two accumulator sets drain under the next
+// tile's MMAs, but read A twice as often: GEMM 1 164, GEMM 2 217 us.
 // The planes take 16 bytes per operand element: plans whose workspace would pass FX_PLANES_MAX and calls on a
 // smaller workspace (heff_apply_noalloc) run on the FP64 units (apply.cu).
 //
